@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cstdint>
+#include <vector>
 
 namespace gw {
 
@@ -150,6 +151,20 @@ template <typename T>
 void launch_fallback_finish64(const double* B_nm, int n_bas, int n_aux, const int* rt, const int* rm, const int* idx,
                               int nf, const double* y64, double* w_re, double* w_im, double* resnorm, T* V,
                               cudaStream_t s, double* V64 = nullptr);
+
+// Nodes of the imaginary-axis stage (freq_nodes.cu): the positions at which it is computed and the matrix that gives
+// every grid column of W from them.
+struct FreqNodes {
+  std::vector<int> col;       // W column per position: position 0 is the static point (column n_g), then grid columns
+  int n_diff = 0;             // positions 1 .. n_diff hold W_g - W_0 (difference form)
+  std::vector<double> C;      // [positions][n_g]: W[r][g] = sum_p C[p][g] value_p
+};
+// Nodes for the ascending positive grid xi whose first n_diff points are difference columns, for poles in
+// [D_min, inf); false where the nodes would save less than a quarter of the n_g + 1 points or the grid is not
+// ascending and positive (the stage then runs at every point).
+bool freq_nodes(const std::vector<double>& xi, int n_diff, double D_min, FreqNodes& out);
+// Every grid column of W [R][n_g + 1] from the node columns (col, C: device copies of FreqNodes).
+cudaError_t launch_w_expand(double* W, long R, int n_g, int n_pos, const int* col, const double* C, cudaStream_t s);
 
 // R term reduction per target over its right-hand sides [start[t], start[t+1]).
 // W[r][g] += W[r][n_g] for g < n_cols (table [R][n_g + 1]): columns held as differences from the static one.

@@ -85,7 +85,11 @@ struct gw_plan {
   std::vector<double> sh_buf;
   int ns_iters_last = 0;
   int ns_kmax = 0;
-  int ns_ndiff = 0;           // lowest grid points whose W column is built in the difference form
+  int ns_ndiff = 0;           // positions 1 .. ns_ndiff of the imaginary-axis stage are difference columns
+  gw::FreqNodes nodes;        // mixed: grid points the stage is computed at, for the smallest pair energy nodes_D
+  double nodes_D = -1.0;
+  bool nodes_ok = false;
+  DevBuf sk_C;                // device copy of nodes.C
   std::vector<DevBuf*> bufs;
   int tc_tiles_n = 0;          // N_aux the tile-order table of the Pi kernel was built for
   DevBuf ws_mat, ws_info, ws_scratch, ws_gout, ws_xi, tc_part, tc_kind, tc_par, tc_err, tc_w, tc_tiles, ns_E, ns_X, ns_X2, ns_Xa, ns_Xb, ns_T, ns_lam,
@@ -106,7 +110,7 @@ struct gw_plan {
   std::vector<Mark> marks;
 
   gw_plan() {
-    DevBuf* all[] = {&ws_mat, &ws_info, &ws_scratch, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &mr_V, &mr_U, &mr_S, &mr_vprev,
+    DevBuf* all[] = {&ws_mat, &ws_info, &ws_scratch, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
                      &mr_v, &mr_d1, &mr_d2, &mr_x, &mr_st, &mr_rt, &mr_rm, &mr_xf, &mr_wre, &mr_wim,
                      &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
                      &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_lu, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS};
@@ -270,7 +274,8 @@ gw_status tc_weighted_syrk(gw_plan* P, const int* kinds, const double* params, i
 // Newton-Schulz X <- 2X - (X eps) X from the closed-form first iterate 2a I - a^2 eps (a = 2/(1 + lambda_max)),
 // converging quadratically because the spectrum of eps lies in [1, lambda_max]; the last iterate is written as
 // eps^-1 - 1, and W[r][g] = b_r^T (eps_g^-1 - 1) b_r is reduced straight out of one more GEMM.
-gw_status ns_w_table(gw_plan* P, int g0, int nc) {
+// Positions [g0, g0 + nc) of the stage, at the frequencies xi_pos[0 .. nc).
+gw_status ns_w_table(gw_plan* P, int g0, int nc, const double* xi_pos) {
   const int n = P->cfg.n_aux, ldn = gw::tc_ld(n);
   const int R = P->n_t * P->n_bas, n_g1 = P->n_g + 1;
   const size_t mat = (size_t)n * n, smat = (size_t)n * ldn, sz = smat * nc;
@@ -411,7 +416,7 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc) {
     }
     b0 = 1;
   }
-  // positions [b0, b1) of this chunk are difference columns (position p > 0 holds grid point p - 1)
+  // positions [b0, b1) of this chunk are difference columns
   const int b1 = std::max(b0, std::min(nc, P->ns_ndiff + 1 - g0));
   const size_t t1 = tick(P);
   if (b0 > 0) CK(wred(Xs[cur], 1, g0));
@@ -423,7 +428,7 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc) {
     const gw::TcOperand E0{{e0, e0 + smat, e0 + 2 * smat}};
     std::vector<int> kinds(nb, 4);
     std::vector<double> xis(nb);
-    for (int b = 0; b < nb; ++b) xis[b] = P->h_xi[g0 + b0 + b - 1];
+    for (int b = 0; b < nb; ++b) xis[b] = xi_pos[b0 + b];
     // M_b in FP32 (ws_mat: eps is no longer needed) and split (ns_E)
     float* Mf = as<float>(P->ws_mat);
     TRY(tc_weighted_syrk(P, kinds.data(), xis.data(), nb, 0, 0, Mf, 0, /*reset_err=*/false));
@@ -483,6 +488,11 @@ gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
   const int n_g1 = P->n_g + 1;
   const int R = P->n_t * P->n_bas;
   const bool use_tc = (P->cfg.precision == GW_PREC_MIXED);
+  // difference-form columns: grid points with xi_g below a tenth of the smallest pair energy (there
+  // |Pi(i xi_g) - Pi(0)| <= 1% of |Pi(0)|)
+  int n_diff = 0;
+  if (use_tc)
+    while (n_diff < P->n_g && P->h_xi[n_diff] < 0.1 * P->D_min) ++n_diff;
   // frequency matrices held at once: <= 8 GiB (and the split-operand budget on the tensor-core path)
   const size_t per = (size_t)n * n * sizeof(T);
   int chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_g1, ws_bytes(P) / per));
@@ -490,29 +500,50 @@ gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
     const size_t per_ns = (size_t)n * gw::tc_ld(n) * 24 + (size_t)n * n * 8;   // split E, Xa, Xb, T; FP32 X, eps
     chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)chunk, ws_bytes(P) / per_ns));
   }
+  // mixed precision, one rank: the stage runs at the nodes of the grid (FreqNodes, 35 to 40 of 129 points) and the
+  // other columns follow from them; the nodes' 1e-8 is far below the BF16-part products' error.  FP64 plans, sharded
+  // plans (each rank owns a block of columns) and plans that the caller gave room for fewer than three matrices run at
+  // every grid point, so the chunked form of that path stays in use at sizes that can be checked; so do plans of one
+  // 128-row tile a matrix, whose 129 points are one wave and cost less than the search for the nodes (a (H2O)_1 job
+  // took 4.68 ms with nodes, 4.48 without; a (H2O)_3 one 4.6 with, 6.8 without).
+  const bool use_nodes = use_tc && n > 128 && P->sh_world == 1 && !(P->cfg.workspace_mb > 0 && chunk < 3);
+  if (use_nodes && P->nodes_D != P->D_min) {
+    P->nodes_D = -1.0;
+    P->nodes_ok = gw::freq_nodes(P->h_xi, n_diff, P->D_min, P->nodes);
+    if (P->nodes_ok) {
+      TRY(ensure(P, P->sk_C, sizeof(double) * P->nodes.C.size()));
+      CK(cudaMemcpyAsync(P->sk_C.p, P->nodes.C.data(), sizeof(double) * P->nodes.C.size(), cudaMemcpyHostToDevice,
+                         P->stream));
+    }
+    P->nodes_D = P->D_min;
+  }
+  const bool nodes = use_nodes && P->nodes_ok;
+  P->ns_ndiff = nodes ? P->nodes.n_diff : n_diff;
+  // processing order: the static point xi = 0 first, then the grid ascending; gout maps position -> W column
+  std::vector<int> gout;
+  if (nodes) {
+    gout = P->nodes.col;
+  } else {
+    gout.resize(n_g1);
+    gout[0] = P->n_g;
+    for (int g = 0; g < P->n_g; ++g) gout[g + 1] = g;
+  }
+  const int n_pos = (int)gout.size();
+  chunk = std::min(chunk, n_pos);
   TRY(ensure(P, P->ws_mat, per * chunk));
   TRY(ensure(P, P->ws_info, sizeof(int) * chunk));
-  TRY(ensure(P, P->ws_gout, sizeof(int) * n_g1));
+  TRY(ensure(P, P->ws_gout, sizeof(int) * n_pos));
   const int n_cta = gw::trsm_w_default_ctas();
-  TRY(ensure(P, P->ws_scratch, sizeof(T) * gw::trsm_w_scratch_elems<T>(n, n_cta)));
-  // processing order: the static point xi = 0 first, then the grid ascending; gout maps position -> W column
-  std::vector<int> gout(n_g1);
-  gout[0] = P->n_g;
-  for (int g = 0; g < P->n_g; ++g) gout[g + 1] = g;
-  CK(cudaMemcpyAsync(P->ws_gout.p, gout.data(), sizeof(int) * n_g1, cudaMemcpyHostToDevice, P->stream));
-  std::vector<double> xi_all(n_g1);
-  for (int i = 0; i < n_g1; ++i) xi_all[i] = gout[i] < P->n_g ? P->h_xi[gout[i]] : 0.0;
-  TRY(ensure(P, P->ws_xi, sizeof(double) * n_g1));
-  CK(cudaMemcpyAsync(P->ws_xi.p, xi_all.data(), sizeof(double) * n_g1, cudaMemcpyHostToDevice, P->stream));
+  if (!use_tc) TRY(ensure(P, P->ws_scratch, sizeof(T) * gw::trsm_w_scratch_elems<T>(n, n_cta)));
+  CK(cudaMemcpyAsync(P->ws_gout.p, gout.data(), sizeof(int) * n_pos, cudaMemcpyHostToDevice, P->stream));
+  std::vector<double> xi_all(n_pos);
+  for (int i = 0; i < n_pos; ++i) xi_all[i] = gout[i] < P->n_g ? P->h_xi[gout[i]] : 0.0;
+  TRY(ensure(P, P->ws_xi, sizeof(double) * n_pos));
+  CK(cudaMemcpyAsync(P->ws_xi.p, xi_all.data(), sizeof(double) * n_pos, cudaMemcpyHostToDevice, P->stream));
   P->ns_kmax = 0;
-  // difference-form columns: grid points with xi_g below a tenth of the smallest pair energy (there
-  // |Pi(i xi_g) - Pi(0)| <= 1% of |Pi(0)|)
-  P->ns_ndiff = 0;
-  if (use_tc)
-    while (P->ns_ndiff < P->n_g && P->h_xi[P->ns_ndiff] < 0.1 * P->D_min) ++P->ns_ndiff;
   // positions this rank computes: its block [p0, p1), from position 0 when the block holds difference-form
   // columns (they need eps(0)^-1); columns outside the block are zeroed before the sum across ranks
-  int p0 = 0, p1 = n_g1;
+  int p0 = 0, p1 = n_pos;
   if (P->sh_world > 1) gw_shard_columns(P->n_g, P->sh_rank, P->sh_world, &p0, &p1);
   const int p_begin = (use_tc && p0 > 0 && p0 <= P->ns_ndiff) ? 0 : p0;
   if (use_tc || P->sh_world > 1)
@@ -535,7 +566,7 @@ gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
     if (use_tc) {
       CK(cudaStreamSynchronize(P->stream));
       ms_pi += now_ms(P, P->ev0, P->ev1);
-      TRY(ns_w_table(P, g0, nc));
+      TRY(ns_w_table(P, g0, nc, xi_all.data() + g0));
       continue;
     }
     size_t t1 = tick(P);
@@ -552,7 +583,10 @@ gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
       if (info[i] != 0)
         return fail(P, GW_ERR_NUMERIC, "Cholesky of eps(i xi) failed at frequency %d, pivot %d", g0 + i, info[i]);
   }
-  if (use_tc && P->ns_ndiff > 0) LAUNCH(gw::launch_w_add_static(P->d_W, R, P->n_g, P->ns_ndiff, P->stream));
+  if (nodes)
+    LAUNCH(CK(gw::launch_w_expand(P->d_W, R, P->n_g, n_pos, as<int>(P->ws_gout), as<double>(P->sk_C), P->stream)));
+  else if (use_tc && P->ns_ndiff > 0)
+    LAUNCH(gw::launch_w_add_static(P->d_W, R, P->n_g, P->ns_ndiff, P->stream));
   P->stats.ms_pi = ms_pi;
   if (P->sh_world > 1) {
     // keep the owned columns (positions [p0, p1): position 0 is column n_g, position p > 0 is column p - 1), then
@@ -2062,6 +2096,7 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
     const u64 per_ns = n * ldn * 24 + n * n * 8;                             // Newton-Schulz split/FP32 iterates
     b += capped(per_ns, per_ns * n_g1) + 6 * n * ldn + 4 * n_g1;             // + the split eps(0)^-1 - 1
     b += 8 * n * n_g1 + 16 * n_g1;                                           // spectrum-estimate vectors
+    b += 8 * n_g1 * std::min<u64>(n_g1, 256);                                // matrix of the grid nodes
   } else {
     b += 8 * (u64)gw::trsm_w_scratch_elems<double>(c->n_aux, gw::trsm_w_default_ctas());
   }
