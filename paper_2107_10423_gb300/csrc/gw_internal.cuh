@@ -10,22 +10,17 @@ namespace gw {
 
 // ---------------------------------------------------------------- dense kernels (kernels_dense.cu)
 // Every kernel below takes the pair energies D_k (k < n_ov, the columns of B) as an array Dk.
-// Pi_PQ(i xi_g) = -4 sum_k B[P][k] B[Q][k] D_k/(D_k^2 + xi_g^2)  (Sec. 3.3, eta = 0), for n_xi points.
-// mode 0 writes Pi, mode 1 writes eps = 1 - Pi.  out: [n_xi][n_aux][n_aux] full symmetric.
-template <typename T>
-void launch_pi_syrk(const T* B, const double* Dk, long n_ov, int n_aux, const double* xi, int n_xi, T* out, int mode,
-                    cudaStream_t s);
-
-// Dense complex real-axis matrix A = 1 - Pi(x) as two real [n_aux][n_aux] halves (dense fallback).
-void launch_pi_complex_dense(const double* B, const double* Dk, long n_ov, int n_aux, double x, double eta, double* Ar,
-                             double* Ai, cudaStream_t s);
-
 // In-place lower Cholesky of `batch` SPD matrices A[b] = base + b*stride (row-major n x n).
 // info[b] = 0 on success, j+1 if pivot j was not positive.
 template <typename T>
 void launch_cholesky(T* base, int n, long stride, int batch, int* info, cudaStream_t s);
 
-// W table from Cholesky factors: for matrices g in [0, n_g): y = L_g^-1 b_r for rows r of Bn [R][n],
+// X_b = L_b^-1 (full n x n, zeros above the diagonal) from lower factors L_b at stride `stride`.
+cudaError_t launch_tri_inv(const double* L, long stride, int n, int batch, double* X, long xstride, cudaStream_t s);
+// W[r][c] = -|Bn_r|^2 for c < n_cols.
+cudaError_t launch_w_minus_norm(const double* Bn, int n, long R, int n_cols, double* W, cudaStream_t s);
+
+// W table from Cholesky factors (gw_w_table_noalloc): for matrices g in [0, n_g): y = L_g^-1 b_r for rows r of Bn [R][n],
 // W[r*w_ld + g_out[g]] = |y|^2 - |b|^2 = b^T(eps^-1 - 1)b.  scratch: [n_cta][n][64] elements of T.
 template <typename T>
 cudaError_t launch_trsm_w(const T* Lbase, long Lstride, int n, int n_g, const int* g_out, const T* Bn, int R,

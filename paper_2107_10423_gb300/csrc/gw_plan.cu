@@ -2,6 +2,7 @@
 // Algorithm 1 (imaginary-axis screening, then the per-state QP loop with batched residue solves).
 #include "gw.h"
 #include "gw_internal.cuh"
+#include "oz_gemm.cuh"
 #include "pi_tc.cuh"
 
 #include <algorithm>
@@ -92,7 +93,8 @@ struct gw_plan {
   DevBuf sk_C;                // device copy of nodes.C
   std::vector<DevBuf*> bufs;
   int tc_tiles_n = 0;          // N_aux the tile-order table of the Pi kernel was built for
-  DevBuf ws_mat, ws_info, ws_scratch, ws_gout, ws_xi, tc_part, tc_kind, tc_par, tc_err, tc_w, tc_tiles, ns_E, ns_X, ns_X2, ns_Xa, ns_Xb, ns_T, ns_lam,
+  DevBuf oz_A, oz_B, oz_X, oz_sc, oz_w;   // FP64 products on the tensor cores: digits, inverse factors, scales, weights
+  DevBuf ws_mat, ws_info, ws_gout, ws_xi, tc_part, tc_kind, tc_par, tc_err, tc_w, tc_tiles, ns_E, ns_X, ns_X2, ns_Xa, ns_Xb, ns_T, ns_lam,
       ns_E0, ns_vec;
   DevBuf mr_V, mr_U, mr_S, mr_vprev, mr_v, mr_d1, mr_d2, mr_x, mr_st, mr_rt, mr_rm, mr_xf, mr_wre, mr_wim,
       mr_dwre, mr_it, mr_res, mr_cnt, mr_Vhi, mr_Vlo, mr_Uhi, mr_Ulo, mr_Vlo2, mr_Ulo2, mr_V64;
@@ -110,7 +112,7 @@ struct gw_plan {
   std::vector<Mark> marks;
 
   gw_plan() {
-    DevBuf* all[] = {&ws_mat, &ws_info, &ws_scratch, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
+    DevBuf* all[] = {&oz_A, &oz_B, &oz_X, &oz_sc, &oz_w, &ws_mat, &ws_info, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
                      &mr_v, &mr_d1, &mr_d2, &mr_x, &mr_st, &mr_rt, &mr_rm, &mr_xf, &mr_wre, &mr_wim,
                      &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
                      &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_lu, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS};
@@ -481,9 +483,126 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc, const double* xi_pos) {
   return GW_OK;
 }
 
+// ---------------------------------------------------------------- FP64 products by digits (oz_gemm.cu)
+// Bytes a digit buffer may take (at least one matrix's smallest piece).
+size_t oz_cap(const gw_plan* P) { return std::min<size_t>(ws_bytes(P), (size_t)1 << 30); }
+
+gw_status oz_check(gw_plan* P) {
+  int herr = 0;
+  CK(cudaMemcpyAsync(&herr, P->tc_err.p, sizeof(int), cudaMemcpyDeviceToHost, P->stream));
+  CK(cudaStreamSynchronize(P->stream));
+  if (herr != 0) return fail(P, GW_ERR_TIMEOUT, "tensor-core FP64 product: bounded wait ran out (code %d)", herr);
+  return GW_OK;
+}
+
+// K columns a weighted product holds at once: all of them, or as many (a multiple of 128) as the cap allows for the
+// digits of B and of one weighted copy.
+int oz_slab(size_t cap, int n, int K) {
+  const size_t per_col = 2 * (size_t)gw::OZ_S * n * sizeof(__nv_bfloat16);
+  if (per_col * gw::oz_ld(K) <= cap) return K;
+  return (int)std::min<size_t>(K, std::max<size_t>(128, cap / per_col / 128 * 128));
+}
+
+// out_b = f(B diag(w_b) B^T) in FP64 for nb entries (weights of kind 0, 1, 2 as in tc_pair_weights).
+gw_status oz_weighted_syrk(gw_plan* P, const int* kinds, const double* params, int nb, int mode_even, int mode_odd,
+                           double* out) {
+  const int n = P->cfg.n_aux, K = P->n_ov;
+  const size_t cap = oz_cap(P);
+  const int slab = oz_slab(cap, n, K);
+  const size_t one = gw::oz_elems(n, slab);
+  // entries at once: their digits within the cap, pairs kept together (even and odd entries have their own modes)
+  int eg = (int)std::min<size_t>(nb, std::max<size_t>(1, cap / (one * sizeof(__nv_bfloat16))));
+  eg = std::min(eg, 32768);
+  if (eg > 1 && eg < nb) eg &= ~1;
+  TRY(ensure(P, P->oz_A, sizeof(__nv_bfloat16) * one * eg));
+  TRY(ensure(P, P->oz_B, sizeof(__nv_bfloat16) * one));
+  TRY(ensure(P, P->oz_w, sizeof(double) * (size_t)K * eg));
+  TRY(ensure(P, P->oz_sc, sizeof(double) * ((size_t)n * (eg + 1) + eg)));
+  TRY(ensure(P, P->tc_kind, sizeof(int) * nb));
+  TRY(ensure(P, P->tc_par, sizeof(double) * nb));
+  TRY(ensure(P, P->tc_err, sizeof(int)));
+  CK(cudaMemcpyAsync(P->tc_kind.p, kinds, sizeof(int) * nb, cudaMemcpyHostToDevice, P->stream));
+  CK(cudaMemcpyAsync(P->tc_par.p, params, sizeof(double) * nb, cudaMemcpyHostToDevice, P->stream));
+  CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
+  double* scB = as<double>(P->oz_sc);
+  double* scA = scB + n;
+  double* scw = scA + (size_t)n * eg;
+  __nv_bfloat16* dB = as<__nv_bfloat16>(P->oz_B);
+  __nv_bfloat16* dA = as<__nv_bfloat16>(P->oz_A);
+  CK(gw::oz_row_scale(P->d_B_ia, n, K, K, scB, P->stream));
+  P->stats.n_kernel_launches += 1;
+  for (int b0 = 0; b0 < nb; b0 += eg) {
+    const int ne = std::min(eg, nb - b0);
+    CK(gw::oz_pair_weights(P->d_D, K, as<int>(P->tc_kind) + b0, as<double>(P->tc_par) + b0, P->cfg.eta, ne,
+                           as<double>(P->oz_w), P->stream));
+    CK(gw::oz_row_scale(as<double>(P->oz_w), ne, K, K, scw, P->stream));
+    for (int k0 = 0; k0 < K; k0 += slab) {
+      const int kc = std::min(slab, K - k0);
+      if (b0 == 0 || slab < K) CK(gw::oz_split(P->d_B_ia, 0, n, k0, kc, K, scB, 1, dB, P->stream));
+      CK(gw::oz_split_weighted(P->d_B_ia, n, k0, kc, K, scB, as<double>(P->oz_w), K, scw, ne, dA, scA, P->stream));
+      gw::OzEpi ep{};
+      ep.kind = gw::OZ_EPI_STORE;
+      ep.lower = 1;
+      ep.mode_even = (b0 & 1) ? mode_odd : mode_even;
+      ep.mode_odd = (b0 & 1) ? mode_even : mode_odd;
+      ep.accumulate = k0 > 0;
+      ep.out = out + (size_t)b0 * n * n;
+      ep.out_bstride = (long)n * n;
+      ep.ldo = n;
+      CK(gw::oz_gemm(gw::OzOperand{dA, scA, 1}, gw::OzOperand{dB, scB, 0}, ne, n, n, kc, ep, as<int>(P->tc_err),
+                     P->stream));
+      P->stats.n_kernel_launches += 3;
+    }
+    P->stats.n_kernel_launches += 2;
+  }
+  return GW_OK;
+}
+
+// W[r][gidx[b]] += |L_b^-1 b_r|^2 for nc Cholesky factors L (ws_mat) and every row of B_nm: the inverse factors, their
+// digits and one digit product per block of rows, summed in its epilogue.
+gw_status oz_w_columns(gw_plan* P, const double* L, int nc, const int* gidx) {
+  const int n = P->cfg.n_aux, n_g1 = P->n_g + 1;
+  const long R = (long)P->n_t * P->n_bas;
+  const size_t cap = oz_cap(P), per = gw::oz_elems(n, n) * sizeof(__nv_bfloat16);
+  const int sub = (int)std::min<size_t>(nc, std::max<size_t>(1, cap / (per + sizeof(double) * n * n)));
+  const int rc = (int)std::min<size_t>((size_t)R, std::max<size_t>(128, cap / (per / n)));
+  TRY(ensure(P, P->oz_X, sizeof(double) * (size_t)n * n * sub));
+  TRY(ensure(P, P->oz_A, sizeof(__nv_bfloat16) * gw::oz_elems(rc, n)));
+  TRY(ensure(P, P->oz_B, per * sub));
+  TRY(ensure(P, P->oz_sc, sizeof(double) * ((size_t)R + (size_t)n * sub)));
+  TRY(ensure(P, P->tc_err, sizeof(int)));
+  CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
+  double* scR = as<double>(P->oz_sc);
+  double* scX = scR + R;
+  double* X = as<double>(P->oz_X);
+  CK(gw::oz_row_scale(P->d_B_nm, (int)R, n, n, scR, P->stream));
+  for (int b0 = 0; b0 < nc; b0 += sub) {
+    const int nb = std::min(sub, nc - b0);
+    CK(gw::launch_tri_inv(L + (size_t)b0 * n * n, (long)n * n, n, nb, X, (long)n * n, P->stream));
+    CK(gw::oz_row_scale(X, n * nb, n, n, scX, P->stream));
+    CK(gw::oz_split(X, (long)n * n, n, 0, n, n, scX, nb, as<__nv_bfloat16>(P->oz_B), P->stream));
+    for (long r0 = 0; r0 < R; r0 += rc) {
+      const int nr = (int)std::min<long>(rc, R - r0);
+      if (b0 == 0 || rc < R)
+        CK(gw::oz_split(P->d_B_nm + r0 * n, 0, nr, 0, n, n, scR + r0, 1, as<__nv_bfloat16>(P->oz_A), P->stream));
+      gw::OzEpi ep{};
+      ep.kind = gw::OZ_EPI_SUMSQ;
+      ep.acc = P->d_W + r0 * n_g1;
+      ep.ldw = n_g1;
+      ep.gidx = gidx + b0;
+      CK(gw::oz_gemm(gw::OzOperand{as<__nv_bfloat16>(P->oz_A), scR + r0, 0},
+                     gw::OzOperand{as<__nv_bfloat16>(P->oz_B), scX, 1}, nb, nr, n, n, ep, as<int>(P->tc_err),
+                     P->stream));
+      P->stats.n_kernel_launches += 2;
+    }
+    P->stats.n_kernel_launches += 3;
+  }
+  return GW_OK;
+}
+
 // ---------------------------------------------------------------- imaginary-axis screening
 template <typename T>
-gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
+gw_status screening_T(gw_plan* P) {
   const int n = P->cfg.n_aux;
   const int n_g1 = P->n_g + 1;
   const int R = P->n_t * P->n_bas;
@@ -533,8 +652,6 @@ gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
   TRY(ensure(P, P->ws_mat, per * chunk));
   TRY(ensure(P, P->ws_info, sizeof(int) * chunk));
   TRY(ensure(P, P->ws_gout, sizeof(int) * n_pos));
-  const int n_cta = gw::trsm_w_default_ctas();
-  if (!use_tc) TRY(ensure(P, P->ws_scratch, sizeof(T) * gw::trsm_w_scratch_elems<T>(n, n_cta)));
   CK(cudaMemcpyAsync(P->ws_gout.p, gout.data(), sizeof(int) * n_pos, cudaMemcpyHostToDevice, P->stream));
   std::vector<double> xi_all(n_pos);
   for (int i = 0; i < n_pos; ++i) xi_all[i] = gout[i] < P->n_g ? P->h_xi[gout[i]] : 0.0;
@@ -546,8 +663,10 @@ gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
   int p0 = 0, p1 = n_pos;
   if (P->sh_world > 1) gw_shard_columns(P->n_g, P->sh_rank, P->sh_world, &p0, &p1);
   const int p_begin = (use_tc && p0 > 0 && p0 <= P->ns_ndiff) ? 0 : p0;
-  if (use_tc || P->sh_world > 1)
-    CK(cudaMemsetAsync(P->d_W, 0, sizeof(double) * (size_t)R * n_g1, P->stream));   // W is accumulated / summed
+  if (use_tc)
+    CK(cudaMemsetAsync(P->d_W, 0, sizeof(double) * (size_t)R * n_g1, P->stream));   // W is accumulated
+  else
+    LAUNCH(CK(gw::launch_w_minus_norm(P->d_B_nm, n, R, n_g1, P->d_W, P->stream)));
   std::vector<int> info(chunk);
   double ms_pi = 0.0;
   for (int g0 = p_begin; g0 < p1; g0 += chunk) {
@@ -558,9 +677,10 @@ gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
       TRY(tc_weighted_syrk(P, kinds.data(), xi_all.data() + g0, nc, 1, 1, reinterpret_cast<float*>(P->ws_mat.p), 0));
     } else {
       const size_t t0 = tick(P);
-      LAUNCH(gw::launch_pi_syrk<T>(B, P->d_D, P->n_ov, n, as<double>(P->ws_xi) + g0, nc,
-                                   as<T>(P->ws_mat), 1, P->stream));
+      std::vector<int> kinds(nc, 0);
+      TRY(oz_weighted_syrk(P, kinds.data(), xi_all.data() + g0, nc, 1, 1, as<double>(P->ws_mat)));
       mark(P, 1, t0, (double)nc * n * n * P->n_ov);
+      TRY(oz_check(P));
     }
     CK(cudaEventRecord(P->ev1, P->stream));
     if (use_tc) {
@@ -570,12 +690,12 @@ gw_status screening_T(gw_plan* P, const T* B, const T* Bn) {
       continue;
     }
     size_t t1 = tick(P);
-    LAUNCH(gw::launch_cholesky<T>(as<T>(P->ws_mat), n, (long)n * n, nc, as<int>(P->ws_info), P->stream));
+    LAUNCH(gw::launch_cholesky<double>(as<double>(P->ws_mat), n, (long)n * n, nc, as<int>(P->ws_info), P->stream));
     mark(P, 2, t1, (double)nc * n * n * (double)n / 3.0);
     t1 = tick(P);
-    LAUNCH(gw::launch_trsm_w<T>(as<T>(P->ws_mat), (long)n * n, n, nc, as<int>(P->ws_gout) + g0, Bn, R, P->d_W,
-                                n_g1, as<T>(P->ws_scratch), n_cta, P->stream));
+    TRY(oz_w_columns(P, as<double>(P->ws_mat), nc, as<int>(P->ws_gout) + g0));
     mark(P, 3, t1, (double)nc * (double)n * n * R);
+    TRY(oz_check(P));
     CK(cudaMemcpyAsync(info.data(), P->ws_info.p, sizeof(int) * nc, cudaMemcpyDeviceToHost, P->stream));
     CK(cudaStreamSynchronize(P->stream));
     ms_pi += now_ms(P, P->ev0, P->ev1);
@@ -612,9 +732,9 @@ gw_status ensure_screening(gw_plan* P) {
   CK(cudaEventRecord(a, P->stream));
   gw_status st;
   if (P->cfg.precision == GW_PREC_MIXED)
-    st = screening_T<float>(P, P->d_B_ia_f, P->d_B_nm_f);
+    st = screening_T<float>(P);
   else
-    st = screening_T<double>(P, P->d_B_ia, P->d_B_nm);
+    st = screening_T<double>(P);
   if (st != GW_OK) { cudaEventDestroy(a); cudaEventDestroy(b); return st; }
   CK(cudaEventRecord(b, P->stream));
   CK(cudaEventSynchronize(b));
@@ -702,11 +822,16 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
       }
     } else {
       const size_t t0 = tick(P);
-      for (int k = 0; k < nf; ++k)
-        LAUNCH(gw::launch_pi_complex_dense(P->d_B_ia, P->d_D, P->n_ov, n, hx[k0 + k],
-                                           P->cfg.eta, reinterpret_cast<double*>(A) + 2 * mat * k,
-                                           reinterpret_cast<double*>(A) + 2 * mat * k + mat, P->stream));
-      mark(P, 6, t0, 4.0 * nf * (double)mat * P->n_ov);
+      std::vector<int> kinds(2 * nf);
+      std::vector<double> par(2 * nf);
+      for (int k = 0; k < nf; ++k) {
+        kinds[2 * k] = 1;
+        kinds[2 * k + 1] = 2;
+        par[2 * k] = par[2 * k + 1] = hx[k0 + k];
+      }
+      TRY(oz_weighted_syrk(P, kinds.data(), par.data(), 2 * nf, 1, 2, reinterpret_cast<double*>(A)));
+      mark(P, 6, t0, 2.0 * nf * (double)mat * P->n_ov);
+      TRY(oz_check(P));
     }
     LAUNCH(gw::launch_fallback_rhs<T>(P->d_B_nm, P->n_bas, n, rt, rm, as<int>(P->fb_idx) + k0, nf, as<T>(P->fb_y),
                                       P->stream));
@@ -1601,10 +1726,6 @@ gw_status gw_polarizability(gw_plan_t P, const double* xi, int n_xi, double* pi_
   }
   if (n_xi <= 0) return fail(P, GW_ERR_ARG, "n_xi must be positive");
   const int n = P->cfg.n_aux;
-  DevBuf& dxi = P->ws_xi;
-  gw_status st = ensure(P, dxi, sizeof(double) * n_xi);
-  if (st != GW_OK) return st;
-  CK(cudaMemcpyAsync(dxi.p, xi, sizeof(double) * n_xi, cudaMemcpyHostToDevice, P->stream));
   CK(cudaEventRecord(P->ev0, P->stream));
   if (P->cfg.precision == GW_PREC_MIXED) {
     TRY(ensure(P, P->ws_mat, sizeof(float) * (size_t)n * n * n_xi));
@@ -1619,12 +1740,13 @@ gw_status gw_polarizability(gw_plan_t P, const double* xi, int n_xi, double* pi_
     }
   } else {
     TRY(ensure(P, P->ws_mat, sizeof(double) * (size_t)n * n * n_xi));
-    LAUNCH(gw::launch_pi_syrk<double>(P->d_B_ia, P->d_D, P->n_ov, n, as<double>(dxi), n_xi,
-                                      as<double>(P->ws_mat), 0, P->stream));
+    std::vector<int> kinds(n_xi, 0);
+    TRY(oz_weighted_syrk(P, kinds.data(), xi, n_xi, 0, 0, as<double>(P->ws_mat)));
     CK(cudaEventRecord(P->ev1, P->stream));
     if (pi_out)
       CK(cudaMemcpyAsync(pi_out, P->ws_mat.p, sizeof(double) * (size_t)n * n * n_xi, cudaMemcpyDeviceToHost,
                          P->stream));
+    TRY(oz_check(P));
   }
   CK(cudaStreamSynchronize(P->stream));
   P->stats.ms_pi = now_ms(P, P->ev0, P->ev1);
@@ -2098,7 +2220,14 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
     b += 8 * n * n_g1 + 16 * n_g1;                                           // spectrum-estimate vectors
     b += 8 * n_g1 * std::min<u64>(n_g1, 256);                                // matrix of the grid nodes
   } else {
-    b += 8 * (u64)gw::trsm_w_scratch_elems<double>(c->n_aux, gw::trsm_w_default_ctas());
+    // digit products: B and its weighted copies, or the inverse factors, their digits and those of B_nm's rows
+    const u64 cap = std::min<u64>(ws, (u64)1 << 30), nb = std::max<u64>(n_g1, 2 * std::max<u64>(1, ws / (2 * n * n * ts)));
+    const u64 slab = (u64)oz_slab((size_t)cap, c->n_aux, (int)std::min<u64>(n_ov, 2147483647ull));
+    const u64 one = 2 * (u64)gw::oz_elems(c->n_aux, (int)slab), per = 2 * (u64)gw::oz_elems(c->n_aux, c->n_aux);
+    const u64 eg = std::min(nb, std::max<u64>(1, cap / one)), sub = std::min(n_g1, std::max<u64>(1, cap / (per + 8 * n * n)));
+    const u64 rc = std::min<u64>(rows, std::max<u64>(128, cap / (per / n)));
+    b += std::max(one * eg, rc * (per / n)) + std::max(one, per * sub) + 8 * n * n * sub;
+    b += 8 * n_ov * eg + 8 * std::max((n + 1) * (eg + 1), rows + n * sub) + 12 * nb;
   }
   // residue batch (at most one right-hand side per target and state at a time)
   u64 batch = c->max_rhs_batch > 0 ? (u64)c->max_rhs_batch

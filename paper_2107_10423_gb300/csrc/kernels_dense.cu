@@ -1,5 +1,4 @@
 // Dense kernels of the CD-G0W0 path (SIMT, templated on the arithmetic type):
-//  * Pi(i xi) symmetric rank-N_ov update (Sec. 3.3, equation after "wauxbas"), lower tiles + mirror;
 //  * batched in-place Cholesky of eps(i xi) = 1 - Pi (SPD, Sec. 3.3 text after "inn");
 //  * triangular solves that turn the factors into the table W^c_nm(i xi) (Algorithm 1, imaginary-grid loop);
 //  * the two skinny GEMMs of the matrix-free residue operator 1 - Pi(x) (Sec. 3.3, MINRES paragraph).
@@ -17,132 +16,6 @@ constexpr int TM = 64;     // tile rows
 constexpr int TN = 64;     // tile cols
 constexpr int TK = 16;     // k step
 constexpr int NT = 256;    // threads per CTA (16 x 16, 4 x 4 outputs each)
-
-// ------------------------------------------------------------------ Pi(i xi) SYRK
-// grid.x: lower-triangular tile index (bi >= bj), grid.y: frequency index.
-template <typename T>
-__global__ void __launch_bounds__(NT) pi_syrk_kernel(const T* __restrict__ B, const double* __restrict__ Dk,
-                                                     long n_ov, int n_aux,
-                                                     const double* __restrict__ xi, T* __restrict__ out, int mode) {
-  __shared__ T As[TK][TM + 4];
-  __shared__ T Bs[TK][TN + 4];
-  // decode lower tile (bi, bj) from linear index t = bi*(bi+1)/2 + bj
-  int t = blockIdx.x;
-  int bi = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
-  while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
-  while (bi * (bi + 1) / 2 > t) --bi;
-  int bj = t - bi * (bi + 1) / 2;
-  const int g = blockIdx.y;
-  const double x2 = xi[g] * xi[g];
-  const int p0 = bi * TM, q0 = bj * TN;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  T acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-  const int lr = tid >> 2, lk = (tid & 3) * 4;
-  for (long k0 = 0; k0 < n_ov; k0 += TK) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      long k = k0 + lk + u;
-      T wa = T(0), va = T(0), vb = T(0);
-      if (k < n_ov) {
-        const double D = Dk[k];
-        wa = (T)(-4.0 * D / (D * D + x2));
-        if (p0 + lr < n_aux) va = B[(long)(p0 + lr) * n_ov + k];
-        if (q0 + lr < n_aux) vb = B[(long)(q0 + lr) * n_ov + k];
-      }
-      As[lk + u][lr] = va * wa;
-      Bs[lk + u][lr] = vb;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      T a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-  T* o = out + (long)g * n_aux * n_aux;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int p = p0 + ty + 16 * i;
-    if (p >= n_aux) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int q = q0 + tx + 16 * j;
-      if (q >= n_aux || q > p) continue;
-      T v = acc[i][j];
-      if (mode == 1) v = (p == q ? T(1) : T(0)) - v;
-      o[(long)p * n_aux + q] = v;
-      o[(long)q * n_aux + p] = v;
-    }
-  }
-}
-
-// Complex real-axis Pi(x) as A = 1 - Pi, two real halves (dense fallback only).
-__global__ void __launch_bounds__(NT) pi_complex_kernel(const double* __restrict__ B, const double* __restrict__ Dk,
-                                                        long n_ov, int n_aux, double x, double eta,
-                                                        double* __restrict__ Ar, double* __restrict__ Ai) {
-  __shared__ double Asr[TK][TM + 4];
-  __shared__ double Asi[TK][TM + 4];
-  __shared__ double Bs[TK][TN + 4];
-  const int p0 = blockIdx.y * TM, q0 = blockIdx.x * TN;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double accr[4][4], acci[4][4];
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) accr[i][j] = acci[i][j] = 0.0;
-  const int lr = tid >> 2, lk = (tid & 3) * 4;
-  const double e2 = eta * eta;
-  for (long k0 = 0; k0 < n_ov; k0 += TK) {
-    for (int u = 0; u < 4; ++u) {
-      long k = k0 + lk + u;
-      double cr = 0, ci = 0, va = 0, vb = 0;
-      if (k < n_ov) {
-        const double D = Dk[k];
-        double a1 = x - D, a2 = -x - D;
-        double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
-        cr = 2.0 * (a1 / d1 + a2 / d2);
-        ci = 2.0 * (-eta / d1 - eta / d2);
-        if (p0 + lr < n_aux) va = B[(long)(p0 + lr) * n_ov + k];
-        if (q0 + lr < n_aux) vb = B[(long)(q0 + lr) * n_ov + k];
-      }
-      Asr[lk + u][lr] = va * cr;
-      Asi[lk + u][lr] = va * ci;
-      Bs[lk + u][lr] = vb;
-    }
-    __syncthreads();
-    for (int kk = 0; kk < TK; ++kk) {
-      double ar[4], ai[4], b[4];
-      for (int i = 0; i < 4; ++i) { ar[i] = Asr[kk][ty + 16 * i]; ai[i] = Asi[kk][ty + 16 * i]; }
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-      for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) {
-          accr[i][j] = fma(ar[i], b[j], accr[i][j]);
-          acci[i][j] = fma(ai[i], b[j], acci[i][j]);
-        }
-    }
-    __syncthreads();
-  }
-  for (int i = 0; i < 4; ++i) {
-    int p = p0 + ty + 16 * i;
-    if (p >= n_aux) continue;
-    for (int j = 0; j < 4; ++j) {
-      int q = q0 + tx + 16 * j;
-      if (q >= n_aux) continue;
-      Ar[(long)p * n_aux + q] = (p == q ? 1.0 : 0.0) - accr[i][j];
-      Ai[(long)p * n_aux + q] = -acci[i][j];
-    }
-  }
-}
 
 // ------------------------------------------------------------------ batched Cholesky, one CTA per matrix
 constexpr int CH_NB = 32;
@@ -231,6 +104,94 @@ __global__ void __launch_bounds__(CH_THREADS) cholesky_kernel(T* base, int n, lo
     __syncthreads();
   }
   if (tid == 0) info[blockIdx.x] = bad;
+}
+
+// ------------------------------------------------------------------ inverse of the Cholesky factors
+// X = L^-1 (lower, zeros above the diagonal) for a batch of factors.  CTA (J, b) builds the 64 columns of block J:
+//   X_JJ = L_JJ^-1,  X_IJ = -L_II^-1 sum_{J <= K < I} L_IK X_KJ,
+// every column block on its own, so (n / 64) CTAs a matrix; n^3/6 FP64 FMAs a matrix, bound by the FP64 pipe.
+__global__ void __launch_bounds__(NT) tri_inv_kernel(const double* __restrict__ Lb, long stride, int n,
+                                                     double* __restrict__ Xb, long xstride) {
+  __shared__ double As[TK][TM + 4];
+  __shared__ double Bs[TK][TN + 4];
+  extern __shared__ double tri_sm[];
+  double* Ts = tri_sm;                  // [64][65]
+  double* Ls = tri_sm + 64 * 65;        // [64][65]
+  const double* L = Lb + (long)blockIdx.y * stride;
+  double* X = Xb + (long)blockIdx.y * xstride;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int J = blockIdx.x, nJ = (n + 63) / 64, c0 = J * 64;
+  for (int i = tid; i < c0 * 64; i += NT) {          // zeros above the diagonal block
+    const int r = i >> 6, c = c0 + (i & 63);
+    if (c < n) X[(long)r * n + c] = 0.0;
+  }
+  for (int I = J; I < nJ; ++I) {
+    const int r0 = I * 64, nr = min(64, n - r0);
+    double acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = (I == J && ty + 16 * i == tx + 16 * j) ? 1.0 : 0.0;
+    for (int k0 = c0; k0 < r0; k0 += TK) {
+      {
+        const int r = tid >> 2, k4 = (tid & 3) * 4, kr = tid >> 4, c4 = (tid & 15) * 4;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          As[k4 + u][r] = r0 + r < n ? L[(long)(r0 + r) * n + k0 + k4 + u] : 0.0;
+          Bs[kr][c4 + u] = c0 + c4 + u < n ? X[(long)(k0 + kr) * n + c0 + c4 + u] : 0.0;
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int kk = 0; kk < TK; ++kk) {
+        double a[4], b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = fma(-a[i], b[j], acc[i][j]);
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) Ts[(ty + 16 * i) * 65 + tx + 16 * j] = acc[i][j];
+    for (int idx = tid; idx < 64 * 64; idx += NT) {
+      const int r = idx >> 6, c = idx & 63;
+      Ls[r * 65 + c] = (r < nr && c <= r) ? L[(long)(r0 + r) * n + r0 + c] : 0.0;
+    }
+    __syncthreads();
+    if (tid < 64)
+      for (int p = 0; p < nr; ++p) {
+        double v = Ts[p * 65 + tid];
+        for (int q = 0; q < p; ++q) v = fma(-Ls[p * 65 + q], Ts[q * 65 + tid], v);
+        Ts[p * 65 + tid] = v / Ls[p * 65 + p];
+      }
+    __syncthreads();
+    for (int idx = tid; idx < 64 * 64; idx += NT) {
+      const int r = idx >> 6, c = idx & 63;
+      if (r < nr && c0 + c < n) X[(long)(r0 + r) * n + c0 + c] = (I == J && c > r) ? 0.0 : Ts[r * 65 + c];
+    }
+    __threadfence_block();
+    __syncthreads();
+  }
+}
+
+// W[r][col] = -|b_r|^2 for every column of the table (the sums of squares of L^-1 b_r are then added).
+__global__ void __launch_bounds__(128) w_minus_norm_kernel(const double* __restrict__ Bn, int n, long R, int n_cols,
+                                                           double* __restrict__ W) {
+  const int lane = threadIdx.x & 31;
+  for (long r = blockIdx.x * 4L + (threadIdx.x >> 5); r < R; r += gridDim.x * 4L) {
+    double s = 0.0;
+    for (int p = lane; p < n; p += 32) s = fma(Bn[r * n + p], Bn[r * n + p], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    for (int c = lane; c < n_cols; c += 32) W[r * n_cols + c] = -s;
+  }
 }
 
 // ------------------------------------------------------------------ TRSM -> W table
@@ -795,23 +756,23 @@ void launch_deriv_resonant(const double* V64, const double* B, long n_ov, int n_
 
 // ------------------------------------------------------------------ launchers
 template <typename T>
-void launch_pi_syrk(const T* B, const double* Dk, long n_ov, int n_aux, const double* xi, int n_xi, T* out, int mode,
-                    cudaStream_t s) {
-  int nb = (n_aux + TM - 1) / TM;
-  dim3 grid(nb * (nb + 1) / 2, n_xi);
-  pi_syrk_kernel<T><<<grid, NT, 0, s>>>(B, Dk, n_ov, n_aux, xi, out, mode);
-}
-
-void launch_pi_complex_dense(const double* B, const double* Dk, long n_ov, int n_aux, double x, double eta, double* Ar,
-                             double* Ai, cudaStream_t s) {
-  int nb = (n_aux + TM - 1) / TM;
-  dim3 grid(nb, nb);
-  pi_complex_kernel<<<grid, NT, 0, s>>>(B, Dk, n_ov, n_aux, x, eta, Ar, Ai);
-}
-
-template <typename T>
 void launch_cholesky(T* base, int n, long stride, int batch, int* info, cudaStream_t s) {
   cholesky_kernel<T><<<batch, CH_THREADS, 0, s>>>(base, n, stride, info);
+}
+
+cudaError_t launch_tri_inv(const double* L, long stride, int n, int batch, double* X, long xstride, cudaStream_t s) {
+  if (n <= 0 || batch <= 0) return cudaSuccess;
+  if (batch > 65535) return cudaErrorInvalidValue;
+  const int smem = (int)sizeof(double) * 2 * 64 * 65;
+  const cudaError_t e = cudaFuncSetAttribute(tri_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  tri_inv_kernel<<<dim3((n + 63) / 64, batch), NT, smem, s>>>(L, stride, n, X, xstride);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_w_minus_norm(const double* Bn, int n, long R, int n_cols, double* W, cudaStream_t s) {
+  if (R > 0) w_minus_norm_kernel<<<(unsigned)(R < 4 * 4096 ? (R + 3) / 4 : 4096), 128, 0, s>>>(Bn, n, R, n_cols, W);
+  return cudaGetLastError();
 }
 
 int trsm_w_default_ctas() {
@@ -857,12 +818,6 @@ void launch_op_gemm2(const T* U, const T* B, int n_aux, int n_ov, int nr, const 
 }
 
 #define GW_INST(T)                                                                                              \
-  template void launch_pi_syrk<T>(const T*, const double*, long, int, const double*, int, T*, int,             \
-                                  cudaStream_t);                                                                \
-  template void launch_cholesky<T>(T*, int, long, int, int*, cudaStream_t);                                     \
-  template size_t trsm_w_scratch_elems<T>(int, int);                                                            \
-  template cudaError_t launch_trsm_w<T>(const T*, long, int, int, const int*, const T*, int, double*, int, T*,   \
-                                        int, cudaStream_t);                                                     \
   template void launch_op_gemm1<T>(const T*, const T*, const double*, long, int, const double*, double, int,    \
                                    T*, int, cudaStream_t, double*, double, long, const int*);                   \
   template void launch_op_gemm2<T>(const T*, const T*, int, int, int, const T*, T*, int, cudaStream_t,          \
@@ -870,6 +825,10 @@ void launch_op_gemm2(const T* U, const T* B, int n_aux, int n_ov, int nr, const 
 GW_INST(double)
 GW_INST(float)
 #undef GW_INST
+template void launch_cholesky<double>(double*, int, long, int, int*, cudaStream_t);
+template size_t trsm_w_scratch_elems<double>(int, int);
+template cudaError_t launch_trsm_w<double>(const double*, long, int, int, const int*, const double*, int, double*, int,
+                                           double*, int, cudaStream_t);
 
 }  // namespace gw
 

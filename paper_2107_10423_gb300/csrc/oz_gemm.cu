@@ -1,0 +1,519 @@
+// FP64 products on the BF16 tensor cores (after Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix
+// multiplication", 2012): every operand row is scaled by a power of two to 63-bit integers and cut into eight balanced
+// base-256 digits, which BF16 holds exactly;
+//   A[m][k] B[n][k] = 2^(ea + eb - 124) sum_{i,j} a_i b_j 256^(14 - i - j),  a_i, b_j in [-128, 127],
+// and the products with i + j = d (d <= 7; the rest is below 2^-64 of the rows' scales) are summed per d in the
+// tensor core's FP32 accumulators over K = 128 at a time.  |a_i b_j| <= 2^14, so such a sum of at most 8 x 128 terms
+// stays within 2^24 and every partial sum is an integer that FP32 holds: the tensor core adds without error.  The
+// drain warps add the integers into two 64-bit fixed-point sums per element (d < 4 and d >= 4), again exactly, and one
+// rounding to FP64 ends the element.  The only errors are the 2^-63 (of the row's scale) of the digits, the dropped
+// products and that rounding, less than an FP64 FMA chain makes.
+//
+// Why: FP64 runs at two multiply-adds a clock and SM on this chip (0.58 T/s in all), the digits' 36 BF16 products at
+// about 50 times that in the tensor cores.  What bounds it: shared-memory reads of the M128 N64 K16 products (6 KiB
+// each at 128 B a clock: 48 clocks, where the tensor core alone would take 32), then the drains, which the single
+// TMEM buffer (8 sums x 64 columns = all 512) does not overlap with the next 128 of K.
+#include "oz_gemm.cuh"
+#include "tc_ptx.cuh"
+
+#include <algorithm>
+#include <cstdint>
+
+namespace gw {
+namespace {
+using namespace ptx;
+
+constexpr int S = OZ_S;
+constexpr int BM = 128, BN = 64, BK = 32;
+constexpr int KCHUNK = 4;                        // k-blocks per exact sum (K = 128)
+constexpr int STAGES = 2;
+constexpr int A_BYTES = S * BM * BK * 2;         // 64 KiB
+constexpr int B_BYTES = S * BN * BK * 2;         // 32 KiB
+constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int BAR_OFF = STAGES * STAGE_BYTES;
+constexpr int SMEM_BYTES = BAR_OFF + 1024 + 128;
+constexpr int DRAIN_WARPS = 8;
+constexpr int THREADS = 32 * (DRAIN_WARPS + 2);
+constexpr uint32_t TMEM_COLS = 512;
+static_assert(S * BN <= (int)TMEM_COLS, "one accumulator of BN columns per digit sum");
+static_assert(SMEM_BYTES + 1024 <= 232448, "shared memory per block");
+// kind::f16 instruction descriptor: D = F32, A = B = BF16, both K-major, N = 64, M = 128
+constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+                           ((uint32_t)(BM >> 4) << 24);
+constexpr uint32_t SBO64 = 8 * 64, SWZ64 = 4;    // 64-byte rows, 64-byte swizzle
+
+struct OzMaps {
+  CUtensorMap a, b;
+};
+
+// grid.x: tile x K range, grid.y: entry.  Warps 0-7 drain (TMEM lane quarter = warp & 3, column half = warp >> 2),
+// warp 8 TMA, warp 9 MMA.
+__global__ void __launch_bounds__(THREADS, 1)
+    oz_gemm_kernel(const __grid_constant__ OzMaps maps, int M, int N, int K, int a_batched, int b_batched,
+                   const double* __restrict__ sca, const double* __restrict__ scb, const OzEpi ep,
+                   int* __restrict__ err) {
+  if (ep.run_if && *ep.run_if == 0) return;      // uniform over the grid: nothing is allocated yet
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* smem = smem_raw + (base - raw);
+  const uint32_t bar0 = base + BAR_OFF;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + BAR_OFF + 64);
+  auto full = [bar0](int s) { return bar0 + 8u * (uint32_t)s; };
+  auto empty = [bar0](int s) { return bar0 + 8u * (uint32_t)(STAGES + s); };
+  const uint32_t acc_full = bar0 + 8u * (2 * STAGES), acc_empty = acc_full + 8u, fin = acc_full + 16u;
+  __shared__ int s_abort;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ksplit = ep.kind == OZ_EPI_PART ? ep.ksplit : 1;
+  const int ks = blockIdx.x % ksplit, tile = blockIdx.x / ksplit, b = blockIdx.y;
+  int bm, bn;
+  if (ep.kind == OZ_EPI_STORE && ep.lower) {     // row block bm holds the column blocks 0 .. 2 bm + 1
+    bm = (int)((sqrt(4.0 * tile + 1.0) - 1.0) * 0.5);
+    while ((bm + 1) * (bm + 2) <= tile) ++bm;
+    while (bm * (bm + 1) > tile) --bm;
+    bn = tile - bm * (bm + 1);
+  } else {
+    const int nbn = (N + BN - 1) / BN;
+    bm = tile / nbn;
+    bn = tile % nbn;
+  }
+  const int m0 = bm * BM, n0 = bn * BN;
+  if (m0 >= M || n0 >= N) return;                // the lower enumeration's last column block may lie past N
+  const int nk_all = ((ep.kind == OZ_EPI_SUMSQ ? min(K, n0 + BN) : K) + BK - 1) / BK;
+  // K ranges in whole chunks
+  const int nch = (nk_all + KCHUNK - 1) / KCHUNK;
+  const int c0 = (int)((long)nch * ks / ksplit), c1 = (int)((long)nch * (ks + 1) / ksplit);
+  const int kb0 = c0 * KCHUNK, nk = min(nk_all, c1 * KCHUNK) - kb0;
+
+  if (threadIdx.x == 0) {
+    s_abort = 0;
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(full(s), 1);
+      mbar_init(empty(s), 1);
+    }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, DRAIN_WARPS);
+    mbar_init(fin, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == DRAIN_WARPS) {
+    if (lane == 0) {
+      // ---------------- TMA producer: one box of all eight digits per operand and k-block
+      int issued = 0;
+      bool ok = true;
+      for (int kb = 0; kb < nk && ok; ++kb) {
+        const int s = kb % STAGES, u = kb / STAGES;
+        if (u > 0 && !mbar_wait(empty(s), (u - 1) & 1, err, 71)) { ok = false; break; }
+        if (*(volatile int*)&s_abort) { ok = false; break; }
+        const uint32_t st = base + s * STAGE_BYTES;
+        mbar_expect_tx(full(s), STAGE_BYTES);
+        tma_load_3d(st, &maps.a, (kb0 + kb) * BK, m0, a_batched ? b * S : 0, full(s));
+        tma_load_3d(st + A_BYTES, &maps.b, (kb0 + kb) * BK, n0, b_batched ? b * S : 0, full(s));
+        issued = kb + 1;
+      }
+      if (!ok) {
+        s_abort = 1;
+        for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
+          mbar_wait(full(kb % STAGES), (kb / STAGES) & 1, err, 72);
+      }
+    }
+  } else if (warp == DRAIN_WARPS + 1) {
+    if (lane == 0) {
+      // ---------------- MMA issuer
+      const uint64_t dA = sdesc(base, SBO64, SWZ64), dB = sdesc(base + A_BYTES, SBO64, SWZ64);
+      bool ok = true;
+      for (int kb = 0; kb < nk && ok; ++kb) {
+        const int s = kb % STAGES, u = kb / STAGES, c = kb / KCHUNK;
+        const bool first = kb % KCHUNK == 0;
+        if (first && c > 0 && !mbar_wait(acc_empty, (c - 1) & 1, err, 73)) { ok = false; break; }
+        if (!mbar_wait(full(s), u & 1, err, 74)) { ok = false; break; }
+        if (*(volatile int*)&s_abort) { ok = false; break; }
+        tc_fence_after();
+        const uint64_t a0 = dA + (uint64_t)((s * STAGE_BYTES) >> 4), b0 = dB + (uint64_t)((s * STAGE_BYTES) >> 4);
+#pragma unroll 1
+        for (int k = 0; k < BK / 16; ++k) {
+#pragma unroll 1
+          for (int i = 0; i < S; ++i) {
+            const uint64_t ad = a0 + (uint64_t)(i * ((BM * BK * 2) >> 4) + 2 * k);
+            for (int j = 0; i + j < S; ++j)
+              mma_bf16(tmem + (uint32_t)((i + j) * BN), ad, b0 + (uint64_t)(j * ((BN * BK * 2) >> 4) + 2 * k), IDESC,
+                       (first && k == 0 && i == 0) ? 0u : 1u);
+          }
+        }
+        mma_commit(empty(s));
+        if (kb % KCHUNK == KCHUNK - 1 || kb == nk - 1) mma_commit(acc_full);
+      }
+      if (!ok) s_abort = 1;
+      mma_commit(fin);             // every product issued above has completed once this flips
+      mbar_wait(fin, 0, err, 76);
+    }
+  }
+  bool ok = true;
+  const int q = warp & 3, h = (warp >> 2) & 1;
+  long long hi[32], lo[32];
+  if (warp < DRAIN_WARPS) {
+    // ---------------- drain: integers of the digit sums into the fixed-point sums
+#pragma unroll
+    for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
+    const int nchunks = (nk + KCHUNK - 1) / KCHUNK;
+    const uint32_t addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * 32);
+    for (int c = 0; c < nchunks; ++c) {
+      ok = !*(volatile int*)&s_abort && mbar_wait(acc_full, c & 1, err, 75);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+#pragma unroll
+      for (int d = 0; d < S; ++d) {
+        uint32_t v[32];
+        tmem_ld32(addr + (uint32_t)(d * BN), v);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const int x = __float2int_rn(__uint_as_float(v[j]));
+          if (d < 4) hi[j] += (long long)x * (1ll << (8 * (3 - d)));
+          else lo[j] += (long long)x * (1ll << (8 * (7 - d)));
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty);
+    }
+    if (!ok) s_abort = 1;
+  }
+  __syncwarp();
+  const bool all_ok = __syncthreads_and(ok && !*(volatile int*)&s_abort) != 0;
+  if (all_ok && warp < DRAIN_WARPS) {
+    const int m = m0 + q * 32 + lane, c = n0 + h * 32;
+    const double sm = m < M ? sca[(a_batched ? (long)b * M : 0) + m] * 1.4551915228366852e-11 : 0.0;   // 2^-36
+    const double* sn = scb + (b_batched ? (long)b * N : 0);
+    if (ep.kind == OZ_EPI_SUMSQ) {
+      // this row's sum over the tile's columns; hi 2^12 + lo 2^-20 is within 2^-60 of the scales' product and needs
+      // one conversion an element on the FP64 pipe instead of two
+      double t = 0.0;
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (c + j < N) {
+          const double v = (double)((hi[j] << 12) + (lo[j] >> 20)) * sn[c + j];
+          t = fma(v, v, t);
+        }
+      if (m < M) atomicAdd(ep.acc + (long)m * ep.ldw + ep.gidx[b], t * (sm * sm) * 5.9604644775390625e-08);   // 2^-24
+    } else if (ep.kind == OZ_EPI_PART) {
+      if (m < M) {
+        double* o = ep.part + ((long)ks * M + m) * N;
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          if (c + j < N) o[c + j] = fma((double)lo[j], 2.3283064365386963e-10, (double)hi[j]) * sm * sn[c + j];
+      }
+    } else {
+      const int mode = (b & 1) ? ep.mode_odd : ep.mode_even;
+      double* o = ep.out + (long)b * ep.out_bstride;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const int n = c + j;
+        if (m >= M || n >= N || (ep.lower && n > m)) continue;
+        double v = fma((double)lo[j], 2.3283064365386963e-10, (double)hi[j]) * sm * sn[n];
+        const long at = (long)m * ep.ldo + n;
+        if (mode != 0) v = -v;
+        if (ep.accumulate) v += o[at];
+        else if (mode == 1 && m == n) v += 1.0;
+        o[at] = v;
+        if (ep.lower && n < m) o[(long)n * ep.ldo + m] = v;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+  }
+}
+
+typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+PFN_encodeTiled encoder() {
+  static PFN_encodeTiled fn = nullptr;
+  if (!fn) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+            cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<PFN_encodeTiled>(p);
+  }
+  return fn;
+}
+
+// [batch * S][rows][ld] digits, boxes of BK columns x box_rows rows x S digits.
+bool map_digits(CUtensorMap* map, const void* ptr, int rows, int K, long planes, int box_rows) {
+  PFN_encodeTiled enc = encoder();
+  if (!enc || (reinterpret_cast<uintptr_t>(ptr) & 15)) return false;
+  const cuuint64_t ld = (cuuint64_t)oz_ld(K);
+  cuuint64_t dims[3] = {ld, (cuuint64_t)rows, (cuuint64_t)planes};
+  cuuint64_t strides[2] = {ld * 2, ld * 2 * (cuuint64_t)rows};
+  cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, (cuuint32_t)S};
+  cuuint32_t es[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// ------------------------------------------------------------------ digits
+// 63-bit integer of x scaled by 2^(62 - e), rounded to nearest (ties away), for |x| <= 2^e; pure integer arithmetic
+// (the FP64 pipe runs at 1/64 of the integer one).
+__device__ __forceinline__ long long to_fixed(double x, int e) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+  const int be = (int)((bits >> 52) & 0x7ff);
+  unsigned long long m = bits & 0xfffffffffffffull;
+  if (be) m |= 1ull << 52;
+  const int sh = (be ? be : 1) - 1075 + 62 - e;        // value = m 2^(be - 1075)
+  unsigned long long v;
+  if (sh >= 0) v = sh < 11 ? m << sh : 0ull;           // |x| <= 2^e keeps sh <= 10
+  else v = sh > -55 ? (m + (1ull << (-sh - 1))) >> (-sh) : 0ull;
+  return (bits >> 63) ? -(long long)v : (long long)v;
+}
+
+__device__ __forceinline__ int scale_exp(double sc) {   // sc is a power of two (or NaN: any exponent will do)
+  return (int)((__double_as_longlong(sc) >> 52) & 0x7ff) - 1023;
+}
+
+// Digits of eight consecutive elements: out[i] = the eight BF16 of digit i.
+__device__ __forceinline__ void digits8(const long long (&x)[8], uint4 (&out)[S]) {
+  uint32_t w[S][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    unsigned long long y[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) y[t] = (unsigned long long)x[2 * p + t] + 0x0080808080808080ull;
+#pragma unroll
+    for (int i = 0; i < S; ++i) {                      // digit 0 is the top byte (signed), the others byte - 128
+      float f[2];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const uint32_t byte = (uint32_t)(y[t] >> (8 * (S - 1 - i))) & 0xffu;
+        f[t] = i == 0 ? __uint_as_float(0x4b000000u | (byte ^ 0x80u)) - 8388736.f
+                      : __uint_as_float(0x4b000000u | byte) - 8388736.f;
+      }
+      __nv_bfloat162 v = __floats2bfloat162_rn(f[0], f[1]);
+      w[i][p] = *reinterpret_cast<uint32_t*>(&v);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < S; ++i) out[i] = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+}
+
+// One thread: eight columns of one row of entry blockIdx.z: x itself (a matrix per entry at stride xbs), or one x
+// times the entry's weights.
+template <bool WEIGHTED>
+__global__ void __launch_bounds__(128) oz_split_kernel(const double* __restrict__ x, long xbs, int rows, int k0,
+                                                       int cols, long ld, const double* __restrict__ sc,
+                                                       const double* __restrict__ w, long ldw,
+                                                       const double* __restrict__ wsc,
+                                                       __nv_bfloat16* __restrict__ dig, double* __restrict__ sc_out,
+                                                       int ldd) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.z;
+  const int c = 8 * g;
+  if (c >= ldd) return;
+  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+    const double s0 = sc[(WEIGHTED ? 0 : (long)b * rows) + r];
+    int e = scale_exp(s0);
+    if (WEIGHTED) {
+      const double sw = wsc[b];
+      e += scale_exp(sw);
+      if (g == 0) sc_out[(long)b * rows + r] = s0 * sw;
+    }
+    const double* xr = x + (WEIGHTED ? 0 : (long)b * xbs) + (long)r * ld + k0;
+    long long f[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      double v = 0.0;
+      if (c + t < cols) v = WEIGHTED ? xr[c + t] * w[(long)b * ldw + k0 + c + t] : xr[c + t];
+      f[t] = to_fixed(v, e);
+    }
+    uint4 d[S];
+    digits8(f, d);
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+      *reinterpret_cast<uint4*>(dig + (((long)b * S + i) * rows + r) * ldd + c) = d[i];
+  }
+}
+
+// Transposed operand: block of 32 source columns (operand rows) x 64 source rows through shared memory.
+__global__ void __launch_bounds__(256) oz_split_t_kernel(const double* __restrict__ x, int rows, int cols, long ld,
+                                                         const double* __restrict__ sc,
+                                                         __nv_bfloat16* __restrict__ dig, int ldd) {
+  __shared__ double t[64][33];
+  const int c0 = blockIdx.x * 32, p0 = blockIdx.y * 64;
+  for (int i = threadIdx.x; i < 64 * 32; i += 256) {
+    const int p = p0 + (i >> 5), c = c0 + (i & 31);
+    t[i >> 5][i & 31] = (p < rows && c < cols) ? x[(long)p * ld + c] : 0.0;
+  }
+  __syncthreads();
+  const int cc = threadIdx.x >> 3, g = threadIdx.x & 7;     // 32 operand rows x 8 groups of eight
+  const int c = c0 + cc, p = p0 + 8 * g;
+  if (c >= cols || p >= ldd) return;
+  const int e = scale_exp(sc[c]);
+  long long f[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) f[u] = to_fixed(t[8 * g + u][cc], e);
+  uint4 d[S];
+  digits8(f, d);
+#pragma unroll
+  for (int i = 0; i < S; ++i) *reinterpret_cast<uint4*>(dig + ((long)i * cols + c) * ldd + p) = d[i];
+}
+
+// Power of two from the largest magnitude's bits: 2^e with |x| <= 2^e (the next power), exponents kept inside
+// [-900, 900] so that products of scales stay finite; NaN if the row holds a NaN or an infinity.
+__device__ __forceinline__ double scale_of(unsigned long long mx) {
+  if (mx >= 0x7ff0000000000000ull) return __longlong_as_double(0x7ff8000000000000ll);
+  int e = (int)(mx >> 52) - 1022;                 // 2^e > |x|
+  if (mx == 0) e = 0;
+  if (e < -900) e = -900;
+  if (e > 900) return __longlong_as_double(0x7ff8000000000000ll);
+  return __longlong_as_double((long long)(1023 + e) << 52);
+}
+
+__global__ void __launch_bounds__(256) oz_row_scale_kernel(const double* __restrict__ x, long cols, long ld,
+                                                           double* __restrict__ sc) {
+  __shared__ unsigned long long red[8];
+  const long r = blockIdx.x;
+  unsigned long long mx = 0;
+  for (long k = threadIdx.x; k < cols; k += 256) {
+    const unsigned long long v = (unsigned long long)__double_as_longlong(x[r * ld + k]) & 0x7fffffffffffffffull;
+    mx = v > mx ? v : mx;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = v > mx ? v : mx;
+  }
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) mx = red[i] > mx ? red[i] : mx;
+    sc[r] = scale_of(mx);
+  }
+}
+
+__global__ void __launch_bounds__(256) oz_col_scale_kernel(const double* __restrict__ x, int rows, int cols, long ld,
+                                                           double* __restrict__ sc) {
+  __shared__ unsigned long long red[8][33];
+  const int c = blockIdx.x * 32 + (threadIdx.x & 31), w = threadIdx.x >> 5;
+  unsigned long long mx = 0;
+  if (c < cols)
+    for (int p = w; p < rows; p += 8) {
+      const unsigned long long v = (unsigned long long)__double_as_longlong(x[(long)p * ld + c]) & 0x7fffffffffffffffull;
+      mx = v > mx ? v : mx;
+    }
+  red[w][threadIdx.x & 31] = mx;
+  __syncthreads();
+  if (w == 0 && c < cols) {
+    for (int i = 1; i < 8; ++i) mx = red[i][threadIdx.x] > mx ? red[i][threadIdx.x] : mx;
+    sc[c] = scale_of(mx);
+  }
+}
+
+__global__ void oz_weight_kernel(const double* __restrict__ Dk, int K, const int* __restrict__ kinds,
+                                 const double* __restrict__ params, double eta, double* __restrict__ w) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
+  if (k >= K) return;
+  const int kind = kinds[b];
+  const double D = Dk[k], p = params[b];
+  double v;
+  if (kind == 0) {
+    v = -4.0 * D / (D * D + p * p);
+  } else {
+    const double a1 = p - D, a2 = -p - D, e2 = eta * eta;
+    const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
+    v = kind == 1 ? 2.0 * (a1 / d1 + a2 / d2) : 2.0 * (-eta / d1 - eta / d2);
+  }
+  w[(long)b * K + k] = v;
+}
+
+}  // namespace
+
+int oz_ld(int K) { return (K + 7) / 8 * 8; }
+size_t oz_elems(int rows, int K) { return (size_t)S * rows * oz_ld(K); }
+
+cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int batch, int M, int N, int K, const OzEpi& ep, int* err,
+                    cudaStream_t s) {
+  if (batch <= 0 || M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
+  if (batch > 65535) return cudaErrorInvalidValue;
+  OzMaps maps;
+  if (!map_digits(&maps.a, A.dig, M, K, (long)S * (A.batched ? batch : 1), BM) ||
+      !map_digits(&maps.b, B.dig, N, K, (long)S * (B.batched ? batch : 1), BN))
+    return cudaErrorInvalidValue;
+  static bool attr = false;
+  if (!attr) {
+    const cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  const long nbm = (M + BM - 1) / BM, nbn = (N + BN - 1) / BN;
+  const long tiles = ep.kind == OZ_EPI_STORE && ep.lower ? nbm * (nbm + 1) : nbm * nbn;
+  const long gx = tiles * (ep.kind == OZ_EPI_PART ? ep.ksplit : 1);
+  oz_gemm_kernel<<<dim3((unsigned)gx, batch), THREADS, SMEM_BYTES, s>>>(maps, M, N, K, A.batched, B.batched, A.sc, B.sc,
+                                                                       ep, err);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_row_scale(const double* x, int rows, long cols, long ld, double* sc, cudaStream_t s) {
+  if (rows > 0) oz_row_scale_kernel<<<rows, 256, 0, s>>>(x, cols, ld, sc);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_col_scale(const double* x, int rows, int cols, long ld, double* sc, cudaStream_t s) {
+  if (cols > 0) oz_col_scale_kernel<<<(cols + 31) / 32, 256, 0, s>>>(x, rows, cols, ld, sc);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_split(const double* x, long xbs, int rows, int k0, int cols, long ld, const double* sc, int nb,
+                     __nv_bfloat16* dig, cudaStream_t s) {
+  const int ldd = oz_ld(cols);
+  if (nb > 65535) return cudaErrorInvalidValue;
+  if (rows > 0 && cols > 0 && nb > 0)
+    oz_split_kernel<false><<<dim3((ldd / 8 + 127) / 128, std::min(rows, 65535), nb), 128, 0, s>>>(
+        x, xbs, rows, k0, cols, ld, sc, nullptr, 0, nullptr, dig, nullptr, ldd);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long ld, const double* sc, const double* w,
+                              long ldw, const double* wsc, int nb, __nv_bfloat16* dig, double* sc_out,
+                              cudaStream_t s) {
+  const int ldd = oz_ld(cols);
+  if (nb > 65535) return cudaErrorInvalidValue;
+  if (rows > 0 && cols > 0 && nb > 0)
+    oz_split_kernel<true><<<dim3((ldd / 8 + 127) / 128, std::min(rows, 65535), nb), 128, 0, s>>>(
+        x, 0, rows, k0, cols, ld, sc, w, ldw, wsc, dig, sc_out, ldd);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_split_transpose(const double* x, int rows, int cols, long ld, const double* sc, __nv_bfloat16* dig,
+                               cudaStream_t s) {
+  const int ldd = oz_ld(rows);
+  if (rows > 0 && cols > 0)
+    oz_split_t_kernel<<<dim3((cols + 31) / 32, (ldd + 63) / 64), 256, 0, s>>>(x, rows, cols, ld, sc, dig, ldd);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_pair_weights(const double* Dk, int K, const int* kinds, const double* params, double eta, int nb,
+                            double* w, cudaStream_t s) {
+  if (K > 0 && nb > 0) oz_weight_kernel<<<dim3((K + 255) / 256, nb), 256, 0, s>>>(Dk, K, kinds, params, eta, w);
+  return cudaGetLastError();
+}
+
+}  // namespace gw

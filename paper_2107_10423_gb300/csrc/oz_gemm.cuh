@@ -1,0 +1,60 @@
+// FP64 products on the BF16 tensor cores by exact integer digits (oz_gemm.cu).
+#pragma once
+#include <cuda_runtime.h>
+#include <cuda_bf16.h>
+#include <cstddef>
+
+namespace gw {
+
+constexpr int OZ_S = 8;              // digits per operand element
+
+// Digit operand: dig [batch][OZ_S][rows][ld] BF16 and sc [batch][rows] (the power of two of each row).
+struct OzOperand {
+  const __nv_bfloat16* dig;
+  const double* sc;
+  int batched;                       // 0: one matrix for every entry
+};
+
+enum { OZ_EPI_STORE = 0, OZ_EPI_PART = 1, OZ_EPI_SUMSQ = 2 };
+struct OzEpi {
+  int kind;
+  // OZ_EPI_STORE: out_b[m][n] = f(v) (f: 0 v, 1 delta_mn - v, 2 -v; even / odd entries), added to what is there when
+  // accumulate; lower != 0 computes the lower tiles and mirrors them
+  int mode_even, mode_odd, lower, accumulate;
+  double* out;
+  long out_bstride;
+  int ldo;
+  // OZ_EPI_PART: part[ks][m][n] = v of this K range (row length N)
+  double* part;
+  int ksplit;
+  // OZ_EPI_SUMSQ: acc[m * ldw + gidx[b]] += sum_n v[m][n]^2; the B rows are lower triangular (row n ends at column n)
+  double* acc;
+  int ldw;
+  const int* gidx;
+  const int* run_if;                 // if not NULL: the launch does nothing when *run_if == 0
+};
+
+int oz_ld(int K);                    // row length of the digit arrays
+size_t oz_elems(int rows, int K);    // BF16 elements of one matrix's digits
+// out_b[m][n] = f(sum_k A_b[m][k] B_b[n][k]) for b < batch.  *err receives a code if a bounded wait ran out.
+cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int batch, int M, int N, int K, const OzEpi& ep, int* err,
+                    cudaStream_t s);
+
+// Row scales sc[r] = 2^e >= max_k |x[r][k]| (NaN for a row with a NaN or infinity); rows of `cols` at stride ld.
+cudaError_t oz_row_scale(const double* x, int rows, long cols, long ld, double* sc, cudaStream_t s);
+// Digits of rows x_b[r][k0 .. k0 + cols) (stride ld, matrices b < nb at stride xbs) with the rows' scales sc [nb][rows].
+cudaError_t oz_split(const double* x, long xbs, int rows, int k0, int cols, long ld, const double* sc, int nb,
+                     __nv_bfloat16* dig, cudaStream_t s);
+// Digits of the transpose: row c of the operand is column c of x [rows][ld] (cols operand rows of length rows).
+cudaError_t oz_split_transpose(const double* x, int rows, int cols, long ld, const double* sc, __nv_bfloat16* dig,
+                               cudaStream_t s);
+cudaError_t oz_col_scale(const double* x, int rows, int cols, long ld, double* sc, cudaStream_t s);
+// Digits of x[r][k] w[b][k] for nb weight rows: scales sc_out[b][r] = sc[r] * wsc[b] (wsc from oz_row_scale of w).
+cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long ld, const double* sc, const double* w,
+                              long ldw, const double* wsc, int nb, __nv_bfloat16* dig, double* sc_out,
+                              cudaStream_t s);
+// FP64 weights w[b][k] of tc_pair_weights' kinds (row length K).
+cudaError_t oz_pair_weights(const double* Dk, int K, const int* kinds, const double* params, double eta, int nb,
+                            double* w, cudaStream_t s);
+
+}  // namespace gw
