@@ -41,6 +41,11 @@ void launch_op_gemm1(const T* V, const T* B, const double* Dk, long n_ov, int n_
                      int nr, T* U, int mode, cudaStream_t s, double* dw = nullptr,
                      double cut = 0.0, long ldb = 0,    // ldb: row length of B (0 = n_ov)
                      const int* run_if = nullptr);      // device flag: the launch does nothing if *run_if == 0
+// The same in FP64 for few right-hand sides (no padding of the rows): gemm1 modes 0 and 2 (no cut), gemm2 modes 0, 1.
+void launch_op_rows1(const double* V, const double* B, const double* Dk, long n_ov, int n_aux, const double* x,
+                     double eta, int nr, double* U, int mode, cudaStream_t s, double* dw, const int* run_if);
+void launch_op_rows2(const double* U, const double* B, int n_aux, long n_ov, int nr, const double* V, double* out,
+                     int mode, cudaStream_t s, const int* run_if);
 // Double-float (FP32 pair, 48-bit) versions of op_gemm1 mode 0 and op_gemm2 mode 1 for the refinement residual:
 // V, U, out FP64; B as its split Bh + Bl (launch_df_split of the FP64 B_ia): Bh [n_aux][ldh] is the FP32 rounding
 // of B (the plan's FP32 copy), Bl [n_aux][n_ov] the rounding of the remainder.  launch_df_split writes h only if it

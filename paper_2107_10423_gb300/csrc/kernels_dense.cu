@@ -548,6 +548,95 @@ __global__ void __launch_bounds__(NT) op_gemm2_kernel(const T* __restrict__ U, c
   }
 }
 
+// ------------------------------------------------------------------ the operator for few right-hand sides
+// FP64 runs at two multiply-adds a clock and SM, so the 64-row tiles above spend their time on padding when a batch has
+// 2 to 16 rows (91 us a product at n_aux 84, 95 pairs, 2 rows; 4 us here).  gemm1: 16 columns x 16 slices of the
+// contraction a CTA, RM rows; gemm2: one warp per output column.
+template <int RM>
+__global__ void __launch_bounds__(256) op_rows1_kernel(const double* __restrict__ V, const double* __restrict__ B,
+                                                       const double* __restrict__ Dk, long n_ov, int n_aux,
+                                                       const double* __restrict__ xs, double eta, int M,
+                                                       double* __restrict__ U, int mode, double* __restrict__ dw,
+                                                       const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  __shared__ double red[16][RM][17];
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const long k = blockIdx.x * 16L + tx;
+  const int m0 = blockIdx.y * RM;
+  double acc[RM];
+#pragma unroll
+  for (int i = 0; i < RM; ++i) acc[i] = 0.0;
+  if (k < n_ov)
+#pragma unroll 4
+    for (int P = ty; P < n_aux; P += 16) {
+      const double b = B[(long)P * n_ov + k];
+#pragma unroll
+      for (int i = 0; i < RM; ++i) acc[i] = fma(m0 + i < M ? V[(long)(m0 + i) * n_aux + P] : 0.0, b, acc[i]);
+    }
+#pragma unroll
+  for (int i = 0; i < RM; ++i) red[ty][i][tx] = acc[i];
+  __syncthreads();
+  const int pr = ty;                              // the CTA's pair of rows this thread finishes
+  const bool on = pr < RM / 2 && m0 + 2 * pr < M && k < n_ov;
+  double sum = 0.0;
+  if (on) {
+    double tr = 0.0, ti = 0.0;
+    for (int q = 0; q < 16; ++q) {
+      tr += red[q][2 * pr][tx];
+      ti -= red[q][2 * pr + 1][tx];
+    }
+    const int r = m0 + 2 * pr;
+    const double x = xs[r >> 1], D = Dk[k], e2 = eta * eta;
+    const double a1 = x - D, a2 = -x - D;
+    const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
+    if (mode == 2) {
+      const double q1r = (a1 * a1 - e2) / (d1 * d1), q1i = -2.0 * a1 * eta / (d1 * d1);
+      const double q2r = (a2 * a2 - e2) / (d2 * d2), q2i = -2.0 * a2 * eta / (d2 * d2);
+      sum = 2.0 * (-q1r + q2r) * (tr * tr - ti * ti) - 2.0 * (-q1i + q2i) * (2.0 * tr * ti);
+    } else {
+      const double cr = 2.0 * (a1 / d1 + a2 / d2), ci = -2.0 * eta * (1.0 / d1 + 1.0 / d2);
+      U[(long)r * n_ov + k] = cr * tr - ci * ti;
+      U[(long)(r + 1) * n_ov + k] = cr * ti + ci * tr;
+    }
+  }
+  if (mode == 2 && pr < RM / 2) {                 // whole half warps: 16 lanes of one pair
+    const unsigned mask = RM / 2 > 1 ? 0xffffffffu : 0xffffu;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(mask, sum, o);
+    if (tx == 0 && m0 + 2 * pr < M) atomicAdd(dw + ((m0 + 2 * pr) >> 1), sum);
+  }
+}
+
+template <int RM>
+__global__ void __launch_bounds__(128) op_rows2_kernel(const double* __restrict__ U, const double* __restrict__ B,
+                                                       int n_aux, long n_ov, int M, const double* __restrict__ V,
+                                                       double* __restrict__ out, int mode,
+                                                       const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  const int P = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31, m0 = blockIdx.y * RM;
+  if (P >= n_aux) return;
+  const double* b = B + (long)P * n_ov;
+  double acc[RM];
+#pragma unroll
+  for (int i = 0; i < RM; ++i) acc[i] = 0.0;
+#pragma unroll 4
+  for (long k = lane; k < n_ov; k += 32) {
+    const double v = b[k];
+#pragma unroll
+    for (int i = 0; i < RM; ++i) acc[i] = fma(m0 + i < M ? U[(long)(m0 + i) * n_ov + k] : 0.0, v, acc[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < RM; ++i) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+    const int r = m0 + i;
+    if (lane == 0 && r < M) {
+      const double vin = mode == 1 ? V[(long)r * n_aux + P] : 0.0;
+      out[(long)r * n_aux + P] = mode == 1 ? ((r & 1) ? -vin : vin) - acc[i] : acc[i];
+    }
+  }
+}
+
 // ------------------------------------------------------------------ double-float GEMMs (refinement residual)
 // A double x is carried as the FP32 pair (h, l), h = fl(x), l = fl(x - h): 48 significant bits.  A multiply-add
 // s += a b takes the product exactly to FP32 pair precision (h*h by an FMA error term, plus the two cross terms)
@@ -800,6 +889,25 @@ cudaError_t launch_trsm_w(const T* Lbase, long Lstride, int n, int n_g, const in
   void* args[] = {(void*)&Lbase, (void*)&Lstride, (void*)&n, (void*)&n_g, (void*)&g_out, (void*)&Bn,
                   (void*)&R, (void*)&W, (void*)&w_ld, (void*)&scratch};
   return cudaLaunchKernel((const void*)trsm_w_kernel<T>, dim3(grid), dim3(NT), args, smem, s);
+}
+
+void launch_op_rows1(const double* V, const double* B, const double* Dk, long n_ov, int n_aux, const double* x,
+                     double eta, int nr, double* U, int mode, cudaStream_t s, double* dw, const int* run_if) {
+  const unsigned gx = (unsigned)((n_ov + 15) / 16);
+  if (nr == 1)
+    op_rows1_kernel<2><<<dim3(gx, 1), 256, 0, s>>>(V, B, Dk, n_ov, n_aux, x, eta, 2, U, mode, dw, run_if);
+  else if (nr > 1)
+    op_rows1_kernel<4><<<dim3(gx, (nr + 1) / 2), 256, 0, s>>>(V, B, Dk, n_ov, n_aux, x, eta, 2 * nr, U, mode, dw,
+                                                              run_if);
+}
+
+void launch_op_rows2(const double* U, const double* B, int n_aux, long n_ov, int nr, const double* V, double* out,
+                     int mode, cudaStream_t s, const int* run_if) {
+  const unsigned gx = (n_aux + 3) / 4;
+  if (nr == 1)
+    op_rows2_kernel<2><<<dim3(gx, 1), 128, 0, s>>>(U, B, n_aux, n_ov, 2, V, out, mode, run_if);
+  else if (nr > 1)
+    op_rows2_kernel<4><<<dim3(gx, (nr + 1) / 2), 128, 0, s>>>(U, B, n_aux, n_ov, 2 * nr, V, out, mode, run_if);
 }
 
 template <typename T>

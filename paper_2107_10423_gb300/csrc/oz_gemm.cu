@@ -444,6 +444,134 @@ __global__ void oz_weight_kernel(const double* __restrict__ Dk, int K, const int
   w[(long)b * K + k] = v;
 }
 
+// ------------------------------------------------------------------ residue operator
+__device__ __forceinline__ unsigned long long block_max(unsigned long long mx, unsigned long long* red) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = v > mx ? v : mx;
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) mx = red[i] > mx ? red[i] : mx;
+  return mx;
+}
+
+__device__ __forceinline__ unsigned long long mag(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+
+// Digits of one row by the whole block, eight columns a thread.
+__device__ __forceinline__ void row_to_digits(const double* xr, int cols, int ldd, double sc, int rows, int r,
+                                              __nv_bfloat16* dig) {
+  const int e = scale_exp(sc);
+  for (int c = 8 * (int)threadIdx.x; c < ldd; c += 8 * blockDim.x) {
+    long long f[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) f[t] = to_fixed(c + t < cols ? xr[c + t] : 0.0, e);
+    uint4 d[S];
+    digits8(f, d);
+#pragma unroll
+    for (int i = 0; i < S; ++i) *reinterpret_cast<uint4*>(dig + ((long)i * rows + r) * ldd + c) = d[i];
+  }
+}
+
+__global__ void __launch_bounds__(128) oz_row_digits_kernel(const double* __restrict__ x, int rows, int cols, long ld,
+                                                            double* __restrict__ sc, __nv_bfloat16* __restrict__ dig,
+                                                            int ldd, const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  __shared__ unsigned long long red[4];
+  const int r = blockIdx.x;
+  const double* xr = x + (long)r * ld;
+  unsigned long long mx = 0;
+  for (int c = threadIdx.x; c < cols; c += blockDim.x) mx = max(mx, mag(xr[c]));
+  const double s = scale_of(block_max(mx, red));
+  if (threadIdx.x == 0) sc[r] = s;
+  row_to_digits(xr, cols, ldd, s, rows, r, dig);
+}
+
+__global__ void oz_pole_weight_kernel(const double* __restrict__ Dk, int K, const double* __restrict__ xs, double eta,
+                                      double2* __restrict__ cw) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+  if (k >= K) return;
+  const double x = xs[j], D = Dk[k], a1 = x - D, a2 = -x - D, e2 = eta * eta;
+  const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
+  cw[(long)j * K + k] = make_double2(2.0 * (a1 / d1 + a2 / d2), -2.0 * eta * (1.0 / d1 + 1.0 / d2));
+}
+
+// One CTA per right-hand side: the weights cost four FP64 multiply-adds a pair (their divisions are done once per
+// batch, not per iteration), the rest is memory traffic: T and cw in, U and 32 bytes of digits out.
+__global__ void __launch_bounds__(256) oz_pole_apply_kernel(double* __restrict__ T, int K,
+                                                            const double2* __restrict__ cw, int rows,
+                                                            double* __restrict__ sc, __nv_bfloat16* __restrict__ dig,
+                                                            int ldd, const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  __shared__ unsigned long long red[8];
+  const int j = blockIdx.x;
+  double* t0 = T + (long)(2 * j) * K;
+  double* t1 = t0 + K;
+  const double2* c = cw + (long)j * K;
+  unsigned long long m0 = 0, m1 = 0;
+  for (int k = threadIdx.x; k < K; k += blockDim.x) {
+    const double tr = t0[k], ti = -t1[k];
+    const double2 w = c[k];
+    const double u = w.x * tr - w.y * ti, v = w.x * ti + w.y * tr;
+    t0[k] = u;
+    t1[k] = v;
+    m0 = max(m0, mag(u));
+    m1 = max(m1, mag(v));
+  }
+  const double s0 = scale_of(block_max(m0, red)), s1 = scale_of(block_max(m1, red));
+  if (threadIdx.x == 0) {
+    sc[2 * j] = s0;
+    sc[2 * j + 1] = s1;
+  }
+  __syncthreads();
+  row_to_digits(t0, K, ldd, s0, rows, 2 * j, dig);
+  row_to_digits(t1, K, ldd, s1, rows, 2 * j + 1, dig);
+}
+
+__global__ void __launch_bounds__(256) oz_part_reduce_kernel(const double* __restrict__ part, int ksplit, long N, int n,
+                                                             const double* __restrict__ V, int mode,
+                                                             double* __restrict__ out,
+                                                             const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  for (long i = blockIdx.x * 256L + threadIdx.x; i < N; i += gridDim.x * 256L) {
+    double v = 0.0;
+    for (int q = 0; q < ksplit; ++q) v += part[q * N + i];
+    if (mode == 1) v = (((i / n) & 1) ? -V[i] : V[i]) - v;
+    out[i] = v;
+  }
+}
+
+__global__ void __launch_bounds__(256) oz_pole_derivative_kernel(const double* __restrict__ T, int K,
+                                                                 const double* __restrict__ Dk,
+                                                                 const double* __restrict__ xs, double eta,
+                                                                 double* __restrict__ dw) {
+  __shared__ double red[8];
+  const int j = blockIdx.x;
+  const double* t0 = T + (long)(2 * j) * K;
+  const double* t1 = t0 + K;
+  const double x = xs[j], e2 = eta * eta;
+  double sum = 0.0;
+  for (int k = threadIdx.x; k < K; k += blockDim.x) {
+    const double tr = t0[k], ti = -t1[k], D = Dk[k];
+    const double a1 = x - D, a2 = -x - D;
+    const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
+    const double q1r = (a1 * a1 - e2) / (d1 * d1), q1i = -2.0 * a1 * eta / (d1 * d1);
+    const double q2r = (a2 * a2 - e2) / (d2 * d2), q2i = -2.0 * a2 * eta / (d2 * d2);
+    const double cr = 2.0 * (-q1r + q2r), ci = 2.0 * (-q1i + q2i);
+    sum += cr * (tr * tr - ti * ti) - ci * (2.0 * tr * ti);
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) sum += red[i];
+    dw[j] = sum;
+  }
+}
+
 }  // namespace
 
 int oz_ld(int K) { return (K + 7) / 8 * 8; }
@@ -513,6 +641,40 @@ cudaError_t oz_split_transpose(const double* x, int rows, int cols, long ld, con
 cudaError_t oz_pair_weights(const double* Dk, int K, const int* kinds, const double* params, double eta, int nb,
                             double* w, cudaStream_t s) {
   if (K > 0 && nb > 0) oz_weight_kernel<<<dim3((K + 255) / 256, nb), 256, 0, s>>>(Dk, K, kinds, params, eta, w);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_row_digits(const double* x, int rows, int cols, long ld, double* sc, __nv_bfloat16* dig,
+                          const int* run_if, cudaStream_t s) {
+  if (rows > 0 && cols > 0) oz_row_digits_kernel<<<rows, 128, 0, s>>>(x, rows, cols, ld, sc, dig, oz_ld(cols), run_if);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_pole_weights(const double* Dk, int K, const double* xs, double eta, int nr, double2* cw,
+                            cudaStream_t s) {
+  if (nr > 65535) return cudaErrorInvalidValue;
+  if (nr > 0 && K > 0) oz_pole_weight_kernel<<<dim3((K + 255) / 256, nr), 256, 0, s>>>(Dk, K, xs, eta, cw);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_pole_apply(double* T, int K, const double2* cw, int nr, double* sc, __nv_bfloat16* dig,
+                          const int* run_if, cudaStream_t s) {
+  if (nr > 0) oz_pole_apply_kernel<<<nr, 256, 0, s>>>(T, K, cw, 2 * nr, sc, dig, oz_ld(K), run_if);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_part_reduce(const double* part, int ksplit, int rows, int n, const double* V, int mode, double* out,
+                           const int* run_if, cudaStream_t s) {
+  const long N = (long)rows * n;
+  if (N > 0)
+    oz_part_reduce_kernel<<<(unsigned)std::min<long>((N + 255) / 256, 2048), 256, 0, s>>>(part, ksplit, N, n, V, mode,
+                                                                                          out, run_if);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_pole_derivative(const double* T, int K, const double* Dk, const double* xs, double eta, int nr,
+                               double* dw, cudaStream_t s) {
+  if (nr > 0) oz_pole_derivative_kernel<<<nr, 256, 0, s>>>(T, K, Dk, xs, eta, dw);
   return cudaGetLastError();
 }
 

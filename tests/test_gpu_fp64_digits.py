@@ -60,3 +60,26 @@ def test_non_finite_input_is_a_numeric_error(gwlib, bad):
         with pytest.raises(gw.GWError) as e:
             p.screening()
     assert e.value.status == gw.GW_ERR_NUMERIC
+
+
+# one right-hand side, an odd few (SIMT rows), the first digit batch (16 rows: 8 right-hand sides) and a ragged larger
+# one, sizes on both sides of the 2^23 multiply-add line; max_rhs_batch splits the list into batches of unequal size
+@pytest.mark.parametrize("n_rhs,n_aux,n_virt,batch", [(1, 65, 20, 0), (3, 130, 33, 0), (8, 390, 150, 0),
+                                                      (37, 257, 95, 0), (70, 257, 95, 33), (9, 84, 19, 4)])
+def test_residues_fp64(gwlib, n_rhs, n_aux, n_virt, batch):
+    from paper_2107_10423_gb300 import gw
+    s = _system(n_aux, 9, n_virt)
+    B, Bn = s.b_ia(), s.b_nm()
+    r = np.random.default_rng(n_rhs)
+    m, x = r.integers(0, s.n_bas, n_rhs), r.uniform(-0.4, 0.4, n_rhs)     # inside the gap: MINRES converges
+    with gw.Plan(s.eps, s.n_occ, B, Bn, s.targets, minres_tol=1e-13, minres_maxit=200, minres_fallback_tol=1e-10,
+                 max_rhs_batch=batch) as p:
+        out = p.residues(np.zeros(n_rhs, dtype=np.int32), m, x)
+    assert not out["used_fallback"].any()
+    for j in range(n_rhs):
+        w, dw = O.w_corr_and_deriv(O.pi_complex(s.eps, s.n_occ, B, x[j], 1e-3),
+                                   O.dpi_complex(s.eps, s.n_occ, B, x[j], 1e-3), Bn[0, m[j]])
+        # relative residual 1e-13 times the condition number of 1 - Pi(x) in the gap (below 100) on W and dW
+        assert abs(out["w_re"][j] - w.real) < 1e-10 * max(1, abs(w))
+        assert abs(out["w_im"][j] - w.imag) < 1e-10 * max(1, abs(w))
+        assert abs(out["dw_re"][j] - dw.real) < 1e-9 * max(1, abs(dw))
