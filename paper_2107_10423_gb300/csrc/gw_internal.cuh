@@ -29,24 +29,22 @@ template <typename T>
 size_t trsm_w_scratch_elems(int n, int n_cta);
 int trsm_w_default_ctas();
 
-// Matrix-free operator of the residue systems (MINRES), for a batch of nr right-hand sides.
+// Matrix-free FP64 operator of the residue systems (MINRES), for a batch of nr right-hand sides.
 // V: [2nr][n_aux] pairs (u, v) encoding z = u - i v.
-// gemm1: mode 0: U[2j..2j+1][k] = c_k(x_j) * t_k, t = B^T z, with c_k(x) = 2[1/(x-D_k+i eta) + 1/(-x-D_k+i eta)];
-//   mode 2: dw[j] += sum_k Re(c'_k(x_j) t_k^2) in FP64, c' the x-derivative (dw zeroed by the caller, U unused), skipping the pairs
-//   with |x_j - D_k| < cut or |-x_j - D_k| < cut (added by launch_deriv_resonant).
+// gemm1: U[2j..2j+1][k] = c_k(x_j) * t_k, t = B^T z, with c_k(x) = 2[1/(x-D_k+i eta) + 1/(-x-D_k+i eta)].
 // gemm2: S[r][P] = sum_k U[r][k] B[P][k]; mode 0 writes S (= [Re; Im] of Pi z),
 //   mode 1 writes the real embedding [u - S_re; -v - S_im] of (1 - Pi) z.
+// run_if: device flag, the launch does nothing if *run_if == 0.
+void launch_op_gemm1(const double* V, const double* B, const double* Dk, long n_ov, int n_aux, const double* x,
+                     double eta, int nr, double* U, cudaStream_t s, const int* run_if = nullptr);
+void launch_op_gemm2(const double* U, const double* B, int n_aux, long n_ov, int nr, const double* V, double* out,
+                     int mode, cudaStream_t s, const int* run_if = nullptr);
+// dw[j] += sum_k Re(c'_k(x_j) t_k^2) in FP64, c' the x-derivative (dw zeroed by the caller), skipping the pairs with
+// |x_j - D_k| < cut or |-x_j - D_k| < cut (added by launch_deriv_resonant); ldb: row length of B.
 template <typename T>
-void launch_op_gemm1(const T* V, const T* B, const double* Dk, long n_ov, int n_aux, const double* x, double eta,
-                     int nr, T* U, int mode, cudaStream_t s, double* dw = nullptr,
-                     double cut = 0.0, long ldb = 0,    // ldb: row length of B (0 = n_ov)
-                     const int* run_if = nullptr);      // device flag: the launch does nothing if *run_if == 0
-// The same in FP64 for few right-hand sides (no padding of the rows): gemm1 modes 0 and 2 (no cut), gemm2 modes 0, 1.
-void launch_op_rows1(const double* V, const double* B, const double* Dk, long n_ov, int n_aux, const double* x,
-                     double eta, int nr, double* U, int mode, cudaStream_t s, double* dw, const int* run_if);
-void launch_op_rows2(const double* U, const double* B, int n_aux, long n_ov, int nr, const double* V, double* out,
-                     int mode, cudaStream_t s, const int* run_if);
-// Double-float (FP32 pair, 48-bit) versions of op_gemm1 mode 0 and op_gemm2 mode 1 for the refinement residual:
+void launch_deriv(const T* V, const T* B, const double* Dk, long n_ov, int n_aux, const double* x, double eta, int nr,
+                  double* dw, double cut, long ldb, cudaStream_t s);
+// Double-float (FP32 pair, 48-bit) versions of op_gemm1 and op_gemm2 mode 1 for the refinement residual:
 // V, U, out FP64; B as its split Bh + Bl (launch_df_split of the FP64 B_ia): Bh [n_aux][ldh] is the FP32 rounding
 // of B (the plan's FP32 copy), Bl [n_aux][n_ov] the rounding of the remainder.  launch_df_split writes h only if it
 // is not NULL.
@@ -55,15 +53,11 @@ void launch_op_gemm1_df(const double* V, const float* Bh, const float* Bl, long 
                         int n_aux, const double* x, double eta, int nr, double* U, cudaStream_t s);
 void launch_op_gemm2_df(const double* U, const float* Bh, const float* Bl, long ldh, int n_aux, int n_ov, int nr,
                         const double* V, double* out, cudaStream_t s);
-// The pairs that mode 2 skips, in FP64: dw[j] += Re(c'_k(x_j) t_k^2) with t from the FP64 rows of V64 and the FP64
+// The pairs that launch_deriv skips, in FP64: dw[j] += Re(c'_k(x_j) t_k^2) with t from the FP64 rows of V64 and the FP64
 // B_ia [n_aux][n_ov]; Dsort ascending pair energies with their pair indices kidx.
 void launch_deriv_resonant(const double* V64, const double* B, long n_ov, int n_aux, const double* Dsort,
                            const int* kidx, const double* xs, int nr, double eta, double cut, double* dw,
                            cudaStream_t s);
-template <typename T>
-void launch_op_gemm2(const T* U, const T* B, int n_aux, int n_ov, int nr, const T* V, T* out, int mode,
-                     cudaStream_t s, const int* run_if = nullptr);
-
 // ---------------------------------------------------------------- CD kernels (kernels_cd.cu)
 // Sigma_x of each target; occ_t (device [n_t], or NULL for n_occ everywhere): occupied states of its spin.
 void launch_sigma_x(const double* B_nm, int n_t, int n_bas, int n_aux, int n_occ, double* sx, cudaStream_t s,
@@ -101,9 +95,6 @@ void launch_minres_finish(const double* B_nm, int n_bas, int n_aux, const int* r
                           const double* x, const MinresState* st, double* w_re, double* w_im, int* iters,
                           double* resnorm, T* V, cudaStream_t s, double* V64 = nullptr);
 
-// Batched complex LU with partial pivoting (kernels_lu.cu): matrices b at Ar + b*stride, Ai + b*stride.
-template <typename T>
-void launch_zlu(T* Ar, T* Ai, long stride, int n, int batch, int* piv, int* info, cudaStream_t s);
 // Spectral-decomposition route (kernels_sd.cu): the Casida matrix M = D^1/2 (D + 4 B^T B) D^1/2 [Np][Np] (Np = N
 // rounded up to even, identity padding) and T = I; one cyclic Jacobi sweep of M (rotations accumulated in T, cs [Np]
 // work space); off[0] / off[1] = squared off-diagonal / diagonal Frobenius norms; Omega [N], V = 2 B D^1/2 T
@@ -118,15 +109,21 @@ cudaError_t sd_weights(const double* B, const double* Dk, const double* M, const
 cudaError_t sd_sigma(const double* w2, const double* Om, int N, int n_bas, const double* eps, const int* tmap,
                      const int* spin, const int* occ_t, int n_occ, const double* omega, int npts, double eta,
                      double* S, double* dS, cudaStream_t s);
-// Blocked FP32 LU of `batch` complex matrices (planes A and A + plane, matrix stride `stride`) with the trailing
-// updates on the tensor cores; same factors and pivot convention as launch_zlu.  work: work_elems BF16, at least
-// zlu_tc_work_elems(n, 1) (one matrix's split panel operands); the updates run in sub-batches that fit it.
-size_t zlu_tc_work_elems(int n, int batch);
-cudaError_t launch_zlu_tc(float* A, long stride, long plane, int n, int batch, int* piv, int* info,
-                          __nv_bfloat16* work, size_t work_elems, int* err, cudaStream_t s);
+// Blocked LU of `batch` complex matrices (planes A and A + plane, matrix stride `stride`, FP32 or FP64) with partial
+// pivoting, in place, trailing updates on the tensor cores.  perm [batch][n]: the row order as launch_zlu_solve reads it
+// (the original row at each row of the factors; the sequential swaps for n > 16384, FP64 8192); info[b]: 0, or the first zero pivot's column + 1.  Work space: work of work_elems BF16 (at least
+// zlu_operand_elems(n, 1, fp64); the batch runs in sub-batches that fit it), idx zlu_index_ints, linv zlu_linv_elems,
+// scales zlu_scale_elems (FP64 only).
+size_t zlu_operand_elems(int n, int batch, bool fp64);
+size_t zlu_index_ints(int batch);
+size_t zlu_linv_elems(int batch);
+size_t zlu_scale_elems(int n, int batch);
 template <typename T>
-void launch_zlu_solve(const T* Ar, const T* Ai, long stride, int n, int batch, const int* piv, T* yr, T* yi,
-                      long ystride, cudaStream_t s);
+cudaError_t launch_zlu(T* A, long stride, long plane, int n, int batch, int* perm, int* info, __nv_bfloat16* work,
+                       size_t work_elems, int* idx, T* linv, double* scales, int* err, cudaStream_t s);
+template <typename T>
+cudaError_t launch_zlu_solve(const T* Ar, const T* Ai, long stride, int n, int batch, const int* perm, T* yr, T* yi,
+                             long ystride, cudaStream_t s);
 // Fallback bookkeeping: for k < nf with slot index idx[k] (into the MINRES batch), set y planes = (b, 0) before
 // the solve (stage 0), or after it write W = b^T y - b^T b, resnorm 0 and the (u, v) = (y_r, -y_i) rows of V.
 template <typename T>

@@ -93,8 +93,7 @@ struct gw_plan {
   DevBuf sk_C;                // device copy of nodes.C
   std::vector<DevBuf*> bufs;
   int tc_tiles_n = 0;          // N_aux the tile-order table of the Pi kernel was built for
-  DevBuf oz_A, oz_B, oz_X, oz_sc, oz_w, op_B, op_BT, op_sc, op_scv, op_V, op_U, op_cw, op_part;
-  bool op_digits = false;           // op_B and op_BT hold the digits of B_ia and of its transpose (made per call)
+  DevBuf oz_A, oz_B, oz_X, oz_sc, oz_w, op_BT, op_sc, op_V;
     // FP64 products on the tensor cores: digits, inverse factors, scales, weights
   DevBuf ws_mat, ws_info, ws_gout, ws_xi, tc_part, tc_kind, tc_par, tc_err, tc_w, tc_tiles, ns_E, ns_X, ns_X2, ns_Xa, ns_Xb, ns_T, ns_lam,
       ns_E0, ns_vec;
@@ -102,7 +101,7 @@ struct gw_plan {
       mr_dwre, mr_it, mr_res, mr_cnt, mr_Vhi, mr_Vlo, mr_Uhi, mr_Ulo, mr_Vlo2, mr_Ulo2, mr_V64;
   DevBuf sg_I, sg_dI, sg_R, sg_dR, sg_om, sg_start, sg_coef, sg_act, sg_tmap, qp_st, qp_om0;
   DevBuf fb_A, fb_y, fb_piv, fb_info, fb_idx, fb_y64, fb_V32, fb_S32, fb_Vp, fb_Up, fb_x, fb_V64, fb_U64, fb_S64, fb_sel,
-      fb_pos, fb_rho, fb_xs, fb_Bl, fb_lu;
+      fb_pos, fb_rho, fb_xs, fb_Bl, fb_lu, fb_sw, fb_linv, fb_lus;
   int* h_cnt = nullptr;       // pinned
   std::string err;
   gw_stats stats{};
@@ -114,10 +113,10 @@ struct gw_plan {
   std::vector<Mark> marks;
 
   gw_plan() {
-    DevBuf* all[] = {&oz_A, &oz_B, &oz_X, &oz_sc, &oz_w, &op_B, &op_BT, &op_sc, &op_scv, &op_V, &op_U, &op_cw, &op_part, &ws_mat, &ws_info, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
+    DevBuf* all[] = {&oz_A, &oz_B, &oz_X, &oz_sc, &oz_w, &op_BT, &op_sc, &op_V, &ws_mat, &ws_info, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
                      &mr_v, &mr_d1, &mr_d2, &mr_x, &mr_st, &mr_rt, &mr_rm, &mr_xf, &mr_wre, &mr_wim,
                      &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
-                     &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_lu, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS};
+                     &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_lu, &fb_sw, &fb_linv, &fb_lus, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS};
     bufs.assign(all, all + sizeof(all) / sizeof(all[0]));
   }
 };
@@ -754,10 +753,10 @@ gw_status ensure_third_parts(gw_plan* P);
 // Half-width (Ha) of the window around each resonance x = +-D_ia whose derivative terms are computed in FP64.
 constexpr double kResonantCut = 0.1;
 
-// BF16 elements of the blocked LU's split panel operands for a fallback batch of fb matrices: the whole batch, or
-// as many matrices as fit in 1 GiB (at least one); the panel updates then run in sub-batches.
-size_t lu_work_elems(int n, long fb) {
-  const size_t one = gw::zlu_tc_work_elems(n, 1);
+// BF16 elements of the blocked LU's panel operands for a fallback batch of fb matrices: the whole batch, or as many
+// matrices as fit in 1 GiB (at least one); the LU then runs in sub-batches.
+size_t lu_work_elems(int n, long fb, bool fp64) {
+  const size_t one = gw::zlu_operand_elems(n, 1, fp64);
   const size_t cap = std::max(one, ((size_t)1 << 29) / std::max<size_t>(one, 1) * one);
   return std::min(one * (size_t)std::max(1L, fb), cap);
 }
@@ -793,8 +792,11 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
     TRY(ensure(P, P->fb_rho, sizeof(double) * fb));
     TRY(ensure(P, P->fb_sel, sizeof(int) * fb));
     TRY(ensure(P, P->fb_pos, sizeof(int) * fb));
-    TRY(ensure(P, P->fb_lu, sizeof(__nv_bfloat16) * lu_work_elems(n, fb)));
   }
+  TRY(ensure(P, P->fb_lu, sizeof(__nv_bfloat16) * lu_work_elems(n, fb, sizeof(T) == 8)));
+  TRY(ensure(P, P->fb_sw, sizeof(int) * gw::zlu_index_ints(fb)));
+  TRY(ensure(P, P->fb_linv, sizeof(T) * gw::zlu_linv_elems(fb)));
+  if (sizeof(T) == 8) TRY(ensure(P, P->fb_lus, sizeof(double) * gw::zlu_scale_elems(n, fb)));
   CK(cudaMemcpyAsync(P->fb_idx.p, need.data(), sizeof(int) * nneed, cudaMemcpyHostToDevice, P->stream));
   std::vector<double> hx(nneed);
   {
@@ -838,20 +840,15 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
     LAUNCH(gw::launch_fallback_rhs<T>(P->d_B_nm, P->n_bas, n, rt, rm, as<int>(P->fb_idx) + k0, nf, as<T>(P->fb_y),
                                       P->stream));
     const size_t tl = tick(P);
-    if (sizeof(T) == 4) {
-      // FP32 factors, trailing updates on the tensor cores (about FP32-accurate six-product split); a bounded
-      // wait that runs out in its GEMMs is reported by the refinement operator's check below
-      CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
-      CK(gw::launch_zlu_tc(reinterpret_cast<float*>(A), (long)(2 * mat), (long)mat, n, nf, as<int>(P->fb_piv),
-                           as<int>(P->fb_info), as<__nv_bfloat16>(P->fb_lu), P->fb_lu.bytes / sizeof(__nv_bfloat16),
-                           as<int>(P->tc_err), P->stream));
-      P->stats.n_kernel_launches += 5 * ((n + 63) / 64);
-    } else {
-      LAUNCH(gw::launch_zlu<T>(A, A + mat, (long)(2 * mat), n, nf, as<int>(P->fb_piv), as<int>(P->fb_info),
-                               P->stream));
-    }
-    LAUNCH(gw::launch_zlu_solve<T>(A, A + mat, (long)(2 * mat), n, nf, as<int>(P->fb_piv), as<T>(P->fb_y),
-                                   as<T>(P->fb_y) + n, 2L * n, P->stream));
+    // trailing updates on the tensor cores (FP32: about FP32-accurate six-product split; FP64: exact digits); a bounded
+    // wait that runs out in them is reported by the check below (FP64) or by the refinement operator's (mixed)
+    CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
+    CK(gw::launch_zlu<T>(A, (long)(2 * mat), (long)mat, n, nf, as<int>(P->fb_piv), as<int>(P->fb_info),
+                         as<__nv_bfloat16>(P->fb_lu), P->fb_lu.bytes / sizeof(__nv_bfloat16), as<int>(P->fb_sw),
+                         as<T>(P->fb_linv), as<double>(P->fb_lus), as<int>(P->tc_err), P->stream));
+    P->stats.n_kernel_launches += 4 * ((n + 63) / 64);
+    LAUNCH(CK(gw::launch_zlu_solve<T>(A, A + mat, (long)(2 * mat), n, nf, as<int>(P->fb_piv), as<T>(P->fb_y),
+                                      as<T>(P->fb_y) + n, 2L * n, P->stream)));
     mark(P, 7, tl, nf * (8.0 / 3.0 * (double)n * n * n + 8.0 * (double)n * n));
     if (sizeof(T) == 4) {
       // iterative refinement with the FP32 factors (matrix-free residuals), solution accumulated in FP64
@@ -868,8 +865,8 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
         mark(P, 8, tr, 2.0 * 2.0 * (2.0 * nf) * n * (double)P->n_ov);
         LAUNCH(gw::launch_refine(1, P->d_B_nm, P->n_bas, n, rt, rm, idx, nf, y32, as<double>(P->fb_y64),
                                  as<float>(P->fb_V32), as<float>(P->fb_S32), P->stream));
-        LAUNCH(gw::launch_zlu_solve<T>(A, A + mat, (long)(2 * mat), n, nf, as<int>(P->fb_piv), as<T>(P->fb_y),
-                                       as<T>(P->fb_y) + n, 2L * n, P->stream));
+        LAUNCH(CK(gw::launch_zlu_solve<T>(A, A + mat, (long)(2 * mat), n, nf, as<int>(P->fb_piv), as<T>(P->fb_y),
+                                          as<T>(P->fb_y) + n, 2L * n, P->stream)));
         LAUNCH(gw::launch_refine(2, P->d_B_nm, P->n_bas, n, rt, rm, idx, nf, y32, as<double>(P->fb_y64),
                                  as<float>(P->fb_V32), nullptr, P->stream, nullptr, nullptr,
                                  P->cfg.refine_tol > 0.0 ? as<double>(P->fb_rho) : nullptr));
@@ -917,17 +914,17 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
             LAUNCH(gw::launch_op_gemm2_df(as<double>(P->fb_U64), P->d_B_ia_f, as<float>(P->fb_Bl), P->ld_f, n,
                                           P->n_ov, m, as<double>(P->fb_V64), as<double>(P->fb_S64), P->stream));
           } else {
-            LAUNCH(gw::launch_op_gemm1<double>(as<double>(P->fb_V64), P->d_B_ia, P->d_D, P->n_ov, n, as<double>(P->fb_xs), P->cfg.eta, m,
-                                               as<double>(P->fb_U64), 0, P->stream));
-            LAUNCH(gw::launch_op_gemm2<double>(as<double>(P->fb_U64), P->d_B_ia, n, P->n_ov, m,
-                                               as<double>(P->fb_V64), as<double>(P->fb_S64), 1, P->stream));
+            LAUNCH(gw::launch_op_gemm1(as<double>(P->fb_V64), P->d_B_ia, P->d_D, P->n_ov, n, as<double>(P->fb_xs),
+                                       P->cfg.eta, m, as<double>(P->fb_U64), P->stream));
+            LAUNCH(gw::launch_op_gemm2(as<double>(P->fb_U64), P->d_B_ia, n, P->n_ov, m, as<double>(P->fb_V64),
+                                       as<double>(P->fb_S64), 1, P->stream));
           }
           mark(P, 8, tr, 2.0 * 2.0 * (2.0 * m) * n * (double)P->n_ov);
           LAUNCH(gw::launch_refine(1, P->d_B_nm, P->n_bas, n, rt, rm, idx, nf, y32, as<double>(P->fb_y64),
                                    as<float>(P->fb_V32), nullptr, P->stream, as<double>(P->fb_S64),
                                    as<int>(P->fb_pos)));
-          LAUNCH(gw::launch_zlu_solve<T>(A, A + mat, (long)(2 * mat), n, nf, as<int>(P->fb_piv), as<T>(P->fb_y),
-                                         as<T>(P->fb_y) + n, 2L * n, P->stream));
+          LAUNCH(CK(gw::launch_zlu_solve<T>(A, A + mat, (long)(2 * mat), n, nf, as<int>(P->fb_piv), as<T>(P->fb_y),
+                                            as<T>(P->fb_y) + n, 2L * n, P->stream)));
           LAUNCH(gw::launch_refine(2, P->d_B_nm, P->n_bas, n, rt, rm, idx, nf, y32, as<double>(P->fb_y64),
                                    as<float>(P->fb_V32), nullptr, P->stream));
           P->stats.n_refine_fp64 += m;
@@ -938,6 +935,7 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
     } else {
       LAUNCH(gw::launch_fallback_finish<T>(P->d_B_nm, P->n_bas, n, rt, rm, as<int>(P->fb_idx) + k0, nf,
                                            as<T>(P->fb_y), w_re, w_im, resnorm, as<T>(P->mr_V), P->stream));
+      TRY(oz_check(P));
     }
     CK(cudaMemcpyAsync(info.data(), P->fb_info.p, sizeof(int) * nf, cudaMemcpyDeviceToHost, P->stream));
     CK(cudaStreamSynchronize(P->stream));
@@ -1028,100 +1026,41 @@ gw_status tc_operator3(gw_plan* P, int nf, const double* xf, const float* V32, f
   return GW_OK;
 }
 
-// ---------------------------------------------------------------- FP64 residue operator
-// Three forms by size.  Few rows (2 nr of them): SIMT kernels without row padding.  From 16 rows and 2^23 multiply-adds
-// a product on, digit products: at n_aux 377, 1695 pairs and 80 rows one product takes 0.03 ms there and 0.43 (gemm1)
-// or 1.76 (gemm2) in the 64 x 64 tiles, which remain for B too large to hold as digits (32 bytes an element).
-enum { OP_ROWS = 0, OP_DIGITS = 1, OP_TILES = 2 };
-bool op_digits_fit(size_t ws, int n, long K) {
-  return gw::oz_elems(n, (int)K) + gw::oz_elems((int)K, n) <= ws / 2 / sizeof(__nv_bfloat16);
-}
-int op_form(const gw_plan* P, int nr) {
-  const int n = P->cfg.n_aux;
-  const long K = P->n_ov;
-  if (2 * nr >= 16 && 2.0 * nr * n * K >= 8388608.0 && op_digits_fit(ws_bytes(P), n, K)) return OP_DIGITS;
-  return 2 * nr <= 16 || 2.0 * nr * n * K < 8388608.0 ? OP_ROWS : OP_TILES;
-}
-// K ranges of the second product: about one wave of CTAs.
-int op_ksplit(int rows, int n, int K) {
-  const int tiles = ((rows + 127) / 128) * ((n + 63) / 64), nch = (K + 127) / 128;
-  return std::max(1, std::min(nch, 148 / std::max(1, tiles)));
-}
+// ---------------------------------------------------------------- FP64 derivative pass
+// dW/dx = y^T Pi'(x) y for the rows V (y) of nr right-hand sides: t = V B by exact digits, then the weighted sum; where
+// the digits of B^T (16 bytes an element) do not fit, the fused FP64 product.
+bool deriv_digits_fit(size_t ws, int n, long K) { return gw::oz_elems((int)K, n) <= ws / 4 / sizeof(__nv_bfloat16); }
 
-// Buffers of the operator for batches of up to `batch` right-hand sides, and the weights of this one.
-gw_status op_prepare(gw_plan* P, int form, int batch, int nr, const double* xf) {
-  if (form != OP_DIGITS) return GW_OK;
-  const int n = P->cfg.n_aux, K = P->n_ov, M = 2 * batch;
-  TRY(ensure(P, P->tc_err, sizeof(int)));
-  TRY(ensure(P, P->op_sc, sizeof(double) * ((size_t)n + K)));
-  TRY(ensure(P, P->op_scv, sizeof(double) * 2 * (size_t)M));
-  TRY(ensure(P, P->op_B, sizeof(__nv_bfloat16) * gw::oz_elems(n, K)));
-  TRY(ensure(P, P->op_BT, sizeof(__nv_bfloat16) * gw::oz_elems(K, n)));
-  TRY(ensure(P, P->op_V, sizeof(__nv_bfloat16) * gw::oz_elems(M, n)));
-  TRY(ensure(P, P->op_U, sizeof(__nv_bfloat16) * gw::oz_elems(M, K)));
-  TRY(ensure(P, P->op_cw, sizeof(double2) * (size_t)batch * K));
-  TRY(ensure(P, P->op_part, sizeof(double) * (size_t)op_ksplit(2 * nr, n, K) * 2 * nr * n));
-  double* sc = as<double>(P->op_sc);
-  if (!P->op_digits) {
-    CK(gw::oz_row_scale(P->d_B_ia, n, K, K, sc, P->stream));
-    CK(gw::oz_split(P->d_B_ia, 0, n, 0, K, K, sc, 1, as<__nv_bfloat16>(P->op_B), P->stream));
-    CK(gw::oz_col_scale(P->d_B_ia, n, K, K, sc + n, P->stream));
-    CK(gw::oz_split_transpose(P->d_B_ia, n, K, K, sc + n, as<__nv_bfloat16>(P->op_BT), P->stream));
-    P->op_digits = true;
-    P->stats.n_kernel_launches += 4;
-  }
-  CK(gw::oz_pole_weights(P->d_D, K, xf, P->cfg.eta, nr, as<double2>(P->op_cw), P->stream));
-  P->stats.n_kernel_launches += 1;
-  return GW_OK;
-}
-
-// T = V B (mr_U) by digits.
-gw_status op_product1(gw_plan* P, int nr, const double* V, const int* run_if) {
+gw_status derivative64(gw_plan* P, int batch, int nr, const double* xf, const double* V, double* dw, bool* have_BT) {
   const int n = P->cfg.n_aux, K = P->n_ov, M = 2 * nr;
-  double* sc = as<double>(P->op_sc);
-  double* scV = as<double>(P->op_scv);
-  CK(gw::oz_row_digits(V, M, n, n, scV, as<__nv_bfloat16>(P->op_V), run_if, P->stream));
-  gw::OzEpi e1{};
-  e1.kind = gw::OZ_EPI_STORE;
-  e1.out = as<double>(P->mr_U);
-  e1.ldo = K;
-  e1.run_if = run_if;
-  CK(gw::oz_gemm(gw::OzOperand{as<__nv_bfloat16>(P->op_V), scV, 0}, gw::OzOperand{as<__nv_bfloat16>(P->op_BT), sc + n, 0},
-                 1, M, K, n, e1, as<int>(P->tc_err), P->stream));
-  P->stats.n_kernel_launches += 2;
-  return GW_OK;
-}
-
-// S = Pi(x) z (mode 0: [Re; Im]) or the embedded (1 - Pi(x)) z (mode 1) for the rows V [2 nr][n].
-gw_status op_apply(gw_plan* P, int form, int batch, int nr, const double* xf, const double* V, double* S, int mode,
-                   const int* run_if) {
-  const int n = P->cfg.n_aux, K = P->n_ov;
-  double* U = as<double>(P->mr_U);
-  if (form == OP_TILES) {
-    LAUNCH(gw::launch_op_gemm1<double>(V, P->d_B_ia, P->d_D, K, n, xf, P->cfg.eta, nr, U, 0, P->stream, nullptr, 0.0, 0,
-                                       run_if));
-    LAUNCH(gw::launch_op_gemm2<double>(U, P->d_B_ia, n, K, nr, V, S, mode, P->stream, run_if));
+  // below 2^23 multiply-adds a digit product has no more than a wave of short tiles to gain
+  if ((double)M * n * K < 8388608.0 || !deriv_digits_fit(ws_bytes(P), n, K)) {
+    LAUNCH(gw::launch_deriv<double>(V, P->d_B_ia, P->d_D, K, n, xf, P->cfg.eta, nr, dw, 0.0, K, P->stream));
     return GW_OK;
   }
-  if (form == OP_ROWS) {
-    LAUNCH(gw::launch_op_rows1(V, P->d_B_ia, P->d_D, K, n, xf, P->cfg.eta, nr, U, 0, P->stream, nullptr, run_if));
-    LAUNCH(gw::launch_op_rows2(U, P->d_B_ia, n, K, nr, V, S, mode, P->stream, run_if));
-    return GW_OK;
+  TRY(ensure(P, P->tc_err, sizeof(int)));
+  TRY(ensure(P, P->op_sc, sizeof(double) * (K + 2 * (size_t)batch)));
+  TRY(ensure(P, P->op_BT, sizeof(__nv_bfloat16) * gw::oz_elems(K, n)));
+  TRY(ensure(P, P->op_V, sizeof(__nv_bfloat16) * gw::oz_elems(2 * batch, n)));
+  double* scB = as<double>(P->op_sc);
+  double* scV = scB + K;
+  if (!*have_BT) {                      // once per residue call
+    CK(gw::oz_col_scale(P->d_B_ia, n, K, K, scB, P->stream));
+    CK(gw::oz_split_transpose(P->d_B_ia, n, K, K, scB, as<__nv_bfloat16>(P->op_BT), P->stream));
+    P->stats.n_kernel_launches += 2;
+    *have_BT = true;
   }
-  double* sc = as<double>(P->op_sc);
-  double* scU = as<double>(P->op_scv) + 2 * batch;
-  TRY(op_product1(P, nr, V, run_if));
-  CK(gw::oz_pole_apply(U, K, as<double2>(P->op_cw), nr, scU, as<__nv_bfloat16>(P->op_U), run_if, P->stream));
-  gw::OzEpi e2{};
-  e2.kind = gw::OZ_EPI_PART;
-  e2.part = as<double>(P->op_part);
-  e2.ksplit = op_ksplit(2 * nr, n, K);
-  e2.run_if = run_if;
-  CK(gw::oz_gemm(gw::OzOperand{as<__nv_bfloat16>(P->op_U), scU, 0}, gw::OzOperand{as<__nv_bfloat16>(P->op_B), sc, 0}, 1,
-                 2 * nr, n, K, e2, as<int>(P->tc_err), P->stream));
-  CK(gw::oz_part_reduce(as<double>(P->op_part), e2.ksplit, 2 * nr, n, V, mode, S, run_if, P->stream));
+  CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
+  CK(gw::oz_row_digits(V, M, n, n, scV, as<__nv_bfloat16>(P->op_V), P->stream));
+  gw::OzEpi e{};
+  e.kind = gw::OZ_EPI_STORE;
+  e.out = as<double>(P->mr_U);
+  e.ldo = K;
+  CK(gw::oz_gemm(gw::OzOperand{as<__nv_bfloat16>(P->op_V), scV, 0}, gw::OzOperand{as<__nv_bfloat16>(P->op_BT), scB, 0},
+                 1, M, K, n, e, as<int>(P->tc_err), P->stream));
+  CK(gw::oz_pole_derivative(as<double>(P->mr_U), K, P->d_D, xf, P->cfg.eta, nr, dw, P->stream));
   P->stats.n_kernel_launches += 3;
-  return GW_OK;
+  return oz_check(P);
 }
 
 // ---------------------------------------------------------------- batched residue solves
@@ -1161,7 +1100,7 @@ gw_status residues_T(gw_plan* P, int nr_total, const int* d_rt, const int* d_rm,
     CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
   }
   const double eta = P->cfg.eta;
-  P->op_digits = false;
+  bool have_BT = false;
   std::vector<double> h_res;
   for (int j0 = 0; j0 < nr_total; j0 += batch) {
     const int nr = std::min(batch, nr_total - j0);
@@ -1170,14 +1109,13 @@ gw_status residues_T(gw_plan* P, int nr_total, const int* d_rt, const int* d_rm,
     const double* xf = d_xf + j0;
     LAUNCH(gw::launch_gather_rhs<T>(P->d_B_nm, P->n_bas, n, rt, rm, nr, as<T>(P->mr_V), P->stream));
     // rhs = Pi(x) b
-    int form = OP_TILES;
     if (tcop) {
       TRY(tc_operator(P, nr, xf, reinterpret_cast<const float*>(P->mr_V.p), reinterpret_cast<float*>(P->mr_S.p), 0));
     } else {
-      form = op_form(P, nr);
-      TRY(op_prepare(P, form, batch, nr, xf));
-      if (form == OP_DIGITS) CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
-      TRY(op_apply(P, form, batch, nr, xf, as<double>(P->mr_V), as<double>(P->mr_S), 0, nullptr));
+      LAUNCH(gw::launch_op_gemm1(as<double>(P->mr_V), P->d_B_ia, P->d_D, n_ov, n, xf, eta, nr, as<double>(P->mr_U),
+                                 P->stream));
+      LAUNCH(gw::launch_op_gemm2(as<double>(P->mr_U), P->d_B_ia, n, n_ov, nr, as<double>(P->mr_V),
+                                 as<double>(P->mr_S), 0, P->stream));
     }
     LAUNCH(gw::launch_minres_init<T>(as<T>(P->mr_S), nr, n, as<double>(P->mr_vprev), as<double>(P->mr_v),
                                      as<double>(P->mr_d1), as<double>(P->mr_d2), as<double>(P->mr_x),
@@ -1199,7 +1137,11 @@ gw_status residues_T(gw_plan* P, int nr_total, const int* d_rt, const int* d_rm,
           cap = tc_operator(P, nr, xf, reinterpret_cast<const float*>(P->mr_V.p),
                             reinterpret_cast<float*>(P->mr_S.p), 1, cnt);
         } else {
-          cap = op_apply(P, form, batch, nr, xf, as<double>(P->mr_V), as<double>(P->mr_S), 1, cnt);
+          gw::launch_op_gemm1(as<double>(P->mr_V), P->d_B_ia, P->d_D, n_ov, n, xf, eta, nr, as<double>(P->mr_U),
+                              P->stream, cnt);
+          gw::launch_op_gemm2(as<double>(P->mr_U), P->d_B_ia, n, n_ov, nr, as<double>(P->mr_V), as<double>(P->mr_S), 1,
+                              P->stream, cnt);
+          P->stats.n_kernel_launches += 2;
         }
         if (cudaMemsetAsync(cnt, 0, sizeof(int), P->stream) != cudaSuccess) cap = GW_ERR_CUDA;
         gw::launch_minres_step<T>(as<T>(P->mr_S), nr, n, P->cfg.minres_tol, as<double>(P->mr_vprev),
@@ -1235,7 +1177,7 @@ gw_status residues_T(gw_plan* P, int nr_total, const int* d_rt, const int* d_rm,
       if (tg != (size_t)-1 && tg1 != (size_t)-1) P->marks.push_back({4, tg, tg1, op_flops * ran});
       P->stats.launches_kernel[4] += ran;
     }
-    if (tcop || form == OP_DIGITS) {
+    if (tcop) {
       int herr = 0;
       CK(cudaMemcpyAsync(&herr, P->tc_err.p, sizeof(int), cudaMemcpyDeviceToHost, P->stream));
       CK(cudaStreamSynchronize(P->stream));
@@ -1261,23 +1203,14 @@ gw_status residues_T(gw_plan* P, int nr_total, const int* d_rt, const int* d_rm,
     CK(cudaMemsetAsync(dw_re + j0, 0, sizeof(double) * nr, P->stream));
     const size_t td = tick(P);
     if (d64) {
-      LAUNCH(gw::launch_op_gemm1<double>(V64, P->d_B_ia, P->d_D, P->n_ov, n, xf, eta, nr,
-                                         nullptr, 2, P->stream, dw_re + j0));
+      LAUNCH(gw::launch_deriv<double>(V64, P->d_B_ia, P->d_D, n_ov, n, xf, eta, nr, dw_re + j0, 0.0, n_ov, P->stream));
     } else if (sizeof(T) == 4) {
-      LAUNCH(gw::launch_op_gemm1<float>(as<float>(P->mr_V), P->d_B_ia_f, P->d_D, P->n_ov, n, xf, eta, nr, nullptr, 2,
-                                        P->stream, dw_re + j0, kResonantCut, P->ld_f));
+      LAUNCH(gw::launch_deriv<float>(as<float>(P->mr_V), P->d_B_ia_f, P->d_D, n_ov, n, xf, eta, nr, dw_re + j0,
+                                     kResonantCut, P->ld_f, P->stream));
       LAUNCH(gw::launch_deriv_resonant(V64, P->d_B_ia, n_ov, n, P->d_Dsort, P->d_Dkidx, xf, nr, eta, kResonantCut,
                                        dw_re + j0, P->stream));
-    } else if (form == OP_DIGITS) {
-      TRY(op_product1(P, nr, as<double>(P->mr_V), nullptr));
-      LAUNCH(CK(gw::oz_pole_derivative(as<double>(P->mr_U), n_ov, P->d_D, xf, eta, nr, dw_re + j0, P->stream)));
-      TRY(oz_check(P));
-    } else if (form == OP_ROWS) {
-      LAUNCH(gw::launch_op_rows1(as<double>(P->mr_V), P->d_B_ia, P->d_D, n_ov, n, xf, eta, nr, nullptr, 2, P->stream,
-                                 dw_re + j0, nullptr));
     } else {
-      LAUNCH(gw::launch_op_gemm1<double>(as<double>(P->mr_V), P->d_B_ia, P->d_D, P->n_ov, n, xf, eta, nr, nullptr, 2,
-                                         P->stream, dw_re + j0));
+      TRY(derivative64(P, batch, nr, xf, as<double>(P->mr_V), dw_re + j0, &have_BT));
     }
     mark(P, 4, td, 2.0 * (2.0 * nr) * n * (double)n_ov);
   }
@@ -2337,10 +2270,8 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
                                    : std::max<u64>(1, std::min<u64>((ws / 2) / (2 * n_ov * ts), 2048));
   batch = std::min(batch, std::max<u64>(1, rows));
   b += batch * (4 * n * ts + 2 * n_ov * ts + 10 * n * 8 + 64);               // V, S, U, Lanczos vectors, state
-  if (!mixed && op_digits_fit((size_t)ws, c->n_aux, (long)n_ov)) {             // digits of B, B^T, V, U; pole weights
-    b += 16 * (n * ldo + n_ov * ldn + 2 * batch * (ldn + ldo)) + 16 * batch * n_ov + 8 * (n + n_ov + 4 * batch);
-    b += 8 * std::max<u64>(2 * batch * n, 148 * 128 * 64);                      // partial products, one wave of tiles
-  }
+  if (!mixed && deriv_digits_fit((size_t)ws, c->n_aux, (long)n_ov))            // digits of B^T and V
+    b += 16 * (n_ov * ldn + 2 * batch * ldn) + 8 * (n_ov + 2 * batch);
   if (mixed) {
     b += batch * (16 * n + 8 * ldn + 8 * ldo);                               // FP64 solutions, split V and U
     if (c->op_parts >= 3) b += batch * (4 * ldn + 4 * ldo);
@@ -2353,8 +2284,9 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
   if (mixed) {
     b += fb * (16 * n + 16 * n + 12 * ldn + 12 * ldo + 40);                  // FP64 solutions, V/S, split parts
     b += fb * (32 * n + 16 * n_ov) + 4 * n * n_ov;                           // FP64-residual vectors, df lo part of B
-    b += 2 * (u64)lu_work_elems(c->n_aux, (long)std::min<u64>(fb, 1u << 30));            // blocked-LU split operands
   }
+  b += 2 * (u64)lu_work_elems(c->n_aux, (long)std::min<u64>(fb, 1u << 30), !mixed);      // blocked-LU operands
+  b += fb * (4 * (u64)gw::zlu_index_ints(1) + ts * (u64)gw::zlu_linv_elems(1) + (mixed ? 0 : 8 * (u64)gw::zlu_scale_elems(c->n_aux, 1)));
   *bytes = b;
   return GW_OK;
 }

@@ -1,7 +1,8 @@
 // Dense kernels of the CD-G0W0 path (SIMT, templated on the arithmetic type):
 //  * batched in-place Cholesky of eps(i xi) = 1 - Pi (SPD, Sec. 3.3 text after "inn");
 //  * triangular solves that turn the factors into the table W^c_nm(i xi) (Algorithm 1, imaginary-grid loop);
-//  * the two skinny GEMMs of the matrix-free residue operator 1 - Pi(x) (Sec. 3.3, MINRES paragraph).
+//  * the two skinny products of the FP64 matrix-free residue operator 1 - Pi(x) (Sec. 3.3, MINRES paragraph) and the
+//    derivative pass.
 #include "gw_internal.cuh"
 #include "gw.h"
 
@@ -309,15 +310,14 @@ __global__ void __launch_bounds__(NT) trsm_w_kernel(const T* __restrict__ Lbase,
   }
 }
 
-// ------------------------------------------------------------------ residue operator GEMMs
-// gemm1: rows r in [0, 2nr), cols k in [0, n_ov): acc = sum_P V[r][P] B[P][k]  (B is N-contiguous here)
+// ------------------------------------------------------------------ derivative pass
+// dw[j] += sum_k Re(c'_k(x_j) t_k^2) in FP64, t = V B over rows r in [0, 2nr) and the columns k (B is N-contiguous), the
+// reduction fused into the product's epilogue (no N_ov-sized output); pairs within `cut` of resonance left out.
 template <typename T>
-__global__ void __launch_bounds__(NT) op_gemm1_kernel(const T* __restrict__ V, const T* __restrict__ B,
-                                                      const double* __restrict__ Dk, long n_ov,
-                                                      int n_aux, const double* __restrict__ xs, double eta, int nr,
-                                                      T* __restrict__ U, int mode, double* __restrict__ dw,
-                                                      double cut, long ldb, const int* __restrict__ run_if) {
-  if (run_if && *run_if == 0) return;
+__global__ void __launch_bounds__(NT) deriv_kernel(const T* __restrict__ V, const T* __restrict__ B,
+                                                   const double* __restrict__ Dk, long n_ov, int n_aux,
+                                                   const double* __restrict__ xs, double eta, int nr,
+                                                   double* __restrict__ dw, double cut, long ldb) {
   __shared__ T As[TK][TM + 4];
   __shared__ T Bs[TK][TN + 4];
   const int M = 2 * nr;
@@ -361,58 +361,32 @@ __global__ void __launch_bounds__(NT) op_gemm1_kernel(const T* __restrict__ V, c
     __syncthreads();
   }
   const double e2 = eta * eta;
-  if (mode == 2) {
-    // derivative pass fused with its reduction: dw[j] += sum_k Re(c'_k(x_j) t_k^2) in FP64 (no U round trip),
-    // c' = 2[-(a1 - i eta)^2/d1^2 + (a2 - i eta)^2/d2^2]
-#pragma unroll
-    for (int ip = 0; ip < 2; ++ip) {
-      const int r = m0 + 2 * ty + 32 * ip;
-      double sum = 0.0;
-      if (r < M) {
-        const double x = xs[r >> 1];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const long k = k0c + tx + 16 * j;
-          if (k >= n_ov) continue;
-          const double tr = (double)acc[2 * ip][j], ti = -(double)acc[2 * ip + 1][j];
-          const double D = Dk[k];
-          const double a1 = x - D, a2 = -x - D;
-          if (fabs(a1) < cut || fabs(a2) < cut) continue;   // near resonance: FP64 pass (deriv_resonant)
-          const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
-          const double q1r = (a1 * a1 - e2) / (d1 * d1), q1i = -2.0 * a1 * eta / (d1 * d1);
-          const double q2r = (a2 * a2 - e2) / (d2 * d2), q2i = -2.0 * a2 * eta / (d2 * d2);
-          const double cr = 2.0 * (-q1r + q2r), ci = 2.0 * (-q1i + q2i);
-          sum += cr * (tr * tr - ti * ti) - ci * (2.0 * tr * ti);
-        }
-      }
-      // the 16 lanes tx of one ty hold the same row: reduce within each half warp
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if (tx == 0 && r < M) atomicAdd(dw + (r >> 1), sum);
-    }
-    return;
-  }
+  // c' = 2[-(a1 - i eta)^2/d1^2 + (a2 - i eta)^2/d2^2]
 #pragma unroll
   for (int ip = 0; ip < 2; ++ip) {
-    int r = m0 + 2 * ty + 32 * ip;           // even row of the pair
-    if (r >= M) continue;
-    int jr = r >> 1;
-    double x = xs[jr];
+    const int r = m0 + 2 * ty + 32 * ip;
+    double sum = 0.0;
+    if (r < M) {
+      const double x = xs[r >> 1];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      long k = k0c + tx + 16 * j;
-      if (k >= n_ov) continue;
-      double tr = (double)acc[2 * ip][j], ti = -(double)acc[2 * ip + 1][j];
-      const double D = Dk[k];
-      double a1 = x - D, a2 = -x - D;
-      double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
-      const double cr = 2.0 * (a1 / d1 + a2 / d2);
-      const double ci = -2.0 * eta * (1.0 / d1 + 1.0 / d2);
-      const double outr = cr * tr - ci * ti;
-      const double outi = cr * ti + ci * tr;
-      U[(long)r * n_ov + k] = (T)outr;
-      U[(long)(r + 1) * n_ov + k] = (T)outi;
+      for (int j = 0; j < 4; ++j) {
+        const long k = k0c + tx + 16 * j;
+        if (k >= n_ov) continue;
+        const double tr = (double)acc[2 * ip][j], ti = -(double)acc[2 * ip + 1][j];
+        const double D = Dk[k];
+        const double a1 = x - D, a2 = -x - D;
+        if (fabs(a1) < cut || fabs(a2) < cut) continue;   // near resonance: FP64 pass (deriv_resonant)
+        const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
+        const double q1r = (a1 * a1 - e2) / (d1 * d1), q1i = -2.0 * a1 * eta / (d1 * d1);
+        const double q2r = (a2 * a2 - e2) / (d2 * d2), q2i = -2.0 * a2 * eta / (d2 * d2);
+        const double cr = 2.0 * (-q1r + q2r), ci = 2.0 * (-q1i + q2i);
+        sum += cr * (tr * tr - ti * ti) - ci * (2.0 * tr * ti);
+      }
     }
+    // the 16 lanes tx of one ty hold the same row: reduce within each half warp
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (tx == 0 && r < M) atomicAdd(dw + (r >> 1), sum);
   }
 }
 
@@ -490,151 +464,88 @@ __global__ void __launch_bounds__(256) deriv_resonant_kernel(const double* __res
   }
 }
 
-// gemm2: rows r in [0, 2nr), cols P in [0, n_aux): acc = sum_k U[r][k] B[P][k]  (both K-contiguous)
-template <typename T>
-__global__ void __launch_bounds__(NT) op_gemm2_kernel(const T* __restrict__ U, const T* __restrict__ B, int n_aux,
-                                                      long n_ov, int nr, const T* __restrict__ V,
-                                                      T* __restrict__ out, int mode, const int* __restrict__ run_if) {
+// ------------------------------------------------------------------ FP64 residue operator
+// One output a thread, one row a warp: a CTA takes CR rows x 32 columns, its warps without a row do nothing.  FP64 runs
+// at two multiply-adds a clock and SM (16 clocks a warp instruction), so a tile must not pad: 64 x 64 tiles spent 91 us
+// on a product of 2 rows, 84 and 95 long, and 3.2 ms on one of 382 rows, 504 and 3040 long on 48 CTAs (here 4 us and
+// 1.1 ms, the FP64 pipe's own time).  Every output is one chain of FMAs in ascending order, as in those tiles: MINRES
+// amplifies a last-bit difference of its operator to 1e-2 of a residual norm within 25 steps near a resonance, so the
+// order is kept (products by exact digits take a sixth of the time, but round differently).
+constexpr int CR = 8, CK = 32;
+
+// gemm1: t = V B, then U[2j], U[2j + 1] = Re, Im of c_k(x_j) (t[2j] - i t[2j + 1]).
+__global__ void __launch_bounds__(256) op_chain1_kernel(const double* __restrict__ V, const double* __restrict__ B,
+                                                        const double* __restrict__ Dk, long n_ov, int n_aux,
+                                                        const double* __restrict__ xs, double eta, int M,
+                                                        double* __restrict__ U, const int* __restrict__ run_if) {
   if (run_if && *run_if == 0) return;
-  __shared__ T As[TK][TM + 4];
-  __shared__ T Bs[TK][TN + 4];
-  const int M = 2 * nr;
-  const int m0 = blockIdx.y * TM;
-  const int q0 = blockIdx.x * TN;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  T acc[4][4];
+  __shared__ double As[CR][CK];
+  __shared__ double Bs[CK][32];
+  __shared__ double Ts[CR][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, m0 = blockIdx.y * CR, r = m0 + w;
+  const long k = blockIdx.x * 32L + lane;
+  double acc = 0.0;
+  for (int p0 = 0; p0 < n_aux; p0 += CK) {
+    As[w][lane] = (r < M && p0 + lane < n_aux) ? V[(long)r * n_aux + p0 + lane] : 0.0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int u = 0; u < CK / 8; ++u) {
+      const int P = p0 + w + 8 * u;
+      Bs[w + 8 * u][lane] = (P < n_aux && k < n_ov) ? B[(long)P * n_ov + k] : 0.0;
+    }
+    __syncthreads();
+    if (r < M)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-  const int lr = tid >> 2, lk = (tid & 3) * 4;
-  for (long k0 = 0; k0 < n_ov; k0 += TK) {
+      for (int kk = 0; kk < CK; ++kk) acc = fma(As[w][kk], Bs[kk][lane], acc);
+    __syncthreads();
+  }
+  Ts[w][lane] = acc;
+  __syncthreads();
+  if ((w & 1) || r >= M || k >= n_ov) return;
+  const double tr = acc, ti = -Ts[w + 1][lane];
+  // every rounding spelled out, for the same reason
+  const double x = xs[r >> 1], e2 = __dmul_rn(eta, eta);
+  const double D = Dk[k];
+  const double a1 = x - D, a2 = -x - D;
+  const double d1 = fma(a1, a1, e2), d2 = fma(a2, a2, e2);
+  const double cr = 2.0 * __dadd_rn(a1 / d1, a2 / d2);
+  const double ci = -2.0 * eta * __dadd_rn(1.0 / d1, 1.0 / d2);
+  const double outr = fma(cr, tr, -__dmul_rn(ci, ti));
+  const double outi = fma(ci, tr, __dmul_rn(cr, ti));
+  U[(long)r * n_ov + k] = outr;
+  U[(long)(r + 1) * n_ov + k] = outi;
+}
+
+// gemm2: out[r][P] = sum_k U[r][k] B[P][k] (mode 0), or the embedding [u - acc; -v - acc] (mode 1).
+__global__ void __launch_bounds__(256) op_chain2_kernel(const double* __restrict__ U, const double* __restrict__ B,
+                                                        int n_aux, long n_ov, int M, const double* __restrict__ V,
+                                                        double* __restrict__ out, int mode,
+                                                        const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  __shared__ double As[CR][CK];
+  __shared__ double Bs[32][CK + 1];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, m0 = blockIdx.y * CR, r = m0 + w;
+  const int q0 = blockIdx.x * 32, P = q0 + lane;
+  double acc = 0.0;
+  for (long k0 = 0; k0 < n_ov; k0 += CK) {
+    const long k = k0 + lane;
+    As[w][lane] = (r < M && k < n_ov) ? U[(long)r * n_ov + k] : 0.0;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      long k = k0 + lk + u;
-      As[lk + u][lr] = (m0 + lr < M && k < n_ov) ? U[(long)(m0 + lr) * n_ov + k] : T(0);
-      Bs[lk + u][lr] = (q0 + lr < n_aux && k < n_ov) ? B[(long)(q0 + lr) * n_ov + k] : T(0);
+      const int q = w + 8 * u;
+      Bs[q][lane] = (q0 + q < n_aux && k < n_ov) ? B[(long)(q0 + q) * n_ov + k] : 0.0;
     }
     __syncthreads();
+    if (r < M)
 #pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      T a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][2 * ty + (i & 1) + 32 * (i >> 1)];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
+      for (int kk = 0; kk < CK; ++kk) acc = fma(As[w][kk], Bs[lane][kk], acc);
     __syncthreads();
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int r = m0 + 2 * ty + (i & 1) + 32 * (i >> 1);
-    if (r >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int P = q0 + tx + 16 * j;
-      if (P >= n_aux) continue;
-      T v = acc[i][j];
-      if (mode == 1) {
-        T vin = V[(long)r * n_aux + P];
-        v = ((r & 1) ? -vin : vin) - v;
-      }
-      out[(long)r * n_aux + P] = v;
-    }
+  if (r >= M || P >= n_aux) return;
+  if (mode == 1) {
+    const double vin = V[(long)r * n_aux + P];
+    acc = ((r & 1) ? -vin : vin) - acc;
   }
-}
-
-// ------------------------------------------------------------------ the operator for few right-hand sides
-// FP64 runs at two multiply-adds a clock and SM, so the 64-row tiles above spend their time on padding when a batch has
-// 2 to 16 rows (91 us a product at n_aux 84, 95 pairs, 2 rows; 4 us here).  gemm1: 16 columns x 16 slices of the
-// contraction a CTA, RM rows; gemm2: one warp per output column.
-template <int RM>
-__global__ void __launch_bounds__(256) op_rows1_kernel(const double* __restrict__ V, const double* __restrict__ B,
-                                                       const double* __restrict__ Dk, long n_ov, int n_aux,
-                                                       const double* __restrict__ xs, double eta, int M,
-                                                       double* __restrict__ U, int mode, double* __restrict__ dw,
-                                                       const int* __restrict__ run_if) {
-  if (run_if && *run_if == 0) return;
-  __shared__ double red[16][RM][17];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const long k = blockIdx.x * 16L + tx;
-  const int m0 = blockIdx.y * RM;
-  double acc[RM];
-#pragma unroll
-  for (int i = 0; i < RM; ++i) acc[i] = 0.0;
-  if (k < n_ov)
-#pragma unroll 4
-    for (int P = ty; P < n_aux; P += 16) {
-      const double b = B[(long)P * n_ov + k];
-#pragma unroll
-      for (int i = 0; i < RM; ++i) acc[i] = fma(m0 + i < M ? V[(long)(m0 + i) * n_aux + P] : 0.0, b, acc[i]);
-    }
-#pragma unroll
-  for (int i = 0; i < RM; ++i) red[ty][i][tx] = acc[i];
-  __syncthreads();
-  const int pr = ty;                              // the CTA's pair of rows this thread finishes
-  const bool on = pr < RM / 2 && m0 + 2 * pr < M && k < n_ov;
-  double sum = 0.0;
-  if (on) {
-    double tr = 0.0, ti = 0.0;
-    for (int q = 0; q < 16; ++q) {
-      tr += red[q][2 * pr][tx];
-      ti -= red[q][2 * pr + 1][tx];
-    }
-    const int r = m0 + 2 * pr;
-    const double x = xs[r >> 1], D = Dk[k], e2 = eta * eta;
-    const double a1 = x - D, a2 = -x - D;
-    const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
-    if (mode == 2) {
-      const double q1r = (a1 * a1 - e2) / (d1 * d1), q1i = -2.0 * a1 * eta / (d1 * d1);
-      const double q2r = (a2 * a2 - e2) / (d2 * d2), q2i = -2.0 * a2 * eta / (d2 * d2);
-      sum = 2.0 * (-q1r + q2r) * (tr * tr - ti * ti) - 2.0 * (-q1i + q2i) * (2.0 * tr * ti);
-    } else {
-      const double cr = 2.0 * (a1 / d1 + a2 / d2), ci = -2.0 * eta * (1.0 / d1 + 1.0 / d2);
-      U[(long)r * n_ov + k] = cr * tr - ci * ti;
-      U[(long)(r + 1) * n_ov + k] = cr * ti + ci * tr;
-    }
-  }
-  if (mode == 2 && pr < RM / 2) {                 // whole half warps: 16 lanes of one pair
-    const unsigned mask = RM / 2 > 1 ? 0xffffffffu : 0xffffu;
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(mask, sum, o);
-    if (tx == 0 && m0 + 2 * pr < M) atomicAdd(dw + ((m0 + 2 * pr) >> 1), sum);
-  }
-}
-
-template <int RM>
-__global__ void __launch_bounds__(128) op_rows2_kernel(const double* __restrict__ U, const double* __restrict__ B,
-                                                       int n_aux, long n_ov, int M, const double* __restrict__ V,
-                                                       double* __restrict__ out, int mode,
-                                                       const int* __restrict__ run_if) {
-  if (run_if && *run_if == 0) return;
-  const int P = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31, m0 = blockIdx.y * RM;
-  if (P >= n_aux) return;
-  const double* b = B + (long)P * n_ov;
-  double acc[RM];
-#pragma unroll
-  for (int i = 0; i < RM; ++i) acc[i] = 0.0;
-#pragma unroll 4
-  for (long k = lane; k < n_ov; k += 32) {
-    const double v = b[k];
-#pragma unroll
-    for (int i = 0; i < RM; ++i) acc[i] = fma(m0 + i < M ? U[(long)(m0 + i) * n_ov + k] : 0.0, v, acc[i]);
-  }
-#pragma unroll
-  for (int i = 0; i < RM; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-    const int r = m0 + i;
-    if (lane == 0 && r < M) {
-      const double vin = mode == 1 ? V[(long)r * n_aux + P] : 0.0;
-      out[(long)r * n_aux + P] = mode == 1 ? ((r & 1) ? -vin : vin) - acc[i] : acc[i];
-    }
-  }
+  out[(long)r * n_aux + P] = acc;
 }
 
 // ------------------------------------------------------------------ double-float GEMMs (refinement residual)
@@ -891,48 +802,29 @@ cudaError_t launch_trsm_w(const T* Lbase, long Lstride, int n, int n_g, const in
   return cudaLaunchKernel((const void*)trsm_w_kernel<T>, dim3(grid), dim3(NT), args, smem, s);
 }
 
-void launch_op_rows1(const double* V, const double* B, const double* Dk, long n_ov, int n_aux, const double* x,
-                     double eta, int nr, double* U, int mode, cudaStream_t s, double* dw, const int* run_if) {
-  const unsigned gx = (unsigned)((n_ov + 15) / 16);
-  if (nr == 1)
-    op_rows1_kernel<2><<<dim3(gx, 1), 256, 0, s>>>(V, B, Dk, n_ov, n_aux, x, eta, 2, U, mode, dw, run_if);
-  else if (nr > 1)
-    op_rows1_kernel<4><<<dim3(gx, (nr + 1) / 2), 256, 0, s>>>(V, B, Dk, n_ov, n_aux, x, eta, 2 * nr, U, mode, dw,
-                                                              run_if);
+void launch_op_gemm1(const double* V, const double* B, const double* Dk, long n_ov, int n_aux, const double* x,
+                     double eta, int nr, double* U, cudaStream_t s, const int* run_if) {
+  const dim3 grid((unsigned)((n_ov + 31) / 32), (2 * nr + CR - 1) / CR);
+  if (nr > 0) op_chain1_kernel<<<grid, 256, 0, s>>>(V, B, Dk, n_ov, n_aux, x, eta, 2 * nr, U, run_if);
 }
 
-void launch_op_rows2(const double* U, const double* B, int n_aux, long n_ov, int nr, const double* V, double* out,
+void launch_op_gemm2(const double* U, const double* B, int n_aux, long n_ov, int nr, const double* V, double* out,
                      int mode, cudaStream_t s, const int* run_if) {
-  const unsigned gx = (n_aux + 3) / 4;
-  if (nr == 1)
-    op_rows2_kernel<2><<<dim3(gx, 1), 128, 0, s>>>(U, B, n_aux, n_ov, 2, V, out, mode, run_if);
-  else if (nr > 1)
-    op_rows2_kernel<4><<<dim3(gx, (nr + 1) / 2), 128, 0, s>>>(U, B, n_aux, n_ov, 2 * nr, V, out, mode, run_if);
+  const dim3 grid((n_aux + 31) / 32, (2 * nr + CR - 1) / CR);
+  if (nr > 0) op_chain2_kernel<<<grid, 256, 0, s>>>(U, B, n_aux, n_ov, 2 * nr, V, out, mode, run_if);
 }
 
 template <typename T>
-void launch_op_gemm1(const T* V, const T* B, const double* Dk, long n_ov, int n_aux, const double* x, double eta,
-                     int nr, T* U, int mode, cudaStream_t s, double* dw, double cut, long ldb, const int* run_if) {
-  dim3 grid((unsigned)((n_ov + TN - 1) / TN), (2 * nr + TM - 1) / TM);
-  op_gemm1_kernel<T><<<grid, NT, 0, s>>>(V, B, Dk, n_ov, n_aux, x, eta, nr, U, mode, dw, cut,
-                                         ldb > 0 ? ldb : n_ov, run_if);
+void launch_deriv(const T* V, const T* B, const double* Dk, long n_ov, int n_aux, const double* x, double eta, int nr,
+                  double* dw, double cut, long ldb, cudaStream_t s) {
+  const dim3 grid((unsigned)((n_ov + TN - 1) / TN), (2 * nr + TM - 1) / TM);
+  if (nr > 0) deriv_kernel<T><<<grid, NT, 0, s>>>(V, B, Dk, n_ov, n_aux, x, eta, nr, dw, cut, ldb);
 }
 
-template <typename T>
-void launch_op_gemm2(const T* U, const T* B, int n_aux, int n_ov, int nr, const T* V, T* out, int mode,
-                     cudaStream_t s, const int* run_if) {
-  dim3 grid((n_aux + TN - 1) / TN, (2 * nr + TM - 1) / TM);
-  op_gemm2_kernel<T><<<grid, NT, 0, s>>>(U, B, n_aux, (long)n_ov, nr, V, out, mode, run_if);
-}
-
-#define GW_INST(T)                                                                                              \
-  template void launch_op_gemm1<T>(const T*, const T*, const double*, long, int, const double*, double, int,    \
-                                   T*, int, cudaStream_t, double*, double, long, const int*);                   \
-  template void launch_op_gemm2<T>(const T*, const T*, int, int, int, const T*, T*, int, cudaStream_t,          \
-                                   const int*);
-GW_INST(double)
-GW_INST(float)
-#undef GW_INST
+template void launch_deriv<double>(const double*, const double*, const double*, long, int, const double*, double, int,
+                                   double*, double, long, cudaStream_t);
+template void launch_deriv<float>(const float*, const float*, const double*, long, int, const double*, double, int,
+                                  double*, double, long, cudaStream_t);
 template void launch_cholesky<double>(double*, int, long, int, int*, cudaStream_t);
 template size_t trsm_w_scratch_elems<double>(int, int);
 template cudaError_t launch_trsm_w<double>(const double*, long, int, int, const int*, const double*, int, double*, int,

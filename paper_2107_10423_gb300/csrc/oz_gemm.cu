@@ -14,6 +14,7 @@
 // each at 128 B a clock: 48 clocks, where the tensor core alone would take 32), then the drains, which the single
 // TMEM buffer (8 sums x 64 columns = all 512) does not overlap with the next 128 of K.
 #include "oz_gemm.cuh"
+#include "oz_digits.cuh"
 #include "tc_ptx.cuh"
 
 #include <algorithm>
@@ -22,8 +23,8 @@
 namespace gw {
 namespace {
 using namespace ptx;
+using namespace oz;
 
-constexpr int S = OZ_S;
 constexpr int BM = 128, BN = 64, BK = 32;
 constexpr int KCHUNK = 4;                        // k-blocks per exact sum (K = 128)
 constexpr int STAGES = 2;
@@ -46,13 +47,12 @@ struct OzMaps {
   CUtensorMap a, b;
 };
 
-// grid.x: tile x K range, grid.y: entry.  Warps 0-7 drain (TMEM lane quarter = warp & 3, column half = warp >> 2),
+// grid.x: tile, grid.y: entry.  Warps 0-7 drain (TMEM lane quarter = warp & 3, column half = warp >> 2),
 // warp 8 TMA, warp 9 MMA.
 __global__ void __launch_bounds__(THREADS, 1)
     oz_gemm_kernel(const __grid_constant__ OzMaps maps, int M, int N, int K, int a_batched, int b_batched,
                    const double* __restrict__ sca, const double* __restrict__ scb, const OzEpi ep,
                    int* __restrict__ err) {
-  if (ep.run_if && *ep.run_if == 0) return;      // uniform over the grid: nothing is allocated yet
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -65,8 +65,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   __shared__ int s_abort;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ksplit = ep.kind == OZ_EPI_PART ? ep.ksplit : 1;
-  const int ks = blockIdx.x % ksplit, tile = blockIdx.x / ksplit, b = blockIdx.y;
+  const int tile = blockIdx.x, b = blockIdx.y;
   int bm, bn;
   if (ep.kind == OZ_EPI_STORE && ep.lower) {     // row block bm holds the column blocks 0 .. 2 bm + 1
     bm = (int)((sqrt(4.0 * tile + 1.0) - 1.0) * 0.5);
@@ -80,11 +79,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
   const int m0 = bm * BM, n0 = bn * BN;
   if (m0 >= M || n0 >= N) return;                // the lower enumeration's last column block may lie past N
-  const int nk_all = ((ep.kind == OZ_EPI_SUMSQ ? min(K, n0 + BN) : K) + BK - 1) / BK;
-  // K ranges in whole chunks
-  const int nch = (nk_all + KCHUNK - 1) / KCHUNK;
-  const int c0 = (int)((long)nch * ks / ksplit), c1 = (int)((long)nch * (ks + 1) / ksplit);
-  const int kb0 = c0 * KCHUNK, nk = min(nk_all, c1 * KCHUNK) - kb0;
+  const int nk = ((ep.kind == OZ_EPI_SUMSQ ? min(K, n0 + BN) : K) + BK - 1) / BK;
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -120,8 +115,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (*(volatile int*)&s_abort) { ok = false; break; }
         const uint32_t st = base + s * STAGE_BYTES;
         mbar_expect_tx(full(s), STAGE_BYTES);
-        tma_load_3d(st, &maps.a, (kb0 + kb) * BK, m0, a_batched ? b * S : 0, full(s));
-        tma_load_3d(st + A_BYTES, &maps.b, (kb0 + kb) * BK, n0, b_batched ? b * S : 0, full(s));
+        tma_load_3d(st, &maps.a, kb * BK, m0, a_batched ? b * S : 0, full(s));
+        tma_load_3d(st + A_BYTES, &maps.b, kb * BK, n0, b_batched ? b * S : 0, full(s));
         issued = kb + 1;
       }
       if (!ok) {
@@ -210,12 +205,13 @@ __global__ void __launch_bounds__(THREADS, 1)
           t = fma(v, v, t);
         }
       if (m < M) atomicAdd(ep.acc + (long)m * ep.ldw + ep.gidx[b], t * (sm * sm) * 5.9604644775390625e-08);   // 2^-24
-    } else if (ep.kind == OZ_EPI_PART) {
+    } else if (ep.kind == OZ_EPI_SUB2) {
       if (m < M) {
-        double* o = ep.part + ((long)ks * M + m) * N;
+        double* o = ep.out + (long)b * ep.out_bstride + (m < ep.half ? (long)m * ep.ldo
+                                                                     : ep.plane + (long)(m - ep.half) * ep.ldo);
 #pragma unroll
         for (int j = 0; j < 32; ++j)
-          if (c + j < N) o[c + j] = fma((double)lo[j], 2.3283064365386963e-10, (double)hi[j]) * sm * sn[c + j];
+          if (c + j < N) o[c + j] -= fma((double)lo[j], 2.3283064365386963e-10, (double)hi[j]) * sm * sn[c + j];
       }
     } else {
       const int mode = (b & 1) ? ep.mode_odd : ep.mode_even;
@@ -274,49 +270,6 @@ bool map_digits(CUtensorMap* map, const void* ptr, int rows, int K, long planes,
 }
 
 // ------------------------------------------------------------------ digits
-// 63-bit integer of x scaled by 2^(62 - e), rounded to nearest (ties away), for |x| <= 2^e; pure integer arithmetic
-// (the FP64 pipe runs at 1/64 of the integer one).
-__device__ __forceinline__ long long to_fixed(double x, int e) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  const int be = (int)((bits >> 52) & 0x7ff);
-  unsigned long long m = bits & 0xfffffffffffffull;
-  if (be) m |= 1ull << 52;
-  const int sh = (be ? be : 1) - 1075 + 62 - e;        // value = m 2^(be - 1075)
-  unsigned long long v;
-  if (sh >= 0) v = sh < 11 ? m << sh : 0ull;           // |x| <= 2^e keeps sh <= 10
-  else v = sh > -55 ? (m + (1ull << (-sh - 1))) >> (-sh) : 0ull;
-  return (bits >> 63) ? -(long long)v : (long long)v;
-}
-
-__device__ __forceinline__ int scale_exp(double sc) {   // sc is a power of two (or NaN: any exponent will do)
-  return (int)((__double_as_longlong(sc) >> 52) & 0x7ff) - 1023;
-}
-
-// Digits of eight consecutive elements: out[i] = the eight BF16 of digit i.
-__device__ __forceinline__ void digits8(const long long (&x)[8], uint4 (&out)[S]) {
-  uint32_t w[S][4];
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    unsigned long long y[2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) y[t] = (unsigned long long)x[2 * p + t] + 0x0080808080808080ull;
-#pragma unroll
-    for (int i = 0; i < S; ++i) {                      // digit 0 is the top byte (signed), the others byte - 128
-      float f[2];
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const uint32_t byte = (uint32_t)(y[t] >> (8 * (S - 1 - i))) & 0xffu;
-        f[t] = i == 0 ? __uint_as_float(0x4b000000u | (byte ^ 0x80u)) - 8388736.f
-                      : __uint_as_float(0x4b000000u | byte) - 8388736.f;
-      }
-      __nv_bfloat162 v = __floats2bfloat162_rn(f[0], f[1]);
-      w[i][p] = *reinterpret_cast<uint32_t*>(&v);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < S; ++i) out[i] = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
-}
-
 // One thread: eight columns of one row of entry blockIdx.z: x itself (a matrix per entry at stride xbs), or one x
 // times the entry's weights.
 template <bool WEIGHTED>
@@ -377,17 +330,6 @@ __global__ void __launch_bounds__(256) oz_split_t_kernel(const double* __restric
   for (int i = 0; i < S; ++i) *reinterpret_cast<uint4*>(dig + ((long)i * cols + c) * ldd + p) = d[i];
 }
 
-// Power of two from the largest magnitude's bits: 2^e with |x| <= 2^e (the next power), exponents kept inside
-// [-900, 900] so that products of scales stay finite; NaN if the row holds a NaN or an infinity.
-__device__ __forceinline__ double scale_of(unsigned long long mx) {
-  if (mx >= 0x7ff0000000000000ull) return __longlong_as_double(0x7ff8000000000000ll);
-  int e = (int)(mx >> 52) - 1022;                 // 2^e > |x|
-  if (mx == 0) e = 0;
-  if (e < -900) e = -900;
-  if (e > 900) return __longlong_as_double(0x7ff8000000000000ll);
-  return __longlong_as_double((long long)(1023 + e) << 52);
-}
-
 __global__ void __launch_bounds__(256) oz_row_scale_kernel(const double* __restrict__ x, long cols, long ld,
                                                            double* __restrict__ sc) {
   __shared__ unsigned long long red[8];
@@ -444,7 +386,7 @@ __global__ void oz_weight_kernel(const double* __restrict__ Dk, int K, const int
   w[(long)b * K + k] = v;
 }
 
-// ------------------------------------------------------------------ residue operator
+// ------------------------------------------------------------------ derivative pass
 __device__ __forceinline__ unsigned long long block_max(unsigned long long mx, unsigned long long* red) {
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
@@ -455,10 +397,6 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long mx, u
   __syncthreads();
   for (int i = 0; i < (int)(blockDim.x >> 5); ++i) mx = red[i] > mx ? red[i] : mx;
   return mx;
-}
-
-__device__ __forceinline__ unsigned long long mag(double v) {
-  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
 
 // Digits of one row by the whole block, eight columns a thread.
@@ -478,8 +416,7 @@ __device__ __forceinline__ void row_to_digits(const double* xr, int cols, int ld
 
 __global__ void __launch_bounds__(128) oz_row_digits_kernel(const double* __restrict__ x, int rows, int cols, long ld,
                                                             double* __restrict__ sc, __nv_bfloat16* __restrict__ dig,
-                                                            int ldd, const int* __restrict__ run_if) {
-  if (run_if && *run_if == 0) return;
+                                                            int ldd) {
   __shared__ unsigned long long red[4];
   const int r = blockIdx.x;
   const double* xr = x + (long)r * ld;
@@ -488,60 +425,6 @@ __global__ void __launch_bounds__(128) oz_row_digits_kernel(const double* __rest
   const double s = scale_of(block_max(mx, red));
   if (threadIdx.x == 0) sc[r] = s;
   row_to_digits(xr, cols, ldd, s, rows, r, dig);
-}
-
-__global__ void oz_pole_weight_kernel(const double* __restrict__ Dk, int K, const double* __restrict__ xs, double eta,
-                                      double2* __restrict__ cw) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-  if (k >= K) return;
-  const double x = xs[j], D = Dk[k], a1 = x - D, a2 = -x - D, e2 = eta * eta;
-  const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
-  cw[(long)j * K + k] = make_double2(2.0 * (a1 / d1 + a2 / d2), -2.0 * eta * (1.0 / d1 + 1.0 / d2));
-}
-
-// One CTA per right-hand side: the weights cost four FP64 multiply-adds a pair (their divisions are done once per
-// batch, not per iteration), the rest is memory traffic: T and cw in, U and 32 bytes of digits out.
-__global__ void __launch_bounds__(256) oz_pole_apply_kernel(double* __restrict__ T, int K,
-                                                            const double2* __restrict__ cw, int rows,
-                                                            double* __restrict__ sc, __nv_bfloat16* __restrict__ dig,
-                                                            int ldd, const int* __restrict__ run_if) {
-  if (run_if && *run_if == 0) return;
-  __shared__ unsigned long long red[8];
-  const int j = blockIdx.x;
-  double* t0 = T + (long)(2 * j) * K;
-  double* t1 = t0 + K;
-  const double2* c = cw + (long)j * K;
-  unsigned long long m0 = 0, m1 = 0;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const double tr = t0[k], ti = -t1[k];
-    const double2 w = c[k];
-    const double u = w.x * tr - w.y * ti, v = w.x * ti + w.y * tr;
-    t0[k] = u;
-    t1[k] = v;
-    m0 = max(m0, mag(u));
-    m1 = max(m1, mag(v));
-  }
-  const double s0 = scale_of(block_max(m0, red)), s1 = scale_of(block_max(m1, red));
-  if (threadIdx.x == 0) {
-    sc[2 * j] = s0;
-    sc[2 * j + 1] = s1;
-  }
-  __syncthreads();
-  row_to_digits(t0, K, ldd, s0, rows, 2 * j, dig);
-  row_to_digits(t1, K, ldd, s1, rows, 2 * j + 1, dig);
-}
-
-__global__ void __launch_bounds__(256) oz_part_reduce_kernel(const double* __restrict__ part, int ksplit, long N, int n,
-                                                             const double* __restrict__ V, int mode,
-                                                             double* __restrict__ out,
-                                                             const int* __restrict__ run_if) {
-  if (run_if && *run_if == 0) return;
-  for (long i = blockIdx.x * 256L + threadIdx.x; i < N; i += gridDim.x * 256L) {
-    double v = 0.0;
-    for (int q = 0; q < ksplit; ++q) v += part[q * N + i];
-    if (mode == 1) v = (((i / n) & 1) ? -V[i] : V[i]) - v;
-    out[i] = v;
-  }
 }
 
 __global__ void __launch_bounds__(256) oz_pole_derivative_kernel(const double* __restrict__ T, int K,
@@ -593,8 +476,7 @@ cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int batch, int M, in
   }
   const long nbm = (M + BM - 1) / BM, nbn = (N + BN - 1) / BN;
   const long tiles = ep.kind == OZ_EPI_STORE && ep.lower ? nbm * (nbm + 1) : nbm * nbn;
-  const long gx = tiles * (ep.kind == OZ_EPI_PART ? ep.ksplit : 1);
-  oz_gemm_kernel<<<dim3((unsigned)gx, batch), THREADS, SMEM_BYTES, s>>>(maps, M, N, K, A.batched, B.batched, A.sc, B.sc,
+  oz_gemm_kernel<<<dim3((unsigned)tiles, batch), THREADS, SMEM_BYTES, s>>>(maps, M, N, K, A.batched, B.batched, A.sc, B.sc,
                                                                        ep, err);
   return cudaGetLastError();
 }
@@ -645,30 +527,8 @@ cudaError_t oz_pair_weights(const double* Dk, int K, const int* kinds, const dou
 }
 
 cudaError_t oz_row_digits(const double* x, int rows, int cols, long ld, double* sc, __nv_bfloat16* dig,
-                          const int* run_if, cudaStream_t s) {
-  if (rows > 0 && cols > 0) oz_row_digits_kernel<<<rows, 128, 0, s>>>(x, rows, cols, ld, sc, dig, oz_ld(cols), run_if);
-  return cudaGetLastError();
-}
-
-cudaError_t oz_pole_weights(const double* Dk, int K, const double* xs, double eta, int nr, double2* cw,
-                            cudaStream_t s) {
-  if (nr > 65535) return cudaErrorInvalidValue;
-  if (nr > 0 && K > 0) oz_pole_weight_kernel<<<dim3((K + 255) / 256, nr), 256, 0, s>>>(Dk, K, xs, eta, cw);
-  return cudaGetLastError();
-}
-
-cudaError_t oz_pole_apply(double* T, int K, const double2* cw, int nr, double* sc, __nv_bfloat16* dig,
-                          const int* run_if, cudaStream_t s) {
-  if (nr > 0) oz_pole_apply_kernel<<<nr, 256, 0, s>>>(T, K, cw, 2 * nr, sc, dig, oz_ld(K), run_if);
-  return cudaGetLastError();
-}
-
-cudaError_t oz_part_reduce(const double* part, int ksplit, int rows, int n, const double* V, int mode, double* out,
-                           const int* run_if, cudaStream_t s) {
-  const long N = (long)rows * n;
-  if (N > 0)
-    oz_part_reduce_kernel<<<(unsigned)std::min<long>((N + 255) / 256, 2048), 256, 0, s>>>(part, ksplit, N, n, V, mode,
-                                                                                          out, run_if);
+                          cudaStream_t s) {
+  if (rows > 0 && cols > 0) oz_row_digits_kernel<<<rows, 128, 0, s>>>(x, rows, cols, ld, sc, dig, oz_ld(cols));
   return cudaGetLastError();
 }
 

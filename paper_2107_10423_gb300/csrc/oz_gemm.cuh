@@ -15,7 +15,7 @@ struct OzOperand {
   int batched;                       // 0: one matrix for every entry
 };
 
-enum { OZ_EPI_STORE = 0, OZ_EPI_PART = 1, OZ_EPI_SUMSQ = 2 };
+enum { OZ_EPI_STORE = 0, OZ_EPI_SUMSQ = 1, OZ_EPI_SUB2 = 2 };
 struct OzEpi {
   int kind;
   // OZ_EPI_STORE: out_b[m][n] = f(v) (f: 0 v, 1 delta_mn - v, 2 -v; even / odd entries), added to what is there when
@@ -24,14 +24,13 @@ struct OzEpi {
   double* out;
   long out_bstride;
   int ldo;
-  // OZ_EPI_PART: part[ks][m][n] = v of this K range (row length N)
-  double* part;
-  int ksplit;
   // OZ_EPI_SUMSQ: acc[m * ldw + gidx[b]] += sum_n v[m][n]^2; the B rows are lower triangular (row n ends at column n)
   double* acc;
   int ldw;
   const int* gidx;
-  const int* run_if;                 // if not NULL: the launch does nothing when *run_if == 0
+  // OZ_EPI_SUB2: out_b[m][n] -= v for m < half, out_b[plane + (m - half) ldo + n] -= v below (ldo, out_bstride as above)
+  long plane;
+  int half;
 };
 
 int oz_ld(int K);                    // row length of the digit arrays
@@ -57,20 +56,10 @@ cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long 
 cudaError_t oz_pair_weights(const double* Dk, int K, const int* kinds, const double* params, double eta, int nb,
                             double* w, cudaStream_t s);
 
-// ---- residue operator of FP64 plans (rows 2j, 2j + 1 of V, T, U belong to right-hand side j)
 // Row scales and digits of x [rows][cols] (row length ld) in one launch.
 cudaError_t oz_row_digits(const double* x, int rows, int cols, long ld, double* sc, __nv_bfloat16* dig,
-                          const int* run_if, cudaStream_t s);
-// cw[j][k] = c_k(x_j) = 2[1/(x - D + i eta) + 1/(-x - D + i eta)].
-cudaError_t oz_pole_weights(const double* Dk, int K, const double* xs, double eta, int nr, double2* cw,
-                            cudaStream_t s);
-// U = c (t_r + i t_i), t_r = T[2j], t_i = -T[2j + 1], as row scales and digits (T is overwritten by U).
-cudaError_t oz_pole_apply(double* T, int K, const double2* cw, int nr, double* sc, __nv_bfloat16* dig,
-                          const int* run_if, cudaStream_t s);
-// out[r][p] = v (mode 0) or (r odd ? -V : V)[r][p] - v (mode 1), v = the sum of the ksplit partial products.
-cudaError_t oz_part_reduce(const double* part, int ksplit, int rows, int n, const double* V, int mode, double* out,
-                           const int* run_if, cudaStream_t s);
-// dw[j] = sum_k Re(c'_k(x_j) t_k^2).
+                          cudaStream_t s);
+// dw[j] = sum_k Re(c'_k(x_j) t_k^2), t_k = T[2j][k] - i T[2j + 1][k].
 cudaError_t oz_pole_derivative(const double* T, int K, const double* Dk, const double* xs, double eta, int nr,
                                double* dw, cudaStream_t s);
 
