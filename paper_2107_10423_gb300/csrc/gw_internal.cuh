@@ -39,6 +39,11 @@ void launch_op_gemm1(const double* V, const double* B, const double* Dk, long n_
                      double eta, int nr, double* U, cudaStream_t s, const int* run_if = nullptr);
 void launch_op_gemm2(const double* U, const double* B, int n_aux, long n_ov, int nr, const double* V, double* out,
                      int mode, cudaStream_t s, const int* run_if = nullptr);
+// Both products in FP32 for up to kSkinnyRhs right-hand sides: B FP32 [n_aux][ldb] (rows 16-byte aligned, zero padded),
+// U [2 nr][ldb] work space, S as in gemm2.
+constexpr int kSkinnyRhs = 4;
+void launch_op_skinny(const float* V, const float* B, long ldb, const double* Dk, int n_ov, int n_aux, const double* x,
+                      float eta, int nr, float* U, float* S, int mode, cudaStream_t s, const int* run_if);
 // dw[j] += sum_k Re(c'_k(x_j) t_k^2) in FP64, c' the x-derivative (dw zeroed by the caller), skipping the pairs with
 // |x_j - D_k| < cut or |-x_j - D_k| < cut (added by launch_deriv_resonant); ldb: row length of B.
 template <typename T>

@@ -98,11 +98,10 @@ struct gw_plan {
   DevBuf ws_mat, ws_info, ws_gout, ws_xi, tc_part, tc_kind, tc_par, tc_err, tc_w, tc_tiles, ns_E, ns_X, ns_X2, ns_Xa, ns_Xb, ns_T, ns_lam,
       ns_E0, ns_vec;
   DevBuf mr_V, mr_U, mr_S, mr_vprev, mr_v, mr_d1, mr_d2, mr_x, mr_st, mr_rt, mr_rm, mr_xf, mr_wre, mr_wim,
-      mr_dwre, mr_it, mr_res, mr_cnt, mr_Vhi, mr_Vlo, mr_Uhi, mr_Ulo, mr_Vlo2, mr_Ulo2, mr_V64;
+      mr_dwre, mr_it, mr_res, mr_cnt, mr_Vhi, mr_Vlo, mr_Uhi, mr_Ulo, mr_Vlo2, mr_Ulo2, mr_V64, mr_part;
   DevBuf sg_I, sg_dI, sg_R, sg_dR, sg_om, sg_start, sg_coef, sg_act, sg_tmap, qp_st, qp_om0;
   DevBuf fb_A, fb_y, fb_piv, fb_info, fb_idx, fb_y64, fb_V32, fb_S32, fb_Vp, fb_Up, fb_x, fb_V64, fb_U64, fb_S64, fb_sel,
       fb_pos, fb_rho, fb_xs, fb_Bl, fb_lu, fb_sw, fb_linv, fb_lus;
-  int* h_cnt = nullptr;       // pinned
   std::string err;
   gw_stats stats{};
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
@@ -115,7 +114,7 @@ struct gw_plan {
   gw_plan() {
     DevBuf* all[] = {&oz_A, &oz_B, &oz_X, &oz_sc, &oz_w, &op_BT, &op_sc, &op_V, &ws_mat, &ws_info, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
                      &mr_v, &mr_d1, &mr_d2, &mr_x, &mr_st, &mr_rt, &mr_rm, &mr_xf, &mr_wre, &mr_wim,
-                     &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
+                     &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &mr_part, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
                      &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_lu, &fb_sw, &fb_linv, &fb_lus, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS};
     bufs.assign(all, all + sizeof(all) / sizeof(all[0]));
   }
@@ -952,6 +951,12 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
 gw_status tc_operator(gw_plan* P, int nr, const double* xf, const float* V32, float* S32, int mode,
                       const int* run_if = nullptr) {
   const int n = P->cfg.n_aux, n_ov = P->n_ov;
+  if (nr <= gw::kSkinnyRhs) {
+    LAUNCH(gw::launch_op_skinny(V32, P->d_B_ia_f, P->ld_f, P->d_D, n_ov, n, xf, (float)P->cfg.eta, nr,
+                                as<float>(P->mr_U), S32, mode, P->stream, run_if));
+    P->stats.n_kernel_launches++;
+    return GW_OK;
+  }
   const int ldov = gw::tc_ld(n_ov);
   const bool three = P->cfg.op_parts >= 3;
   if (three) TRY(ensure_third_parts(P));
@@ -974,8 +979,12 @@ gw_status tc_operator(gw_plan* P, int nr, const double* xf, const float* V32, fl
   const int ns = three ? 3 : 2;
   CK(gw::tc_gemm_ex(Vop, 1, BT, 0, ns, 2 * nr, n_ov, n, 0, e1, as<int>(P->tc_err), P->stream));
   gw::TcEpi e2{};
-  e2.kind = mode == 0 ? gw::TC_EPI_STORE : gw::TC_EPI_EMBED;
-  e2.out = S32;
+  // the second product's contraction is the long one: over few output tiles it is split in K ranges (at 50 rows,
+  // 629 x 4675, 62 us on 5 CTAs before)
+  const int ks = gw::tc_ksplit(2 * nr, n, n_ov);
+  e2.kind = ks > 1 ? gw::TC_EPI_PART : (mode == 0 ? gw::TC_EPI_STORE : gw::TC_EPI_EMBED);
+  e2.out = ks > 1 ? as<float>(P->mr_part) : S32;
+  e2.ksplit = ks;
   e2.ldo = n;
   e2.vin = V32;
   e2.ldv = n;
@@ -984,6 +993,10 @@ gw_status tc_operator(gw_plan* P, int nr, const double* xf, const float* V32, fl
   const gw::TcOperand Bop{{P->d_Bhi, P->d_Blo, three ? P->d_Blo2 : nullptr}};
   CK(gw::tc_gemm_ex(Uop, 1, Bop, 0, ns, 2 * nr, n, n_ov, 0, e2, as<int>(P->tc_err), P->stream));
   P->stats.n_kernel_launches += 3;
+  if (ks > 1) {
+    CK(gw::tc_part_reduce(as<float>(P->mr_part), ks, 2 * nr, n, V32, mode, S32, run_if, P->stream));
+    P->stats.n_kernel_launches++;
+  }
   return GW_OK;
 }
 
@@ -1078,7 +1091,7 @@ gw_status residues_T(gw_plan* P, int nr_total, const int* d_rt, const int* d_rm,
   batch = std::min(batch, std::max(1, nr_total));
   TRY(ensure(P, P->mr_V, sizeof(T) * 2 * (size_t)batch * n));
   TRY(ensure(P, P->mr_S, sizeof(T) * 2 * (size_t)batch * n));
-  TRY(ensure(P, P->mr_U, sizeof(T) * 2 * (size_t)batch * n_ov));
+  TRY(ensure(P, P->mr_U, sizeof(T) * 2 * (size_t)batch * (sizeof(T) == 4 ? P->ld_f : n_ov)));
   const bool d64 = (sizeof(T) == 4) && P->cfg.deriv_fp64;
   if (sizeof(T) == 4) TRY(ensure(P, P->mr_V64, sizeof(double) * 2 * (size_t)batch * n));
   double* V64 = (sizeof(T) == 4) ? as<double>(P->mr_V64) : nullptr;
@@ -1088,6 +1101,12 @@ gw_status residues_T(gw_plan* P, int nr_total, const int* d_rt, const int* d_rm,
   TRY(ensure(P, P->mr_cnt, sizeof(int)));
   const bool tcop = (sizeof(T) == 4) && P->d_BThi != nullptr;
   if (tcop) {
+    // partial products of the full batch and of the last, smaller one
+    const int last = nr_total % batch ? nr_total % batch : batch;
+    for (int nr : {batch, last}) {
+      const int ks = gw::tc_ksplit(2 * nr, n, n_ov);
+      if (nr > gw::kSkinnyRhs && ks > 1) TRY(ensure(P, P->mr_part, sizeof(float) * (size_t)ks * 2 * nr * n));
+    }
     TRY(ensure(P, P->mr_Vhi, sizeof(__nv_bfloat16) * 2 * (size_t)batch * gw::tc_ld(n)));
     TRY(ensure(P, P->mr_Vlo, sizeof(__nv_bfloat16) * 2 * (size_t)batch * gw::tc_ld(n)));
     TRY(ensure(P, P->mr_Uhi, sizeof(__nv_bfloat16) * 2 * (size_t)batch * gw::tc_ld(n_ov)));
@@ -1499,7 +1518,6 @@ static void free_plan(gw_plan* P) {
   if (P->d_Bnhi) cudaFree(P->d_Bnhi);
   if (P->d_Bnlo) cudaFree(P->d_Bnlo);
   if (P->d_Bnlo2) cudaFree(P->d_Bnlo2);
-  if (P->h_cnt) cudaFreeHost(P->h_cnt);
   if (P->ev0) cudaEventDestroy(P->ev0);
   if (P->ev1) cudaEventDestroy(P->ev1);
   if (P->ev2) cudaEventDestroy(P->ev2);
@@ -1541,7 +1559,6 @@ static gw_status plan_create_impl(gw_plan* P, const gw_config* cfg, const double
   CK(cudaEventCreate(&P->ev0));
   CK(cudaEventCreate(&P->ev1));
   CK(cudaEventCreate(&P->ev2));
-  CK(cudaMallocHost(&P->h_cnt, sizeof(int)));
   const int n = cfg->n_aux;
   P->h_eps.assign(eps, eps + P->n_bas);
   P->h_eps_s[0] = P->h_eps;
@@ -2275,6 +2292,7 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
   if (mixed) {
     b += batch * (16 * n + 8 * ldn + 8 * ldo);                               // FP64 solutions, split V and U
     if (c->op_parts >= 3) b += batch * (4 * ldn + 4 * ldo);
+    b += batch * 8 * (ldf - n_ov) + 4 * (u64)152 * 128 * 128;                // U rows' padding, partial products
   }
   b += 48 * std::max<u64>(1, rows) + 8 * 6 * (u64)n_t + 64;                  // residue lists, Sigma scratch
   // dense fallback batch

@@ -548,6 +548,155 @@ __global__ void __launch_bounds__(256) op_chain2_kernel(const double* __restrict
   out[(long)r * n_aux + P] = acc;
 }
 
+// ------------------------------------------------------------------ FP32 residue operator for few rows
+// Mixed plans, up to eight rows (four right-hand sides: HOMO and LUMO jobs).  A 128-row tensor tile would be padding,
+// and its CTAs as few as the output has column tiles: at 4 rows, 3024 x 109440, a product took 1.6 ms on 24 CTAs; here
+// it is one pass over B at 6 TB/s (0.22 ms), in FP32 instead of BF16 parts.  At 126 x 190 4 us against 9.
+// Sums run in chains of 64 (gemm2) or one slice's 1/8 of the contraction (gemm1) before they are added.
+constexpr int SKC = 128;             // gemm1 columns a CTA: 32 lanes x 4
+template <int RM>
+__global__ void __launch_bounds__(256) op_skinny1_kernel(const float* __restrict__ V, const float* __restrict__ B,
+                                                         long ldb, const double* __restrict__ Dk, int n_ov, int n_aux,
+                                                         const double* __restrict__ xs, float eta, int M,
+                                                         float* __restrict__ U, const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  __shared__ float Vs[256][RM];
+  __shared__ float red[8][RM][SKC];
+  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+  const long k = blockIdx.x * (long)SKC + 4 * lane;
+  float tot[RM][4];
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) tot[i][c] = 0.f;
+  for (int p0 = 0; p0 < n_aux; p0 += 256) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+      Vs[threadIdx.x][i] = (i < M && p0 + (int)threadIdx.x < n_aux) ? V[(long)i * n_aux + p0 + threadIdx.x] : 0.f;
+    __syncthreads();
+    const int pe = min(32, n_aux - p0 - 32 * sl);
+    float acc[RM][4];
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
+    if (k < ldb)
+#pragma unroll 8
+      for (int t = 0; t < pe; ++t) {
+        const float4 b = *reinterpret_cast<const float4*>(B + (long)(p0 + 32 * sl + t) * ldb + k);
+#pragma unroll
+        for (int i = 0; i < RM; ++i) {
+          const float v = Vs[32 * sl + t][i];
+          acc[i][0] = fmaf(v, b.x, acc[i][0]);
+          acc[i][1] = fmaf(v, b.y, acc[i][1]);
+          acc[i][2] = fmaf(v, b.z, acc[i][2]);
+          acc[i][3] = fmaf(v, b.w, acc[i][3]);
+        }
+      }
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) tot[i][c] += acc[i][c];
+  }
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) red[sl][i][4 * lane + c] = tot[i][c];
+  __syncthreads();
+  const float e2 = eta * eta;
+  for (int it = threadIdx.x; it < SKC * (RM / 2); it += 256) {
+    const int c = it % SKC, pr = it / SKC;
+    const long kk = blockIdx.x * (long)SKC + c;
+    if (2 * pr >= M || kk >= ldb) continue;
+    float tr = 0.f, ti = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      tr += red[q][2 * pr][c];
+      ti -= red[q][2 * pr + 1][c];
+    }
+    float ur = 0.f, ui = 0.f;                      // zero in the rows' padding
+    if (kk < n_ov) {
+      const double x = xs[pr], D = Dk[kk];
+      const float a1 = (float)(x - D), a2 = (float)(-x - D);
+      const float d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
+      const float cr = 2.f * (a1 / d1 + a2 / d2);
+      const float ci = -2.f * eta * (1.f / d1 + 1.f / d2);
+      ur = cr * tr - ci * ti;
+      ui = cr * ti + ci * tr;
+    }
+    U[(long)(2 * pr) * ldb + kk] = ur;
+    U[(long)(2 * pr + 1) * ldb + kk] = ui;
+  }
+}
+
+// Four rows P of B a CTA, its eight warps over the contraction.
+template <int RM>
+__global__ void __launch_bounds__(256) op_skinny2_kernel(const float* __restrict__ U, const float* __restrict__ B,
+                                                         long ldb, int n_aux, int M, const float* __restrict__ V,
+                                                         float* __restrict__ out, int mode,
+                                                         const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  __shared__ float red[8][4][RM];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, P0 = blockIdx.x * 4;
+  float tot[4][RM];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int i = 0; i < RM; ++i) tot[p][i] = 0.f;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (long k0 = 4L * threadIdx.x; k0 < ldb; k0 += 1024 * 16) {
+    float acc[4][RM];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int i = 0; i < RM; ++i) acc[p][i] = 0.f;
+#pragma unroll 2
+    for (int t = 0; t < 16; ++t) {
+      const long k = k0 + 1024L * t;
+      if (k >= ldb) break;
+      float4 b[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+        b[p] = P0 + p < n_aux ? *reinterpret_cast<const float4*>(B + (long)(P0 + p) * ldb + k) : zero;
+#pragma unroll
+      for (int i = 0; i < RM; ++i) {
+        if (i >= M) break;
+        const float4 u = *reinterpret_cast<const float4*>(U + (long)i * ldb + k);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          acc[p][i] = fmaf(u.x, b[p].x, acc[p][i]);
+          acc[p][i] = fmaf(u.y, b[p].y, acc[p][i]);
+          acc[p][i] = fmaf(u.z, b[p].z, acc[p][i]);
+          acc[p][i] = fmaf(u.w, b[p].w, acc[p][i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int i = 0; i < RM; ++i) tot[p][i] += acc[p][i];
+  }
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int i = 0; i < RM; ++i) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) tot[p][i] += __shfl_xor_sync(0xffffffffu, tot[p][i], o);
+      if (lane == 0) red[w][p][i] = tot[p][i];
+    }
+  __syncthreads();
+  if (threadIdx.x < 4 * RM) {
+    const int p = threadIdx.x / RM, i = threadIdx.x % RM;
+    if (i < M && P0 + p < n_aux) {
+      float s = 0.f;
+      for (int q = 0; q < 8; ++q) s += red[q][p][i];
+      const long at = (long)i * n_aux + P0 + p;
+      out[at] = mode == 1 ? ((i & 1) ? -V[at] : V[at]) - s : s;
+    }
+  }
+}
+
 // ------------------------------------------------------------------ double-float GEMMs (refinement residual)
 // A double x is carried as the FP32 pair (h, l), h = fl(x), l = fl(x - h): 48 significant bits.  A multiply-add
 // s += a b takes the product exactly to FP32 pair precision (h*h by an FMA error term, plus the two cross terms)
@@ -812,6 +961,21 @@ void launch_op_gemm2(const double* U, const double* B, int n_aux, long n_ov, int
                      int mode, cudaStream_t s, const int* run_if) {
   const dim3 grid((n_aux + 31) / 32, (2 * nr + CR - 1) / CR);
   if (nr > 0) op_chain2_kernel<<<grid, 256, 0, s>>>(U, B, n_aux, n_ov, 2 * nr, V, out, mode, run_if);
+}
+
+void launch_op_skinny(const float* V, const float* B, long ldb, const double* Dk, int n_ov, int n_aux, const double* x,
+                      float eta, int nr, float* U, float* S, int mode, cudaStream_t s, const int* run_if) {
+  const unsigned g1 = (unsigned)((ldb + SKC - 1) / SKC), g2 = (n_aux + 3) / 4;
+  if (nr == 1) {
+    op_skinny1_kernel<2><<<g1, 256, 0, s>>>(V, B, ldb, Dk, n_ov, n_aux, x, eta, 2, U, run_if);
+    op_skinny2_kernel<2><<<g2, 256, 0, s>>>(U, B, ldb, n_aux, 2, V, S, mode, run_if);
+  } else if (nr == 2) {
+    op_skinny1_kernel<4><<<g1, 256, 0, s>>>(V, B, ldb, Dk, n_ov, n_aux, x, eta, 4, U, run_if);
+    op_skinny2_kernel<4><<<g2, 256, 0, s>>>(U, B, ldb, n_aux, 4, V, S, mode, run_if);
+  } else if (nr <= kSkinnyRhs) {
+    op_skinny1_kernel<8><<<g1, 256, 0, s>>>(V, B, ldb, Dk, n_ov, n_aux, x, eta, 2 * nr, U, run_if);
+    op_skinny2_kernel<8><<<g2, 256, 0, s>>>(U, B, ldb, n_aux, 2 * nr, V, S, mode, run_if);
+  }
 }
 
 template <typename T>

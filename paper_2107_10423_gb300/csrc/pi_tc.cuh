@@ -6,7 +6,8 @@
 #include <vector>
 
 namespace gw {
-enum { TC_EPI_STORE = 0, TC_EPI_CPAIR = 1, TC_EPI_EMBED = 2, TC_EPI_AXPBY = 3, TC_EPI_WRED = 4, TC_EPI_SUB2 = 5 };
+enum { TC_EPI_STORE = 0, TC_EPI_CPAIR = 1, TC_EPI_EMBED = 2, TC_EPI_AXPBY = 3, TC_EPI_WRED = 4, TC_EPI_SUB2 = 5,
+       TC_EPI_PART = 6 };
 
 // Epilogue of the tensor-core GEMM (passed by value to the kernel).
 struct TcEpi {
@@ -45,6 +46,8 @@ struct TcEpi {
   long plane;
   int half;
   long limit;                 // TC_EPI_SUB2: elements writable from out (an index beyond it is recorded, code 66)
+  // TC_EPI_PART: out[z][m][n] = v of K range z of ksplit (row length N; one batch entry); tc_part_reduce adds them
+  int ksplit;
   // if not NULL: the whole launch does nothing when *run_if == 0 (device flag, read once at kernel start)
   const int* run_if;
 };
@@ -100,6 +103,11 @@ struct TcOperand {
 // products (BF16x3), nsplit 3 the six products with part indices i + j <= 2 (about FP32-accurate).
 cudaError_t tc_gemm_ex(const TcOperand& A, int batch, const TcOperand& B, int b_batched, int nsplit, int M, int N,
                        int K, int lower, const TcEpi& ep, int* err, cudaStream_t s);
+// K ranges worth taking for an M x N x K product (1: none), and the sum of its partial products: out[r][c] = sum (mode
+// 0) or the residue operator's embedding (r odd ? -vin : vin)[r][c] - sum (mode 1).
+int tc_ksplit(int M, int N, int K);
+cudaError_t tc_part_reduce(const float* part, int ksplit, int rows, int n, const float* vin, int mode, float* out,
+                           const int* run_if, cudaStream_t s);
 // rows x cols FP32 (row length lds) split into BF16 hi/lo rows of tc_ld(cols) elements (zero padded).
 cudaError_t tc_split_rows(const float* src, int rows, int cols, int lds, __nv_bfloat16* hi, __nv_bfloat16* lo,
                           cudaStream_t s, __nv_bfloat16* lo2 = nullptr);

@@ -12,6 +12,7 @@
 
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 
@@ -202,6 +203,12 @@ __device__ void epilogue(const TcEpi& ep, const float* stg, int m0, int n0, int 
         atomicAdd(ep.W + (long)n * ep.wld + ep.gidx[b], acc);
       }
     }
+  } else if (ep.kind == TC_EPI_PART) {
+    float* o = ep.out + (long)blockIdx.z * M * N;
+    for (int idx = threadIdx.x; idx < BM * BN; idx += THREADS) {
+      const int rr = idx / BN, cc = idx % BN, m = m0 + rr, n = n0 + cc;
+      if (m < M && n < N) o[(long)m * N + n] = stg[rr * (BN + 1) + cc];
+    }
   } else if (ep.kind == TC_EPI_SUB2) {
     float* o = ep.out + (long)b * ep.out_bstride;
     for (int base = threadIdx.x; base < BM * BN; base += THREADS * EPI_U) {
@@ -286,7 +293,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     bn = blockIdx.x % nbn;
   }
   const int m0 = bm * BM, n0 = bn * BN, b = blockIdx.y;
-  const int nk = (K + BK - 1) / BK;
+  // this CTA's range of k-blocks (grid.z > 1: TC_EPI_PART)
+  const int nk_all = (K + BK - 1) / BK, kb0 = (int)((long)nk_all * blockIdx.z / gridDim.z);
+  const int nk = (int)((long)nk_all * (blockIdx.z + 1) / gridDim.z) - kb0;
   const int nchunks = (nk + CHUNK - 1) / CHUNK;
 
   uint32_t full[STAGES], empty[STAGES];
@@ -334,10 +343,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint32_t st = base + s * STAGE_BYTES;
         mbar_expect_tx(full[s], STAGE_BYTES);
 #pragma unroll
-        for (int i = 0; i < NSP; ++i) tma_load_3d(st + i * TILE_BYTES, &maps.a[i], kb * BK, m0, b, full[s]);
+        for (int i = 0; i < NSP; ++i) tma_load_3d(st + i * TILE_BYTES, &maps.a[i], (kb0 + kb) * BK, m0, b, full[s]);
 #pragma unroll
         for (int j = 0; j < NSP; ++j)
-          tma_load_3d(st + (NSP + j) * TILE_BYTES, &maps.b[j], kb * BK, n0, b_batched ? b : 0, full[s]);
+          tma_load_3d(st + (NSP + j) * TILE_BYTES, &maps.b[j], (kb0 + kb) * BK, n0, b_batched ? b : 0, full[s]);
         issued = kb + 1;
       }
     }
@@ -461,7 +470,7 @@ cudaError_t tc_gemm_ex(const TcOperand& A, int batch, const TcOperand& B, int b_
       return cudaErrorInvalidValue;
   const int nbm = (M + BM - 1) / BM, nbn = (N + BN - 1) / BN;
   const int tiles = lower ? nbm * (nbm + 1) / 2 : nbm * nbn;
-  dim3 grid(tiles, batch);
+  dim3 grid(tiles, batch, ep.kind == TC_EPI_PART ? std::max(1, ep.ksplit) : 1);
   if (nsplit == 2) {
     static bool attr = false;
     if (!attr) {
@@ -482,6 +491,34 @@ cudaError_t tc_gemm_ex(const TcOperand& A, int batch, const TcOperand& B, int b_
     tc_gemm_kernel<3><<<grid, THREADS, TcCfg<3>::SMEM_BYTES, s>>>(maps, M, N, K, lower, b_batched, ep, err);
   }
   return cudaGetLastError();
+}
+
+// out[r][c] = s (mode 0) or the embedding (r odd ? -vin : vin) - s (mode 1), s = the ksplit partial products in order.
+__global__ void __launch_bounds__(256) tc_part_reduce_kernel(const float* __restrict__ part, int ksplit, long N, int n,
+                                                             const float* __restrict__ vin, int mode,
+                                                             float* __restrict__ out, const int* __restrict__ run_if) {
+  if (run_if && *run_if == 0) return;
+  for (long i = blockIdx.x * 256L + threadIdx.x; i < N; i += gridDim.x * 256L) {
+    float s = 0.f;
+    for (int q = 0; q < ksplit; ++q) s += part[q * N + i];
+    if (mode == 1) s = (((i / n) & 1) ? -vin[i] : vin[i]) - s;
+    out[i] = s;
+  }
+}
+
+cudaError_t tc_part_reduce(const float* part, int ksplit, int rows, int n, const float* vin, int mode, float* out,
+                           const int* run_if, cudaStream_t s) {
+  const long N = (long)rows * n;
+  if (N > 0)
+    tc_part_reduce_kernel<<<(unsigned)std::min<long>((N + 255) / 256, 2048), 256, 0, s>>>(part, ksplit, N, n, vin, mode,
+                                                                                          out, run_if);
+  return cudaGetLastError();
+}
+
+// K ranges for a product of few tiles: about one wave of CTAs, each with at least eight k-blocks.
+int tc_ksplit(int M, int N, int K) {
+  const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN), nk = (K + BK - 1) / BK;
+  return std::max(1, std::min(nk / 8, 152 / std::max(1, tiles)));
 }
 
 cudaError_t tc_gemm(const __nv_bfloat16* Ahi, const __nv_bfloat16* Alo, int batch, const __nv_bfloat16* Bhi,
