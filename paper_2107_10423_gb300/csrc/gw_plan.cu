@@ -362,7 +362,7 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc, const double* xi_pos) {
     et.ldh = ldn;
     et.oh_bstride = (long)smat;
     // S = X eps   (eps is symmetric, so it is its own K-major B operand)
-    CK(gw::tc_gemm_ex(Xs[cur], nc, E, 1, ns, n, n, n, 0, et, as<int>(P->tc_err), P->stream));
+    CK(gw::tc_gemm_ex(Xs[cur], nc, E, 1, ns, n, n, n, et, as<int>(P->tc_err), P->stream));
     gw::TcEpi ex{};
     ex.kind = gw::TC_EPI_AXPBY;
     ex.xin = Xf[xf];
@@ -380,7 +380,7 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc, const double* xi_pos) {
     ex.oh_bstride = (long)smat;
     // X <- 2X - S X = 2X - X eps X  (X symmetric: X is its own transpose as the B operand); the last iterate is
     // written as X - I
-    CK(gw::tc_gemm_ex(T, nc, Xs[cur], 1, ns, n, n, n, 0, ex, as<int>(P->tc_err), P->stream));
+    CK(gw::tc_gemm_ex(T, nc, Xs[cur], 1, ns, n, n, n, ex, as<int>(P->tc_err), P->stream));
     cur = 1 - cur;
     P->stats.n_kernel_launches += 2;
   }
@@ -402,7 +402,7 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc, const double* xi_pos) {
     ew.gidx = as<int>(P->ws_gout) + pos;
     ew.bvec = P->d_B_nm_f;
     ew.ldb = n;
-    return gw::tc_gemm_ex(A, nb, Bn, 0, 3, n, R, n, 0, ew, as<int>(P->tc_err), P->stream);
+    return gw::tc_gemm_ex(A, nb, Bn, 0, 3, n, R, n, ew, as<int>(P->tc_err), P->stream);
   };
   auto shift = [&](const gw::TcOperand& op, int b) {
     return gw::TcOperand{{op.p[0] + b * smat, op.p[1] + b * smat, op.p[2] + b * smat}};
@@ -448,7 +448,7 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc, const double* xi_pos) {
     e1.out = C;
     e1.out_bstride = (long)mat;
     e1.ldo = n;
-    CK(gw::tc_gemm_ex(E, nb, E0, 0, 3, n, n, n, 0, e1, as<int>(P->tc_err), P->stream));
+    CK(gw::tc_gemm_ex(E, nb, E0, 0, 3, n, n, n, e1, as<int>(P->tc_err), P->stream));
     // C_b^T = eps_0^-1 M_b, split, as the K-major operand of the next product
     for (int b = 0; b < nb; ++b)
       CK(gw::tc_transpose_split(C + b * mat, n, n, const_cast<__nv_bfloat16*>(T.p[0]) + b * smat,
@@ -467,7 +467,7 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc, const double* xi_pos) {
     e2.olo2 = const_cast<__nv_bfloat16*>(Xs[1 - cur].p[2]);
     e2.ldh = ldn;
     e2.oh_bstride = (long)smat;
-    CK(gw::tc_gemm_ex(shift(Xs[cur], b0), nb, T, 1, 3, n, n, n, 0, e2, as<int>(P->tc_err), P->stream));
+    CK(gw::tc_gemm_ex(shift(Xs[cur], b0), nb, T, 1, 3, n, n, n, e2, as<int>(P->tc_err), P->stream));
     mark(P, 2, t2, 2.0 * 2.0 * nb * (double)n * n * n);
     const size_t t3 = tick(P);
     CK(wred(Xs[1 - cur], nb, g0 + b0));
@@ -977,7 +977,7 @@ gw_status tc_operator(gw_plan* P, int nr, const double* xf, const float* V32, fl
   const gw::TcOperand Vop{{as<__nv_bfloat16>(P->mr_Vhi), as<__nv_bfloat16>(P->mr_Vlo), vlo2}};
   const gw::TcOperand BT{{P->d_BThi, P->d_BTlo, three ? P->d_BTlo2 : nullptr}};
   const int ns = three ? 3 : 2;
-  CK(gw::tc_gemm_ex(Vop, 1, BT, 0, ns, 2 * nr, n_ov, n, 0, e1, as<int>(P->tc_err), P->stream));
+  CK(gw::tc_gemm_ex(Vop, 1, BT, 0, ns, 2 * nr, n_ov, n, e1, as<int>(P->tc_err), P->stream));
   gw::TcEpi e2{};
   // the second product's contraction is the long one: over few output tiles it is split in K ranges (at 50 rows,
   // 629 x 4675, 62 us on 5 CTAs before)
@@ -991,7 +991,7 @@ gw_status tc_operator(gw_plan* P, int nr, const double* xf, const float* V32, fl
   e2.run_if = run_if;
   const gw::TcOperand Uop{{as<__nv_bfloat16>(P->mr_Uhi), as<__nv_bfloat16>(P->mr_Ulo), ulo2}};
   const gw::TcOperand Bop{{P->d_Bhi, P->d_Blo, three ? P->d_Blo2 : nullptr}};
-  CK(gw::tc_gemm_ex(Uop, 1, Bop, 0, ns, 2 * nr, n, n_ov, 0, e2, as<int>(P->tc_err), P->stream));
+  CK(gw::tc_gemm_ex(Uop, 1, Bop, 0, ns, 2 * nr, n, n_ov, e2, as<int>(P->tc_err), P->stream));
   P->stats.n_kernel_launches += 3;
   if (ks > 1) {
     CK(gw::tc_part_reduce(as<float>(P->mr_part), ks, 2 * nr, n, V32, mode, S32, run_if, P->stream));
@@ -1021,7 +1021,7 @@ gw_status tc_operator3(gw_plan* P, int nf, const double* xf, const float* V32, f
   e1.ldh = gw::tc_ld(n_ov);
   const gw::TcOperand Vop{{vp, vp + sv, vp + 2 * sv}};
   const gw::TcOperand BT{{P->d_BThi, P->d_BTlo, P->d_BTlo2}};
-  CK(gw::tc_gemm_ex(Vop, 1, BT, 0, 3, 2 * nf, n_ov, n, 0, e1, as<int>(P->tc_err), P->stream));
+  CK(gw::tc_gemm_ex(Vop, 1, BT, 0, 3, 2 * nf, n_ov, n, e1, as<int>(P->tc_err), P->stream));
   gw::TcEpi e2{};
   e2.kind = gw::TC_EPI_EMBED;
   e2.out = S32;
@@ -1030,7 +1030,7 @@ gw_status tc_operator3(gw_plan* P, int nf, const double* xf, const float* V32, f
   e2.ldv = n;
   const gw::TcOperand Uop{{up, up + su, up + 2 * su}};
   const gw::TcOperand Bop{{P->d_Bhi, P->d_Blo, P->d_Blo2}};
-  CK(gw::tc_gemm_ex(Uop, 1, Bop, 0, 3, 2 * nf, n, n_ov, 0, e2, as<int>(P->tc_err), P->stream));
+  CK(gw::tc_gemm_ex(Uop, 1, Bop, 0, 3, 2 * nf, n, n_ov, e2, as<int>(P->tc_err), P->stream));
   P->stats.n_kernel_launches += 3;
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, P->tc_err.p, sizeof(int), cudaMemcpyDeviceToHost, P->stream));

@@ -1039,7 +1039,7 @@ cudaError_t launch_zlu(T* A, long stride, long plane, int n, int batch, int* per
         ep.half = m;
         ep.limit = limb - ((long)kend * n + kend);
         const TcOperand ao{{lp[0], lp[1], lp[2]}}, bo{{ub[0], ub[1], ub[2]}};
-        e = tc_gemm_ex(ao, nb, bo, 1, 3, 2 * m, m, TC_LDK, 0, ep, err, s);
+        e = tc_gemm_ex(ao, nb, bo, 1, 3, 2 * m, m, TC_LDK, ep, err, s);
         if (e != cudaSuccess) return e;
       }
     }

@@ -12,8 +12,7 @@ enum { TC_EPI_STORE = 0, TC_EPI_CPAIR = 1, TC_EPI_EMBED = 2, TC_EPI_AXPBY = 3, T
 // Epilogue of the tensor-core GEMM (passed by value to the kernel).
 struct TcEpi {
   int kind;
-  // TC_EPI_STORE: out_b[m][n] (row length ldo) = v, delta_mn - v or -v (mode for even / odd batch entries)
-  int mode_even, mode_odd;
+  // TC_EPI_STORE: out_b[m][n] (row length ldo) = v
   float* out;
   long out_bstride;
   int ldo;
@@ -89,12 +88,6 @@ cudaError_t tc_pi_panel_split(const float* B, long ldb, int n, int K, __nv_bfloa
 void tc_pi_fused_tile_order(int n, std::vector<uint32_t>& tiles);
 // The split the autotuner chose for a shape with the given largest feasible split, or 0 if it has not seen it.
 int tc_pi_fused_ksplit(int n, int K, int nb, int max_ctas, int max_split);
-// out_b = f(A_b Bm^T) for b < batch, out [batch][M][N] FP32; lower != 0 computes lower tiles and mirrors.
-// mode_even / mode_odd for even / odd b: 0 v, 1 delta - v, 2 -v.  *err (device) receives a nonzero code if a
-// bounded wait inside the kernel ran out.
-cudaError_t tc_gemm(const __nv_bfloat16* Ahi, const __nv_bfloat16* Alo, int batch, const __nv_bfloat16* Bhi,
-                    const __nv_bfloat16* Blo, int M, int N, int K, int lower, int mode_even, int mode_odd, float* out,
-                    int* err, cudaStream_t s);
 // Split operand: parts p[0..nsplit) of [batch][rows][tc_ld(K)] BF16 (hi, lo[, lo2]).
 struct TcOperand {
   const __nv_bfloat16* p[3];
@@ -102,7 +95,7 @@ struct TcOperand {
 // General form: B may also be batched (b_batched != 0: Bm_b has the same batch count as A); nsplit 2 uses three
 // products (BF16x3), nsplit 3 the six products with part indices i + j <= 2 (about FP32-accurate).
 cudaError_t tc_gemm_ex(const TcOperand& A, int batch, const TcOperand& B, int b_batched, int nsplit, int M, int N,
-                       int K, int lower, const TcEpi& ep, int* err, cudaStream_t s);
+                       int K, const TcEpi& ep, int* err, cudaStream_t s);
 // K ranges worth taking for an M x N x K product (1: none), and the sum of its partial products: out[r][c] = sum (mode
 // 0) or the residue operator's embedding (r odd ? -vin : vin)[r][c] - sum (mode 1).
 int tc_ksplit(int M, int N, int K);

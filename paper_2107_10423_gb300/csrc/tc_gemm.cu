@@ -9,6 +9,7 @@
 // Every mbarrier wait is bounded: on timeout the kernel records an error code and unwinds.
 #include "pi_tc.cuh"
 #include "gw_internal.cuh"
+#include "tc_ptx.cuh"
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -132,93 +133,127 @@ __device__ __forceinline__ void split_store(float v, __nv_bfloat16* hi, __nv_bfl
   if (lo2) lo2[o] = __float2bfloat16_rn(r - __bfloat162float(m));
 }
 
-__device__ void epilogue(const TcEpi& ep, const float* stg, int m0, int n0, int M, int N, int b, int lower,
-                         int* err) {
+// FP32 pair sum s += a b (48 bits: exact product by an FMA error term, Knuth's TwoSum), for reductions that would
+// otherwise take three operations an element on the FP64 pipe (16 clocks a warp each).
+__device__ __forceinline__ void df_fma(float a, float b, float& sh, float& sl) {
+  const float p = __fmul_rn(a, b), pe = __fmaf_rn(a, b, -p);
+  const float t = __fadd_rn(sh, p), v = __fsub_rn(t, sh);
+  const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, v)), __fsub_rn(p, v));
+  sl = __fadd_rn(sl, __fadd_rn(e, pe));
+  sh = t;
+}
+
+// stg: [BM][TN + 1] staged tile; aux: 4 TN floats of shared memory.
+template <int TN, int NTH>
+__device__ void epilogue(const TcEpi& ep, const float* stg, float* aux, int m0, int n0, int M, int N, int b, int* err) {
+  constexpr int LDS_ = TN + 1;
   if (ep.kind == TC_EPI_STORE) {
-    const int mode = (b & 1) ? ep.mode_odd : ep.mode_even;
     float* o = ep.out + (long)b * ep.out_bstride;
-    for (int idx = threadIdx.x; idx < BM * BN; idx += THREADS) {
-      const int rr = idx / BN, cc = idx % BN;
+    for (int idx = threadIdx.x; idx < BM * TN; idx += NTH) {
+      const int rr = idx / TN, cc = idx % TN;
       const int m = m0 + rr, n = n0 + cc;
-      if (m >= M || n >= N) continue;
-      if (lower && n > m) continue;
-      float v = stg[rr * (BN + 1) + cc];
-      v = mode == 0 ? v : (mode == 1 ? ((m == n ? 1.f : 0.f) - v) : -v);
-      o[(long)m * ep.ldo + n] = v;
-    }
-    if (lower) {
-      for (int idx = threadIdx.x; idx < BM * BN; idx += THREADS) {
-        const int cc = idx / BM, rr = idx % BM;
-        const int m = m0 + rr, n = n0 + cc;
-        if (m >= M || n >= N || n >= m) continue;
-        const float v = stg[rr * (BN + 1) + cc];
-        o[(long)n * ep.ldo + m] = mode == 0 ? v : -v;
-      }
+      if (m < M && n < N) o[(long)m * ep.ldo + n] = stg[rr * LDS_ + cc];
     }
   } else if (ep.kind == TC_EPI_CPAIR) {
     // rows (2j, 2j+1) hold B^T u and B^T v of z_j = u - i v; column k is the pair ia.
     // w = c_k(x_j) (t_r + i t_i) with t = B^T z, c_k(x) = 2[1/(x - D_k + i eta) + 1/(-x - D_k + i eta)];
-    // Re w and Im w go to rows 2j, 2j+1 of the split operand of the second GEMM.
+    // Re w and Im w go to rows 2j, 2j+1 of the split operand of the second GEMM.  x and D enter as FP32 pairs, split
+    // once a row and column: x - D in FP64 for every element was four operations on the FP64 pipe, 8 us a tile.
+    float* Dh = aux;
+    float* Dl = aux + TN;
+    float* xh = aux + 2 * TN;
+    float* xl = xh + BM / 2;
+    for (int i = threadIdx.x; i < TN + BM / 2; i += NTH) {
+      const bool col = i < TN;
+      const int at = col ? n0 + i : (m0 >> 1) + i - TN;
+      const double v = col ? (at < N ? ep.Dk[at] : 0.0) : (at < (M >> 1) ? ep.x[at] : 0.0);
+      const float h = (float)v, l = (float)(v - (double)h);
+      if (col) { Dh[i] = h; Dl[i] = l; } else { xh[i - TN] = h; xl[i - TN] = l; }
+    }
+    __syncthreads();
     const float e2 = ep.eta * ep.eta;
-    for (int idx = threadIdx.x; idx < (BM / 2) * BN; idx += THREADS) {
-      const int pr = idx / BN, cc = idx % BN;
+    for (int idx = threadIdx.x; idx < (BM / 2) * TN; idx += NTH) {
+      const int pr = idx / TN, cc = idx % TN;
       const int m = m0 + 2 * pr, n = n0 + cc;
       if (m >= M || n >= N) continue;
-      const double x = ep.x[m >> 1], D = ep.Dk[n];
-      const float a1 = (float)(x - D), a2 = (float)(-x - D);
+      const float a1 = (xh[pr] - Dh[cc]) + (xl[pr] - Dl[cc]), a2 = -((xh[pr] + Dh[cc]) + (xl[pr] + Dl[cc]));
       const float d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
       const float cr = 2.f * (a1 / d1 + a2 / d2);
       const float ci = -2.f * ep.eta * (1.f / d1 + 1.f / d2);
-      const float tr = stg[(2 * pr) * (BN + 1) + cc], ti = -stg[(2 * pr + 1) * (BN + 1) + cc];
+      const float tr = stg[(2 * pr) * LDS_ + cc], ti = -stg[(2 * pr + 1) * LDS_ + cc];
       split_store(cr * tr - ci * ti, ep.ohi, ep.olo, (long)m * ep.ldh + n, ep.olo2);
       split_store(cr * ti + ci * tr, ep.ohi, ep.olo, (long)(m + 1) * ep.ldh + n, ep.olo2);
     }
   } else if (ep.kind == TC_EPI_AXPBY) {
-    // EPI_U elements per thread and pass: their global reads are issued together before any store
-    for (int base = threadIdx.x; base < BM * BN; base += THREADS * EPI_U) {
-      float xv[EPI_U];
+    // two columns a thread (the split rows are 16-byte multiples, so pairs stay aligned); EPI_U pairs a pass, whose
+    // global reads are issued together before any store
+    for (int base = threadIdx.x; base < BM * TN / 2; base += NTH * EPI_U) {
+      float2 xv[EPI_U];
 #pragma unroll
       for (int u = 0; u < EPI_U; ++u) {
-        const int idx = base + u * THREADS, rr = idx / BN, cc = idx % BN, m = m0 + rr, n = n0 + cc;
-        xv[u] = (ep.xin && idx < BM * BN && m < M && n < N)
-                    ? ep.xin[(long)b * ep.x_bstride + (long)m * ep.ldo + n] : 0.f;
+        const int idx = base + u * NTH, rr = idx / (TN / 2), cc = 2 * (idx % (TN / 2)), m = m0 + rr, n = n0 + cc;
+        xv[u] = make_float2(0.f, 0.f);
+        if (ep.xin && idx < BM * TN / 2 && m < M && n < N) {
+          const float* x = ep.xin + (long)b * ep.x_bstride + (long)m * ep.ldo + n;
+          xv[u].x = x[0];
+          if (n + 1 < N) xv[u].y = x[1];
+        }
       }
 #pragma unroll
       for (int u = 0; u < EPI_U; ++u) {
-        const int idx = base + u * THREADS, rr = idx / BN, cc = idx % BN, m = m0 + rr, n = n0 + cc;
-        if (idx >= BM * BN || m >= M || n >= N) continue;
-        const float y = ep.gamma * stg[rr * (BN + 1) + cc] + (m == n ? ep.beta : 0.f) + ep.alpha * xv[u];
-        if (ep.out) ep.out[(long)b * ep.out_bstride + (long)m * ep.ldo + n] = y;
-        if (ep.ohi) split_store(y, ep.ohi, ep.olo, (long)b * ep.oh_bstride + (long)m * ep.ldh + n, ep.olo2);
+        const int idx = base + u * NTH, rr = idx / (TN / 2), cc = 2 * (idx % (TN / 2)), m = m0 + rr, n = n0 + cc;
+        if (idx >= BM * TN / 2 || m >= M || n >= N) continue;
+        const float y0 = ep.gamma * stg[rr * LDS_ + cc] + (m == n ? ep.beta : 0.f) + ep.alpha * xv[u].x;
+        const float y1 = n + 1 < N ? ep.gamma * stg[rr * LDS_ + cc + 1] + (m == n + 1 ? ep.beta : 0.f) +
+                                         ep.alpha * xv[u].y
+                                   : 0.f;              // the row's padding
+        if (ep.out) {
+          float* o = ep.out + (long)b * ep.out_bstride + (long)m * ep.ldo + n;
+          o[0] = y0;
+          if (n + 1 < N) o[1] = y1;
+        }
+        if (ep.ohi) {
+          const long o = (long)b * ep.oh_bstride + (long)m * ep.ldh + n;
+          const __nv_bfloat162 h = __floats2bfloat162_rn(y0, y1);
+          const float r0 = y0 - __low2float(h), r1 = y1 - __high2float(h);
+          const __nv_bfloat162 l = __floats2bfloat162_rn(r0, r1);
+          *reinterpret_cast<__nv_bfloat162*>(ep.ohi + o) = h;
+          *reinterpret_cast<__nv_bfloat162*>(ep.olo + o) = l;
+          if (ep.olo2)
+            *reinterpret_cast<__nv_bfloat162*>(ep.olo2 + o) = __floats2bfloat162_rn(r0 - __low2float(l),
+                                                                                    r1 - __high2float(l));
+        }
       }
     }
   } else if (ep.kind == TC_EPI_WRED) {
     // column n of the tile: sum over the tile's rows m of bvec[n][m] * v[m][n], added into W
-    if (threadIdx.x < BN) {
+    if (threadIdx.x < TN) {
       const int cc = threadIdx.x, n = n0 + cc;
       if (n < N) {
-        const float* bv = ep.bvec + (long)n * ep.ldb;
-        double acc = 0.0;
-        for (int rr = 0; rr < BM && m0 + rr < M; ++rr) acc += (double)bv[m0 + rr] * stg[rr * (BN + 1) + cc];
-        atomicAdd(ep.W + (long)n * ep.wld + ep.gidx[b], acc);
+        const float* bv = ep.bvec + (long)n * ep.ldb + m0;
+        float sh = 0.f, sl = 0.f;
+        const int rows = min(BM, M - m0);
+#pragma unroll 8
+        for (int rr = 0; rr < rows; ++rr) df_fma(bv[rr], stg[rr * LDS_ + cc], sh, sl);
+        atomicAdd(ep.W + (long)n * ep.wld + ep.gidx[b], (double)sh + (double)sl);
       }
     }
   } else if (ep.kind == TC_EPI_PART) {
     float* o = ep.out + (long)blockIdx.z * M * N;
-    for (int idx = threadIdx.x; idx < BM * BN; idx += THREADS) {
-      const int rr = idx / BN, cc = idx % BN, m = m0 + rr, n = n0 + cc;
-      if (m < M && n < N) o[(long)m * N + n] = stg[rr * (BN + 1) + cc];
+    for (int idx = threadIdx.x; idx < BM * TN; idx += NTH) {
+      const int rr = idx / TN, cc = idx % TN, m = m0 + rr, n = n0 + cc;
+      if (m < M && n < N) o[(long)m * N + n] = stg[rr * LDS_ + cc];
     }
   } else if (ep.kind == TC_EPI_SUB2) {
     float* o = ep.out + (long)b * ep.out_bstride;
-    for (int base = threadIdx.x; base < BM * BN; base += THREADS * EPI_U) {
+    for (int base = threadIdx.x; base < BM * TN; base += NTH * EPI_U) {
       long off[EPI_U];
       float cv[EPI_U];
 #pragma unroll
       for (int u = 0; u < EPI_U; ++u) {
-        const int idx = base + u * THREADS, rr = idx / BN, cc = idx % BN, m = m0 + rr, n = n0 + cc;
+        const int idx = base + u * NTH, rr = idx / TN, cc = idx % TN, m = m0 + rr, n = n0 + cc;
         off[u] = -1;
-        if (idx < BM * BN && m < M && n < N) {
+        if (idx < BM * TN && m < M && n < N) {
           const long o1 = m < ep.half ? (long)m * ep.ldo + n : ep.plane + (long)(m - ep.half) * ep.ldo + n;
           if ((long)b * ep.out_bstride + o1 >= ep.limit || o1 < 0) atomicCAS(err, 0, 66);
           else off[u] = o1;
@@ -227,45 +262,42 @@ __device__ void epilogue(const TcEpi& ep, const float* stg, int m0, int n0, int 
       }
 #pragma unroll
       for (int u = 0; u < EPI_U; ++u) {
-        const int idx = base + u * THREADS, rr = idx / BN, cc = idx % BN;
-        if (off[u] >= 0) o[off[u]] = cv[u] - stg[rr * (BN + 1) + cc];
+        const int idx = base + u * NTH, rr = idx / TN, cc = idx % TN;
+        if (off[u] >= 0) o[off[u]] = cv[u] - stg[rr * LDS_ + cc];
       }
     }
   } else if (ep.kind == TC_EPI_EMBED) {
     // real 2n embedding of (1 - Pi) z: rows 2j: u - (B w)_r, rows 2j+1: -v - (B w)_i
-    for (int base = threadIdx.x; base < BM * BN; base += THREADS * EPI_U) {
+    for (int base = threadIdx.x; base < BM * TN; base += NTH * EPI_U) {
       float vv[EPI_U];
 #pragma unroll
       for (int u = 0; u < EPI_U; ++u) {
-        const int idx = base + u * THREADS, rr = idx / BN, cc = idx % BN, m = m0 + rr, n = n0 + cc;
-        vv[u] = (idx < BM * BN && m < M && n < N) ? ep.vin[(long)m * ep.ldv + n] : 0.f;
+        const int idx = base + u * NTH, rr = idx / TN, cc = idx % TN, m = m0 + rr, n = n0 + cc;
+        vv[u] = (idx < BM * TN && m < M && n < N) ? ep.vin[(long)m * ep.ldv + n] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < EPI_U; ++u) {
-        const int idx = base + u * THREADS, rr = idx / BN, cc = idx % BN, m = m0 + rr, n = n0 + cc;
-        if (idx >= BM * BN || m >= M || n >= N) continue;
-        ep.out[(long)m * ep.ldo + n] = ((m & 1) ? -vv[u] : vv[u]) - stg[rr * (BN + 1) + cc];
+        const int idx = base + u * NTH, rr = idx / TN, cc = idx % TN, m = m0 + rr, n = n0 + cc;
+        if (idx >= BM * TN || m >= M || n >= N) continue;
+        ep.out[(long)m * ep.ldo + n] = ((m & 1) ? -vv[u] : vv[u]) - stg[rr * LDS_ + cc];
       }
     }
   }
 }
 
-// grid.x: output tile (lower-triangular enumeration when `lower`), grid.y: batch entry.
+// grid.x: output tile, grid.y: batch entry, grid.z: K range.
 // Warp roles: warps 0-3 drain the accumulator (TMEM lane quarter = warp), warp 4 issues TMA, warp 5 issues MMA.
 // The contraction is cut into chunks of CHUNK k-blocks; each chunk accumulates in one of two TMEM buffers and
 // is then added into FP32 registers by the drain warps (round to nearest), so no partial sum runs through more
 // than 4 * CHUNK tensor-core accumulates of the dominant hi*hi product (the tensor-core accumulator loses about
 // one ulp per accumulate, which over long K leaves a systematic relative error).
-// mode_even / mode_odd select the epilogue for even / odd batch entries:
-//   0: v    1: delta_mn - v    2: -v
 struct TcMaps {
   CUtensorMap a[3], b[3];
 };
 
 template <int NSP>
 __global__ void __launch_bounds__(THREADS, 1)
-    tc_gemm_kernel(const __grid_constant__ TcMaps maps, int M, int N, int K, int lower, int b_batched, const TcEpi ep,
-                   int* __restrict__ err) {
+    tc_gemm_kernel(const __grid_constant__ TcMaps maps, int M, int N, int K, int b_batched, const TcEpi ep, int* __restrict__ err) {
   constexpr int STAGES = TcCfg<NSP>::STAGES;
   constexpr int STAGE_BYTES = TcCfg<NSP>::STAGE_BYTES;
   constexpr int CHUNK = TcCfg<NSP>::CHUNK;
@@ -280,18 +312,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   __shared__ int s_abort;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int bm, bn;
-  if (lower) {
-    int t = blockIdx.x;
-    bm = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
-    while ((bm + 1) * (bm + 2) / 2 <= t) ++bm;
-    while (bm * (bm + 1) / 2 > t) --bm;
-    bn = t - bm * (bm + 1) / 2;
-  } else {
-    const int nbn = (N + BN - 1) / BN;
-    bm = blockIdx.x / nbn;
-    bn = blockIdx.x % nbn;
-  }
+  const int nbn = (N + BN - 1) / BN;
+  const int bm = blockIdx.x / nbn, bn = blockIdx.x % nbn;
   const int m0 = bm * BM, n0 = bn * BN, b = blockIdx.y;
   // this CTA's range of k-blocks (grid.z > 1: TC_EPI_PART)
   const int nk_all = (K + BK - 1) / BK, kb0 = (int)((long)nk_all * blockIdx.z / gridDim.z);
@@ -415,7 +437,199 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int j = 0; j < BN; ++j) stg[r * (BN + 1) + j] = acc[j];
   }
   __syncthreads();
-  if (all_ok) epilogue(ep, stg, m0, n0, M, N, b, lower, err);
+  if (all_ok) epilogue<BN, THREADS>(ep, stg, stg + BM * (BN + 1), m0, n0, M, N, b, err);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+  }
+}
+
+// ------------------------------------------------------------------ 128 x 256 tiles
+// The same product in M128 N256 instructions.  What bounds it: L2 -> SM traffic (about 37 B a clock and SM on this
+// chip) and shared-memory reads; a 128 x 128 tile moves 64 (three parts) or 85 B a clock at full tensor rate, this one
+// 47 or 62, and reads 12 KiB of shared memory per 128 clocks instead of 16.
+// Accumulators: TMEM columns [0, 256) the hi*hi sum of BIGC k-blocks (of 32), [256, 512) the cross terms of SMALLC.
+// A k-block's cross terms are issued first, so the drain of the previous hi*hi sum runs beside them; the cross terms are
+// 2^-8 of the sum, so their accumulator may run four times as long for the same error.  Eight drain warps (TMEM lane
+// quarter = warp & 3, column half = warp >> 2) add both into FP32 registers, rounded to nearest.
+constexpr int WN = 256, WK = 32;
+template <int NSP>
+struct WideCfg {
+  static constexpr int BIGC = NSP == 2 ? 8 : 2, SMALLC = 4 * BIGC;
+  static constexpr int STAGES = NSP == 2 ? 4 : 3;
+  static constexpr int A_TILE = BM * WK * 2, B_TILE = WN * WK * 2;
+  static constexpr int STAGE_BYTES = NSP * (A_TILE + B_TILE);
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+  static_assert(BM * (WN + 1) * 4 + 4 * WN * 4 <= STAGES * STAGE_BYTES, "the staged tile reuses the ring");
+};
+constexpr long kWideMinTiles = 120;
+constexpr int WDRAIN = 8, WTHREADS = 32 * (WDRAIN + 2);
+constexpr uint32_t WIDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(WN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+
+template <int NSP>
+__global__ void __launch_bounds__(WTHREADS, 1)
+    tc_gemm_wide_kernel(const __grid_constant__ TcMaps maps, int M, int N, int K, int b_batched, const TcEpi ep,
+                        int* __restrict__ err) {
+  using C = WideCfg<NSP>;
+  constexpr int STAGES = C::STAGES;
+  if (ep.run_if && *ep.run_if == 0) return;     // uniform over the grid: nothing is allocated yet
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* smem = smem_raw + (base - raw);
+  const uint32_t bar0 = base + STAGES * C::STAGE_BYTES;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + STAGES * C::STAGE_BYTES + 128);
+  auto full = [bar0](int s) { return bar0 + 8u * (uint32_t)s; };
+  auto empty = [bar0](int s) { return bar0 + 8u * (uint32_t)(STAGES + s); };
+  const uint32_t acc_full = bar0 + 8u * (2 * STAGES), big_empty = acc_full + 8u, small_empty = acc_full + 16u,
+                 fin = acc_full + 24u;
+  __shared__ int s_abort;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nbn = (N + WN - 1) / WN;
+  const int m0 = (blockIdx.x / nbn) * BM, n0 = (blockIdx.x % nbn) * WN, b = blockIdx.y;
+  const int nk = (K + WK - 1) / WK;
+
+  if (threadIdx.x == 0) {
+    s_abort = 0;
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(full(s), 1);
+      mbar_init(empty(s), 1);
+    }
+    mbar_init(acc_full, 1);
+    mbar_init(big_empty, WDRAIN);
+    mbar_init(small_empty, WDRAIN);
+    mbar_init(fin, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+
+  float acc[128];
+  bool ok = true;
+  if (warp == WDRAIN) {
+    if (lane == 0) {
+      // ---------------- TMA producer
+      int issued = 0;
+      bool go = true;
+      for (int kb = 0; kb < nk && go; ++kb) {
+        const int s = kb % STAGES, u = kb / STAGES;
+        if (u > 0 && !mbar_wait(empty(s), (u - 1) & 1, err, 1)) go = false;
+        if (!go || *(volatile int*)&s_abort) { go = false; break; }
+        const uint32_t st = base + s * C::STAGE_BYTES;
+        mbar_expect_tx(full(s), C::STAGE_BYTES);
+#pragma unroll
+        for (int i = 0; i < NSP; ++i) tma_load_3d(st + i * C::A_TILE, &maps.a[i], kb * WK, m0, b, full(s));
+#pragma unroll
+        for (int j = 0; j < NSP; ++j)
+          tma_load_3d(st + NSP * C::A_TILE + j * C::B_TILE, &maps.b[j], kb * WK, n0, b_batched ? b : 0, full(s));
+        issued = kb + 1;
+      }
+      if (!go) {
+        s_abort = 1;
+        for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
+          mbar_wait(full(kb % STAGES), (kb / STAGES) & 1, err, 4);
+      }
+    }
+  } else if (warp == WDRAIN + 1) {
+    if (lane == 0) {
+      // ---------------- MMA issuer
+      bool go = true;
+      uint32_t nbig = 0, nsmall = 0;
+      const uint64_t dA = ptx::sdesc(base, 8 * 64, 4), dB = ptx::sdesc(base + NSP * C::A_TILE, 8 * 64, 4);
+      for (int kb = 0; kb < nk; ++kb) {
+        const int s = kb % STAGES, u = kb / STAGES;
+        const bool bfirst = kb % C::BIGC == 0, sfirst = kb % C::SMALLC == 0;
+        if (!mbar_wait(full(s), u & 1, err, 2)) { go = false; break; }
+        if (*(volatile int*)&s_abort) { go = false; break; }
+        if (sfirst && kb > 0) {
+          if (!mbar_wait(small_empty, nsmall & 1u, err, 6)) { go = false; break; }
+          ++nsmall;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t a0 = dA + (uint64_t)((s * C::STAGE_BYTES) >> 4), b0 = dB + (uint64_t)((s * C::STAGE_BYTES) >> 4);
+#pragma unroll
+        for (int k = 0; k < WK / 16; ++k)
+#pragma unroll
+          for (int i = 0; i < NSP; ++i)
+#pragma unroll
+            for (int j = 0; j + i < NSP; ++j)
+              if (i + j > 0)
+                ptx::mma_bf16(tmem + WN, a0 + (uint64_t)((i * C::A_TILE) >> 4) + 2 * k,
+                              b0 + (uint64_t)((j * C::B_TILE) >> 4) + 2 * k, WIDESC,
+                              (sfirst && k == 0 && i == 0 && j == 1) ? 0u : 1u);
+        if (bfirst && kb > 0) {
+          if (!mbar_wait(big_empty, nbig & 1u, err, 5)) { go = false; break; }
+          ++nbig;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+#pragma unroll
+        for (int k = 0; k < WK / 16; ++k)
+          ptx::mma_bf16(tmem, a0 + 2 * k, b0 + 2 * k, WIDESC, (bfirst && k == 0) ? 0u : 1u);
+        mma_commit(empty(s));
+        if (kb % C::BIGC == C::BIGC - 1 || kb == nk - 1) mma_commit(acc_full);
+      }
+      if (!go) s_abort = 1;
+      mma_commit(fin);             // every product issued above has completed once this flips
+      mbar_wait(fin, 0, err, 7);
+    }
+  } else {
+    // ---------------- drain warps
+    const uint32_t addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 128);
+#pragma unroll
+    for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+    const int nchunks = (nk + C::BIGC - 1) / C::BIGC;
+    for (int c = 0; c < nchunks; ++c) {
+      ok = !*(volatile int*)&s_abort && mbar_wait(acc_full, c & 1, err, 3);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        uint32_t v[32];
+        tmem_ld32(addr + (uint32_t)(g * 32), v);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[g * 32 + j] += __uint_as_float(v[j]);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(big_empty) : "memory");
+      if (c % (C::SMALLC / C::BIGC) == C::SMALLC / C::BIGC - 1 || c == nchunks - 1) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          uint32_t v[32];
+          tmem_ld32(addr + (uint32_t)(WN + g * 32), v);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) acc[g * 32 + j] += __uint_as_float(v[j]);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(small_empty) : "memory");
+      }
+    }
+    if (!ok) s_abort = 1;
+  }
+  __syncwarp();
+  const bool all_ok = __syncthreads_and(ok && !*(volatile int*)&s_abort) != 0;
+  float* stg = reinterpret_cast<float*>(smem);     // [BM][WN + 1], reuses the operand ring
+  if (all_ok && warp < WDRAIN) {
+    const int r = (warp & 3) * 32 + lane, c = (warp >> 2) * 128;
+#pragma unroll
+    for (int j = 0; j < 128; ++j) stg[r * (WN + 1) + c + j] = acc[j];
+  }
+  __syncthreads();
+  if (all_ok) epilogue<WN, WTHREADS>(ep, stg, stg + BM * (WN + 1), m0, n0, M, N, b, err);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
@@ -441,15 +655,16 @@ PFN_encodeTiled get_encode() {
   return fn;
 }
 
-bool make_map(CUtensorMap* map, const void* ptr, int rows, int K, int ld, int batch) {
+bool make_map(CUtensorMap* map, const void* ptr, int rows, int K, int ld, int batch, int box_k, int box_rows,
+              CUtensorMapSwizzle swz) {
   PFN_encodeTiled enc = get_encode();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)batch};
   cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)ld * 2 * rows};
-  cuuint32_t box[3] = {BK, BM, 1};
+  cuuint32_t box[3] = {(cuuint32_t)box_k, (cuuint32_t)box_rows, 1};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, batch > 0 ? 3 : 2, const_cast<void*>(ptr), dims, strides,
-                   box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                   box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
@@ -459,37 +674,50 @@ bool make_map(CUtensorMap* map, const void* ptr, int rows, int K, int ld, int ba
 int tc_ld(int K) { return (K + 7) / 8 * 8; }
 
 cudaError_t tc_gemm_ex(const TcOperand& A, int batch, const TcOperand& B, int b_batched, int nsplit, int M, int N,
-                       int K, int lower, const TcEpi& ep, int* err, cudaStream_t s) {
+                       int K, const TcEpi& ep, int* err, cudaStream_t s) {
   const int ld = tc_ld(K);
   TcMaps maps;
   const int bb = b_batched ? batch : 1;
   if (nsplit != 2 && nsplit != 3) return cudaErrorInvalidValue;
+  // 128 x 256 tiles wherever they are enough CTAs for the chip; products of fewer tiles and split-K products run in
+  // 128 x 128 tiles, twice the CTAs
+  const long nbm = (M + BM - 1) / BM, wide_tiles = nbm * ((N + WN - 1) / WN);
+  const bool wide = ep.kind != TC_EPI_PART && N > BN && wide_tiles * batch >= kWideMinTiles;
   for (int i = 0; i < nsplit; ++i)
-    if (!A.p[i] || !B.p[i] || !make_map(&maps.a[i], A.p[i], M, K, ld, batch) ||
-        !make_map(&maps.b[i], B.p[i], N, K, ld, bb))
+    if (!A.p[i] || !B.p[i] ||
+        !make_map(&maps.a[i], A.p[i], M, K, ld, batch, wide ? WK : BK, BM,
+                  wide ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map(&maps.b[i], B.p[i], N, K, ld, bb, wide ? WK : BK, wide ? WN : BN,
+                  wide ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B))
       return cudaErrorInvalidValue;
-  const int nbm = (M + BM - 1) / BM, nbn = (N + BN - 1) / BN;
-  const int tiles = lower ? nbm * (nbm + 1) / 2 : nbm * nbn;
-  dim3 grid(tiles, batch, ep.kind == TC_EPI_PART ? std::max(1, ep.ksplit) : 1);
-  if (nsplit == 2) {
-    static bool attr = false;
-    if (!attr) {
-      cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           TcCfg<2>::SMEM_BYTES);
-      if (e != cudaSuccess) return e;
-      attr = true;
-    }
-    tc_gemm_kernel<2><<<grid, THREADS, TcCfg<2>::SMEM_BYTES, s>>>(maps, M, N, K, lower, b_batched, ep, err);
-  } else {
-    static bool attr = false;
-    if (!attr) {
-      cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           TcCfg<3>::SMEM_BYTES);
-      if (e != cudaSuccess) return e;
-      attr = true;
-    }
-    tc_gemm_kernel<3><<<grid, THREADS, TcCfg<3>::SMEM_BYTES, s>>>(maps, M, N, K, lower, b_batched, ep, err);
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         TcCfg<2>::SMEM_BYTES);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(tc_gemm_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<3>::SMEM_BYTES);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(tc_gemm_wide_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               WideCfg<2>::SMEM_BYTES);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(tc_gemm_wide_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               WideCfg<3>::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    attr = true;
   }
+  if (wide) {
+    const dim3 grid((unsigned)wide_tiles, batch);
+    if (nsplit == 2)
+      tc_gemm_wide_kernel<2><<<grid, WTHREADS, WideCfg<2>::SMEM_BYTES, s>>>(maps, M, N, K, b_batched, ep, err);
+    else
+      tc_gemm_wide_kernel<3><<<grid, WTHREADS, WideCfg<3>::SMEM_BYTES, s>>>(maps, M, N, K, b_batched, ep, err);
+    return cudaGetLastError();
+  }
+  const dim3 grid((unsigned)(nbm * ((N + BN - 1) / BN)), batch, ep.kind == TC_EPI_PART ? std::max(1, ep.ksplit) : 1);
+  if (nsplit == 2)
+    tc_gemm_kernel<2><<<grid, THREADS, TcCfg<2>::SMEM_BYTES, s>>>(maps, M, N, K, b_batched, ep, err);
+  else
+    tc_gemm_kernel<3><<<grid, THREADS, TcCfg<3>::SMEM_BYTES, s>>>(maps, M, N, K, b_batched, ep, err);
   return cudaGetLastError();
 }
 
@@ -519,20 +747,6 @@ cudaError_t tc_part_reduce(const float* part, int ksplit, int rows, int n, const
 int tc_ksplit(int M, int N, int K) {
   const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN), nk = (K + BK - 1) / BK;
   return std::max(1, std::min(nk / 8, 152 / std::max(1, tiles)));
-}
-
-cudaError_t tc_gemm(const __nv_bfloat16* Ahi, const __nv_bfloat16* Alo, int batch, const __nv_bfloat16* Bhi,
-                    const __nv_bfloat16* Blo, int M, int N, int K, int lower, int mode_even, int mode_odd, float* out,
-                    int* err, cudaStream_t s) {
-  TcEpi ep{};
-  ep.kind = TC_EPI_STORE;
-  ep.mode_even = mode_even;
-  ep.mode_odd = mode_odd;
-  ep.out = out;
-  ep.out_bstride = (long)M * N;
-  ep.ldo = N;
-  const TcOperand a{{Ahi, Alo, nullptr}}, bo{{Bhi, Blo, nullptr}};
-  return tc_gemm_ex(a, batch, bo, 0, 2, M, N, K, lower, ep, err, s);
 }
 
 // B^T split: out[k][m] = B[m][k] as BF16 hi/lo, rows of length tc_ld(M).  32 x 32 tiles through shared memory.
