@@ -111,9 +111,29 @@ cudaError_t sd_jacobi_sweep(double* M, double* T, int Np, double* cs, cudaStream
 cudaError_t sd_offdiag(const double* M, int Np, double* off, cudaStream_t s);
 cudaError_t sd_weights(const double* B, const double* Dk, const double* M, const double* T, const double* Bn,
                        int n_aux, int N, int Np, int R, double* Om, double* V, double* w2, cudaStream_t s);
+// part [npts][sd_sigma_parts][2] is work space.
+int sd_sigma_parts(int n_bas, int N);
 cudaError_t sd_sigma(const double* w2, const double* Om, int N, int n_bas, const double* eps, const int* tmap,
                      const int* spin, const int* occ_t, int n_occ, const double* omega, int npts, double eta,
-                     double* S, double* dS, cudaStream_t s);
+                     double* part, double* S, double* dS, cudaStream_t s);
+// Direct route (N <= sd_direct_max()): A [N][ld] (overwritten) = Q T Q^T with reflectors H [N][ld], beta, d, e [N]
+// (p_buf [4 N], bar one counter, *err set if a wait ran out); then eigenvectors Z (rows, length ld) of A from T by
+// bisection (lam), twisted factorisations (W1, W2 [N][ldw]) and the reflectors; nrm [N] work space.
+int sd_direct_max();
+cudaError_t sd_tridiagonal(double* A, int N, long ld, double* H, double* beta, double* d, double* e, double* p_buf,
+                           unsigned* bar, int* err, cudaStream_t s);
+cudaError_t sd_tridiagonal_vectors(const double* d, const double* e, int N, double* lam, double* W1, double* W2, long ldw,
+                                   const double* H, const double* beta, long ld, double* nrm, double* Z,
+                                   cudaStream_t s);
+// Refinement step on rows V with S = V M V^T and G = V V^T ([N][N]): norms [3] (off-diagonal and diagonal squares of S,
+// squares of I - G), and C = I + E^T, the factor of the next rows C V.
+cudaError_t sd_eig_norms(const double* S, const double* G, int N, double* norms, cudaStream_t s);
+cudaError_t sd_eig_update(const double* S, double* G, int N, double* C, const double* norms, cudaStream_t s);
+cudaError_t sd_pack_rows(const double* X, int rows, int N, long ld, double* Y, cudaStream_t s);
+cudaError_t sd_twice_sqrt(const double* Dk, int N, double* w, cudaStream_t s);
+// Omega from S and G, and the pole weights from V = 2 B D^1/2 T [n_aux][N].
+cudaError_t sd_rows_weights(const double* S, const double* G, const double* V, const double* Bn, int n_aux, int N, int R,
+                            double* Om, double* w2, cudaStream_t s);
 // Blocked LU of `batch` complex matrices (planes A and A + plane, matrix stride `stride`, FP32 or FP64) with partial
 // pivoting, in place, trailing updates on the tensor cores.  perm [batch][n]: the row order as launch_zlu_solve reads it
 // (the original row at each row of the factors; the sequential swaps for n > 16384, FP64 8192); info[b]: 0, or the first zero pivot's column + 1.  Work space: work of work_elems BF16 (at least

@@ -75,7 +75,7 @@ struct gw_plan {
   __nv_bfloat16* d_Bnlo2 = nullptr;
   bool screening_done = false;
   // spectral-decomposition route (gw_sigma_sd): Casida matrix and eigenvectors, pole weights; valid while sd_done
-  DevBuf sd_M, sd_T, sd_cs, sd_off, sd_Om, sd_V, sd_w2, sd_tmap, sd_om, sd_S, sd_dS;
+  DevBuf sd_M, sd_T, sd_cs, sd_off, sd_Om, sd_V, sd_w2, sd_tmap, sd_om, sd_S, sd_dS, sd_part, sd_x[5], sd_vec;
   bool sd_done = false;
   int sd_sweeps = 0;
   // sharding across ranks (gw_set_shard): frequency positions [sh_p0, sh_p1) of the imaginary-axis stage and the
@@ -115,7 +115,7 @@ struct gw_plan {
     DevBuf* all[] = {&oz_A, &oz_B, &oz_X, &oz_sc, &oz_w, &op_BT, &op_sc, &op_V, &ws_mat, &ws_info, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
                      &mr_v, &mr_d1, &mr_d2, &mr_x, &mr_st, &mr_rt, &mr_rm, &mr_xf, &mr_wre, &mr_wim,
                      &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &mr_part, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
-                     &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_lu, &fb_sw, &fb_linv, &fb_lus, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS};
+                     &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_lu, &fb_sw, &fb_linv, &fb_lus, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS, &sd_part, &sd_x[0], &sd_x[1], &sd_x[2], &sd_x[3], &sd_x[4], &sd_vec};
     bufs.assign(all, all + sizeof(all) / sizeof(all[0]));
   }
 };
@@ -1833,6 +1833,115 @@ gw_status gw_sigma_cd(gw_plan_t P, const double* omega, double* sigma_c, double*
 // the factor 4 into the 2 of each spin block) diagonalised by cyclic Jacobi sweeps in FP64 until the off-diagonal
 // Frobenius norm is below 1e-13 of the diagonal one, then Omega_s and the pole weights of every (target, state).
 constexpr long kSdMaxPairs = 16384;       // O(N_ov^3) work and 2 N_ov^2 doubles of storage
+
+// One N_ov x N_ov FP64 product C = X Y^T by digits, in buffers sd_direct has sized; Yt: Y given transposed (C = X Yt).
+gw_status sd_product(gw_plan* P, const double* X, const double* Y, const double* Yt, double* C) {
+  const int N = P->n_ov;
+  double* sa = as<double>(P->oz_sc);
+  double* sb = sa + N;
+  __nv_bfloat16* da = as<__nv_bfloat16>(P->oz_A);
+  __nv_bfloat16* db = as<__nv_bfloat16>(P->oz_B);
+  CK(gw::oz_row_digits(X, N, N, N, sa, da, P->stream));
+  if (Yt) {
+    CK(gw::oz_col_scale(Yt, N, N, N, sb, P->stream));
+    CK(gw::oz_split_transpose(Yt, N, N, N, sb, db, P->stream));
+  } else if (Y == X) {
+    db = da;
+    sb = sa;
+  } else {
+    CK(gw::oz_row_digits(Y, N, N, N, sb, db, P->stream));
+  }
+  gw::OzEpi ep{};
+  ep.kind = gw::OZ_EPI_STORE;
+  ep.out = C;
+  ep.ldo = N;
+  CK(gw::oz_gemm(gw::OzOperand{da, sa, 0}, gw::OzOperand{db, sb, 0}, 1, N, N, N, ep, as<int>(P->tc_err), P->stream));
+  P->stats.n_kernel_launches += 3;
+  return GW_OK;
+}
+
+// Eigenvectors of the Casida matrix by tridiagonalisation and refinement on digit products (kernels_sd.cu); *ok is 0
+// where the off-diagonal criterion of the Jacobi sweeps is not met (they then start from the matrix in sd_M).
+gw_status sd_direct(gw_plan* P, int Np, bool* ok) {
+  *ok = false;
+  const int N = P->n_ov, n = P->cfg.n_aux, R = P->n_t * P->n_bas;
+  const size_t nn = sizeof(double) * (size_t)N * N;
+  TRY(ensure(P, P->tc_err, sizeof(int)));
+  // everything up front: where the digits (16 N max(N, n) bytes twice) and the five matrices do not fit, the sweeps run
+  // in the memory they have
+  const size_t dg_bytes = sizeof(__nv_bfloat16) * std::max(gw::oz_elems(N, N), gw::oz_elems(n, N));
+  gw_status fit = GW_OK;
+  for (int i = 0; i < 5 && fit == GW_OK; ++i) fit = ensure(P, P->sd_x[i], nn);
+  if (fit == GW_OK) fit = ensure(P, P->sd_vec, sizeof(double) * (9 * (size_t)N + 8));
+  if (fit == GW_OK) fit = ensure(P, P->oz_A, dg_bytes);
+  if (fit == GW_OK) fit = ensure(P, P->oz_B, dg_bytes);
+  if (fit == GW_OK) fit = ensure(P, P->oz_sc, sizeof(double) * (2 * (size_t)std::max(N, n) + N + 1));
+  if (fit != GW_OK) {
+    (void)cudaGetLastError();
+    for (DevBuf& b : P->sd_x) {
+      if (b.p) cudaFree(b.p);
+      count_bytes(P, -(long long)b.bytes);
+      b = DevBuf{};
+    }
+    return GW_OK;
+  }
+  CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
+  double* M = as<double>(P->sd_x[0]);      // the matrix, row length N
+  double* A = as<double>(P->sd_x[1]);      // its working copy; then pivots, S
+  double* H = as<double>(P->sd_x[2]);      // reflectors; then G, C
+  double* W = as<double>(P->sd_x[3]);      // pivots; then M V^T
+  double* V = as<double>(P->sd_x[4]);      // eigenvectors, rows
+  double* vec = as<double>(P->sd_vec);
+  double *dg = vec, *eg = vec + N, *beta = vec + 2 * (size_t)N, *lam = vec + 3 * (size_t)N, *nrm = vec + 4 * (size_t)N,
+         *pb = vec + 5 * (size_t)N, *norms = vec + 9 * (size_t)N;
+  unsigned* bar = reinterpret_cast<unsigned*>(norms + 4);
+  CK(gw::sd_pack_rows(as<double>(P->sd_M), N, N, Np, M, P->stream));
+  CK(cudaMemcpyAsync(A, M, nn, cudaMemcpyDeviceToDevice, P->stream));
+  CK(gw::sd_tridiagonal(A, N, N, H, beta, dg, eg, pb, bar, as<int>(P->tc_err), P->stream));
+  CK(gw::sd_tridiagonal_vectors(dg, eg, N, lam, A, W, N, H, beta, N, nrm, V, P->stream));
+  P->stats.n_kernel_launches += 5;
+  double h[3];
+  for (int it = 0; it < 5; ++it) {
+    TRY(sd_product(P, V, V, nullptr, H));              // G
+    TRY(sd_product(P, V, M, nullptr, W));              // V M (M is symmetric)
+    TRY(sd_product(P, W, V, nullptr, A));              // S
+    CK(gw::sd_eig_norms(A, H, N, norms, P->stream));
+    CK(cudaMemcpyAsync(h, norms, sizeof(h), cudaMemcpyDeviceToHost, P->stream));
+    TRY(oz_check(P));
+    if (!std::isfinite(h[0] + h[1] + h[2]) || h[2] > 0.01) return GW_OK;     // clusters: not a basis
+    // S is as diagonal as the sweeps leave it and the rows are orthonormal to the same level
+    if (it > 0 && h[0] <= 1e-26 * h[1] && h[2] <= 1e-26 * N) {
+      *ok = true;
+      break;
+    }
+    CK(gw::sd_eig_update(A, H, N, W, norms, P->stream));
+    TRY(sd_product(P, W, nullptr, V, A));              // next rows
+    std::swap(V, A);
+    P->stats.n_kernel_launches += 2;
+  }
+  if (!*ok) return GW_OK;
+  // V_aux = 2 B D^1/2 T and the pole weights
+  double* sB = as<double>(P->oz_sc);
+  double* sA = sB + n;
+  double* sV = sA + n;
+  double* sw = sV + N;
+  CK(gw::sd_twice_sqrt(P->d_D, N, dg, P->stream));
+  CK(gw::oz_row_scale(dg, 1, N, N, sw, P->stream));
+  CK(gw::oz_row_scale(P->d_B_ia, n, N, N, sB, P->stream));
+  CK(gw::oz_split_weighted(P->d_B_ia, n, 0, N, N, sB, dg, N, sw, 1, as<__nv_bfloat16>(P->oz_A), sA, P->stream));
+  CK(gw::oz_row_digits(V, N, N, N, sV, as<__nv_bfloat16>(P->oz_B), P->stream));
+  gw::OzEpi ep{};
+  ep.kind = gw::OZ_EPI_STORE;
+  ep.out = as<double>(P->sd_V);
+  ep.ldo = N;
+  CK(gw::oz_gemm(gw::OzOperand{as<__nv_bfloat16>(P->oz_A), sA, 0}, gw::OzOperand{as<__nv_bfloat16>(P->oz_B), sV, 0}, 1, n,
+                 N, N, ep, as<int>(P->tc_err), P->stream));
+  CK(gw::sd_rows_weights(A, H, as<double>(P->sd_V), P->d_B_nm, n, N, R, as<double>(P->sd_Om), as<double>(P->sd_w2),
+                         P->stream));
+  P->stats.n_kernel_launches += 8;
+  return oz_check(P);
+}
+
 gw_status ensure_sd(gw_plan* P) {
   if (P->sd_done) return GW_OK;
   const long N = P->n_ov;
@@ -1849,6 +1958,15 @@ gw_status ensure_sd(gw_plan* P) {
   TRY(ensure(P, P->sd_w2, sizeof(double) * (size_t)R * N));
   LAUNCH(CK(gw::sd_casida_matrix(P->d_B_ia, P->d_D, n, (int)N, Np, as<double>(P->sd_M), as<double>(P->sd_T),
                                  P->stream)));
+  if (N >= 8 && N <= gw::sd_direct_max()) {
+    bool ok = false;
+    TRY(sd_direct(P, Np, &ok));
+    if (ok) {
+      P->sd_sweeps = 0;
+      P->sd_done = true;
+      return GW_OK;
+    }
+  }
   double off[2] = {1.0, 1.0};
   int sweeps = 0;
   for (; sweeps < 40; ++sweeps) {
@@ -1887,11 +2005,12 @@ gw_status gw_sigma_sd(gw_plan_t P, int n_points, const int* target_idx, const do
   TRY(ensure(P, P->sd_om, sizeof(double) * n_points));
   TRY(ensure(P, P->sd_S, sizeof(double) * n_points));
   TRY(ensure(P, P->sd_dS, sizeof(double) * n_points));
+  TRY(ensure(P, P->sd_part, sizeof(double) * 2 * (size_t)n_points * gw::sd_sigma_parts(P->n_bas, P->n_ov)));
   CK(cudaMemcpyAsync(P->sd_tmap.p, tmap.data(), sizeof(int) * n_points, cudaMemcpyHostToDevice, P->stream));
   CK(cudaMemcpyAsync(P->sd_om.p, omega, sizeof(double) * n_points, cudaMemcpyHostToDevice, P->stream));
   LAUNCH(CK(gw::sd_sigma(as<double>(P->sd_w2), as<double>(P->sd_Om), (int)P->n_ov, P->n_bas, P->d_eps_g,
                          as<int>(P->sd_tmap), P->d_spin, P->d_occ_t, P->cfg.n_occ, as<double>(P->sd_om), n_points,
-                         P->cfg.eta, as<double>(P->sd_S), as<double>(P->sd_dS), P->stream)));
+                         P->cfg.eta, as<double>(P->sd_part), as<double>(P->sd_S), as<double>(P->sd_dS), P->stream)));
   std::vector<double> S(n_points), dS(n_points);
   CK(cudaMemcpyAsync(S.data(), P->sd_S.p, sizeof(double) * n_points, cudaMemcpyDeviceToHost, P->stream));
   CK(cudaMemcpyAsync(dS.data(), P->sd_dS.p, sizeof(double) * n_points, cudaMemcpyDeviceToHost, P->stream));
