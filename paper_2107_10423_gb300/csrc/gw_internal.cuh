@@ -15,12 +15,16 @@ namespace gw {
 template <typename T>
 void launch_cholesky(T* base, int n, long stride, int batch, int* info, cudaStream_t s);
 
+// out_g = Pi(i xi_g) (mode 0) or 1 - Pi(i xi_g) (mode 1), g < n_xi, n_aux x n_aux, on the FP64 pipe.
+void launch_pi_syrk(const double* B, const double* Dk, long n_ov, int n_aux, const double* xi, int n_xi, double* out,
+                    int mode, cudaStream_t s);
+
 // X_b = L_b^-1 (full n x n, zeros above the diagonal) from lower factors L_b at stride `stride`.
 cudaError_t launch_tri_inv(const double* L, long stride, int n, int batch, double* X, long xstride, cudaStream_t s);
 // W[r][c] = -|Bn_r|^2 for c < n_cols.
 cudaError_t launch_w_minus_norm(const double* Bn, int n, long R, int n_cols, double* W, cudaStream_t s);
 
-// W table from Cholesky factors (gw_w_table_noalloc): for matrices g in [0, n_g): y = L_g^-1 b_r for rows r of Bn [R][n],
+// W table from Cholesky factors (gw_w_table_noalloc, small FP64 plans): for matrices g in [0, n_g): y = L_g^-1 b_r for rows r of Bn [R][n],
 // W[r*w_ld + g_out[g]] = |y|^2 - |b|^2 = b^T(eps^-1 - 1)b.  scratch: [n_cta][n][64] elements of T.
 template <typename T>
 cudaError_t launch_trsm_w(const T* Lbase, long Lstride, int n, int n_g, const int* g_out, const T* Bn, int R,

@@ -484,6 +484,7 @@ gw_status ns_w_table(gw_plan* P, int g0, int nc, const double* xi_pos) {
 }
 
 // ---------------------------------------------------------------- FP64 products by digits (oz_gemm.cu)
+constexpr int kSmall64 = 128;        // FP64 plans up to here keep the imaginary axis on the FP64 pipe
 // Bytes a digit buffer may take (at least one matrix's smallest piece).
 size_t oz_cap(const gw_plan* P) { return std::min<size_t>(ws_bytes(P), (size_t)1 << 30); }
 
@@ -607,6 +608,10 @@ gw_status screening_T(gw_plan* P) {
   const int n_g1 = P->n_g + 1;
   const int R = P->n_t * P->n_bas;
   const bool use_tc = (P->cfg.precision == GW_PREC_MIXED);
+  // FP64 plans of one digit tile stay on the FP64 pipe: a tile's padding takes the digits' advantage (n_aux 84, 95 pairs,
+  // 129 points: Pi 0.35 ms and W 0.24, the job by the step tree 6.3 ms either way), and these plans run the QP searches
+  // whose roots, near poles of Sigma, move by 1e-8 with the order in which W is summed.
+  const bool small64 = !use_tc && n <= kSmall64;
   // difference-form columns: grid points with xi_g below a tenth of the smallest pair energy (there
   // |Pi(i xi_g) - Pi(0)| <= 1% of |Pi(0)|)
   int n_diff = 0;
@@ -663,9 +668,9 @@ gw_status screening_T(gw_plan* P) {
   int p0 = 0, p1 = n_pos;
   if (P->sh_world > 1) gw_shard_columns(P->n_g, P->sh_rank, P->sh_world, &p0, &p1);
   const int p_begin = (use_tc && p0 > 0 && p0 <= P->ns_ndiff) ? 0 : p0;
-  if (use_tc)
-    CK(cudaMemsetAsync(P->d_W, 0, sizeof(double) * (size_t)R * n_g1, P->stream));   // W is accumulated
-  else
+  if (use_tc || (small64 && P->sh_world > 1))
+    CK(cudaMemsetAsync(P->d_W, 0, sizeof(double) * (size_t)R * n_g1, P->stream));   // W is accumulated / summed
+  else if (!small64)
     LAUNCH(CK(gw::launch_w_minus_norm(P->d_B_nm, n, R, n_g1, P->d_W, P->stream)));
   std::vector<int> info(chunk);
   double ms_pi = 0.0;
@@ -677,10 +682,15 @@ gw_status screening_T(gw_plan* P) {
       TRY(tc_weighted_syrk(P, kinds.data(), xi_all.data() + g0, nc, 1, 1, reinterpret_cast<float*>(P->ws_mat.p), 0));
     } else {
       const size_t t0 = tick(P);
-      std::vector<int> kinds(nc, 0);
-      TRY(oz_weighted_syrk(P, kinds.data(), xi_all.data() + g0, nc, 1, 1, as<double>(P->ws_mat)));
+      if (small64) {
+        LAUNCH(gw::launch_pi_syrk(P->d_B_ia, P->d_D, P->n_ov, n, as<double>(P->ws_xi) + g0, nc, as<double>(P->ws_mat),
+                                  1, P->stream));
+      } else {
+        std::vector<int> kinds(nc, 0);
+        TRY(oz_weighted_syrk(P, kinds.data(), xi_all.data() + g0, nc, 1, 1, as<double>(P->ws_mat)));
+      }
       mark(P, 1, t0, (double)nc * n * n * P->n_ov);
-      TRY(oz_check(P));
+      if (!small64) TRY(oz_check(P));
     }
     CK(cudaEventRecord(P->ev1, P->stream));
     if (use_tc) {
@@ -693,9 +703,16 @@ gw_status screening_T(gw_plan* P) {
     LAUNCH(gw::launch_cholesky<double>(as<double>(P->ws_mat), n, (long)n * n, nc, as<int>(P->ws_info), P->stream));
     mark(P, 2, t1, (double)nc * n * n * (double)n / 3.0);
     t1 = tick(P);
-    TRY(oz_w_columns(P, as<double>(P->ws_mat), nc, as<int>(P->ws_gout) + g0));
+    if (small64) {
+      const int n_cta = gw::trsm_w_default_ctas();
+      TRY(ensure(P, P->oz_X, sizeof(double) * gw::trsm_w_scratch_elems<double>(n, n_cta)));
+      LAUNCH(gw::launch_trsm_w<double>(as<double>(P->ws_mat), (long)n * n, n, nc, as<int>(P->ws_gout) + g0, P->d_B_nm,
+                                       R, P->d_W, n_g1, as<double>(P->oz_X), n_cta, P->stream));
+    } else {
+      TRY(oz_w_columns(P, as<double>(P->ws_mat), nc, as<int>(P->ws_gout) + g0));
+    }
     mark(P, 3, t1, (double)nc * (double)n * n * R);
-    TRY(oz_check(P));
+    if (!small64) TRY(oz_check(P));
     CK(cudaMemcpyAsync(info.data(), P->ws_info.p, sizeof(int) * nc, cudaMemcpyDeviceToHost, P->stream));
     CK(cudaStreamSynchronize(P->stream));
     ms_pi += now_ms(P, P->ev0, P->ev1);
@@ -2399,6 +2416,7 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
     const u64 eg = std::min(nb, std::max<u64>(1, cap / one)), sub = std::min(n_g1, std::max<u64>(1, cap / (per + 8 * n * n)));
     const u64 rc = std::min<u64>(rows, std::max<u64>(128, cap / (per / n)));
     b += std::max(one * eg, rc * (per / n)) + std::max(one, per * sub) + 8 * n * n * sub;
+    if (c->n_aux <= kSmall64) b += 8 * (u64)gw::trsm_w_scratch_elems<double>(c->n_aux, gw::trsm_w_default_ctas());
     b += 8 * n_ov * eg + 8 * std::max((n + 1) * (eg + 1), rows + n * sub) + 12 * nb;
   }
   // residue batch (at most one right-hand side per target and state at a time)

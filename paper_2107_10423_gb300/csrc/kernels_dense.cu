@@ -1,4 +1,5 @@
 // Dense kernels of the CD-G0W0 path (SIMT, templated on the arithmetic type):
+//  * Pi(i xi) of small FP64 plans;
 //  * batched in-place Cholesky of eps(i xi) = 1 - Pi (SPD, Sec. 3.3 text after "inn");
 //  * triangular solves that turn the factors into the table W^c_nm(i xi) (Algorithm 1, imaginary-grid loop);
 //  * the two skinny products of the FP64 matrix-free residue operator 1 - Pi(x) (Sec. 3.3, MINRES paragraph) and the
@@ -17,6 +18,76 @@ constexpr int TM = 64;     // tile rows
 constexpr int TN = 64;     // tile cols
 constexpr int TK = 16;     // k step
 constexpr int NT = 256;    // threads per CTA (16 x 16, 4 x 4 outputs each)
+
+// ------------------------------------------------------------------ Pi(i xi) SYRK
+// 1 - Pi(i xi) of FP64 plans of at most one 128-row digit tile (screening_T), on the FP64 pipe.
+// grid.x: lower-triangular tile index (bi >= bj), grid.y: frequency index.
+__global__ void __launch_bounds__(NT) pi_syrk_kernel(const double* __restrict__ B, const double* __restrict__ Dk,
+                                                     long n_ov, int n_aux,
+                                                     const double* __restrict__ xi, double* __restrict__ out, int mode) {
+  __shared__ double As[TK][TM + 4];
+  __shared__ double Bs[TK][TN + 4];
+  // decode lower tile (bi, bj) from linear index t = bi*(bi+1)/2 + bj
+  int t = blockIdx.x;
+  int bi = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
+  while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
+  while (bi * (bi + 1) / 2 > t) --bi;
+  int bj = t - bi * (bi + 1) / 2;
+  const int g = blockIdx.y;
+  const double x2 = xi[g] * xi[g];
+  const int p0 = bi * TM, q0 = bj * TN;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  double acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+  const int lr = tid >> 2, lk = (tid & 3) * 4;
+  for (long k0 = 0; k0 < n_ov; k0 += TK) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      long k = k0 + lk + u;
+      double wa = 0.0, va = 0.0, vb = 0.0;
+      if (k < n_ov) {
+        const double D = Dk[k];
+        wa = (-4.0 * D / (D * D + x2));
+        if (p0 + lr < n_aux) va = B[(long)(p0 + lr) * n_ov + k];
+        if (q0 + lr < n_aux) vb = B[(long)(q0 + lr) * n_ov + k];
+      }
+      As[lk + u][lr] = va * wa;
+      Bs[lk + u][lr] = vb;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < TK; ++kk) {
+      double a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+  double* o = out + (long)g * n_aux * n_aux;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    int p = p0 + ty + 16 * i;
+    if (p >= n_aux) continue;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      int q = q0 + tx + 16 * j;
+      if (q >= n_aux || q > p) continue;
+      double v = acc[i][j];
+      if (mode == 1) v = (p == q ? 1.0 : 0.0) - v;
+      o[(long)p * n_aux + q] = v;
+      o[(long)q * n_aux + p] = v;
+    }
+  }
+}
 
 // ------------------------------------------------------------------ batched Cholesky, one CTA per matrix
 constexpr int CH_NB = 32;
@@ -907,6 +978,12 @@ void launch_deriv_resonant(const double* V64, const double* B, long n_ov, int n_
 template <typename T>
 void launch_cholesky(T* base, int n, long stride, int batch, int* info, cudaStream_t s) {
   cholesky_kernel<T><<<batch, CH_THREADS, 0, s>>>(base, n, stride, info);
+}
+
+void launch_pi_syrk(const double* B, const double* Dk, long n_ov, int n_aux, const double* xi, int n_xi, double* out,
+                    int mode, cudaStream_t s) {
+  const int nb = (n_aux + TM - 1) / TM;
+  pi_syrk_kernel<<<dim3(nb * (nb + 1) / 2, n_xi), NT, 0, s>>>(B, Dk, n_ov, n_aux, xi, out, mode);
 }
 
 cudaError_t launch_tri_inv(const double* L, long stride, int n, int batch, double* X, long xstride, cudaStream_t s) {
