@@ -16,22 +16,28 @@
 //
 // Design (one CTA per SM, persistent over work items = (128 x 256 tile, batch entry), entries fastest so that the
 // CTAs running at the same time read the same rows of B):
-//   * TMA streams, per 32-wide k-block, the hi/lo rows of the weighted side (2 x 128 x 32) with the entry's weight
-//     row into a 3-stage A ring that the transform releases, and the BF16 hi/lo tiles of the unweighted side
-//     (2 x 256 x 32) into a 4-stage B ring that the tensor core releases; the transformed tiles go through a
-//     3-stage T ring, also released by the tensor core.  The B loads therefore run up to three k-blocks ahead of
-//     the tensor core, independently of the transform.
-//   * Two transform warpgroups (two threads per row) form b = hi + lo in FP32 (exact: 16 significant bits), multiply
-//     by the weights and split the products into BF16 hi/lo tiles (64-byte swizzle, the tensor core's K-major
-//     layout).  The weight never round-trips through HBM.
+//   * One thread streams by TMA, per 32-wide k-block, the hi/lo rows of the weighted side (2 x 128 x 32) with the
+//     entry's weight row into a 4-stage A ring that the transform releases; another the BF16 hi/lo tiles of the
+//     unweighted side (2 x 256 x 32) into a 3-stage B ring that the tensor core releases; the transformed tiles go
+//     through a 4-stage T ring, also released by the tensor core.  With one thread for both rings the weighted side
+//     could not run ahead of a B stage's release, and the loads alone (transform, drain and two of three products
+//     left out) took 7.0 ms of the 10.0 of 38 entries at N_aux 1800, K 26496; they take 5.8 with two.
+//   * Two transform groups of four warps take the k-blocks in turn, one thread per row: form b = hi + lo in FP32
+//     (exact: 16 significant bits), multiply by the weights and split the products into BF16 hi/lo tiles (64-byte
+//     swizzle, the tensor core's K-major layout).  The weight never round-trips through HBM.  A k-block's transform
+//     is a chain of waits, conversions and a proxy fence that is longer than its MMAs; two groups overlap two of
+//     them (a third group gains nothing and costs a B stage's room).
 //   * One thread issues tcgen05.mma M128 N256 K16 (BF16 in, FP32 accumulate in TMEM): hi*hi + hi*lo + lo*hi.
 //     The tensor core queues little work ahead of the issuing thread, so an instruction that takes 128 cycles
 //     (N = 256) leaves that thread the time for its barrier waits and commits without idling the tensor core;
 //     with N = 128 those waits showed up as idle tensor-core time.
 //   * Accumulation precision: the tensor core's FP32 accumulator loses up to an ulp per accumulate, so no
-//     partial sum runs through more than CHUNK k-blocks (6 CHUNK accumulates) before the drain warpgroup adds it,
+//     partial sum runs through more than CHUNK k-blocks (6 CHUNK accumulates) before the drain warps add it,
 //     rounded to nearest, into an FP32 running sum.  TMEM columns [256, 512) hold the sum (the first chunk of an
-//     item accumulates there directly), [0, 256) the partial of the later chunks.
+//     item accumulates there directly), [0, 256) the partial of the later chunks.  The tensor core waits while a
+//     chunk is drained, so eight warps share it (128 columns each): four took 0.9 of the 10.0 ms, eight 0.4.
+//   Together 9.95 to 8.99 ms (38 entries, N_aux 1800, K 26496) and 1.52 to 1.37 (N_aux 1008, K 12160): what remains is
+//   shared-memory and L2 traffic (48 KiB in and 32 KiB through the transform per 6 MMAs).
 // Every mbarrier wait is bounded; on timeout the kernel records a code in *err, stops every role, waits for its
 // copies and tensor-core work in flight, frees TMEM and returns.
 #include "pi_tc.cuh"
@@ -51,7 +57,11 @@ namespace {
 using namespace ptx;
 
 constexpr int BM = 128, BN = 256, BK = 32;
-constexpr int A_STAGES = 3, B_STAGES = 4, T_STAGES = 3;
+constexpr int TR_GROUPS = 2, TR_GROUP = 4;       // transform: groups of four warps taking the k-blocks in turn
+constexpr int A_STAGES = 4, B_STAGES = 3, T_STAGES = 4;
+// a stage of the A and T rings always belongs to the same transform group, which then sees every phase of its barriers
+// (a wait by parity passes too early for a thread that is two phases behind)
+static_assert(A_STAGES % TR_GROUPS == 0 && T_STAGES % TR_GROUPS == 0, "stages of the transform groups");
 constexpr int A_BYTES = 2 * BM * BK * 2;        // hi/lo rows of the weighted side: 16 KiB
 constexpr int W_BYTES = BK * 4;                 // the entry's weight row [BK] FP32
 constexpr int HB_BYTES = BN * BK * 2;           // one BF16 tile of the unweighted side (256 rows x 64 bytes)
@@ -70,8 +80,10 @@ constexpr int BAR_AF = 0, BAR_AE = BAR_AF + A_STAGES, BAR_BF = BAR_AE + A_STAGES
 static_assert(N_BARS * 8 + 4 <= 256, "barrier area");
 constexpr int SMEM_BYTES = BAR_OFF + 256 + 1024;
 static_assert(SMEM_BYTES + 1024 <= 232448, "shared memory per block (dynamic + static)");
-constexpr int THREADS = 448;                    // warps 0-3 drain + epilogue, 4-11 transform, 12 TMA, 13 MMA
-constexpr int TR_WARPS = 8;
+// warps: drain + epilogue (two per TMEM lane quarter, 128 columns each), transform, TMA of the weighted side, MMA, TMA of
+// the unweighted side
+constexpr int DR_WARPS = 8, TR_WARP0 = DR_WARPS, A_WARP = TR_WARP0 + TR_GROUPS * TR_GROUP, MMA_WARP = A_WARP + 1,
+              B_WARP = A_WARP + 2, THREADS = 32 * (A_WARP + 3);
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t COL_P = 0, COL_S = 256;      // TMEM columns of the partial and of the running sum
 constexpr uint32_t SBO64 = 8 * 64;              // 8-row groups of 64-byte rows
@@ -110,6 +122,25 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// Two FP32 operations in one instruction, each rounded to nearest.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+      "add.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+      "mul.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+
 // Chunk bookkeeping of an item with nki k-blocks: chunk c = kb / CHUNK accumulates into the running sum (c = 0)
 // or into the partial (c >= 1).  The drain warpgroup acts at the end of every chunk c >= 1 (sum += partial, or the
 // epilogue at the item's last k-block) and at the end of a single-chunk item (epilogue).
@@ -146,18 +177,18 @@ __global__ void __launch_bounds__(THREADS, 1)
     s_abort = 0;
     for (int s = 0; s < A_STAGES; ++s) {
       mbar_init(bar(BAR_AF + s), 1);
-      mbar_init(bar(BAR_AE + s), TR_WARPS);    // one arrival per transform warp
+      mbar_init(bar(BAR_AE + s), TR_GROUP);    // one arrival per transform warp of a group
     }
     for (int s = 0; s < B_STAGES; ++s) {
       mbar_init(bar(BAR_BF + s), 1);              // the producer's expect_tx arrival
       mbar_init(bar(BAR_BE + s), 1);              // the MMA thread's commit
     }
     for (int s = 0; s < T_STAGES; ++s) {
-      mbar_init(bar(BAR_TF + s), TR_WARPS);       // one arrival per transform warp
+      mbar_init(bar(BAR_TF + s), TR_GROUP);       // one arrival per transform warp of a group
       mbar_init(bar(BAR_TE + s), 1);              // the MMA thread's commit
     }
     mbar_init(bar(BAR_ACCF), 1);
-    mbar_init(bar(BAR_ACCE), 4);               // one arrival per drain warp
+    mbar_init(bar(BAR_ACCE), DR_WARPS);        // one arrival per drain warp
     mbar_init(bar(BAR_FIN), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -173,49 +204,66 @@ __global__ void __launch_bounds__(THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 12) {
+  if (warp == A_WARP) {
     if (lane == 0) {
-      // ------------------------------------------------------------ TMA producer
-      // A ring (FP32 rows + weight row): released by the transform warps; B ring (BF16 hi/lo of the unweighted
-      // side): released by the tensor core.  Ring positions are stage indices and phase bits.
-      long issued_a = 0, issued_b = 0;
-      uint32_t sa = 0, pa = 0, sb = 0, pb = 0;
-      bool a_wrapped = false, b_wrapped = false;
-      bool ok = true;
+      // ------------------------------------------------------------ TMA producer, weighted side
+      // rows + weight row, released by the transform warps.  Ring positions are stage indices and phase bits.
+      long issued = 0;
+      uint32_t sa = 0, pa = 0;
+      bool wrapped = false, ok = true;
       for (long it = blockIdx.x; it < items && ok; it += gridDim.x) {
         int bm, bn2, b, ks;
         decode_item(it, nb, ksplit, tiles, bm, bn2, b, ks);
         const int kb0 = (int)((long)nk * ks / ksplit), nki = (int)((long)nk * (ks + 1) / ksplit) - kb0;
         for (int kb = 0; kb < nki; ++kb) {
           const int kx = (kb0 + kb) * BK;
-          if (a_wrapped && !mbar_wait(bar(BAR_AE + sa), pa ^ 1u, err, 11)) { ok = false; break; }
+          if (wrapped && !mbar_wait(bar(BAR_AE + sa), pa ^ 1u, err, 11)) { ok = false; break; }
           if (*(volatile int*)&s_abort) { ok = false; break; }
           mbar_expect_tx(bar(BAR_AF + sa), A_TX);
           tma_load_3d(base + sa * A_BYTES, &maps.ah, kx % KP, bm * BM, kx / KP, bar(BAR_AF + sa));
           tma_load_3d(base + sa * A_BYTES + HA_BYTES, &maps.al, kx % KP, bm * BM, kx / KP, bar(BAR_AF + sa));
           tma_load_2d(base + W_OFF + sa * W_BYTES, &maps.w, kx, b, bar(BAR_AF + sa));
-          ++issued_a;
-          if (++sa == A_STAGES) { sa = 0; pa ^= 1u; a_wrapped = true; }
-          if (b_wrapped && !mbar_wait(bar(BAR_BE + sb), pb ^ 1u, err, 13)) { ok = false; break; }
-          if (*(volatile int*)&s_abort) { ok = false; break; }
-          const uint32_t bs = base + B_OFF + sb * BS_BYTES;
-          mbar_expect_tx(bar(BAR_BF + sb), B_TX);
-          tma_load_3d(bs, &maps.bh, kx % KP, bn2 * BN, kx / KP, bar(BAR_BF + sb));
-          tma_load_3d(bs + HB_BYTES, &maps.bl, kx % KP, bn2 * BN, kx / KP, bar(BAR_BF + sb));
-          ++issued_b;
-          if (++sb == B_STAGES) { sb = 0; pb ^= 1u; b_wrapped = true; }
+          ++issued;
+          if (++sa == A_STAGES) { sa = 0; pa ^= 1u; wrapped = true; }
         }
       }
       if (!ok) {
         s_abort = 1;
         // wait for the copies that may still be in flight (the latest phase of each stage)
-        for (long q = issued_a > A_STAGES ? issued_a - A_STAGES : 0; q < issued_a; ++q)
+        for (long q = issued > A_STAGES ? issued - A_STAGES : 0; q < issued; ++q)
           mbar_wait(bar(BAR_AF + (int)(q % A_STAGES)), (uint32_t)((q / A_STAGES) & 1), err, 12);
-        for (long q = issued_b > B_STAGES ? issued_b - B_STAGES : 0; q < issued_b; ++q)
+      }
+    }
+  } else if (warp == B_WARP) {
+    if (lane == 0) {
+      // ------------------------------------------------------------ TMA producer, unweighted side
+      // BF16 hi/lo rows, released by the tensor core.
+      long issued = 0;
+      uint32_t sb = 0, pb = 0;
+      bool wrapped = false, ok = true;
+      for (long it = blockIdx.x; it < items && ok; it += gridDim.x) {
+        int bm, bn2, b, ks;
+        decode_item(it, nb, ksplit, tiles, bm, bn2, b, ks);
+        const int kb0 = (int)((long)nk * ks / ksplit), nki = (int)((long)nk * (ks + 1) / ksplit) - kb0;
+        for (int kb = 0; kb < nki; ++kb) {
+          const int kx = (kb0 + kb) * BK;
+          if (wrapped && !mbar_wait(bar(BAR_BE + sb), pb ^ 1u, err, 13)) { ok = false; break; }
+          if (*(volatile int*)&s_abort) { ok = false; break; }
+          const uint32_t bs = base + B_OFF + sb * BS_BYTES;
+          mbar_expect_tx(bar(BAR_BF + sb), B_TX);
+          tma_load_3d(bs, &maps.bh, kx % KP, bn2 * BN, kx / KP, bar(BAR_BF + sb));
+          tma_load_3d(bs + HB_BYTES, &maps.bl, kx % KP, bn2 * BN, kx / KP, bar(BAR_BF + sb));
+          ++issued;
+          if (++sb == B_STAGES) { sb = 0; pb ^= 1u; wrapped = true; }
+        }
+      }
+      if (!ok) {
+        s_abort = 1;
+        for (long q = issued > B_STAGES ? issued - B_STAGES : 0; q < issued; ++q)
           mbar_wait(bar(BAR_BF + (int)(q % B_STAGES)), (uint32_t)((q / B_STAGES) & 1), err, 14);
       }
     }
-  } else if (warp == 13) {
+  } else if (warp == MMA_WARP) {
     if (lane == 0) {
       // ------------------------------------------------------------ MMA issuer
       // Per k-block: two waits (B tiles landed, transformed tiles written), six M128 N256 K16 MMAs, two commits
@@ -264,62 +312,44 @@ __global__ void __launch_bounds__(THREADS, 1)
       mma_commit(bar(BAR_FIN));
       mbar_wait(bar(BAR_FIN), 0, err, 24);
     }
-  } else if (warp >= 4) {
-    // -------------------------------------------------------------- transform: two threads per row of the tile,
-    // each over 16 of the k-block's 32 columns
-    const int t = threadIdx.x - 128;
-    const int r = t & (BM - 1), h = t >> 7;
-    uint32_t sa = 0, pa = 0, st = 0, pt = 0;
-    bool t_wrapped = false;
+  } else if (warp >= TR_WARP0) {
+    // -------------------------------------------------------------- transform: one thread per row of the tile; the
+    // groups take the k-blocks in turn, so that one's waits and latencies overlap another's work
+    const int r = threadIdx.x & (BM - 1), grp = (warp - TR_WARP0) / TR_GROUP;
+    uint32_t sa = grp, pa = 0, st = grp, pt = 0;       // this group's next stages (every TR_GROUPS-th)
+    long cnt = grp, total = 0;                         // its next k-block, k-blocks before the current item
     bool ok = true;
     for (long it = blockIdx.x; it < items && ok; it += gridDim.x) {
-      int bm, bn2, b, ks;
-      decode_item(it, nb, ksplit, tiles, bm, bn2, b, ks);
+      const int ks = (int)(it % ksplit);
       const int nki = (int)((long)nk * (ks + 1) / ksplit) - (int)((long)nk * ks / ksplit);
-      for (int kb = 0; kb < nki; ++kb) {
+      for (; cnt < total + nki; cnt += TR_GROUPS) {
         bool w_ok = !*(volatile int*)&s_abort && mbar_wait(bar(BAR_AF + sa), pa, err, 31);
-        if (w_ok && t_wrapped) w_ok = mbar_wait(bar(BAR_TE + st), pt ^ 1u, err, 32);
+        if (w_ok && cnt >= T_STAGES) w_ok = mbar_wait(bar(BAR_TE + st), pt ^ 1u, err, 32);
         if (!__all_sync(0xffffffffu, w_ok)) { ok = false; break; }
         const uint8_t* sp = smem + sa * A_BYTES;
         const float* wrow = reinterpret_cast<const float*>(smem + W_OFF + sa * W_BYTES);
-        constexpr int HK = BK / 2;
-        float a[HK], wv[HK];
+        uint8_t* tp = smem + T_OFF + st * TS_BYTES;
 #pragma unroll
-        for (int c = 0; c < HK / 8; ++c) {   // 64-byte swizzle: 16-byte chunk j of row r sits at j ^ ((r >> 1) & 3)
-          const int off = r * 64 + (((h * (HK / 8) + c) ^ ((r >> 1) & 3)) << 4);
+        for (int j = 0; j < BK / 8; ++j) {   // 64-byte swizzle: 16-byte chunk j of row r sits at j ^ ((r >> 1) & 3)
+          const int off = r * 64 + ((j ^ ((r >> 1) & 3)) << 4);
           const uint4 vh = *reinterpret_cast<const uint4*>(sp + off);
           const uint4 vl = *reinterpret_cast<const uint4*>(sp + HA_BYTES + off);
+          const float4 w0 = *reinterpret_cast<const float4*>(wrow + 8 * j);              // broadcast reads
+          const float4 w1 = *reinterpret_cast<const float4*>(wrow + 8 * j + 4);
           const uint32_t hw4[4] = {vh.x, vh.y, vh.z, vh.w}, lw4[4] = {vl.x, vl.y, vl.z, vl.w};
+          const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+          uint32_t hi[4], lo[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const __nv_bfloat162 x = *reinterpret_cast<const __nv_bfloat162*>(&hw4[e]);
             const __nv_bfloat162 y = *reinterpret_cast<const __nv_bfloat162*>(&lw4[e]);
-            a[8 * c + 2 * e] = __low2float(x) + __low2float(y);
-            a[8 * c + 2 * e + 1] = __high2float(x) + __high2float(y);
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < HK / 4; ++c) {
-          const float4 q = *reinterpret_cast<const float4*>(wrow + h * HK + 4 * c);   // broadcast reads
-          wv[4 * c] = q.x;
-          wv[4 * c + 1] = q.y;
-          wv[4 * c + 2] = q.z;
-          wv[4 * c + 3] = q.w;
-        }
-        uint8_t* tp = smem + T_OFF + st * TS_BYTES;
-#pragma unroll
-        for (int jj = 0; jj < HK / 8; ++jj) {  // 64-byte swizzle: 16-byte chunk j of row r sits at j ^ ((r >> 1) & 3)
-          const int j = h * (HK / 8) + jj;
-          uint32_t hi[4], lo[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int k = 8 * jj + 2 * e;
-            const float v0 = a[k] * wv[k], v1 = a[k + 1] * wv[k + 1];
-            hi[e] = pack_bf16(v0, v1);
+            float2 v = make_float2(__low2float(x), __high2float(x));
+            v = mul2(add2(v, make_float2(__low2float(y), __high2float(y))), make_float2(wv[2 * e], wv[2 * e + 1]));
+            hi[e] = pack_bf16(v.x, v.y);
             const __nv_bfloat162 hh = *reinterpret_cast<const __nv_bfloat162*>(&hi[e]);
-            lo[e] = pack_bf16(v0 - __low2float(hh), v1 - __high2float(hh));
+            v = add2(v, make_float2(-__low2float(hh), -__high2float(hh)));
+            lo[e] = pack_bf16(v.x, v.y);
           }
-          const int off = r * 64 + ((j ^ ((r >> 1) & 3)) << 4);
           *reinterpret_cast<uint4*>(tp + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
           *reinterpret_cast<uint4*>(tp + HA_BYTES + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
@@ -329,14 +359,15 @@ __global__ void __launch_bounds__(THREADS, 1)
           mbar_arrive(bar(BAR_TF + st));
           mbar_arrive(bar(BAR_AE + sa));
         }
-        if (++sa == A_STAGES) { sa = 0; pa ^= 1u; }
-        if (++st == T_STAGES) { st = 0; pt ^= 1u; t_wrapped = true; }
+        if ((sa += TR_GROUPS) >= A_STAGES) { sa -= A_STAGES; pa ^= 1u; }
+        if ((st += TR_GROUPS) >= T_STAGES) { st -= T_STAGES; pt ^= 1u; }
       }
+      total += nki;
     }
     if (!ok) s_abort = 1;
   } else {
-    // -------------------------------------------------------------- drain + epilogue (TMEM lane quarter = warp)
-    const int q = warp;
+    // -------------------------------------------------------------- drain + epilogue (TMEM lane quarter = warp mod 4)
+    const int q = warp & 3, g0 = (warp >> 2) * (BN / 64);
     uint32_t n_events = 0;
     bool ok = true;
     for (long it = blockIdx.x; it < items && ok; it += gridDim.x) {
@@ -361,7 +392,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         tc_fence_after();
         const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
-        for (int g = 0; g < BN / 32; ++g) {
+        for (int g = g0; g < g0 + BN / 64; ++g) {
           uint32_t v[32], w[32];
           tmem_ld32(lane_addr + COL_S + (uint32_t)(g * 32), v);
           if (with_p) tmem_ld32(lane_addr + COL_P + (uint32_t)(g * 32), w);
