@@ -74,6 +74,8 @@ struct gw_plan {
   __nv_bfloat16* d_Bnlo = nullptr;
   __nv_bfloat16* d_Bnlo2 = nullptr;
   bool screening_done = false;
+  std::vector<char*> slabs;         // kSlab bytes each, the last one used up to slab_used (plan_alloc)
+  size_t slab_used = 0;
   // spectral-decomposition route (gw_sigma_sd): Casida matrix and eigenvectors, pole weights; valid while sd_done
   DevBuf sd_M, sd_T, sd_cs, sd_off, sd_Om, sd_V, sd_w2, sd_tmap, sd_om, sd_S, sd_dS, sd_part, sd_x[5], sd_vec;
   bool sd_done = false;
@@ -160,26 +162,61 @@ void count_bytes(gw_plan* P, long long delta) {
   P->stats.bytes_device_peak = std::max(P->stats.bytes_device_peak, P->stats.bytes_device);
 }
 
-// Device allocation counted in gw_stats.bytes_device.
+// Device allocations of a plan, counted in gw_stats.bytes_device: buffers up to kSmallBuf come out of slabs that the plan
+// holds until it is destroyed; larger ones are the driver's.  A cudaMalloc with its cudaFree takes 40 to 130 us and a small
+// job has some 60 buffers: a (H2O)_1 job takes 3.70 ms with one each, 3.48 with 4 MiB slabs, 3.25 with these; a (H2O)_5
+// one 15.2, 14.8 and 14.1.
+constexpr size_t kSlab = 32u << 20, kSmallBuf = 8u << 20;
+
+gw_status plan_alloc(gw_plan* P, void** p, size_t bytes) {
+  if (bytes > kSmallBuf) {
+    CK(cudaMalloc(p, bytes));
+    count_bytes(P, (long long)bytes);
+    return GW_OK;
+  }
+  const size_t need = (bytes + 511) & ~(size_t)511;
+  if (P->slabs.empty() || P->slab_used + need > kSlab) {
+    void* q = nullptr;
+    CK(cudaMalloc(&q, kSlab));
+    P->slabs.push_back(static_cast<char*>(q));
+    count_bytes(P, (long long)kSlab);
+    P->slab_used = 0;
+  }
+  *p = P->slabs.back() + P->slab_used;
+  P->slab_used += need;
+  return GW_OK;
+}
+
+bool in_slab(const gw_plan* P, const void* p) {
+  for (const char* q : P->slabs)
+    if (p >= q && p < q + kSlab) return true;
+  return false;
+}
+
+// Gives back a buffer of plan_alloc (bytes as asked for; a slab keeps its share until the plan ends).
+void plan_free(gw_plan* P, void* p, size_t bytes) {
+  if (!p || in_slab(P, p)) return;
+  cudaFree(p);
+  count_bytes(P, -(long long)bytes);
+}
+
 template <typename T>
 gw_status dmalloc(gw_plan* P, T** p, size_t bytes) {
-  CK(cudaMalloc(reinterpret_cast<void**>(p), bytes));
-  count_bytes(P, (long long)bytes);
-  return GW_OK;
+  return plan_alloc(P, reinterpret_cast<void**>(p), bytes);
 }
 
 gw_status ensure(gw_plan* P, DevBuf& b, size_t bytes) {
   if (b.bytes >= bytes && b.p) return GW_OK;
   if (b.p) {
     CK(cudaStreamSynchronize(P->stream));
-    cudaFree(b.p);
-    count_bytes(P, -(long long)b.bytes);
+    // a buffer that grows inside a slab at least doubles: what it leaves behind stays below its final size
+    if (in_slab(P, b.p) && bytes < 2 * b.bytes) bytes = 2 * b.bytes;
+    plan_free(P, b.p, b.bytes);
     b.p = nullptr;
     b.bytes = 0;
   }
   if (bytes == 0) bytes = 16;
-  CK(cudaMalloc(&b.p, bytes));
-  count_bytes(P, (long long)bytes);
+  TRY(plan_alloc(P, &b.p, bytes));
   b.bytes = bytes;
   return GW_OK;
 }
@@ -1509,32 +1546,33 @@ static void free_plan(gw_plan* P) {
   if (!P) return;
   if (P->stream) cudaStreamSynchronize(P->stream);
   for (DevBuf* b : P->bufs)
-    if (b->p) cudaFree(b->p);
+    plan_free(P, b->p, 0);
   double* owned[] = {P->d_eps, P->d_eps_g, P->d_xi, P->d_wt, P->d_sx, P->d_shift, P->d_en, P->d_W};
-  if (P->d_spin) cudaFree(P->d_spin);
-  if (P->d_occ_t) cudaFree(P->d_occ_t);
+  plan_free(P, P->d_spin, 0);
+  plan_free(P, P->d_occ_t, 0);
   for (double* p : owned)
-    if (p) cudaFree(p);
+    plan_free(P, p, 0);
   if (P->own_B) {
-    if (P->d_B_ia) cudaFree(P->d_B_ia);
-    if (P->d_B_nm) cudaFree(P->d_B_nm);
+    plan_free(P, P->d_B_ia, 0);
+    plan_free(P, P->d_B_nm, 0);
   }
-  if (P->d_B_ia_f) cudaFree(P->d_B_ia_f);
-  if (P->d_B_nm_f) cudaFree(P->d_B_nm_f);
-  if (P->d_Bhi) cudaFree(P->d_Bhi);
-  if (P->d_Blo) cudaFree(P->d_Blo);
-  if (P->d_BThi) cudaFree(P->d_BThi);
-  if (P->d_BTlo) cudaFree(P->d_BTlo);
-  if (P->d_Blo2) cudaFree(P->d_Blo2);
-  if (P->d_Bp_hi) cudaFree(P->d_Bp_hi);
-  if (P->d_Bp_lo) cudaFree(P->d_Bp_lo);
-  if (P->d_BTlo2) cudaFree(P->d_BTlo2);
-  if (P->d_D) cudaFree(P->d_D);
-  if (P->d_Dsort) cudaFree(P->d_Dsort);
-  if (P->d_Dkidx) cudaFree(P->d_Dkidx);
-  if (P->d_Bnhi) cudaFree(P->d_Bnhi);
-  if (P->d_Bnlo) cudaFree(P->d_Bnlo);
-  if (P->d_Bnlo2) cudaFree(P->d_Bnlo2);
+  plan_free(P, P->d_B_ia_f, 0);
+  plan_free(P, P->d_B_nm_f, 0);
+  plan_free(P, P->d_Bhi, 0);
+  plan_free(P, P->d_Blo, 0);
+  plan_free(P, P->d_BThi, 0);
+  plan_free(P, P->d_BTlo, 0);
+  plan_free(P, P->d_Blo2, 0);
+  plan_free(P, P->d_Bp_hi, 0);
+  plan_free(P, P->d_Bp_lo, 0);
+  plan_free(P, P->d_BTlo2, 0);
+  plan_free(P, P->d_D, 0);
+  plan_free(P, P->d_Dsort, 0);
+  plan_free(P, P->d_Dkidx, 0);
+  plan_free(P, P->d_Bnhi, 0);
+  plan_free(P, P->d_Bnlo, 0);
+  plan_free(P, P->d_Bnlo2, 0);
+  for (char* q : P->slabs) cudaFree(q);
   if (P->ev0) cudaEventDestroy(P->ev0);
   if (P->ev1) cudaEventDestroy(P->ev1);
   if (P->ev2) cudaEventDestroy(P->ev2);
@@ -1896,8 +1934,7 @@ gw_status sd_direct(gw_plan* P, int Np, bool* ok) {
   if (fit != GW_OK) {
     (void)cudaGetLastError();
     for (DevBuf& b : P->sd_x) {
-      if (b.p) cudaFree(b.p);
-      count_bytes(P, -(long long)b.bytes);
+      plan_free(P, b.p, b.bytes);
       b = DevBuf{};
     }
     return GW_OK;
@@ -2432,6 +2469,7 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
     b += batch * 8 * (ldf - n_ov) + 4 * (u64)152 * 128 * 128;                // U rows' padding, partial products
   }
   b += 48 * std::max<u64>(1, rows) + 8 * 6 * (u64)n_t + 64;                  // residue lists, Sigma scratch
+  b += 3 * kSlab;                                                            // slabs: their ends, buffers that grew
   // dense fallback batch
   const u64 mat2 = 2 * n * n * ts;
   const u64 fb = std::max<u64>(1, ws / mat2);
