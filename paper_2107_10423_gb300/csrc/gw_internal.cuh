@@ -60,8 +60,11 @@ void launch_deriv(const T* V, const T* B, const double* Dk, long n_ov, int n_aux
 void launch_df_split(const double* x, long n, float* h, float* l, cudaStream_t s);
 void launch_op_gemm1_df(const double* V, const float* Bh, const float* Bl, long ldh, const double* Dk, long n_ov,
                         int n_aux, const double* x, double eta, int nr, double* U, cudaStream_t s);
+// part: op_gemm2_df_ranges x 2 nr x n_aux work space where that is more than one range (at most kDfPartTiles 64 x 64 tiles).
+constexpr long kDfPartTiles = 1520;
+int op_gemm2_df_ranges(int n_aux, long n_ov, int nr);
 void launch_op_gemm2_df(const double* U, const float* Bh, const float* Bl, long ldh, int n_aux, int n_ov, int nr,
-                        const double* V, double* out, cudaStream_t s);
+                        const double* V, double* out, double* part, cudaStream_t s);
 // The pairs that launch_deriv skips, in FP64: dw[j] += Re(c'_k(x_j) t_k^2) with t from the FP64 rows of V64 and the FP64
 // B_ia [n_aux][n_ov]; Dsort ascending pair energies with their pair indices kidx.
 void launch_deriv_resonant(const double* V64, const double* B, long n_ov, int n_aux, const double* Dsort,

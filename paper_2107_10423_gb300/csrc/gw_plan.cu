@@ -103,7 +103,7 @@ struct gw_plan {
       mr_dwre, mr_it, mr_res, mr_cnt, mr_Vhi, mr_Vlo, mr_Uhi, mr_Ulo, mr_Vlo2, mr_Ulo2, mr_V64, mr_part;
   DevBuf sg_I, sg_dI, sg_R, sg_dR, sg_om, sg_start, sg_coef, sg_act, sg_tmap, qp_st, qp_om0;
   DevBuf fb_A, fb_y, fb_piv, fb_info, fb_idx, fb_y64, fb_V32, fb_S32, fb_Vp, fb_Up, fb_x, fb_V64, fb_U64, fb_S64, fb_sel,
-      fb_pos, fb_rho, fb_xs, fb_Bl, fb_lu, fb_sw, fb_linv, fb_lus;
+      fb_pos, fb_rho, fb_xs, fb_Bl, fb_part, fb_lu, fb_sw, fb_linv, fb_lus;
   std::string err;
   gw_stats stats{};
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
@@ -117,7 +117,7 @@ struct gw_plan {
     DevBuf* all[] = {&oz_A, &oz_B, &oz_X, &oz_sc, &oz_w, &op_BT, &op_sc, &op_V, &ws_mat, &ws_info, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
                      &mr_v, &mr_d1, &mr_d2, &mr_x, &mr_st, &mr_rt, &mr_rm, &mr_xf, &mr_wre, &mr_wim,
                      &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &mr_part, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
-                     &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_lu, &fb_sw, &fb_linv, &fb_lus, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS, &sd_part, &sd_x[0], &sd_x[1], &sd_x[2], &sd_x[3], &sd_x[4], &sd_vec};
+                     &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_part, &fb_lu, &fb_sw, &fb_linv, &fb_lus, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS, &sd_part, &sd_x[0], &sd_x[1], &sd_x[2], &sd_x[3], &sd_x[4], &sd_vec};
     bufs.assign(all, all + sizeof(all) / sizeof(all[0]));
   }
 };
@@ -964,8 +964,11 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
             LAUNCH(gw::launch_op_gemm1_df(as<double>(P->fb_V64), P->d_B_ia_f, as<float>(P->fb_Bl), P->ld_f, P->d_D,
                                           P->n_ov, n, as<double>(P->fb_xs), P->cfg.eta, m, as<double>(P->fb_U64),
                                           P->stream));
+            const int ks = gw::op_gemm2_df_ranges(n, P->n_ov, m);
+            if (ks > 1) TRY(ensure(P, P->fb_part, sizeof(double) * 2 * (size_t)n * m * ks));
             LAUNCH(gw::launch_op_gemm2_df(as<double>(P->fb_U64), P->d_B_ia_f, as<float>(P->fb_Bl), P->ld_f, n,
-                                          P->n_ov, m, as<double>(P->fb_V64), as<double>(P->fb_S64), P->stream));
+                                          P->n_ov, m, as<double>(P->fb_V64), as<double>(P->fb_S64),
+                                          as<double>(P->fb_part), P->stream));
           } else {
             LAUNCH(gw::launch_op_gemm1(as<double>(P->fb_V64), P->d_B_ia, P->d_D, P->n_ov, n, as<double>(P->fb_xs),
                                        P->cfg.eta, m, as<double>(P->fb_U64), P->stream));
@@ -2477,6 +2480,7 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
   if (mixed) {
     b += fb * (16 * n + 16 * n + 12 * ldn + 12 * ldo + 40);                  // FP64 solutions, V/S, split parts
     b += fb * (32 * n + 16 * n_ov) + 4 * n * n_ov;                           // FP64-residual vectors, df lo part of B
+    b += (u64)gw::kDfPartTiles * 64 * 64 * 8;                                // its K ranges' sums
   }
   b += 2 * (u64)lu_work_elems(c->n_aux, (long)std::min<u64>(fb, 1u << 30), !mixed);      // blocked-LU operands
   b += fb * (4 * (u64)gw::zlu_index_ints(1) + ts * (u64)gw::zlu_linv_elems(1) + (mixed ? 0 : 8 * (u64)gw::zlu_scale_elems(c->n_aux, 1)));

@@ -875,11 +875,16 @@ __global__ void __launch_bounds__(NT) op_gemm1_df_kernel(const double* __restric
   }
 }
 
-// df gemm2: acc[r][P] = sum_k U[r][k] B[P][k]; out = the real embedding [u - acc_re; -v - acc_im] (op_gemm2 mode 1).
+// df gemm2: acc[r][P] = sum_k U[r][k] B[P][k]; out = the real embedding [u - acc_re; -v - acc_im] (op_gemm2 mode 1), or,
+// with grid.z > 1 K ranges of `range` columns, the range's sums in FP64 to part [grid.z][M][n_aux] (df_part_kernel).
+// Bound by the FP32 pipes, 12 instructions a multiply-add; the next tile's loads run under a tile's arithmetic.  One range
+// and loads before each tile: 1.55 ms for 25 right-hand sides at N_aux 630, K 4750 (20 CTAs), 4.3 for 231 at 1008 and
+// 12160, 15.8 for 226 at 1800 and 26496; now 0.17, 3.0 and 12.3.
 __global__ void __launch_bounds__(NT) op_gemm2_df_kernel(const double* __restrict__ U, const float* __restrict__ Bh,
                                                          const float* __restrict__ Bl, long ldh, int n_aux, long n_ov,
                                                          int nr,
-                                                         const double* __restrict__ V, double* __restrict__ out) {
+                                                         const double* __restrict__ V, double* __restrict__ out,
+                                                         int range, double* __restrict__ part) {
   __shared__ float Ah_s[TK][TM + 4], Al_s[TK][TM + 4];
   __shared__ float Bh_s[TK][TN + 4], Bl_s[TK][TN + 4];
   const int M = 2 * nr;
@@ -892,18 +897,31 @@ __global__ void __launch_bounds__(NT) op_gemm2_df_kernel(const double* __restric
 #pragma unroll
     for (int j = 0; j < 4; ++j) ah_[i][j] = al_[i][j] = 0.f;
   const int lr = tid >> 2, lk = (tid & 3) * 4;
-  for (long k0 = 0; k0 < n_ov; k0 += TK) {
+  const long kbeg = (long)blockIdx.z * range, kend = kbeg + range < n_ov ? kbeg + range : n_ov;
+  double av[4];
+  float bh[4], bl[4];
+  auto load = [&](long k0) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const long k = k0 + lk + u;
-      float h = 0.f, l = 0.f;
-      if (m0 + lr < M && k < n_ov) df_split(U[(long)(m0 + lr) * n_ov + k], h, l);
+      const bool in = q0 + lr < n_aux && k < kend;
+      av[u] = m0 + lr < M && k < kend ? U[(long)(m0 + lr) * n_ov + k] : 0.0;
+      bh[u] = in ? Bh[(long)(q0 + lr) * ldh + k] : 0.f;
+      bl[u] = in ? Bl[(long)(q0 + lr) * n_ov + k] : 0.f;
+    }
+  };
+  load(kbeg);
+  for (long k0 = kbeg; k0 < kend; k0 += TK) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      float h, l;
+      df_split(av[u], h, l);
       Ah_s[lk + u][lr] = h;
       Al_s[lk + u][lr] = l;
-      const bool in = q0 + lr < n_aux && k < n_ov;
-      Bh_s[lk + u][lr] = in ? Bh[(long)(q0 + lr) * ldh + k] : 0.f;
-      Bl_s[lk + u][lr] = in ? Bl[(long)(q0 + lr) * n_ov + k] : 0.f;
+      Bh_s[lk + u][lr] = bh[u];
+      Bl_s[lk + u][lr] = bl[u];
     }
+    if (k0 + TK < kend) load(k0 + TK);
     __syncthreads();
 #pragma unroll 4
     for (int kk = 0; kk < TK; ++kk) {
@@ -935,9 +953,24 @@ __global__ void __launch_bounds__(NT) op_gemm2_df_kernel(const double* __restric
       const int P = q0 + tx + 16 * j;
       if (P >= n_aux) continue;
       const double v = (double)ah_[i][j] + (double)al_[i][j];
+      if (gridDim.z > 1) {
+        part[((long)blockIdx.z * M + r) * n_aux + P] = v;
+        continue;
+      }
       const double vin = V[(long)r * n_aux + P];
       out[(long)r * n_aux + P] = ((r & 1) ? -vin : vin) - v;
     }
+  }
+}
+
+// out[r][P] = (r odd ? -V : V)[r][P] - sum of the ranges' parts, in order.
+__global__ void df_part_kernel(const double* __restrict__ part, int ks, int M, int n_aux, const double* __restrict__ V,
+                               double* __restrict__ out) {
+  const long n = (long)M * n_aux;
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    double v = 0.0;
+    for (int z = 0; z < ks; ++z) v += part[z * n + i];
+    out[i] = ((i / n_aux) & 1 ? -V[i] : V[i]) - v;
   }
 }
 
@@ -962,10 +995,32 @@ void launch_op_gemm1_df(const double* V, const float* Bh, const float* Bl, long 
   if (nr > 0) op_gemm1_df_kernel<<<grid, NT, 0, s>>>(V, Bh, Bl, ldh, Dk, n_ov, n_aux, x, eta, nr, U);
 }
 
+// Few right-hand sides leave most SMs without a tile, and a batch's tiles fill their last round badly: K ranges of at
+// least 512 columns, the fewest that fill nine tenths of the rounds (two CTAs an SM), or those that fill them best.
+int op_gemm2_df_ranges(int n_aux, long n_ov, int nr) {
+  const long tiles = (long)((n_aux + TN - 1) / TN) * ((2 * nr + TM - 1) / TM), slots = 304;
+  int best = 1;
+  double best_fill = 0.0;
+  for (int ks = 1; ks <= 16; ++ks) {
+    if (ks > 1 && (ks * tiles > kDfPartTiles || n_ov / ks < 512)) break;
+    const long rounds = (ks * tiles + slots - 1) / slots;
+    const double fill = (double)(ks * tiles) / (double)(rounds * slots);
+    if (fill > best_fill) {
+      best_fill = fill;
+      best = ks;
+    }
+    if (fill >= 0.9) break;
+  }
+  return best;
+}
+
 void launch_op_gemm2_df(const double* U, const float* Bh, const float* Bl, long ldh, int n_aux, int n_ov, int nr,
-                        const double* V, double* out, cudaStream_t s) {
-  const dim3 grid((n_aux + TN - 1) / TN, (2 * nr + TM - 1) / TM);
-  if (nr > 0) op_gemm2_df_kernel<<<grid, NT, 0, s>>>(U, Bh, Bl, ldh, n_aux, (long)n_ov, nr, V, out);
+                        const double* V, double* out, double* part, cudaStream_t s) {
+  if (nr <= 0) return;
+  const int ks = op_gemm2_df_ranges(n_aux, n_ov, nr), range = ((n_ov + ks - 1) / ks + TK - 1) / TK * TK;
+  const dim3 grid((n_aux + TN - 1) / TN, (2 * nr + TM - 1) / TM, ks);
+  op_gemm2_df_kernel<<<grid, NT, 0, s>>>(U, Bh, Bl, ldh, n_aux, (long)n_ov, nr, V, out, range, part);
+  if (ks > 1) df_part_kernel<<<608, 256, 0, s>>>(part, ks, 2 * nr, n_aux, V, out);
 }
 
 void launch_deriv_resonant(const double* V64, const double* B, long n_ov, int n_aux, const double* Dsort,
