@@ -44,7 +44,7 @@ typedef enum {
 } gw_status;
 
 typedef enum {
-  GW_PREC_FP64 = 0,            /* every step in FP64 */
+  GW_PREC_FP64 = 0,            /* every step in FP64, or exact integer digits of FP64 values */
   GW_PREC_MIXED = 1            /* Pi and the W table on tcgen05 tensor cores with BF16 hi+lo split
                                   products (FP32 accumulate); MINRES operator in FP32, Lanczos
                                   recurrences, quadrature and QP search in FP64 */
@@ -167,13 +167,13 @@ gw_status gw_sigma_cd(gw_plan_t plan, const double* omega, double* sigma_c, doub
 
 /* Sigma_c and its omega-derivative by spectral decomposition (Sec. 2.2 and 3.2, the Casida route the paper uses
  * for small systems): the Hermitian Casida problem D^1/2 (D + 4 B_ia^T B_ia) D^1/2 T = T Omega^2 over the pairs
- * (both spin channels for an open-shell plan) is diagonalised once per plan in FP64 (cyclic Jacobi, to 1e-13
- * relative off-diagonal norm), then
+ * (both spin channels for an open-shell plan) is diagonalised once per plan in FP64 (tridiagonalisation with
+ * refinement, or cyclic Jacobi, to 1e-13 relative off-diagonal norm), then
  *   Sigma_c(omega) = sum_m sum_s w_nms^2 / (omega - e_m +/- Omega_s -/+ i eta)  (upper signs for occupied m),
  *   w_nms = b_nm . V_s / sqrt(2 Omega_s),  V = 2 B_ia D^1/2 T.
  * target_idx[p] (or NULL: point p is target p, n_points = n_targets) and omega[p] (host); sigma_c, dsigma_c host
- * [n_points] (real parts), either may be NULL.  O(N_ov^3) work and 2 N_ov^2 doubles: GW_ERR_ARG above
- * N_ov = 16384; GW_ERR_NOT_CONVERGED if 40 Jacobi sweeps do not converge.  The Casida solution is kept until W's
+ * [n_points] (real parts), either may be NULL.  O(N_ov^3) work and 2 N_ov^2 doubles (11 N_ov^2 up to
+ * N_ov = 8192 where they fit): GW_ERR_ARG above N_ov = 16384; GW_ERR_NOT_CONVERGED if 40 Jacobi sweeps do not converge.  The Casida solution is kept until W's
  * energies change (evGW). */
 gw_status gw_sigma_sd(gw_plan_t plan, int n_points, const int* target_idx, const double* omega, double* sigma_c,
                       double* dsigma_c);
@@ -240,7 +240,7 @@ gw_status gw_w_table(gw_plan_t plan, double* out);
 
 /* Timing and counters accumulated since plan creation (host, milliseconds / counts).  ms_kernel and
  * flops_kernel are per kernel class, timed with CUDA events on the plan's stream:
- *   0 Pi on tensor cores (tcgen05, weights applied in the kernel)   1 Pi (SIMT)
+ *   0 Pi on tensor cores (tcgen05, weights applied in the kernel)   1 Pi (FP64)
  *   2 W-table factorisation (Cholesky of 1 - Pi, or the tensor-core Newton-Schulz inverse in mixed mode)
  *   3 W-table reduction (triangular solves, or the tensor-core GEMM into W)
  *   4 MINRES iterations (the operator GEMMs and, since the iterations run as one CUDA graph per batch, the

@@ -142,7 +142,7 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
 }
 
 // Chunk bookkeeping of an item with nki k-blocks: chunk c = kb / CHUNK accumulates into the running sum (c = 0)
-// or into the partial (c >= 1).  The drain warpgroup acts at the end of every chunk c >= 1 (sum += partial, or the
+// or into the partial (c >= 1).  The drain warps act at the end of every chunk c >= 1 (sum += partial, or the
 // epilogue at the item's last k-block) and at the end of a single-chunk item (epilogue).
 __device__ __forceinline__ bool chunk_end(int kb, int nki) { return kb % CHUNK == CHUNK - 1 || kb == nki - 1; }
 __device__ __forceinline__ bool drain_event(int kb, int nki) {

@@ -1,6 +1,7 @@
 """Direct diagonalisation of the Casida matrix (tridiagonalisation, twisted vectors, refinement on digit products) at the
-edges of its ranges (the smallest N_ov, warps and row blocks of 8, digit tiles of 128 and 256) and at exactly degenerate
-levels, where the Jacobi sweeps take over, against the oracle's LAPACK route."""
+edges of its ranges (the smallest N_ov, warps and row blocks of 8, digit tiles of 128 and 256, rows in shared memory up to
+about 1800, wide bisection up to 2800) and at exactly degenerate levels, where the Jacobi sweeps take over, against the
+oracle's LAPACK route."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n_occ,n_virt,n_aux,degenerate", [
     (1, 7, 5, False), (1, 8, 5, False), (3, 11, 20, False), (4, 32, 9, False), (3, 43, 140, False), (4, 64, 60, False),
-    (1, 257, 33, False), (5, 250, 130, False), (4, 32, 9, True), (5, 40, 300, True)])
+    (1, 257, 33, False), (5, 250, 130, False), (12, 160, 40, False), (13, 224, 30, False), (4, 32, 9, True),
+    (5, 40, 300, True)])
 def test_sd_direct(gwlib, n_occ, n_virt, n_aux, degenerate):
     from paper_2107_10423_gb300 import gw
     occ = np.linspace(-1.4, -0.45, n_occ) if n_occ > 1 else np.array([-0.5])
