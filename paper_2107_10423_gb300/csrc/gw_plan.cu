@@ -95,7 +95,7 @@ struct gw_plan {
   DevBuf sk_C;                // device copy of nodes.C
   std::vector<DevBuf*> bufs;
   int tc_tiles_n = 0;          // N_aux the tile-order table of the Pi kernel was built for
-  DevBuf oz_A, oz_B, oz_X, oz_sc, oz_w, op_BT, op_sc, op_V;
+  DevBuf oz_A, oz_B, oz_X, oz_sc, oz_w, oz_part, op_BT, op_sc, op_V;
     // FP64 products on the tensor cores: digits, inverse factors, scales, weights
   DevBuf ws_mat, ws_info, ws_gout, ws_xi, tc_part, tc_kind, tc_par, tc_err, tc_w, tc_tiles, ns_E, ns_X, ns_X2, ns_Xa, ns_Xb, ns_T, ns_lam,
       ns_E0, ns_vec;
@@ -114,7 +114,7 @@ struct gw_plan {
   std::vector<Mark> marks;
 
   gw_plan() {
-    DevBuf* all[] = {&oz_A, &oz_B, &oz_X, &oz_sc, &oz_w, &op_BT, &op_sc, &op_V, &ws_mat, &ws_info, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
+    DevBuf* all[] = {&oz_A, &oz_B, &oz_X, &oz_sc, &oz_w, &oz_part, &op_BT, &op_sc, &op_V, &ws_mat, &ws_info, &ws_gout, &ws_xi, &tc_part, &tc_kind, &tc_par, &tc_err, &tc_w, &tc_tiles, &ns_E, &ns_X, &ns_X2, &ns_Xa, &ns_Xb, &ns_T, &ns_lam, &ns_E0, &ns_vec, &sk_C, &mr_V, &mr_U, &mr_S, &mr_vprev,
                      &mr_v, &mr_d1, &mr_d2, &mr_x, &mr_st, &mr_rt, &mr_rm, &mr_xf, &mr_wre, &mr_wim,
                      &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &mr_part, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
                      &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_part, &fb_lu, &fb_sw, &fb_linv, &fb_lus, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS, &sd_part, &sd_x[0], &sd_x[1], &sd_x[2], &sd_x[3], &sd_x[4], &sd_vec};
@@ -596,14 +596,25 @@ gw_status oz_weighted_syrk(gw_plan* P, const int* kinds, const double* params, i
   return GW_OK;
 }
 
+// Matrices and rows of B_nm of one product of oz_w_columns: the inverse factors with their digits, the rows' digits and
+// the tiles' sums each within the cap.
+void oz_w_blocks(size_t cap, int n, long R, int nc, int* sub, int* rows) {
+  const size_t per = gw::oz_elems(n, n) * sizeof(__nv_bfloat16);
+  *sub = (int)std::min<size_t>(nc, std::max<size_t>(1, cap / (per + sizeof(double) * n * n)));
+  const size_t part = sizeof(double) * gw::oz_sumsq_tiles(n) * (size_t)*sub;
+  *rows = (int)std::min<size_t>((size_t)R, std::max<size_t>(128, std::min(cap / (per / n), cap / part)));
+}
+
 // W[r][gidx[b]] += |L_b^-1 b_r|^2 for nc Cholesky factors L (ws_mat) and every row of B_nm: the inverse factors, their
-// digits and one digit product per block of rows, summed in its epilogue.
+// digits and one digit product per block of rows, squares summed per tile in its epilogue and over the tiles after it.
 gw_status oz_w_columns(gw_plan* P, const double* L, int nc, const int* gidx) {
   const int n = P->cfg.n_aux, n_g1 = P->n_g + 1;
   const long R = (long)P->n_t * P->n_bas;
-  const size_t cap = oz_cap(P), per = gw::oz_elems(n, n) * sizeof(__nv_bfloat16);
-  const int sub = (int)std::min<size_t>(nc, std::max<size_t>(1, cap / (per + sizeof(double) * n * n)));
-  const int rc = (int)std::min<size_t>((size_t)R, std::max<size_t>(128, cap / (per / n)));
+  const size_t per = gw::oz_elems(n, n) * sizeof(__nv_bfloat16);
+  const int tiles = gw::oz_sumsq_tiles(n);
+  int sub, rc;
+  oz_w_blocks(oz_cap(P), n, R, nc, &sub, &rc);
+  TRY(ensure(P, P->oz_part, sizeof(double) * (size_t)tiles * rc * sub));
   TRY(ensure(P, P->oz_X, sizeof(double) * (size_t)n * n * sub));
   TRY(ensure(P, P->oz_A, sizeof(__nv_bfloat16) * gw::oz_elems(rc, n)));
   TRY(ensure(P, P->oz_B, per * sub));
@@ -625,13 +636,12 @@ gw_status oz_w_columns(gw_plan* P, const double* L, int nc, const int* gidx) {
         CK(gw::oz_split(P->d_B_nm + r0 * n, 0, nr, 0, n, n, scR + r0, 1, as<__nv_bfloat16>(P->oz_A), P->stream));
       gw::OzEpi ep{};
       ep.kind = gw::OZ_EPI_SUMSQ;
-      ep.acc = P->d_W + r0 * n_g1;
-      ep.ldw = n_g1;
-      ep.gidx = gidx + b0;
+      ep.part = as<double>(P->oz_part);
       CK(gw::oz_gemm(gw::OzOperand{as<__nv_bfloat16>(P->oz_A), scR + r0, 0},
                      gw::OzOperand{as<__nv_bfloat16>(P->oz_B), scX, 1}, nb, nr, n, n, ep, as<int>(P->tc_err),
                      P->stream));
-      P->stats.n_kernel_launches += 2;
+      CK(gw::oz_sumsq_add(as<double>(P->oz_part), nb, tiles, nr, P->d_W + r0 * n_g1, n_g1, gidx + b0, P->stream));
+      P->stats.n_kernel_launches += 3;
     }
     P->stats.n_kernel_launches += 3;
   }
@@ -2453,9 +2463,11 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
     const u64 cap = std::min<u64>(ws, (u64)1 << 30), nb = std::max<u64>(n_g1, 2 * std::max<u64>(1, ws / (2 * n * n * ts)));
     const u64 slab = (u64)oz_slab((size_t)cap, c->n_aux, (int)std::min<u64>(n_ov, 2147483647ull));
     const u64 one = 2 * (u64)gw::oz_elems(c->n_aux, (int)slab), per = 2 * (u64)gw::oz_elems(c->n_aux, c->n_aux);
-    const u64 eg = std::min(nb, std::max<u64>(1, cap / one)), sub = std::min(n_g1, std::max<u64>(1, cap / (per + 8 * n * n)));
+    const u64 eg = std::min(nb, std::max<u64>(1, cap / one));
+    const u64 sub = std::min(n_g1, std::max<u64>(1, cap / (per + 8 * n * n))), tile = 8 * (u64)gw::oz_sumsq_tiles(c->n_aux) * sub;
     const u64 rc = std::min<u64>(rows, std::max<u64>(128, cap / (per / n)));
     b += std::max(one * eg, rc * (per / n)) + std::max(one, per * sub) + 8 * n * n * sub;
+    b += std::min(tile * rows, std::max(cap, tile * 128));                   // the tiles' sums
     if (c->n_aux <= kSmall64) b += 8 * (u64)gw::trsm_w_scratch_elems<double>(c->n_aux, gw::trsm_w_default_ctas());
     b += 8 * n_ov * eg + 8 * std::max((n + 1) * (eg + 1), rows + n * sub) + 12 * nb;
   }

@@ -204,7 +204,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           const double v = (double)((hi[j] << 12) + (lo[j] >> 20)) * sn[c + j];
           t = fma(v, v, t);
         }
-      if (m < M) atomicAdd(ep.acc + (long)m * ep.ldw + ep.gidx[b], t * (sm * sm) * 5.9604644775390625e-08);   // 2^-24
+      if (m < M)                                                                                    // 2^-24
+        ep.part[((long)b * 2 * ((N + BN - 1) / BN) + 2 * bn + h) * M + m] = t * (sm * sm) * 5.9604644775390625e-08;
     } else if (ep.kind == OZ_EPI_SUB2) {
       if (m < M) {
         double* o = ep.out + (long)b * ep.out_bstride + (m < ep.half ? (long)m * ep.ldo
@@ -236,6 +237,18 @@ __global__ void __launch_bounds__(THREADS, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
+}
+
+// The tiles' sums of OZ_EPI_SUMSQ in ascending order, so that a table repeats itself bit for bit (roots of the QP search
+// move by 1e-8 with the order near poles of Sigma).  One pass over part, 1/64 of the bytes of the rows' digits an entry.
+__global__ void __launch_bounds__(256) oz_sumsq_add_kernel(const double* __restrict__ part, int tiles, int M,
+                                                           double* __restrict__ W, int ldw,
+                                                           const int* __restrict__ gidx) {
+  const int m = blockIdx.x * 256 + threadIdx.x, b = blockIdx.y;
+  if (m >= M) return;
+  double s = 0.0;
+  for (int t = 0; t < tiles; ++t) s += part[((long)b * tiles + t) * M + m];
+  W[(long)m * ldw + gidx[b]] += s;
 }
 
 typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -456,6 +469,16 @@ __global__ void __launch_bounds__(256) oz_pole_derivative_kernel(const double* _
 }
 
 }  // namespace
+
+int oz_sumsq_tiles(int N) { return 2 * ((N + BN - 1) / BN); }     // a warp's 32 columns each
+
+cudaError_t oz_sumsq_add(const double* part, int batch, int tiles, int M, double* W, int ldw, const int* gidx,
+                         cudaStream_t s) {
+  if (batch > 65535) return cudaErrorInvalidValue;
+  if (batch > 0 && M > 0)
+    oz_sumsq_add_kernel<<<dim3((M + 255) / 256, batch), 256, 0, s>>>(part, tiles, M, W, ldw, gidx);
+  return cudaGetLastError();
+}
 
 int oz_ld(int K) { return (K + 7) / 8 * 8; }
 size_t oz_elems(int rows, int K) { return (size_t)S * rows * oz_ld(K); }

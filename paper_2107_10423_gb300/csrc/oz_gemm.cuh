@@ -24,15 +24,18 @@ struct OzEpi {
   double* out;
   long out_bstride;
   int ldo;
-  // OZ_EPI_SUMSQ: acc[m * ldw + gidx[b]] += sum_n v[m][n]^2; the B rows are lower triangular (row n ends at column n)
-  double* acc;
-  int ldw;
-  const int* gidx;
+  // OZ_EPI_SUMSQ: part[b][column tile][m] = sum of v[m][n]^2 over a tile's 32 columns (oz_sumsq_tiles(N) tiles of M values
+  // an entry; oz_sumsq_add sums them); the B rows are lower triangular (row n ends at column n)
+  double* part;
   // OZ_EPI_SUB2: out_b[m][n] -= v for m < half, out_b[plane + (m - half) ldo + n] -= v below (ldo, out_bstride as above)
   long plane;
   int half;
 };
 
+int oz_sumsq_tiles(int N);
+// W[m * ldw + gidx[b]] += sum over the column tiles t of part[b][t][m], t ascending, for b < batch and m < M.
+cudaError_t oz_sumsq_add(const double* part, int batch, int tiles, int M, double* W, int ldw, const int* gidx,
+                         cudaStream_t s);
 int oz_ld(int K);                    // row length of the digit arrays
 size_t oz_elems(int rows, int K);    // BF16 elements of one matrix's digits
 // out_b[m][n] = f(sum_k A_b[m][k] B_b[n][k]) for b < batch.  *err receives a code if a bounded wait ran out.
