@@ -15,9 +15,10 @@ namespace gw {
 template <typename T>
 void launch_cholesky(T* base, int n, long stride, int batch, int* info, cudaStream_t s);
 
-// out_g = Pi(i xi_g) (mode 0) or 1 - Pi(i xi_g) (mode 1), g < n_xi, n_aux x n_aux, on the FP64 pipe.
+// out_g = Pi(i xi_g) (mode 0) or 1 - Pi(i xi_g) (mode 1), g < n_xi, n_aux x n_aux, on the FP64 pipe; flags: only the
+// lower 64 x 64 tiles whose flag [g][tile] is set (oz_cover's).
 void launch_pi_syrk(const double* B, const double* Dk, long n_ov, int n_aux, const double* xi, int n_xi, double* out,
-                    int mode, cudaStream_t s);
+                    int mode, cudaStream_t s, const int* flags = nullptr);
 
 // X_b = L_b^-1 (full n x n, zeros above the diagonal) from lower factors L_b at stride `stride`.
 cudaError_t launch_tri_inv(const double* L, long stride, int n, int batch, double* X, long xstride, cudaStream_t s);

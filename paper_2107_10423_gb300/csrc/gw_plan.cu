@@ -534,28 +534,31 @@ gw_status oz_check(gw_plan* P) {
 }
 
 // K columns a weighted product holds at once: all of them, or as many (a multiple of 128) as the cap allows for the
-// digits of B and of one weighted copy.
+// digits of one entry's two operands.
 int oz_slab(size_t cap, int n, int K) {
   const size_t per_col = 2 * (size_t)gw::OZ_S * n * sizeof(__nv_bfloat16);
   if (per_col * gw::oz_ld(K) <= cap) return K;
   return (int)std::min<size_t>(K, std::max<size_t>(128, cap / per_col / 128 * 128));
 }
 
-// out_b = f(B diag(w_b) B^T) in FP64 for nb entries (weights of kind 0, 1, 2 as in tc_pair_weights).
+// out_b = f(B diag(w_b) B^T) in FP64 for nb entries (weights of kind 0, 1, 2 as in tc_pair_weights).  checked (kind 0,
+// f = v): tiles whose elements the digits cannot give as accurately as an FP64 sum are computed again (oz_cover).
 gw_status oz_weighted_syrk(gw_plan* P, const int* kinds, const double* params, int nb, int mode_even, int mode_odd,
-                           double* out) {
+                           double* out, bool checked = false) {
   const int n = P->cfg.n_aux, K = P->n_ov;
   const size_t cap = oz_cap(P);
   const int slab = oz_slab(cap, n, K);
   const size_t one = gw::oz_elems(n, slab);
   // entries at once: their digits within the cap, pairs kept together (even and odd entries have their own modes)
-  int eg = (int)std::min<size_t>(nb, std::max<size_t>(1, cap / (one * sizeof(__nv_bfloat16))));
+  int eg = (int)std::min<size_t>(nb, std::max<size_t>(1, cap / (2 * one * sizeof(__nv_bfloat16))));
   eg = std::min(eg, 32768);
   if (eg > 1 && eg < nb) eg &= ~1;
+  const int tiles = gw::oz_cover_tiles(n);
   TRY(ensure(P, P->oz_A, sizeof(__nv_bfloat16) * one * eg));
-  TRY(ensure(P, P->oz_B, sizeof(__nv_bfloat16) * one));
-  TRY(ensure(P, P->oz_w, sizeof(double) * (size_t)K * eg));
-  TRY(ensure(P, P->oz_sc, sizeof(double) * ((size_t)n * (eg + 1) + eg)));
+  TRY(ensure(P, P->oz_B, sizeof(__nv_bfloat16) * one * eg));
+  TRY(ensure(P, P->oz_w, (sizeof(double) + sizeof(int)) * (size_t)K * eg));
+  TRY(ensure(P, P->oz_sc, sizeof(double) * 2 * (size_t)n * eg));
+  if (checked) TRY(ensure(P, P->oz_part, sizeof(int) * (size_t)tiles * eg));
   TRY(ensure(P, P->tc_kind, sizeof(int) * nb));
   TRY(ensure(P, P->tc_par, sizeof(double) * nb));
   TRY(ensure(P, P->tc_err, sizeof(int)));
@@ -563,21 +566,20 @@ gw_status oz_weighted_syrk(gw_plan* P, const int* kinds, const double* params, i
   CK(cudaMemcpyAsync(P->tc_par.p, params, sizeof(double) * nb, cudaMemcpyHostToDevice, P->stream));
   CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
   double* scB = as<double>(P->oz_sc);
-  double* scA = scB + n;
-  double* scw = scA + (size_t)n * eg;
+  double* scA = scB + (size_t)n * eg;
+  double* f = as<double>(P->oz_w);
+  int* h = reinterpret_cast<int*>(f + (size_t)K * eg);
   __nv_bfloat16* dB = as<__nv_bfloat16>(P->oz_B);
   __nv_bfloat16* dA = as<__nv_bfloat16>(P->oz_A);
-  CK(gw::oz_row_scale(P->d_B_ia, n, K, K, scB, P->stream));
-  P->stats.n_kernel_launches += 1;
   for (int b0 = 0; b0 < nb; b0 += eg) {
     const int ne = std::min(eg, nb - b0);
-    CK(gw::oz_pair_weights(P->d_D, K, as<int>(P->tc_kind) + b0, as<double>(P->tc_par) + b0, P->cfg.eta, ne,
-                           as<double>(P->oz_w), P->stream));
-    CK(gw::oz_row_scale(as<double>(P->oz_w), ne, K, K, scw, P->stream));
+    CK(gw::oz_pair_weights(P->d_D, K, as<int>(P->tc_kind) + b0, as<double>(P->tc_par) + b0, P->cfg.eta, ne, f, h,
+                           P->stream));
+    if (checked) CK(cudaMemsetAsync(P->oz_part.p, 0, sizeof(int) * (size_t)tiles * ne, P->stream));
     for (int k0 = 0; k0 < K; k0 += slab) {
       const int kc = std::min(slab, K - k0);
-      if (b0 == 0 || slab < K) CK(gw::oz_split(P->d_B_ia, 0, n, k0, kc, K, scB, 1, dB, P->stream));
-      CK(gw::oz_split_weighted(P->d_B_ia, n, k0, kc, K, scB, as<double>(P->oz_w), K, scw, ne, dA, scA, P->stream));
+      CK(gw::oz_split_weighted(P->d_B_ia, n, k0, kc, K, f, h, K, ne, dA, scA, dB, scB, P->stream));
+      if (checked) CK(gw::oz_cover(dA, dB, n, kc, ne, as<int>(P->oz_part), P->stream));
       gw::OzEpi ep{};
       ep.kind = gw::OZ_EPI_STORE;
       ep.lower = 1;
@@ -587,11 +589,14 @@ gw_status oz_weighted_syrk(gw_plan* P, const int* kinds, const double* params, i
       ep.out = out + (size_t)b0 * n * n;
       ep.out_bstride = (long)n * n;
       ep.ldo = n;
-      CK(gw::oz_gemm(gw::OzOperand{dA, scA, 1}, gw::OzOperand{dB, scB, 0}, ne, n, n, kc, ep, as<int>(P->tc_err),
+      CK(gw::oz_gemm(gw::OzOperand{dA, scA, 1}, gw::OzOperand{dB, scB, 1}, ne, n, n, kc, ep, as<int>(P->tc_err),
                      P->stream));
-      P->stats.n_kernel_launches += 3;
+      P->stats.n_kernel_launches += checked ? 3 : 2;
     }
-    P->stats.n_kernel_launches += 2;
+    P->stats.n_kernel_launches += 1;
+    if (checked)
+      LAUNCH(gw::launch_pi_syrk(P->d_B_ia, P->d_D, K, n, as<double>(P->tc_par) + b0, ne, out + (size_t)b0 * n * n, 0,
+                                P->stream, as<int>(P->oz_part)));
   }
   return GW_OK;
 }
@@ -1862,7 +1867,7 @@ gw_status gw_polarizability(gw_plan_t P, const double* xi, int n_xi, double* pi_
   } else {
     TRY(ensure(P, P->ws_mat, sizeof(double) * (size_t)n * n * n_xi));
     std::vector<int> kinds(n_xi, 0);
-    TRY(oz_weighted_syrk(P, kinds.data(), xi, n_xi, 0, 0, as<double>(P->ws_mat)));
+    TRY(oz_weighted_syrk(P, kinds.data(), xi, n_xi, 0, 0, as<double>(P->ws_mat), /*checked=*/true));
     CK(cudaEventRecord(P->ev1, P->stream));
     if (pi_out)
       CK(cudaMemcpyAsync(pi_out, P->ws_mat.p, sizeof(double) * (size_t)n * n * n_xi, cudaMemcpyDeviceToHost,
@@ -1943,7 +1948,7 @@ gw_status sd_direct(gw_plan* P, int Np, bool* ok) {
   if (fit == GW_OK) fit = ensure(P, P->sd_vec, sizeof(double) * (9 * (size_t)N + 8));
   if (fit == GW_OK) fit = ensure(P, P->oz_A, dg_bytes);
   if (fit == GW_OK) fit = ensure(P, P->oz_B, dg_bytes);
-  if (fit == GW_OK) fit = ensure(P, P->oz_sc, sizeof(double) * (2 * (size_t)std::max(N, n) + N + 1));
+  if (fit == GW_OK) fit = ensure(P, P->oz_sc, sizeof(double) * ((size_t)std::max(N, n) + N));
   if (fit != GW_OK) {
     (void)cudaGetLastError();
     for (DevBuf& b : P->sd_x) {
@@ -1988,14 +1993,11 @@ gw_status sd_direct(gw_plan* P, int Np, bool* ok) {
   }
   if (!*ok) return GW_OK;
   // V_aux = 2 B D^1/2 T and the pole weights
-  double* sB = as<double>(P->oz_sc);
-  double* sA = sB + n;
+  double* sA = as<double>(P->oz_sc);
   double* sV = sA + n;
-  double* sw = sV + N;
   CK(gw::sd_twice_sqrt(P->d_D, N, dg, P->stream));
-  CK(gw::oz_row_scale(dg, 1, N, N, sw, P->stream));
-  CK(gw::oz_row_scale(P->d_B_ia, n, N, N, sB, P->stream));
-  CK(gw::oz_split_weighted(P->d_B_ia, n, 0, N, N, sB, dg, N, sw, 1, as<__nv_bfloat16>(P->oz_A), sA, P->stream));
+  CK(gw::oz_split_weighted(P->d_B_ia, n, 0, N, N, dg, nullptr, N, 1, as<__nv_bfloat16>(P->oz_A), sA, nullptr, nullptr,
+                           P->stream));
   CK(gw::oz_row_digits(V, N, N, N, sV, as<__nv_bfloat16>(P->oz_B), P->stream));
   gw::OzEpi ep{};
   ep.kind = gw::OZ_EPI_STORE;
@@ -2005,7 +2007,7 @@ gw_status sd_direct(gw_plan* P, int Np, bool* ok) {
                  N, N, ep, as<int>(P->tc_err), P->stream));
   CK(gw::sd_rows_weights(A, H, as<double>(P->sd_V), P->d_B_nm, n, N, R, as<double>(P->sd_Om), as<double>(P->sd_w2),
                          P->stream));
-  P->stats.n_kernel_launches += 8;
+  P->stats.n_kernel_launches += 6;
   return oz_check(P);
 }
 
@@ -2463,13 +2465,13 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
     const u64 cap = std::min<u64>(ws, (u64)1 << 30), nb = std::max<u64>(n_g1, 2 * std::max<u64>(1, ws / (2 * n * n * ts)));
     const u64 slab = (u64)oz_slab((size_t)cap, c->n_aux, (int)std::min<u64>(n_ov, 2147483647ull));
     const u64 one = 2 * (u64)gw::oz_elems(c->n_aux, (int)slab), per = 2 * (u64)gw::oz_elems(c->n_aux, c->n_aux);
-    const u64 eg = std::min(nb, std::max<u64>(1, cap / one));
+    const u64 eg = std::min(nb, std::max<u64>(1, cap / (2 * one)));
     const u64 sub = std::min(n_g1, std::max<u64>(1, cap / (per + 8 * n * n))), tile = 8 * (u64)gw::oz_sumsq_tiles(c->n_aux) * sub;
     const u64 rc = std::min<u64>(rows, std::max<u64>(128, cap / (per / n)));
-    b += std::max(one * eg, rc * (per / n)) + std::max(one, per * sub) + 8 * n * n * sub;
+    b += std::max(one * eg, rc * (per / n)) + std::max(one * eg, per * sub) + 8 * n * n * sub;
     b += std::min(tile * rows, std::max(cap, tile * 128));                   // the tiles' sums
     if (c->n_aux <= kSmall64) b += 8 * (u64)gw::trsm_w_scratch_elems<double>(c->n_aux, gw::trsm_w_default_ctas());
-    b += 8 * n_ov * eg + 8 * std::max((n + 1) * (eg + 1), rows + n * sub) + 12 * nb;
+    b += 12 * n_ov * eg + 8 * std::max(2 * n * eg, rows + n * sub) + 12 * nb;
   }
   // residue batch (at most one right-hand side per target and state at a time)
   u64 batch = c->max_rhs_batch > 0 ? (u64)c->max_rhs_batch

@@ -20,11 +20,14 @@ constexpr int TK = 16;     // k step
 constexpr int NT = 256;    // threads per CTA (16 x 16, 4 x 4 outputs each)
 
 // ------------------------------------------------------------------ Pi(i xi) SYRK
-// 1 - Pi(i xi) of FP64 plans of at most one 128-row digit tile (screening_T), on the FP64 pipe.
+// Pi(i xi) on the FP64 pipe: 1 - Pi of FP64 plans of at most one 128-row digit tile (screening_T), and the tiles of a
+// digit product that oz_cover flagged (flags: one per tile and frequency, the others are left alone).
 // grid.x: lower-triangular tile index (bi >= bj), grid.y: frequency index.
 __global__ void __launch_bounds__(NT) pi_syrk_kernel(const double* __restrict__ B, const double* __restrict__ Dk,
                                                      long n_ov, int n_aux,
-                                                     const double* __restrict__ xi, double* __restrict__ out, int mode) {
+                                                     const double* __restrict__ xi, double* __restrict__ out, int mode,
+                                                     const int* __restrict__ flags) {
+  if (flags && flags[(long)blockIdx.y * gridDim.x + blockIdx.x] == 0) return;
   __shared__ double As[TK][TM + 4];
   __shared__ double Bs[TK][TN + 4];
   // decode lower tile (bi, bj) from linear index t = bi*(bi+1)/2 + bj
@@ -1036,9 +1039,9 @@ void launch_cholesky(T* base, int n, long stride, int batch, int* info, cudaStre
 }
 
 void launch_pi_syrk(const double* B, const double* Dk, long n_ov, int n_aux, const double* xi, int n_xi, double* out,
-                    int mode, cudaStream_t s) {
+                    int mode, cudaStream_t s, const int* flags) {
   const int nb = (n_aux + TM - 1) / TM;
-  pi_syrk_kernel<<<dim3(nb * (nb + 1) / 2, n_xi), NT, 0, s>>>(B, Dk, n_ov, n_aux, xi, out, mode);
+  pi_syrk_kernel<<<dim3(nb * (nb + 1) / 2, n_xi), NT, 0, s>>>(B, Dk, n_ov, n_aux, xi, out, mode, flags);
 }
 
 cudaError_t launch_tri_inv(const double* L, long stride, int n, int batch, double* X, long xstride, cudaStream_t s) {

@@ -6,8 +6,21 @@
 // tensor core's FP32 accumulators over K = 128 at a time.  |a_i b_j| <= 2^14, so such a sum of at most 8 x 128 terms
 // stays within 2^24 and every partial sum is an integer that FP32 holds: the tensor core adds without error.  The
 // drain warps add the integers into two 64-bit fixed-point sums per element (d < 4 and d >= 4), again exactly, and one
-// rounding to FP64 ends the element.  The only errors are the 2^-63 (of the row's scale) of the digits, the dropped
-// products and that rounding, less than an FP64 FMA chain makes.
+// rounding to FP64 ends the element.
+//
+// Error: besides that rounding, an element is within K 2^-59 sa sb of the exact sum, sa and sb the powers of two of its
+// two rows (the seven dropped products with i + j = 8 are up to 7 x 2^-62 of sa sb a term, the digits' own rounding
+// 2^-62; typical is sqrt(K) 2^-62).  That is relative to the rows' largest elements, not to the sum of |terms| as an FP64
+// chain's K 2^-53: it is the smaller of the two unless the sum of |terms| is below 2^-6 sa sb, which takes rows whose
+// largest elements meet small ones.  Where that matters:
+//   * weighted products sum_k x_mk w_k x_nk share the weight between the rows (x w 2^-h and x 2^h, 4^h ~ |w|): whatever
+//     the spread of the weights (a pair in resonance has 2/eta), sa sb is at most 8 times the geometric mean of the two
+//     diagonal sums of |terms|, t_m and t_n.  The error is then below K 2^-56 sqrt(t_m t_n), an eighth of an FP64 chain's
+//     bound in the same terms, which are those of the Cholesky factorisation that follows;
+//   * polarizabilities handed to the caller are checked element by element (oz_cover) and tiles with a sum of |terms|
+//     below sa sb / 8 are computed again on the FP64 pipe;
+//   * in the other uses (inverse factors against rows of B, LU updates, y^T Pi' y, eigenvector refinement) the results are
+//     no better than the rows' 2-norms allow, and K 2^-59 sa sb is below K 2^-57 |a| |b|, a sixteenth of an FP64 chain's.
 //
 // Why: FP64 runs at two multiply-adds a clock and SM on this chip (0.58 T/s in all), the digits' 36 BF16 products at
 // about 50 times that in the tensor cores.  What bounds it: shared-memory reads of the M128 N64 K16 products (6 KiB
@@ -283,40 +296,182 @@ bool map_digits(CUtensorMap* map, const void* ptr, int rows, int K, long planes,
 }
 
 // ------------------------------------------------------------------ digits
-// One thread: eight columns of one row of entry blockIdx.z: x itself (a matrix per entry at stride xbs), or one x
-// times the entry's weights.
-template <bool WEIGHTED>
+// One thread: eight columns of one row of matrix blockIdx.z (stride xbs).
 __global__ void __launch_bounds__(128) oz_split_kernel(const double* __restrict__ x, long xbs, int rows, int k0,
                                                        int cols, long ld, const double* __restrict__ sc,
-                                                       const double* __restrict__ w, long ldw,
-                                                       const double* __restrict__ wsc,
-                                                       __nv_bfloat16* __restrict__ dig, double* __restrict__ sc_out,
-                                                       int ldd) {
+                                                       __nv_bfloat16* __restrict__ dig, int ldd) {
   const int g = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.z;
   const int c = 8 * g;
   if (c >= ldd) return;
   for (int r = blockIdx.y; r < rows; r += gridDim.y) {
-    const double s0 = sc[(WEIGHTED ? 0 : (long)b * rows) + r];
-    int e = scale_exp(s0);
-    if (WEIGHTED) {
-      const double sw = wsc[b];
-      e += scale_exp(sw);
-      if (g == 0) sc_out[(long)b * rows + r] = s0 * sw;
-    }
-    const double* xr = x + (WEIGHTED ? 0 : (long)b * xbs) + (long)r * ld + k0;
+    const int e = scale_exp(sc[(long)b * rows + r]);
+    const double* xr = x + (long)b * xbs + (long)r * ld + k0;
     long long f[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      double v = 0.0;
-      if (c + t < cols) v = WEIGHTED ? xr[c + t] * w[(long)b * ldw + k0 + c + t] : xr[c + t];
-      f[t] = to_fixed(v, e);
-    }
+    for (int t = 0; t < 8; ++t) f[t] = to_fixed(c + t < cols ? xr[c + t] : 0.0, e);
     uint4 d[S];
     digits8(f, d);
 #pragma unroll
     for (int i = 0; i < S; ++i)
       *reinterpret_cast<uint4*>(dig + (((long)b * S + i) * rows + r) * ldd + c) = d[i];
   }
+}
+
+// Biased exponent of a non-zero finite value (subnormals as 1), 0 for zero, 4096 for NaN and infinities.
+__device__ __forceinline__ int exp_of(double v) {
+  const unsigned long long m = mag(v);
+  const int e = (int)(m >> 52);
+  return e == 0x7ff ? 4096 : (e == 0 && m != 0 ? 1 : e);
+}
+
+// Scale of a row from the largest biased exponent of its non-zero elements (kNoExp: none, 4096 or more: NaN).
+constexpr int kNoExp = -8192, kZeroWeight = -(1 << 20);
+__device__ __forceinline__ double scale_from_exp(int mx) {
+  if (mx == kNoExp) return 1.0;
+  const int e = max(mx - 1022, -900);
+  return e > 900 ? __longlong_as_double(0x7ff8000000000000ll) : __longlong_as_double((long long)(1023 + e) << 52);
+}
+
+// One CTA a row: digits and scale of x f (operand A) and, with PAIR, of x 2^h (operand B) for entry blockIdx.y, each row
+// scaled to its own largest element.  A first pass over the row (cached) finds the two exponents.  One FP64 product an
+// element and pass; the shift by h is integer arithmetic.
+template <bool PAIR>
+__global__ void __launch_bounds__(128) oz_split_weighted_kernel(const double* __restrict__ x, int rows, int k0, int cols,
+                                                                long ld, const double* __restrict__ f,
+                                                                const int* __restrict__ h, long ldw,
+                                                                __nv_bfloat16* __restrict__ digA,
+                                                                double* __restrict__ scA,
+                                                                __nv_bfloat16* __restrict__ digB,
+                                                                double* __restrict__ scB, int ldd) {
+  __shared__ int red[2][4];
+  const int r = blockIdx.x, b = blockIdx.y;
+  const double* xr = x + (long)r * ld + k0;
+  const double* fr = f + (long)b * ldw + k0;
+  const int* hr = PAIR ? h + (long)b * ldw + k0 : nullptr;
+  int ma = kNoExp, mb = kNoExp;
+  for (int c = threadIdx.x; c < cols; c += 128) {
+    const double v = xr[c];
+    const int ea = exp_of(v * fr[c]);
+    if (ea) ma = max(ma, ea);
+    if (PAIR && hr[c] != kZeroWeight) {
+      const int eb = exp_of(v);
+      if (eb) mb = max(mb, eb >= 4096 ? eb : eb + hr[c]);
+    }
+  }
+  ma = __reduce_max_sync(0xffffffffu, ma);
+  mb = __reduce_max_sync(0xffffffffu, mb);
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = ma;
+    red[1][threadIdx.x >> 5] = mb;
+  }
+  __syncthreads();
+  for (int i = 0; i < 4; ++i) {
+    ma = max(ma, red[0][i]);
+    mb = max(mb, red[1][i]);
+  }
+  const double sa = scale_from_exp(ma), sb = scale_from_exp(mb);
+  const int ea = scale_exp(sa), eb = scale_exp(sb);
+  const long at = (long)b * rows + r;
+  if (threadIdx.x == 0) {
+    scA[at] = sa;
+    if (PAIR) scB[at] = sb;
+  }
+  for (int c = 8 * (int)threadIdx.x; c < ldd; c += 8 * 128) {
+    long long fa[8], fb[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const bool in = c + t < cols;
+      const double v = in ? xr[c + t] : 0.0;
+      fa[t] = to_fixed(in ? v * fr[c + t] : 0.0, ea);
+      if (PAIR) {
+        const int hk = in ? hr[c + t] : kZeroWeight;
+        fb[t] = hk == kZeroWeight ? 0ll : to_fixed(v, eb - hk);
+      }
+    }
+    uint4 d[S];
+    digits8(fa, d);
+#pragma unroll
+    for (int i = 0; i < S; ++i) *reinterpret_cast<uint4*>(digA + (((long)b * S + i) * rows + r) * ldd + c) = d[i];
+    if (PAIR) {
+      digits8(fb, d);
+#pragma unroll
+      for (int i = 0; i < S; ++i) *reinterpret_cast<uint4*>(digB + (((long)b * S + i) * rows + r) * ldd + c) = d[i];
+    }
+  }
+}
+
+// Sums of |terms| of the lower 64 x 64 tiles of a digit product, from the two leading digits of each element in FP32: a
+// tile where one is below sa sb / 8 (and neither row is zero) gets its flag.  flags [batch][tiles], tiles in the order of
+// pi_syrk_kernel.  1/36 of the product's multiply-adds on the FP32 pipes: 2.3 ms for 129 entries of n 504, K 3040 at
+// their peak, for products handed to the caller only.
+constexpr int CT = 64, CKK = 16;
+__global__ void __launch_bounds__(256) oz_cover_kernel(const __nv_bfloat16* __restrict__ digA,
+                                                       const __nv_bfloat16* __restrict__ digB, int n, int ldd,
+                                                       int* __restrict__ flags) {
+  __shared__ float As[CKK][CT + 4], Bs[CKK][CT + 4];
+  const int t = blockIdx.x, b = blockIdx.y;
+  int bi = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
+  while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
+  while (bi * (bi + 1) / 2 > t) --bi;
+  const int bj = t - bi * (bi + 1) / 2, p0 = bi * CT, q0 = bj * CT;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lr = tid >> 2, lk = (tid & 3) * 4;
+  const long plane = (long)n * ldd;
+  const __nv_bfloat16* A = digA + (long)b * S * plane + (long)(p0 + lr) * ldd;
+  const __nv_bfloat16* B = digB + (long)b * S * plane + (long)(q0 + lr) * ldd;
+  auto load = [plane](const __nv_bfloat16* p, float (&v)[4]) {       // |x| / 2^e of four elements to 2^-14
+    const __nv_bfloat162* d0 = reinterpret_cast<const __nv_bfloat162*>(p);
+    const __nv_bfloat162* d1 = reinterpret_cast<const __nv_bfloat162*>(p + plane);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float2 a = __bfloat1622float2(d0[u]), c = __bfloat1622float2(d1[u]);
+      v[2 * u] = fabsf(fmaf(a.x, 256.f, c.x)) * 0.00006103515625f;
+      v[2 * u + 1] = fabsf(fmaf(a.y, 256.f, c.y)) * 0.00006103515625f;
+    }
+  };
+  float acc[4][4], sa[4], sb[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    sa[i] = sb[i] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  }
+  for (int k0 = 0; k0 < ldd; k0 += CKK) {
+    const int k = k0 + lk;
+    float va[4] = {0.f, 0.f, 0.f, 0.f}, vb[4] = {0.f, 0.f, 0.f, 0.f};
+    if (k < ldd && p0 + lr < n) load(A + k, va);             // ldd is a multiple of 8
+    if (k < ldd && q0 + lr < n) load(B + k, vb);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      As[lk + u][lr] = va[u];
+      Bs[lk + u][lr] = vb[u];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < CKK; ++kk) {
+      float a[4], c[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        a[i] = As[kk][ty + 16 * i];
+        c[i] = Bs[kk][tx + 16 * i];
+        sa[i] += a[i];
+        sb[i] += c[i];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], c[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+  bool low = false;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int p = p0 + ty + 16 * i, q = q0 + tx + 16 * j;
+      if (p < n && q <= p && sa[i] > 0.f && sb[j] > 0.f && !(acc[i][j] >= 0.125f)) low = true;
+    }
+  if (__syncthreads_or(low) && tid == 0) flags[(long)b * gridDim.x + t] = 1;
 }
 
 // Transposed operand: block of 32 source columns (operand rows) x 64 source rows through shared memory.
@@ -382,8 +537,10 @@ __global__ void __launch_bounds__(256) oz_col_scale_kernel(const double* __restr
   }
 }
 
+// w = f 2^h with 4^h within a factor of two of |w|: the two rows of a weighted product get w 2^-h and 2^h.
 __global__ void oz_weight_kernel(const double* __restrict__ Dk, int K, const int* __restrict__ kinds,
-                                 const double* __restrict__ params, double eta, double* __restrict__ w) {
+                                 const double* __restrict__ params, double eta, double* __restrict__ f,
+                                 int* __restrict__ h) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
   if (k >= K) return;
   const int kind = kinds[b];
@@ -396,7 +553,10 @@ __global__ void oz_weight_kernel(const double* __restrict__ Dk, int K, const int
     const double d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
     v = kind == 1 ? 2.0 * (a1 / d1 + a2 / d2) : 2.0 * (-eta / d1 - eta / d2);
   }
-  w[(long)b * K + k] = v;
+  const long at = (long)b * K + k;
+  const int e = max(min((int)(mag(v) >> 52) - 1023, 1023), -1022), hh = (e + 1) >> 1;
+  h[at] = v == 0.0 ? kZeroWeight : hh;
+  f[at] = v * __longlong_as_double((long long)(1023 - hh) << 52);
 }
 
 // ------------------------------------------------------------------ derivative pass
@@ -519,19 +679,33 @@ cudaError_t oz_split(const double* x, long xbs, int rows, int k0, int cols, long
   const int ldd = oz_ld(cols);
   if (nb > 65535) return cudaErrorInvalidValue;
   if (rows > 0 && cols > 0 && nb > 0)
-    oz_split_kernel<false><<<dim3((ldd / 8 + 127) / 128, std::min(rows, 65535), nb), 128, 0, s>>>(
-        x, xbs, rows, k0, cols, ld, sc, nullptr, 0, nullptr, dig, nullptr, ldd);
+    oz_split_kernel<<<dim3((ldd / 8 + 127) / 128, std::min(rows, 65535), nb), 128, 0, s>>>(x, xbs, rows, k0, cols, ld, sc,
+                                                                                          dig, ldd);
   return cudaGetLastError();
 }
 
-cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long ld, const double* sc, const double* w,
-                              long ldw, const double* wsc, int nb, __nv_bfloat16* dig, double* sc_out,
+cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long ld, const double* f, const int* h,
+                              long ldw, int nb, __nv_bfloat16* digA, double* scA, __nv_bfloat16* digB, double* scB,
                               cudaStream_t s) {
   const int ldd = oz_ld(cols);
   if (nb > 65535) return cudaErrorInvalidValue;
-  if (rows > 0 && cols > 0 && nb > 0)
-    oz_split_kernel<true><<<dim3((ldd / 8 + 127) / 128, std::min(rows, 65535), nb), 128, 0, s>>>(
-        x, 0, rows, k0, cols, ld, sc, w, ldw, wsc, dig, sc_out, ldd);
+  if (rows <= 0 || cols <= 0 || nb <= 0) return cudaGetLastError();
+  if (h)
+    oz_split_weighted_kernel<true><<<dim3(rows, nb), 128, 0, s>>>(x, rows, k0, cols, ld, f, h, ldw, digA, scA, digB, scB,
+                                                                  ldd);
+  else
+    oz_split_weighted_kernel<false><<<dim3(rows, nb), 128, 0, s>>>(x, rows, k0, cols, ld, f, h, ldw, digA, scA, digB, scB,
+                                                                   ldd);
+  return cudaGetLastError();
+}
+
+int oz_cover_tiles(int n) { return (n + CT - 1) / CT * ((n + CT - 1) / CT + 1) / 2; }
+
+cudaError_t oz_cover(const __nv_bfloat16* digA, const __nv_bfloat16* digB, int n, int cols, int nb, int* flags,
+                     cudaStream_t s) {
+  if (nb > 65535) return cudaErrorInvalidValue;
+  if (n > 0 && cols > 0 && nb > 0)
+    oz_cover_kernel<<<dim3(oz_cover_tiles(n), nb), 256, 0, s>>>(digA, digB, n, oz_ld(cols), flags);
   return cudaGetLastError();
 }
 
@@ -544,8 +718,8 @@ cudaError_t oz_split_transpose(const double* x, int rows, int cols, long ld, con
 }
 
 cudaError_t oz_pair_weights(const double* Dk, int K, const int* kinds, const double* params, double eta, int nb,
-                            double* w, cudaStream_t s) {
-  if (K > 0 && nb > 0) oz_weight_kernel<<<dim3((K + 255) / 256, nb), 256, 0, s>>>(Dk, K, kinds, params, eta, w);
+                            double* f, int* h, cudaStream_t s) {
+  if (K > 0 && nb > 0) oz_weight_kernel<<<dim3((K + 255) / 256, nb), 256, 0, s>>>(Dk, K, kinds, params, eta, f, h);
   return cudaGetLastError();
 }
 

@@ -51,13 +51,19 @@ cudaError_t oz_split(const double* x, long xbs, int rows, int k0, int cols, long
 cudaError_t oz_split_transpose(const double* x, int rows, int cols, long ld, const double* sc, __nv_bfloat16* dig,
                                cudaStream_t s);
 cudaError_t oz_col_scale(const double* x, int rows, int cols, long ld, double* sc, cudaStream_t s);
-// Digits of x[r][k] w[b][k] for nb weight rows: scales sc_out[b][r] = sc[r] * wsc[b] (wsc from oz_row_scale of w).
-cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long ld, const double* sc, const double* w,
-                              long ldw, const double* wsc, int nb, __nv_bfloat16* dig, double* sc_out,
+// Digits and scales of x[r][k] f[b][k] (digA, scA [nb][rows]) and, unless h is null, of x[r][k] 2^h[b][k] (digB, scB) for
+// the columns [k0, k0 + cols) and nb rows of weights.
+cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long ld, const double* f, const int* h,
+                              long ldw, int nb, __nv_bfloat16* digA, double* scA, __nv_bfloat16* digB, double* scB,
                               cudaStream_t s);
-// FP64 weights w[b][k] of tc_pair_weights' kinds (row length K).
+// FP64 weights w[b][k] of tc_pair_weights' kinds (row length K) as f 2^h, 4^h ~ |w|.
 cudaError_t oz_pair_weights(const double* Dk, int K, const int* kinds, const double* params, double eta, int nb,
-                            double* w, cudaStream_t s);
+                            double* f, int* h, cudaStream_t s);
+// flags[b][t] = 1 for the lower 64 x 64 tiles t of entry b that hold an element whose sum of |terms| is below an eighth of
+// its two scales' product (others are left as they are); operands of `cols` columns, oz_cover_tiles(n) tiles an entry.
+int oz_cover_tiles(int n);
+cudaError_t oz_cover(const __nv_bfloat16* digA, const __nv_bfloat16* digB, int n, int cols, int nb, int* flags,
+                     cudaStream_t s);
 
 // Row scales and digits of x [rows][cols] (row length ld) in one launch.
 cudaError_t oz_row_digits(const double* x, int rows, int cols, long ld, double* sc, __nv_bfloat16* dig,
