@@ -133,14 +133,22 @@ __device__ __forceinline__ void split_store(float v, __nv_bfloat16* hi, __nv_bfl
   if (lo2) lo2[o] = __float2bfloat16_rn(r - __bfloat162float(m));
 }
 
-// FP32 pair sum s += a b (48 bits: exact product by an FMA error term, Knuth's TwoSum), for reductions that would
-// otherwise take three operations an element on the FP64 pipe (16 clocks a warp each).
-__device__ __forceinline__ void df_fma(float a, float b, float& sh, float& sl) {
+// a + b = s + (returned) without error (Knuth's TwoSum).
+__device__ __forceinline__ float two_sum(float a, float b, float& s) {
+  s = __fadd_rn(a, b);
+  const float v = __fsub_rn(s, a);
+  return __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+}
+
+// s += a b in three FP32 words (the exact product by an FMA error term, then TwoSums down to the third word): more bits
+// than an FP64 sum, which would take three operations an element on the FP64 pipe (16 clocks a warp each) where this
+// takes 22 on the FP32 pipes.
+__device__ __forceinline__ void sum3_fma(float a, float b, float& s0, float& s1, float& s2) {
   const float p = __fmul_rn(a, b), pe = __fmaf_rn(a, b, -p);
-  const float t = __fadd_rn(sh, p), v = __fsub_rn(t, sh);
-  const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, v)), __fsub_rn(p, v));
-  sl = __fadd_rn(sl, __fadd_rn(e, pe));
-  sh = t;
+  const float e0 = two_sum(s0, p, s0);
+  const float e1 = two_sum(s1, pe, s1);
+  const float e2 = two_sum(s1, e0, s1);
+  s2 = __fadd_rn(s2, __fadd_rn(e1, e2));
 }
 
 // stg: [BM][TN + 1] staged tile; aux: 4 TN floats of shared memory.
@@ -231,11 +239,11 @@ __device__ void epilogue(const TcEpi& ep, const float* stg, float* aux, int m0, 
       const int cc = threadIdx.x, n = n0 + cc;
       if (n < N) {
         const float* bv = ep.bvec + (long)n * ep.ldb + m0;
-        float sh = 0.f, sl = 0.f;
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f;
         const int rows = min(BM, M - m0);
 #pragma unroll 8
-        for (int rr = 0; rr < rows; ++rr) df_fma(bv[rr], stg[rr * LDS_ + cc], sh, sl);
-        atomicAdd(ep.W + (long)n * ep.wld + ep.gidx[b], (double)sh + (double)sl);
+        for (int rr = 0; rr < rows; ++rr) sum3_fma(bv[rr], stg[rr * LDS_ + cc], s0, s1, s2);
+        atomicAdd(ep.W + (long)n * ep.wld + ep.gidx[b], (double)s0 + ((double)s1 + (double)s2));
       }
     }
   } else if (ep.kind == TC_EPI_PART) {
