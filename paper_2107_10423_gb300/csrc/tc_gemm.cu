@@ -32,6 +32,7 @@ struct TcCfg {
   static constexpr int STAGES = NSP == 2 ? 3 : 2;
   static constexpr int STAGE_BYTES = 2 * NSP * TILE_BYTES;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+  static_assert(BM * (BN + 1) * 4 + 3 * (BN + BM / 2) * 4 <= STAGES * STAGE_BYTES, "the staged tile reuses the ring");
 };
 // Two chunk buffers x two accumulators (hi*hi alone; every cross product together) x 128 columns.  Keeping the
 // dominant hi*hi product apart leaves its accumulator one accumulate per k-step; the cross terms are 2^8
@@ -151,7 +152,15 @@ __device__ __forceinline__ void sum3_fma(float a, float b, float& s0, float& s1,
   s2 = __fadd_rn(s2, __fadd_rn(e1, e2));
 }
 
-// stg: [BM][TN + 1] staged tile; aux: 4 TN floats of shared memory.
+// a + b as one FP32 value from the three words of each (a = a0 + a1 + a2 exactly), within an ulp whatever cancels.
+__device__ __forceinline__ float sum3(float a0, float a1, float a2, float b0, float b1, float b2) {
+  float s, t, u;
+  const float e0 = two_sum(a0, b0, s), e1 = two_sum(a1, b1, t);
+  const float e2 = two_sum(s, t, u);                   // the first words may cancel to the size of the second ones
+  return __fadd_rn(u, __fadd_rn(e2, __fadd_rn(e0, __fadd_rn(e1, __fadd_rn(a2, b2)))));
+}
+
+// stg: [BM][TN + 1] staged tile; aux: 3 (TN + BM / 2) floats of shared memory.
 template <int TN, int NTH>
 __device__ void epilogue(const TcEpi& ep, const float* stg, float* aux, int m0, int n0, int M, int N, int b, int* err) {
   constexpr int LDS_ = TN + 1;
@@ -165,18 +174,20 @@ __device__ void epilogue(const TcEpi& ep, const float* stg, float* aux, int m0, 
   } else if (ep.kind == TC_EPI_CPAIR) {
     // rows (2j, 2j+1) hold B^T u and B^T v of z_j = u - i v; column k is the pair ia.
     // w = c_k(x_j) (t_r + i t_i) with t = B^T z, c_k(x) = 2[1/(x - D_k + i eta) + 1/(-x - D_k + i eta)];
-    // Re w and Im w go to rows 2j, 2j+1 of the split operand of the second GEMM.  x and D enter as FP32 pairs, split
-    // once a row and column: x - D in FP64 for every element was four operations on the FP64 pipe, 8 us a tile.
-    float* Dh = aux;
-    float* Dl = aux + TN;
-    float* xh = aux + 2 * TN;
-    float* xl = xh + BM / 2;
-    for (int i = threadIdx.x; i < TN + BM / 2; i += NTH) {
+    // Re w and Im w go to rows 2j, 2j+1 of the split operand of the second GEMM.  x and D enter as three FP32 words
+    // (all 53 bits), split once a row and column: x - D in FP64 for every element was four operations on the FP64 pipe,
+    // 8 us a tile.
+    constexpr int XD = TN + BM / 2;                    // columns' D, then rows' x, per word
+    for (int i = threadIdx.x; i < XD; i += NTH) {
       const bool col = i < TN;
       const int at = col ? n0 + i : (m0 >> 1) + i - TN;
       const double v = col ? (at < N ? ep.Dk[at] : 0.0) : (at < (M >> 1) ? ep.x[at] : 0.0);
-      const float h = (float)v, l = (float)(v - (double)h);
-      if (col) { Dh[i] = h; Dl[i] = l; } else { xh[i - TN] = h; xl[i - TN] = l; }
+      const float h = (float)v;
+      const double r = v - (double)h;
+      const float l = (float)r;
+      aux[i] = h;
+      aux[XD + i] = l;
+      aux[2 * XD + i] = (float)(r - (double)l);
     }
     __syncthreads();
     const float e2 = ep.eta * ep.eta;
@@ -184,7 +195,9 @@ __device__ void epilogue(const TcEpi& ep, const float* stg, float* aux, int m0, 
       const int pr = idx / TN, cc = idx % TN;
       const int m = m0 + 2 * pr, n = n0 + cc;
       if (m >= M || n >= N) continue;
-      const float a1 = (xh[pr] - Dh[cc]) + (xl[pr] - Dl[cc]), a2 = -((xh[pr] + Dh[cc]) + (xl[pr] + Dl[cc]));
+      const float x0 = aux[TN + pr], x1 = aux[XD + TN + pr], x2 = aux[2 * XD + TN + pr];
+      const float D0 = aux[cc], D1 = aux[XD + cc], D2 = aux[2 * XD + cc];
+      const float a1 = sum3(x0, x1, x2, -D0, -D1, -D2), a2 = -sum3(x0, x1, x2, D0, D1, D2);
       const float d1 = a1 * a1 + e2, d2 = a2 * a2 + e2;
       const float cr = 2.f * (a1 / d1 + a2 / d2);
       const float ci = -2.f * ep.eta * (1.f / d1 + 1.f / d2);
@@ -470,7 +483,7 @@ struct WideCfg {
   static constexpr int A_TILE = BM * WK * 2, B_TILE = WN * WK * 2;
   static constexpr int STAGE_BYTES = NSP * (A_TILE + B_TILE);
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
-  static_assert(BM * (WN + 1) * 4 + 4 * WN * 4 <= STAGES * STAGE_BYTES, "the staged tile reuses the ring");
+  static_assert(BM * (WN + 1) * 4 + 3 * (WN + BM / 2) * 4 <= STAGES * STAGE_BYTES, "the staged tile reuses the ring");
 };
 constexpr long kWideMinTiles = 120;
 constexpr int WDRAIN = 8, WTHREADS = 32 * (WDRAIN + 2);

@@ -88,6 +88,62 @@ int main() {
 """
 
 
+# Weights c(x) of one right-hand side a pair of rows, with B^T u = 1 and B^T v = 0: rows 2j, 2j + 1 become Re c, Im c.
+# x - D runs down to 1e-13 of x at an eta below that: a1 within an ulp (2^-23), its square twice that, eta^2, the sum, two
+# divisions and a sum half an ulp each: 2^-20 in all; the parts hold 24 bits.
+CPAIR = HEAD + r"""
+int run(int nr, int N, int K, double eta) {
+  std::mt19937_64 g(nr + N);
+  std::uniform_real_distribution<double> u(0.0, 1.0);
+  const int M = 2 * nr;
+  std::vector<double> x(nr), D(N);
+  for (auto& v : x) v = 0.3 + 0.4 * u(g);
+  for (int k = 0; k < N; ++k) D[k] = k % 2 ? x[(k / 2) % nr] * (1.0 + (k % 4 == 1 ? 1 : -1) * std::pow(10.0, -13.0 * u(g)))
+                                           : 20.0 * u(g) + 0.01;
+  std::vector<float> A((size_t)M * K, 0.f), B((size_t)N * K, 0.f);
+  for (int j = 0; j < nr; ++j) A[(size_t)2 * j * K] = 1.f;
+  for (int k = 0; k < N; ++k) B[(size_t)k * K] = 1.f;
+  Split a(A, M, K), b(B, N, K);
+  const int ld = gw::tc_ld(N);
+  gw::TcEpi e{};
+  e.kind = gw::TC_EPI_CPAIR;
+  e.Dk = up(D);
+  e.x = up(x);
+  e.eta = (float)eta;
+  e.ohi = zeros<__nv_bfloat16>((size_t)M * ld);
+  e.olo = zeros<__nv_bfloat16>((size_t)M * ld);
+  e.olo2 = zeros<__nv_bfloat16>((size_t)M * ld);
+  e.ldh = ld;
+  int* err = zeros<int>(1);
+  CK(gw::tc_gemm_ex(a.op(), 1, b.op(), 0, 2, M, N, K, e, err, 0));
+  CK(cudaDeviceSynchronize());
+  const auto h = down(e.ohi, (size_t)M * ld), l = down(e.olo, (size_t)M * ld), t = down(e.olo2, (size_t)M * ld);
+  if (down(err, 1)[0] != 0) return std::printf("wait\n"), 1;
+  const double e1 = (double)(float)eta;
+  double worst = 0.0;
+  for (int j = 0; j < nr; ++j)
+    for (int k = 0; k < N; ++k) {
+      const double a1 = x[j] - D[k], a2 = -x[j] - D[k], d1 = a1 * a1 + e1 * e1, d2 = a2 * a2 + e1 * e1;
+      const double want[2] = {2.0 * (a1 / d1 + a2 / d2), -2.0 * e1 * (1.0 / d1 + 1.0 / d2)};
+      const double size[2] = {2.0 * (std::fabs(a1) / d1 + std::fabs(a2) / d2), -want[1]};
+      for (int c = 0; c < 2; ++c) {
+        const size_t o = (size_t)(2 * j + c) * ld + k;
+        const double v = (double)__bfloat162float(h[o]) + (double)__bfloat162float(l[o]) + (double)__bfloat162float(t[o]);
+        worst = std::max(worst, std::fabs(v - want[c]) / size[c]);
+      }
+    }
+  if (!(worst < std::ldexp(1.0, -20))) return std::printf("nr %d N %d: %.3g\n", nr, N, worst), 1;
+  return 0;
+}
+int main() {
+  if (run(5, 300, 16, 1e-14) || run(64, 1000, 40, 1e-9) || run(128, 60 * 256 - 5, 16, 1e-14) ||
+      run(70, 60 * 256, 24, 1e-3)) return 1;
+  std::printf("ok\n");
+  return 0;
+}
+"""
+
+
 def _run(tmp_path, src):
     nvcc = os.environ.get("NVCC") or ("/usr/local/cuda/bin/nvcc" if os.path.exists("/usr/local/cuda/bin/nvcc")
                                       else shutil.which("nvcc"))
@@ -105,3 +161,7 @@ def _run(tmp_path, src):
 
 def test_w_reduction_keeps_fp64_bits(gwlib, tmp_path):
     _run(tmp_path, WRED)
+
+
+def test_pole_weights_keep_the_bits_of_the_difference(gwlib, tmp_path):
+    _run(tmp_path, CPAIR)
