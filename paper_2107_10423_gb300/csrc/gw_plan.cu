@@ -23,6 +23,7 @@ thread_local std::string g_create_error;
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
+  bool grown = false;        // it has been allocated before
 };
 
 }  // namespace
@@ -119,6 +120,7 @@ struct gw_plan {
                      &mr_dwre, &mr_it, &mr_res, &mr_cnt, &mr_Vhi, &mr_Vlo, &mr_Uhi, &mr_Ulo, &mr_Vlo2, &mr_Ulo2, &mr_V64, &mr_part, &sg_I, &sg_dI, &sg_R, &sg_dR, &sg_om, &sg_start,
                      &sg_coef, &sg_act, &sg_tmap, &qp_st, &qp_om0, &fb_A, &fb_y, &fb_piv, &fb_info, &fb_idx, &fb_y64, &fb_V32, &fb_S32, &fb_Vp, &fb_Up, &fb_x, &fb_V64, &fb_U64, &fb_S64, &fb_sel, &fb_pos, &fb_rho, &fb_xs, &fb_Bl, &fb_part, &fb_lu, &fb_sw, &fb_linv, &fb_lus, &sd_M, &sd_T, &sd_cs, &sd_off, &sd_Om, &sd_V, &sd_w2, &sd_tmap, &sd_om, &sd_S, &sd_dS, &sd_part, &sd_x[0], &sd_x[1], &sd_x[2], &sd_x[3], &sd_x[4], &sd_vec};
     bufs.assign(all, all + sizeof(all) / sizeof(all[0]));
+    static_assert(sizeof(all) / sizeof(all[0]) + 32 <= 160, "kPlanBufs: these and the plan's other arrays");
   }
 };
 
@@ -162,14 +164,23 @@ void count_bytes(gw_plan* P, long long delta) {
   P->stats.bytes_device_peak = std::max(P->stats.bytes_device_peak, P->stats.bytes_device);
 }
 
-// Device allocations of a plan, counted in gw_stats.bytes_device: buffers up to kSmallBuf come out of slabs that the plan
-// holds until it is destroyed; larger ones are the driver's.  A cudaMalloc with its cudaFree takes 40 to 130 us and a small
-// job has some 60 buffers: a (H2O)_1 job takes 3.70 ms with one each, 3.48 with 4 MiB slabs, 3.25 with these; a (H2O)_5
-// one 15.2, 14.8 and 14.1.
+// Device allocations of a plan, counted in gw_stats.bytes_device: a buffer's first allocation, up to kSmallBuf, comes out
+// of slabs that the plan holds until it is destroyed; larger ones and a buffer that has outgrown its share are the
+// driver's.  A cudaMalloc with its cudaFree takes 40 to 130 us and a small job has some 60 buffers: a (H2O)_1 job takes
+// 3.70 ms with one each, 3.48 with 4 MiB slabs, 3.25 with these; a (H2O)_5 one 15.2, 14.8 and 14.1.
+// A slab is left when a buffer of at most kSmallBuf does not fit, so at least 3/4 of it are first allocations, one per
+// buffer: slab_bound follows.
 constexpr size_t kSlab = 32u << 20, kSmallBuf = 8u << 20;
+constexpr size_t kPlanBufs = 160;              // buffers a plan has, work space and others
 
-gw_status plan_alloc(gw_plan* P, void** p, size_t bytes) {
-  if (bytes > kSmallBuf) {
+// Bytes of slabs that a plan may hold beside its other buffers, all of them `bytes` at their final sizes.
+unsigned long long slab_bound(unsigned long long bytes) {
+  const unsigned long long first = std::min<unsigned long long>(bytes, kPlanBufs * kSmallBuf) + 512 * kPlanBufs;
+  return first / 3 * 4 + kSlab;
+}
+
+gw_status plan_alloc(gw_plan* P, void** p, size_t bytes, bool first = true) {
+  if (bytes > kSmallBuf || !first) {
     CK(cudaMalloc(p, bytes));
     count_bytes(P, (long long)bytes);
     return GW_OK;
@@ -207,16 +218,16 @@ gw_status dmalloc(gw_plan* P, T** p, size_t bytes) {
 
 gw_status ensure(gw_plan* P, DevBuf& b, size_t bytes) {
   if (b.bytes >= bytes && b.p) return GW_OK;
+  const bool first = !b.p && !b.grown;
   if (b.p) {
     CK(cudaStreamSynchronize(P->stream));
-    // a buffer that grows inside a slab at least doubles: what it leaves behind stays below its final size
-    if (in_slab(P, b.p) && bytes < 2 * b.bytes) bytes = 2 * b.bytes;
     plan_free(P, b.p, b.bytes);
     b.p = nullptr;
     b.bytes = 0;
+    b.grown = true;
   }
   if (bytes == 0) bytes = 16;
-  TRY(plan_alloc(P, &b.p, bytes));
+  TRY(plan_alloc(P, &b.p, bytes, first));
   b.bytes = bytes;
   return GW_OK;
 }
@@ -822,10 +833,10 @@ gw_status ensure_third_parts(gw_plan* P);
 constexpr double kResonantCut = 0.1;
 
 // BF16 elements of the blocked LU's panel operands for a fallback batch of fb matrices: the whole batch, or as many
-// matrices as fit in 1 GiB (at least one); the LU then runs in sub-batches.
-size_t lu_work_elems(int n, long fb, bool fp64) {
+// matrices as fit in the work space ws, 1 GiB at most (at least one); the LU then runs in sub-batches.
+size_t lu_work_elems(int n, long fb, bool fp64, size_t ws) {
   const size_t one = gw::zlu_operand_elems(n, 1, fp64);
-  const size_t cap = std::max(one, ((size_t)1 << 29) / std::max<size_t>(one, 1) * one);
+  const size_t cap = std::max(one, std::min<size_t>((size_t)1 << 29, ws / 2) / std::max<size_t>(one, 1) * one);
   return std::min(one * (size_t)std::max(1L, fb), cap);
 }
 
@@ -861,7 +872,7 @@ gw_status dense_fallback(gw_plan* P, const std::vector<int>& need, const int* rt
     TRY(ensure(P, P->fb_sel, sizeof(int) * fb));
     TRY(ensure(P, P->fb_pos, sizeof(int) * fb));
   }
-  TRY(ensure(P, P->fb_lu, sizeof(__nv_bfloat16) * lu_work_elems(n, fb, sizeof(T) == 8)));
+  TRY(ensure(P, P->fb_lu, sizeof(__nv_bfloat16) * lu_work_elems(n, fb, sizeof(T) == 8, ws_bytes(P))));
   TRY(ensure(P, P->fb_sw, sizeof(int) * gw::zlu_index_ints(fb)));
   TRY(ensure(P, P->fb_linv, sizeof(T) * gw::zlu_linv_elems(fb)));
   if (sizeof(T) == 8) TRY(ensure(P, P->fb_lus, sizeof(double) * gw::zlu_scale_elems(n, fb)));
@@ -2486,7 +2497,6 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
     b += batch * 8 * (ldf - n_ov) + 4 * (u64)152 * 128 * 128;                // U rows' padding, partial products
   }
   b += 48 * std::max<u64>(1, rows) + 8 * 6 * (u64)n_t + 64;                  // residue lists, Sigma scratch
-  b += 3 * kSlab;                                                            // slabs: their ends, buffers that grew
   // dense fallback batch
   const u64 mat2 = 2 * n * n * ts;
   const u64 fb = std::max<u64>(1, ws / mat2);
@@ -2496,9 +2506,9 @@ gw_status gw_plan_footprint(const gw_config* c, int n_t, unsigned flags, unsigne
     b += fb * (32 * n + 16 * n_ov) + 4 * n * n_ov;                           // FP64-residual vectors, df lo part of B
     b += (u64)gw::kDfPartTiles * 64 * 64 * 8;                                // its K ranges' sums
   }
-  b += 2 * (u64)lu_work_elems(c->n_aux, (long)std::min<u64>(fb, 1u << 30), !mixed);      // blocked-LU operands
+  b += 2 * (u64)lu_work_elems(c->n_aux, (long)std::min<u64>(fb, 1u << 30), !mixed, (size_t)ws);   // blocked-LU operands
   b += fb * (4 * (u64)gw::zlu_index_ints(1) + ts * (u64)gw::zlu_linv_elems(1) + (mixed ? 0 : 8 * (u64)gw::zlu_scale_elems(c->n_aux, 1)));
-  *bytes = b;
+  *bytes = b + slab_bound(b);
   return GW_OK;
 }
 
