@@ -12,10 +12,7 @@
 namespace gw {
 namespace {
 
-constexpr int LU_NB = 32;        // panel width
 constexpr int LU_T = 512;        // threads per CTA
-constexpr int TTM = 64;          // trailing-update tile rows (16 thread rows x 4)
-constexpr int TTN = 128;         // trailing-update tile columns (32 thread columns x 4)
 
 template <typename T>
 struct cplx {
@@ -52,201 +49,12 @@ __device__ int pivot_row(const T* Ar, const T* Ai, int n, int c, int r0, double*
   return bb > 0.0 ? ii : -1;
 }
 
-// The whole LU in one CTA, for matrices with more rows than lu_panel_kernel holds: panels of LU_NB columns, each
-// followed by its U12 solve and trailing update; rows are swapped in full.  info[b]: a zero pivot (column + 1) or 0.
-template <typename T>
-__global__ void __launch_bounds__(LU_T) zlu_kernel(T* Ar_base, T* Ai_base, long stride, int n, int* piv_base,
-                                                   int* info) {
-  const int kbeg = 0, kend = n;
-  extern __shared__ __align__(16) unsigned char sm[];
-  T* Lr = reinterpret_cast<T*>(sm);               // [TTM][LU_NB+1]
-  T* Li = Lr + TTM * (LU_NB + 1);
-  T* Ur = Li + TTM * (LU_NB + 1);                 // [LU_NB][TTN+1]
-  T* Ui = Ur + LU_NB * (TTN + 1);
-  __shared__ double sv[32];
-  __shared__ int si[32];
-  __shared__ T L11r[LU_NB * (LU_NB + 1)], L11i[LU_NB * (LU_NB + 1)];   // strictly lower part of the panel's top block
-  __shared__ T ucol_r[LU_NB], ucol_i[LU_NB];
-  T* Ar = Ar_base + (long)blockIdx.x * stride;
-  T* Ai = Ai_base + (long)blockIdx.x * stride;
-  int* piv = piv_base + (long)blockIdx.x * n;
-  int bad = 0;
-  for (int k0 = kbeg; k0 < kend; k0 += LU_NB) {
-    const int nb = min(LU_NB, kend - k0), k1 = k0 + nb;
-    // ---- panel factorisation (columns k0..k1-1), left-looking with partial pivoting; rows swapped in full.
-    // Column c is brought up to date only when it becomes the pivot column: its U part (rows k0..c-1) by a
-    // triangular solve with L11 (kept in shared memory), its rows below by one matrix-vector pass (thread per
-    // row, contiguous reads), so every panel element is written once.
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int c = k0; c < k1; ++c) {
-      const int cc = c - k0;
-      if (wid == 0) {
-        // U part of column c: u_r = a_rc - sum_{q<r} L11[r][q] u_q, r = k0..c-1 (lane r holds u_r)
-        T vr = lane < cc ? Ar[(long)(k0 + lane) * n + c] : T(0);
-        T vi = lane < cc ? Ai[(long)(k0 + lane) * n + c] : T(0);
-        for (int r = 1; r < cc; ++r) {
-          T ar = T(0), ai = T(0);
-          if (lane < r) {
-            const T lr = L11r[r * (LU_NB + 1) + lane], li = L11i[r * (LU_NB + 1) + lane];
-            ar = lr * vr - li * vi;
-            ai = lr * vi + li * vr;
-          }
-          for (int o = 16; o > 0; o >>= 1) {
-            ar += __shfl_xor_sync(0xffffffffu, ar, o);
-            ai += __shfl_xor_sync(0xffffffffu, ai, o);
-          }
-          if (lane == r) { vr -= ar; vi -= ai; }
-        }
-        if (lane < cc) {
-          ucol_r[lane] = vr;
-          ucol_i[lane] = vi;
-          Ar[(long)(k0 + lane) * n + c] = vr;
-          Ai[(long)(k0 + lane) * n + c] = vi;
-        }
-      }
-      __syncthreads();
-      // rows c..n-1: a_ic -= sum_{q<c} L_iq u_q
-      if (cc > 0) {
-        for (int i = c + threadIdx.x; i < n; i += blockDim.x) {
-          const T* lr = Ar + (long)i * n + k0;
-          const T* li = Ai + (long)i * n + k0;
-          T sr = T(0), si2 = T(0);
-          for (int q = 0; q < cc; ++q) {
-            sr += lr[q] * ucol_r[q] - li[q] * ucol_i[q];
-            si2 += lr[q] * ucol_i[q] + li[q] * ucol_r[q];
-          }
-          Ar[(long)i * n + c] -= sr;
-          Ai[(long)i * n + c] -= si2;
-        }
-      }
-      __threadfence_block();
-      __syncthreads();
-      int p = pivot_row(Ar, Ai, n, c, c, sv, si);
-      if (p < 0) { bad = c + 1; p = c; }
-      if (threadIdx.x == 0) piv[c] = p;
-      if (p != c) {
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-          T t = Ar[(long)c * n + j]; Ar[(long)c * n + j] = Ar[(long)p * n + j]; Ar[(long)p * n + j] = t;
-          t = Ai[(long)c * n + j]; Ai[(long)c * n + j] = Ai[(long)p * n + j]; Ai[(long)p * n + j] = t;
-        }
-      }
-      __threadfence_block();
-      __syncthreads();
-      // L11 row cc (multipliers of columns k0..c-1 of the new pivot row)
-      if (threadIdx.x < cc) {
-        L11r[cc * (LU_NB + 1) + threadIdx.x] = Ar[(long)c * n + k0 + threadIdx.x];
-        L11i[cc * (LU_NB + 1) + threadIdx.x] = Ai[(long)c * n + k0 + threadIdx.x];
-      }
-      const cplx<T> d = {Ar[(long)c * n + c], Ai[(long)c * n + c]};
-      const bool dz = (d.r == T(0) && d.i == T(0));
-      for (int i = c + 1 + threadIdx.x; i < n; i += blockDim.x) {
-        cplx<T> l = {Ar[(long)i * n + c], Ai[(long)i * n + c]};
-        l = dz ? cplx<T>{T(0), T(0)} : cdiv(l, d);
-        Ar[(long)i * n + c] = l.r;
-        Ai[(long)i * n + c] = l.i;
-      }
-      __threadfence_block();
-      __syncthreads();
-    }
-    if (k1 >= kend) break;
-    // ---- U12 = L11^-1 A12 (unit lower), one column per thread, L11 from shared memory
-    for (int j = k1 + threadIdx.x; j < kend; j += blockDim.x) {
-      T* cr = Ar + (long)k0 * n + j;      // column j of the panel rows; solved entries are read back from cache
-      T* ci = Ai + (long)k0 * n + j;
-      for (int r = 1; r < nb; ++r) {
-        T sr = cr[(long)r * n], sI = ci[(long)r * n];
-        for (int q = 0; q < r; ++q) {
-          const T lr = L11r[r * (LU_NB + 1) + q], li = L11i[r * (LU_NB + 1) + q];
-          const T ur = cr[(long)q * n], ui = ci[(long)q * n];
-          sr -= lr * ur - li * ui;
-          sI -= lr * ui + li * ur;
-        }
-        cr[(long)r * n] = sr;
-        ci[(long)r * n] = sI;
-      }
-    }
-    __threadfence_block();
-    __syncthreads();
-    // ---- trailing update A22 -= L21 U12 in TTM x TTN tiles, 4 x 4 complex outputs per thread
-    const int ntm = (n - k1 + TTM - 1) / TTM, ntn = (kend - k1 + TTN - 1) / TTN;
-    const int ty = threadIdx.x >> 5, tx = threadIdx.x & 31;
-    for (int t = 0; t < ntm * ntn; ++t) {
-      const int r0 = k1 + (t / ntn) * TTM, c0 = k1 + (t % ntn) * TTN;
-      for (int idx = threadIdx.x; idx < TTM * LU_NB; idx += blockDim.x) {
-        const int rr = idx / LU_NB, q = idx % LU_NB;
-        const bool okr = (r0 + rr < n) && (q < nb);
-        Lr[rr * (LU_NB + 1) + q] = okr ? Ar[(long)(r0 + rr) * n + k0 + q] : T(0);
-        Li[rr * (LU_NB + 1) + q] = okr ? Ai[(long)(r0 + rr) * n + k0 + q] : T(0);
-      }
-      for (int idx = threadIdx.x; idx < LU_NB * TTN; idx += blockDim.x) {
-        const int q = idx / TTN, cc = idx % TTN;
-        const bool okc = (c0 + cc < kend) && (q < nb);
-        Ur[q * (TTN + 1) + cc] = okc ? Ar[(long)(k0 + q) * n + c0 + cc] : T(0);
-        Ui[q * (TTN + 1) + cc] = okc ? Ai[(long)(k0 + q) * n + c0 + cc] : T(0);
-      }
-      __syncthreads();
-      // this thread's 4 x 4 outputs are loaded before the K loop so that their latency overlaps the FMAs
-      T accr[4][4], acci[4][4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int gi = r0 + ty + 16 * i;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int gj = c0 + tx + 32 * j;
-          const bool in = gi < n && gj < kend;
-          accr[i][j] = in ? Ar[(long)gi * n + gj] : T(0);
-          acci[i][j] = in ? Ai[(long)gi * n + gj] : T(0);
-        }
-      }
-      for (int q = 0; q < nb; ++q) {
-        T lr[4], li[4], ur[4], ui[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          lr[i] = Lr[(ty + 16 * i) * (LU_NB + 1) + q];
-          li[i] = Li[(ty + 16 * i) * (LU_NB + 1) + q];
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          ur[j] = Ur[q * (TTN + 1) + tx + 32 * j];
-          ui[j] = Ui[q * (TTN + 1) + tx + 32 * j];
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            accr[i][j] = fma(-lr[i], ur[j], accr[i][j]);
-            accr[i][j] = fma(li[i], ui[j], accr[i][j]);
-            acci[i][j] = fma(-lr[i], ui[j], acci[i][j]);
-            acci[i][j] = fma(-li[i], ur[j], acci[i][j]);
-          }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int gi = r0 + ty + 16 * i;
-        if (gi >= n) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int gj = c0 + tx + 32 * j;
-          if (gj < kend) {
-            Ar[(long)gi * n + gj] = accr[i][j];
-            Ai[(long)gi * n + gj] = acci[i][j];
-          }
-        }
-      }
-      __syncthreads();
-    }
-    __threadfence_block();
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) info[blockIdx.x] = bad;
-}
-
 // Solve A y = rhs with the LU factors and the row permutation; rhs/y complex in two planes of length n (yr, yi),
 // overwritten in place.  Forward and back substitution in blocks of SB rows: one warp per row sums the contribution of
 // the finished unknowns (held in shared memory) with eight loads in flight, the SB x SB triangle, fetched to shared
 // memory meanwhile, is solved by one warp.  Bound by the factors' one read per solve at what a single SM can fetch
 // (226 matrices of n 1800: 5.3 ms a solve with 32-row blocks, dependent loads and the swaps replayed one by one).
-// SWAPS: for factors of zlu_kernel (n beyond lu_panel_kernel), perm holds its swaps, the unknowns stay in global memory.
+// SWAPS: for n beyond lu_panel_kernel, perm holds the swaps (lu_panel_global_kernel), the unknowns stay in global memory.
 constexpr int SB = 64;
 template <typename T, bool SWAPS>
 __global__ void __launch_bounds__(LU_T) zlu_solve_kernel(const T* Ar_base, const T* Ai_base, long stride, int n,
@@ -407,6 +215,53 @@ __device__ __forceinline__ void warp_pivot(unsigned long long& key, int& row) {
   const unsigned long long mx = ((unsigned long long)mh << 32) | ml;
   row = (int)__reduce_min_sync(0xffffffffu, key == mx ? (unsigned)row : 0x7fffffffu);
   key = mx;
+}
+
+// L11^-1 (unit lower) of a full panel from its multipliers Lr, Li [TC_PW][TC_PW + 1] to linv; X: 2 TC_PW^2 elements of
+// shared memory.  Thread (row tid / 8, columns tid % 8 + 8 t); step q adds row q to the rows below it.  All LU_T threads.
+template <typename T>
+__device__ __forceinline__ void invert_l11(const T* Lr, const T* Li, T* Xr, T* linv) {
+  constexpr int LD = TC_PW + 1;
+  const int tid = threadIdx.x;
+  T* Xi = Xr + TC_PW * TC_PW;
+  const int r = tid >> 3, j0 = tid & 7;
+  T xr[8], xi[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    xr[t] = r == j0 + 8 * t ? T(1) : T(0);
+    xi[t] = T(0);
+    Xr[r * TC_PW + j0 + 8 * t] = xr[t];
+    Xi[r * TC_PW + j0 + 8 * t] = xi[t];
+  }
+  __syncthreads();
+  for (int q = 0; q + 1 < TC_PW; ++q) {
+    if (r > q) {
+      const T lr = Lr[r * LD + q], li = Li[r * LD + q];
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (8 * t <= q) {
+          const T ur = Xr[q * TC_PW + j0 + 8 * t], ui = Xi[q * TC_PW + j0 + 8 * t];
+          xr[t] = fma(-lr, ur, xr[t]);
+          xr[t] = fma(li, ui, xr[t]);
+          xi[t] = fma(-lr, ui, xi[t]);
+          xi[t] = fma(-li, ur, xi[t]);
+        }
+      if (r == q + 1)
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          Xr[r * TC_PW + j0 + 8 * t] = xr[t];
+          Xi[r * TC_PW + j0 + 8 * t] = xi[t];
+        }
+    }
+    __syncthreads();
+  }
+  // [q][row]: column q of L11^-1 contiguous in the row, as lu_cols_kernel reads it
+  T* vi = linv + TC_PW * TC_PW;
+  for (int i = tid; i < TC_PW * TC_PW; i += LU_T) {
+    const int q = i / TC_PW, row = i % TC_PW;
+    linv[i] = Xr[row * TC_PW + q];
+    vi[i] = Xi[row * TC_PW + q];
+  }
 }
 
 template <typename T, int RPT, int NB>
@@ -667,51 +522,106 @@ __global__ void __launch_bounds__(LU_T, 1) lu_panel_kernel(T* Ar_base, T* Ai_bas
     else if (s_bad && info[blockIdx.x] == 0) info[blockIdx.x] = s_bad;
   }
   if (kend >= n) return;
-  // ---- L11^-1 (unit lower) in place of the panel's other shared memory: thread (row tid / 8, columns tid % 8 + 8 t);
-  // step q adds row q to the rows below it
-  T* Xr = Ur;                                       // [TC_PW][TC_PW] over Ur, Ui, stage (and map, read above)
-  T* Xi = Xr + TC_PW * TC_PW;
-  {
-    const int r = tid >> 3, j0 = tid & 7;
-    T xr[8], xi[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      xr[t] = r == j0 + 8 * t ? T(1) : T(0);
-      xi[t] = T(0);
-      Xr[r * TC_PW + j0 + 8 * t] = xr[t];
-      Xi[r * TC_PW + j0 + 8 * t] = xi[t];
-    }
+  invert_l11(Lr, Li, Ur, linv_base + (long)blockIdx.x * 2 * TC_PW * TC_PW);   // over Ur, Ui, stage (and map, read above)
+}
+
+// A panel of more rows than lu_panel_kernel holds, in global memory: columns brought up to date one by one (the rows'
+// multipliers times the column's U part, thread per row), pivot, swap within the panel, scale.  perm[c] receives the row
+// swapped with row c, sw and linv as in lu_panel_kernel.  Bound by the rows' multipliers, read once a column from L2 by
+// one SM: a mixed residue at n 16397 takes 3.8 s (15 ms a panel), an FP64 one at 8203 1.4 s.  The whole matrix in one CTA,
+// which this replaces, would run the trailing updates' (8/3) n^3 at the rate of one SM: minutes.
+template <typename T>
+__global__ void __launch_bounds__(LU_T) lu_panel_global_kernel(T* Ar_base, T* Ai_base, long stride, int n, int k0,
+                                                               int kend, int* perm_base, int* info, int* sw_base,
+                                                               T* linv_base) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  constexpr int LD = TC_PW + 1;
+  T* Lr = reinterpret_cast<T*>(sm);                // [TC_PW][LD] multipliers of the panel's finished rows
+  T* Li = Lr + TC_PW * LD;
+  T* X = Li + TC_PW * LD;                          // [2][TC_PW][TC_PW]
+  __shared__ double sv[32];
+  __shared__ int si[32], pv[TC_PW], row[2 * TC_PW], from[2 * TC_PW];
+  __shared__ T ur[TC_PW], ui[TC_PW];
+  T* Ar = Ar_base + (long)blockIdx.x * stride;
+  T* Ai = Ai_base + (long)blockIdx.x * stride;
+  const int tid = threadIdx.x, pw = kend - k0;
+  int bad = 0;
+  for (int cc = 0; cc < pw; ++cc) {
+    const int c = k0 + cc;
+    // U part of the column: u = L11^-1 (rows k0 .. c - 1)
+    T xr = tid < cc ? Ar[(long)(k0 + tid) * n + c] : T(0), xi = tid < cc ? Ai[(long)(k0 + tid) * n + c] : T(0);
+    if (tid < cc) { ur[tid] = xr; ui[tid] = xi; }
     __syncthreads();
-    for (int q = 0; q + 1 < TC_PW; ++q) {
-      if (r > q) {
-        const T lr = Lr[r * LD + q], li = Li[r * LD + q];
-#pragma unroll
-        for (int t = 0; t < 8; ++t)
-          if (8 * t <= q) {
-            const T ur = Xr[q * TC_PW + j0 + 8 * t], ui = Xi[q * TC_PW + j0 + 8 * t];
-            xr[t] = fma(-lr, ur, xr[t]);
-            xr[t] = fma(li, ui, xr[t]);
-            xi[t] = fma(-lr, ui, xi[t]);
-            xi[t] = fma(-li, ur, xi[t]);
-          }
-        if (r == q + 1)
-#pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            Xr[r * TC_PW + j0 + 8 * t] = xr[t];
-            Xi[r * TC_PW + j0 + 8 * t] = xi[t];
-          }
+    for (int q = 0; q + 1 < cc; ++q) {
+      if (tid > q && tid < cc) {
+        const T lr = Lr[tid * LD + q], li = Li[tid * LD + q];
+        xr -= lr * ur[q] - li * ui[q];
+        xi -= lr * ui[q] + li * ur[q];
+        if (tid == q + 1) { ur[tid] = xr; ui[tid] = xi; }
       }
       __syncthreads();
     }
-    // [q][row]: column q of L11^-1 contiguous in the row, as lu_cols_kernel reads it
-    T* vr = linv_base + (long)blockIdx.x * 2 * TC_PW * TC_PW;
-    T* vi = vr + TC_PW * TC_PW;
-    for (int i = tid; i < TC_PW * TC_PW; i += LU_T) {
-      const int q = i / TC_PW, row = i % TC_PW;
-      vr[i] = Xr[row * TC_PW + q];
-      vi[i] = Xi[row * TC_PW + q];
+    if (tid < cc) {
+      Ar[(long)(k0 + tid) * n + c] = xr;
+      Ai[(long)(k0 + tid) * n + c] = xi;
     }
+    if (cc > 0)
+      for (int i = c + tid; i < n; i += LU_T) {    // rows c .. n - 1
+        const T* lr = Ar + (long)i * n + k0;
+        const T* li = Ai + (long)i * n + k0;
+        T sr = T(0), s2 = T(0);
+        for (int q = 0; q < cc; ++q) {
+          sr += lr[q] * ur[q] - li[q] * ui[q];
+          s2 += lr[q] * ui[q] + li[q] * ur[q];
+        }
+        Ar[(long)i * n + c] -= sr;
+        Ai[(long)i * n + c] -= s2;
+      }
+    __syncthreads();
+    int p = pivot_row(Ar, Ai, n, c, c, sv, si);
+    if (p < 0) { bad = c + 1; p = c; }
+    if (tid == 0) pv[cc] = p;
+    if (p != c && tid < 2 * pw) {
+      T* A = (tid < pw ? Ar : Ai) + k0 + (tid < pw ? tid : tid - pw);
+      const T t = A[(long)c * n];
+      A[(long)c * n] = A[(long)p * n];
+      A[(long)p * n] = t;
+    }
+    __syncthreads();
+    if (tid < cc) {
+      Lr[cc * LD + tid] = Ar[(long)c * n + k0 + tid];
+      Li[cc * LD + tid] = Ai[(long)c * n + k0 + tid];
+    }
+    const cplx<T> d = {Ar[(long)c * n + c], Ai[(long)c * n + c]};
+    const bool dz = d.r == T(0) && d.i == T(0);
+    for (int i = c + 1 + tid; i < n; i += LU_T) {
+      cplx<T> l = {Ar[(long)i * n + c], Ai[(long)i * n + c]};
+      l = dz ? cplx<T>{T(0), T(0)} : cdiv(l, d);
+      Ar[(long)i * n + c] = l.r;
+      Ai[(long)i * n + c] = l.i;
+    }
+    __syncthreads();
   }
+  int* sw = sw_base + (long)blockIdx.x * SW_LD;
+  if (tid == 0) {
+    // the rows that move and the rows their content comes from: the panel's own rows, in order, then others as met
+    int cnt = pw;
+    for (int j = 0; j < pw; ++j) row[j] = from[j] = k0 + j;
+    for (int j = 0; j < pw; ++j) {
+      int at = pv[j] < kend ? pv[j] - k0 : pw;
+      while (at < cnt && row[at] != pv[j]) ++at;
+      if (at == cnt) { row[at] = from[at] = pv[j]; ++cnt; }
+      const int t = from[j];
+      from[j] = from[at];
+      from[at] = t;
+    }
+    sw[0] = cnt;
+    for (int t = 0; t < cnt; ++t) { sw[1 + 2 * t] = row[t]; sw[2 + 2 * t] = from[t]; }
+    if (k0 == 0) info[blockIdx.x] = bad;
+    else if (bad && info[blockIdx.x] == 0) info[blockIdx.x] = bad;
+  }
+  if (tid < pw) perm_base[(long)blockIdx.x * n + k0 + tid] = pv[tid];
+  if (kend < n) invert_l11(Lr, Li, X, linv_base + (long)blockIdx.x * 2 * TC_PW * TC_PW);
 }
 
 __device__ __forceinline__ void split3(float v, __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2, long o) {
@@ -912,7 +822,7 @@ __global__ void __launch_bounds__(128) lu_digits_l_kernel(const double* Ar_base,
 }  // namespace
 
 namespace {
-// Largest n that lu_panel_kernel holds in registers; beyond it zlu_kernel factors the whole matrix.
+// Largest n that lu_panel_kernel holds in registers; beyond it lu_panel_global_kernel factors the panels.
 template <typename T>
 constexpr int panel_rows() { return (sizeof(T) == 4 ? 32 : 16) * LU_T; }
 
@@ -964,11 +874,12 @@ cudaError_t launch_cols(T* A, long plane, long stride, int n, int batch, int k0,
 }
 
 template <typename T>
-cudaError_t whole_lu(T* A, long plane, long stride, int n, int batch, int* swaps, int* info, cudaStream_t s) {
-  const size_t smem = sizeof(T) * (2 * TTM * (LU_NB + 1) + 2 * LU_NB * (TTN + 1));
-  const cudaError_t e = cudaFuncSetAttribute(zlu_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t global_panel(T* A, long plane, long stride, int n, int batch, int k0, int kend, int* perm, int* info, int* sw,
+                         T* linv, cudaStream_t s) {
+  const int smem = (int)sizeof(T) * 2 * (TC_PW * (TC_PW + 1) + TC_PW * TC_PW);
+  const cudaError_t e = cudaFuncSetAttribute(lu_panel_global_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  zlu_kernel<T><<<batch, LU_T, smem, s>>>(A, A + plane, stride, n, swaps, info);
+  lu_panel_global_kernel<T><<<batch, LU_T, smem, s>>>(A, A + plane, stride, n, k0, kend, perm, info, sw, linv);
   return cudaGetLastError();
 }
 }  // namespace
@@ -988,7 +899,7 @@ cudaError_t launch_zlu(T* A, long stride, long plane, int n, int batch, int* per
   constexpr bool D = sizeof(T) == 8;
   if (batch <= 0) return cudaSuccess;
   if (plane + (long)n * n > stride || batch > 65535) return cudaErrorInvalidValue;
-  if (n > panel_rows<T>()) return whole_lu<T>(A, plane, stride, n, batch, perm, info, s);
+  const bool global = n > panel_rows<T>();
   // the operands of one panel update are held for sub-batches of bs matrices
   const size_t per = zlu_operand_elems(n, 1, D);
   if (n > TC_PW && work_elems < per) return cudaErrorInvalidValue;
@@ -999,7 +910,9 @@ cudaError_t launch_zlu(T* A, long stride, long plane, int n, int batch, int* per
     int* sw = idx;
     for (int k0 = 0; k0 < n; k0 += TC_PW) {
       const int kend = std::min(k0 + TC_PW, n);
-      cudaError_t e = launch_panel(Ab, plane, stride, n, nb, k0, kend, perm + (long)b0 * n, info + b0, sw, linv, s);
+      cudaError_t e =
+          global ? global_panel(Ab, plane, stride, n, nb, k0, kend, perm + (long)b0 * n, info + b0, sw, linv, s)
+                 : launch_panel(Ab, plane, stride, n, nb, k0, kend, perm + (long)b0 * n, info + b0, sw, linv, s);
       if (e != cudaSuccess) return e;
       const int m = n - kend;
       const long lsz = (long)nb * 2 * m * TC_LDK, usz = (long)nb * m * TC_LDK;     // elements of one part or digit
