@@ -172,9 +172,10 @@ gw_status gw_sigma_cd(gw_plan_t plan, const double* omega, double* sigma_c, doub
  *   Sigma_c(omega) = sum_m sum_s w_nms^2 / (omega - e_m +/- Omega_s -/+ i eta)  (upper signs for occupied m),
  *   w_nms = b_nm . V_s / sqrt(2 Omega_s),  V = 2 B_ia D^1/2 T.
  * target_idx[p] (or NULL: point p is target p, n_points = n_targets) and omega[p] (host); sigma_c, dsigma_c host
- * [n_points] (real parts), either may be NULL.  O(N_ov^3) work and 2 N_ov^2 doubles (11 N_ov^2 up to
- * N_ov = 8192 where they fit): GW_ERR_ARG above N_ov = 16384; GW_ERR_NOT_CONVERGED if 40 Jacobi sweeps do not converge.  The Casida solution is kept until W's
- * energies change (evGW). */
+ * [n_points] (real parts), either may be NULL.  O(N_ov^3) work and, while it is diagonalised, 2 N_ov^2 doubles (11 N_ov^2
+ * up to N_ov = 8192 where they fit): GW_ERR_ARG above N_ov = 16384; GW_ERR_NOT_CONVERGED if 40 Jacobi sweeps do not
+ * converge.  The poles and their weights (N_ov and n_targets n_bas N_ov doubles) are kept until W's energies change
+ * (evGW). */
 gw_status gw_sigma_sd(gw_plan_t plan, int n_points, const int* target_idx, const double* omega, double* sigma_c,
                       double* dsigma_c);
 
@@ -278,7 +279,7 @@ gw_status gw_get_stats(gw_plan_t plan, gw_stats* out);
  * mixed-precision copies, the W table, and every work-space class at the size cfg->workspace_mb caps it to (a class
  * whose single item is larger than the cap is counted at that item's size).  Work space that grows with a call's
  * own arguments is not included: gw_polarizability with explicit frequencies (n_xi matrices) and the right-hand-side
- * lists of gw_residues_minres beyond n_targets * n_bas entries.  *bytes receives the bound.  Returns GW_ERR_ARG for
+ * lists of gw_residues_minres beyond n_targets * n_bas entries; nor is gw_sigma_sd's storage, stated there.  *bytes receives the bound.  Returns GW_ERR_ARG for
  * NULL pointers or non-positive sizes. */
 gw_status gw_plan_footprint(const gw_config* cfg, int n_targets, unsigned flags, unsigned long long* bytes);
 

@@ -232,6 +232,14 @@ gw_status ensure(gw_plan* P, DevBuf& b, size_t bytes) {
   return GW_OK;
 }
 
+// Gives a buffer's memory back to the driver (one in a slab keeps it); the stream must have finished with it.
+void release(gw_plan* P, DevBuf& b) {
+  if (!b.p || in_slab(P, b.p)) return;
+  plan_free(P, b.p, b.bytes);
+  b.p = nullptr;
+  b.bytes = 0;
+}
+
 template <typename T>
 T* as(DevBuf& b) { return reinterpret_cast<T*>(b.p); }
 
@@ -1944,6 +1952,14 @@ gw_status sd_product(gw_plan* P, const double* X, const double* Y, const double*
   return GW_OK;
 }
 
+// Memory of the diagonalisation: the direct route's matrices and digits, and (all) the Casida matrix and eigenvectors.
+void sd_release(gw_plan* P, bool all) {
+  for (DevBuf& b : P->sd_x) release(P, b);
+  for (DevBuf* b : {&P->oz_A, &P->oz_B}) release(P, *b);
+  if (all)
+    for (DevBuf* b : {&P->sd_M, &P->sd_T, &P->sd_V}) release(P, *b);
+}
+
 // Eigenvectors of the Casida matrix by tridiagonalisation and refinement on digit products (kernels_sd.cu); *ok is 0
 // where the off-diagonal criterion of the Jacobi sweeps is not met (they then start from the matrix in sd_M).
 gw_status sd_direct(gw_plan* P, int Np, bool* ok) {
@@ -1962,10 +1978,7 @@ gw_status sd_direct(gw_plan* P, int Np, bool* ok) {
   if (fit == GW_OK) fit = ensure(P, P->oz_sc, sizeof(double) * ((size_t)std::max(N, n) + N));
   if (fit != GW_OK) {
     (void)cudaGetLastError();
-    for (DevBuf& b : P->sd_x) {
-      plan_free(P, b.p, b.bytes);
-      b = DevBuf{};
-    }
+    sd_release(P, false);
     return GW_OK;
   }
   CK(cudaMemsetAsync(P->tc_err.p, 0, sizeof(int), P->stream));
@@ -2041,6 +2054,7 @@ gw_status ensure_sd(gw_plan* P) {
   if (N >= 8 && N <= gw::sd_direct_max()) {
     bool ok = false;
     TRY(sd_direct(P, Np, &ok));
+    sd_release(P, ok);                             // the stream is synchronised
     if (ok) {
       P->sd_sweeps = 0;
       P->sd_done = true;
@@ -2063,6 +2077,7 @@ gw_status ensure_sd(gw_plan* P) {
   LAUNCH(CK(gw::sd_weights(P->d_B_ia, P->d_D, as<double>(P->sd_M), as<double>(P->sd_T), P->d_B_nm, n, (int)N, Np, R,
                            as<double>(P->sd_Om), as<double>(P->sd_V), as<double>(P->sd_w2), P->stream)));
   CK(cudaStreamSynchronize(P->stream));
+  sd_release(P, true);
   P->sd_sweeps = sweeps;
   P->sd_done = true;
   return GW_OK;
