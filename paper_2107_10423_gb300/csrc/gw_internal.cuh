@@ -3,10 +3,52 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <atomic>
 #include <cstdint>
 #include <vector>
 
 namespace gw {
+
+// Runs a set-up that belongs to a device (kernel attributes) once on each, again where it failed; any thread may call it.
+class PerDevice {
+  std::atomic<unsigned long long> done_[2] = {};
+
+ public:
+  template <typename F>
+  cudaError_t run(int dev, F set_up) {
+    if (dev < 0 || dev >= 128) return set_up();
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done_[dev >> 6].load(std::memory_order_acquire) & bit) return cudaSuccess;
+    const cudaError_t e = set_up();              // threads that meet here each run it
+    if (e == cudaSuccess) done_[dev >> 6].fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+  template <typename F>
+  cudaError_t run(F set_up) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? run(dev, set_up) : e;
+  }
+};
+
+// Lets a kernel take all the dynamic shared memory its device has, once per device.  The limit is a property of the kernel
+// that every thread shares: set to each launch's own size, a plan's smaller one between another's call and launch makes
+// that launch fail.
+template <auto Kernel>
+cudaError_t allow_smem() {
+  static PerDevice once;
+  return once.run([] {
+    cudaFuncAttributes a;
+    int dev = 0, most = 0;
+    cudaError_t e = cudaFuncGetAttributes(&a, (const void*)Kernel);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute((const void*)Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               most - (int)a.sharedSizeBytes);
+    return e;
+  });
+}
 
 // ---------------------------------------------------------------- dense kernels (kernels_dense.cu)
 // Every kernel below takes the pair energies D_k (k < n_ov, the columns of B) as an array Dk.

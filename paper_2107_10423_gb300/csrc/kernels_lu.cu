@@ -831,8 +831,7 @@ cudaError_t panel(T* A, long plane, long stride, int n, int batch, int k0, int k
                   T* linv, cudaStream_t s) {
   const size_t work = sizeof(T) * (2 * TC_PW * NB + 2 * NB * 2 * TC_PW) + sizeof(int) * (size_t)(n - k0);
   const size_t smem = sizeof(T) * 2 * TC_PW * (TC_PW + 1) + std::max(work, sizeof(T) * 2 * TC_PW * TC_PW);
-  const cudaError_t e = cudaFuncSetAttribute(lu_panel_kernel<T, RPT, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+  const cudaError_t e = allow_smem<lu_panel_kernel<T, RPT, NB>>();
   if (e != cudaSuccess) return e;
   lu_panel_kernel<T, RPT, NB><<<batch, LU_T, smem, s>>>(A, A + plane, stride, n, k0, kend, perm, info, sw, linv);
   return cudaGetLastError();
@@ -864,7 +863,7 @@ cudaError_t launch_cols(T* A, long plane, long stride, int n, int batch, int k0,
                         __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2, double* usc, long olim, int* err,
                         cudaStream_t s) {
   const int smem = (int)sizeof(T) * (6 * TC_PW * TC_PW + TC_PW);
-  const cudaError_t e = cudaFuncSetAttribute(lu_cols_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = allow_smem<lu_cols_kernel<T>>();
   if (e != cudaSuccess) return e;
   const int gx = (k0 + TC_PW - 1) / TC_PW + (n - kend + TC_PW - 1) / TC_PW;
   if (gx > 0)
@@ -877,7 +876,7 @@ template <typename T>
 cudaError_t global_panel(T* A, long plane, long stride, int n, int batch, int k0, int kend, int* perm, int* info, int* sw,
                          T* linv, cudaStream_t s) {
   const int smem = (int)sizeof(T) * 2 * (TC_PW * (TC_PW + 1) + TC_PW * TC_PW);
-  const cudaError_t e = cudaFuncSetAttribute(lu_panel_global_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = allow_smem<lu_panel_global_kernel<T>>();
   if (e != cudaSuccess) return e;
   lu_panel_global_kernel<T><<<batch, LU_T, smem, s>>>(A, A + plane, stride, n, k0, kend, perm, info, sw, linv);
   return cudaGetLastError();
@@ -966,15 +965,13 @@ cudaError_t launch_zlu_solve(const T* Ar, const T* Ai, long stride, int n, int b
   if (batch <= 0) return cudaSuccess;
   const size_t tri = sizeof(T) * (2 * SB * (SB + 1) + 2 * SB);
   if (n > panel_rows<T>()) {
-    const cudaError_t e = cudaFuncSetAttribute(zlu_solve_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)tri);
+    const cudaError_t e = allow_smem<zlu_solve_kernel<T, true>>();
     if (e != cudaSuccess) return e;
     zlu_solve_kernel<T, true><<<batch, LU_T, tri, s>>>(Ar, Ai, stride, n, perm, yr, yi, ystride);
     return cudaGetLastError();
   }
   const size_t smem = tri + sizeof(T) * 2 * (size_t)n;
-  const cudaError_t e = cudaFuncSetAttribute(zlu_solve_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+  const cudaError_t e = allow_smem<zlu_solve_kernel<T, false>>();
   if (e != cudaSuccess) return e;
   zlu_solve_kernel<T, false><<<batch, LU_T, smem, s>>>(Ar, Ai, stride, n, perm, yr, yi, ystride);
   return cudaGetLastError();

@@ -671,7 +671,7 @@ cudaError_t sd_tridiagonal(double* A, int N, long ld, double* H, double* beta, d
   const bool sm = with_rows <= 220 * 1024;   // N up to about 1800
   const int smem = sm ? (int)with_rows : 3 * N * (int)sizeof(double);
   const void* f = sm ? (const void*)tridiag_kernel<true> : (const void*)tridiag_kernel<false>;
-  c = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  c = sm ? allow_smem<tridiag_kernel<true>>() : allow_smem<tridiag_kernel<false>>();
   if (c == cudaSuccess) c = cudaMemsetAsync(bar, 0, sizeof(unsigned), s);
   if (c != cudaSuccess) return c;
   void* args[] = {(void*)&A, (void*)&N, (void*)&ld, (void*)&H, (void*)&beta, (void*)&d, (void*)&e, (void*)&p_buf,
@@ -686,8 +686,9 @@ cudaError_t sd_tridiagonal_vectors(const double* d, const double* e, int N, doub
   cudaError_t c = cudaGetDevice(&dev);
   if (c == cudaSuccess) c = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int bs = 2 * N * (int)sizeof(double);
-  if (c == cudaSuccess) c = cudaFuncSetAttribute(tri_bisect_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bs);
-  if (c == cudaSuccess) c = cudaFuncSetAttribute(tri_bisect_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bs);
+  if (c == cudaSuccess) c = allow_smem<tri_bisect_kernel<16>>();
+  if (c == cudaSuccess) c = allow_smem<tri_bisect_kernel<4>>();
+  if (c == cudaSuccess) c = allow_smem<tri_back_kernel>();
   if (c != cudaSuccess) return c;
   if (N <= 2800) tri_bisect_kernel<16><<<(N + 7) / 8, 128, bs, s>>>(d, e, N, lam);
   else tri_bisect_kernel<4><<<(N + 31) / 32, 128, bs, s>>>(d, e, N, lam);
@@ -698,8 +699,6 @@ cudaError_t sd_tridiagonal_vectors(const double* d, const double* e, int N, doub
   warps = warps < even ? warps : even;
   warps = warps < 1 ? 1 : (warps > 8 ? 8 : warps);
   const int zs = warps * N * (int)sizeof(double);
-  c = cudaFuncSetAttribute(tri_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, zs);
-  if (c != cudaSuccess) return c;
   tri_back_kernel<<<(N + warps - 1) / warps, 32 * warps, zs, s>>>(H, beta, N, ld, nrm, Z);
   return cudaGetLastError();
 }
