@@ -26,6 +26,7 @@
 // about 50 times that in the tensor cores.  What bounds it: shared-memory reads of the M128 N64 K16 products (6 KiB
 // each at 128 B a clock: 48 clocks, where the tensor core alone would take 32), then the drains, which the single
 // TMEM buffer (8 sums x 64 columns = all 512) does not overlap with the next 128 of K.
+#include "gw_internal.cuh"
 #include "oz_gemm.cuh"
 #include "oz_digits.cuh"
 #include "tc_ptx.cuh"
@@ -651,12 +652,10 @@ cudaError_t oz_gemm(const OzOperand& A, const OzOperand& B, int batch, int M, in
   if (!map_digits(&maps.a, A.dig, M, K, (long)S * (A.batched ? batch : 1), BM) ||
       !map_digits(&maps.b, B.dig, N, K, (long)S * (B.batched ? batch : 1), BN))
     return cudaErrorInvalidValue;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static PerDevice attr;
+  const cudaError_t ae = attr.run(
+      [] { return cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES); });
+  if (ae != cudaSuccess) return ae;
   const long nbm = (M + BM - 1) / BM, nbn = (N + BN - 1) / BN;
   const long tiles = ep.kind == OZ_EPI_STORE && ep.lower ? nbm * (nbm + 1) : nbm * nbn;
   oz_gemm_kernel<<<dim3((unsigned)tiles, batch), THREADS, SMEM_BYTES, s>>>(maps, M, N, K, A.batched, B.batched, A.sc, B.sc,

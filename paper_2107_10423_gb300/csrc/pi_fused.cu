@@ -41,6 +41,7 @@
 // Every mbarrier wait is bounded; on timeout the kernel records a code in *err, stops every role, waits for its
 // copies and tensor-core work in flight, frees TMEM and returns.
 #include "pi_tc.cuh"
+#include "gw_internal.cuh"
 #include "tc_ptx.cuh"
 
 #include <cuda.h>
@@ -643,12 +644,10 @@ cudaError_t tc_pi_fused(int n, int K, const float* w, int nb, const uint32_t* ti
       !map_panel(&maps.bl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Blo, n, P, BN, CU_TENSOR_MAP_SWIZZLE_64B) ||
       !map2d(&maps.w, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w, K, nb, ldw, BK, 1, CU_TENSOR_MAP_SWIZZLE_NONE))
     return cudaErrorInvalidValue;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(pi_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static PerDevice attr;
+  const cudaError_t ae = attr.run(
+      [] { return cudaFuncSetAttribute(pi_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES); });
+  if (ae != cudaSuccess) return ae;
   const int nk = (K + BK - 1) / BK;
   const size_t per_split = (size_t)nb * n * n * sizeof(float);
   auto feasible = [&](int ks) {

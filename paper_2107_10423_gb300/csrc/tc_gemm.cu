@@ -711,8 +711,8 @@ cudaError_t tc_gemm_ex(const TcOperand& A, int batch, const TcOperand& B, int b_
         !make_map(&maps.b[i], B.p[i], N, K, ld, bb, wide ? WK : BK, wide ? WN : BN,
                   wide ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B))
       return cudaErrorInvalidValue;
-  static bool attr = false;
-  if (!attr) {
+  static PerDevice attr;
+  const cudaError_t ae = attr.run([] {
     cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          TcCfg<2>::SMEM_BYTES);
     if (e == cudaSuccess)
@@ -723,9 +723,9 @@ cudaError_t tc_gemm_ex(const TcOperand& A, int batch, const TcOperand& B, int b_
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(tc_gemm_wide_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                WideCfg<3>::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+    return e;
+  });
+  if (ae != cudaSuccess) return ae;
   if (wide) {
     const dim3 grid((unsigned)wide_tiles, batch);
     if (nsplit == 2)
