@@ -448,7 +448,10 @@ def main():
                           "arrivals_4_slots": rnd(live4), "arrivals_1_slot": rnd(live1),
                           "capacity_jobs_per_s_4_slots": round(cap4["jobs_per_s"], 3),
                           "capacity_jobs_per_s_1_slot": round(cap1["jobs_per_s"], 3),
-                          "capacity_p99_latency_s_4_slots": round(cap4["p99_latency_s"], 3)}
+                          "capacity_p99_latency_s_4_slots": round(cap4["p99_latency_s"], 3),
+                          # jobs whose mixed solve failed and that ran again in FP64, with what it said
+                          "capacity_fp64_fallbacks": [cap4["fp64_fallbacks"], cap1["fp64_fallbacks"]],
+                          "capacity_mixed_errors": [cap4["mixed_errors"], cap1["mixed_errors"]]}
         # serial plain-FP64 baseline: the sample's small jobs ((H2O)_n, n <= 3; an FP64 (H2O)_16 job alone takes
         # minutes) solved one after another in FP64, against their latency in the 4-slot mixed run above
         try:

@@ -58,16 +58,20 @@ def run_job(job: Job, precision: str = "mixed", qp: str = "linearised") -> dict:
     mode = gw.GW_QP_LINEARISED if qp == "linearised" else gw.GW_QP_STEPTREE
     tries = [gw.GW_PREC_MIXED, gw.GW_PREC_FP64] if precision == "mixed" else [gw.GW_PREC_FP64]
     last = None
+    retried = {}
     for prec in tries:
         try:
             with gw.Plan(s.eps, s.n_occ, B_ia, B_nm, s.targets, precision=prec,
                          workspace_mb=workspace_for(s)) as p:
                 p.screening()
                 e, z, st = p.qp_solve(mode)
-            return {"e_qp": e, "z": z, "status": st, "precision": "mixed" if prec == gw.GW_PREC_MIXED else "fp64"}
-        except gw.GWError as err:          # mixed failed: fall back to FP64 for this job
+            return {"e_qp": e, "z": z, "status": st, "precision": "mixed" if prec == gw.GW_PREC_MIXED else "fp64",
+                    **retried}
+        except gw.GWError as err:          # mixed failed: fall back to FP64 for this job, and say why
             last = err
-    return {"error": str(last)}
+            if prec == gw.GW_PREC_MIXED:
+                retried = {"mixed_error": str(err)}
+    return {"error": str(last), **retried}
 
 
 class Server:
@@ -142,7 +146,8 @@ def summarize(jobs, makespan: float = None) -> dict:
     return {"jobs": len(jobs), "completed": len(ok), "jobs_per_s": len(ok) / span if span > 0 else None,
             "p50_latency_s": float(np.percentile(lat, 50)), "p99_latency_s": float(np.percentile(lat, 99)),
             "mean_wait_s": float(np.mean([j.start - j.arrival for j in jobs])),
-            "fp64_fallbacks": sum(1 for j in ok if j.result.get("precision") == "fp64")}
+            "fp64_fallbacks": sum(1 for j in ok if j.result.get("precision") == "fp64"),
+            "mixed_errors": {j.job_id: j.result["mixed_error"] for j in jobs if "mixed_error" in j.result}}
 
 
 def make_jobs(stream, n_max: int = None, limit: int = None, mixed: bool = True, inputs: bool = False):
