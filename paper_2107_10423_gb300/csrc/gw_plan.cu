@@ -696,11 +696,11 @@ gw_status screening_T(gw_plan* P) {
     chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)chunk, ws_bytes(P) / per_ns));
   }
   // mixed precision, one rank: the stage runs at the nodes of the grid (FreqNodes, 35 to 40 of 129 points) and the
-  // other columns follow from them; the nodes' 1e-8 is far below the BF16-part products' error.  FP64 plans, sharded
-  // plans (each rank owns a block of columns) and plans that the caller gave room for fewer than three matrices run at
-  // every grid point, so the chunked form of that path stays in use at sizes that can be checked; so do plans of one
-  // 128-row tile a matrix, whose 129 points are one wave and cost less than the search for the nodes (a (H2O)_1 job
-  // took 4.68 ms with nodes, 4.48 without; a (H2O)_3 one 4.6 with, 6.8 without).
+  // other columns follow from them; the nodes' 2e-8 is far below the BF16-part products' error.  FP64 plans and sharded
+  // plans (each rank owns a block of columns) run at every grid point, so do plans whose caller left room for fewer than
+  // three matrices (no need of theirs: the chunked form of the every-point stage, which sharded plans share, is checked
+  // against the oracle there) and plans of one 128-row tile a matrix, whose 129 points are one wave and cost less than the
+  // search for the nodes (a (H2O)_1 job took 4.68 ms with nodes, 4.48 without; a (H2O)_3 one 4.6 with, 6.8 without).
   const bool use_nodes = use_tc && n > 128 && P->sh_world == 1 && !(P->cfg.workspace_mb > 0 && chunk < 3);
   if (use_nodes && P->nodes_D != P->D_min) {
     P->nodes_D = -1.0;

@@ -623,9 +623,15 @@ __global__ void __launch_bounds__(256) op_chain2_kernel(const double* __restrict
 }
 
 // ------------------------------------------------------------------ FP32 residue operator for few rows
-// Mixed plans, up to eight rows (four right-hand sides: HOMO and LUMO jobs).  A 128-row tensor tile would be padding,
-// and its CTAs as few as the output has column tiles: at 4 rows, 3024 x 109440, a product took 1.6 ms on 24 CTAs; here
-// it is one pass over B at 6 TB/s (0.22 ms), in FP32 instead of BF16 parts.  At 126 x 190 4 us against 9.
+// Mixed plans, up to eight rows (four right-hand sides: HOMO and LUMO jobs), where a 128-row tensor tile is padding.
+// A MINRES iteration (operator and recurrences) of 1, 2, 3, 4 right-hand sides here, and of 3, 4, 5 in the tensor tiles:
+//   126 x 190       23   23    24    25 us     34   35   34
+//   629 x 4675      38   40    43    45        52   53   53
+//   1259 x 18950    97  107   116   130        96   93   93
+//   3024 x 109440  598  766  1135  1338       527  527  548
+// So the line is right up to some 10 thousand pairs.  Beyond, the first product reads B at 6 TB/s and the second, whose
+// rows of U come from L2 once per four rows of B, does not keep up with the tensor tiles (they took 1.6 ms a product
+// before theirs was split in K); it stays for its FP32 operands, where the tiles hold 16 bits.
 // Sums run in chains of 64 (gemm2) or one slice's 1/8 of the contraction (gemm1) before they are added.
 constexpr int SKC = 128;             // gemm1 columns a CTA: 32 lanes x 4
 template <int RM>

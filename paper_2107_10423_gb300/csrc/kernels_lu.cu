@@ -192,8 +192,11 @@ constexpr int SW_LD = 4 * TC_PW + 2;        // ints per matrix of the panel's pe
 // column costs two barriers and no global traffic: pivot search by shuffles, the two swapped rows through shared
 // memory, the rank-1 update in registers.  Each NB columns are first brought up to date with the panel's earlier ones
 // (U by one warp per column from L11 in shared memory, then one pass over the rows' earlier multipliers), and the
-// panel's other columns follow the swaps.  Bound by these latencies: about 60 us a panel at n 1800 in FP32, where
-// factoring column by column in global memory took 1.4 ms.  NB shrinks as rows a thread grow, to stay in 64 registers.
+// panel's other columns follow the swaps.  Bound by the latency of its loads (the rows' earlier multipliers, 8 bytes a
+// thread; 152 matrices share L2) and of the columns' barriers: the first panel at n 1800 takes 0.71 ms in FP32 (0.38 on
+// average over the matrix; 0.85 and 0.43 for 152 matrices at once) and 5.1 ms in FP64 (16 clocks a warp instruction),
+// where factoring column by column in global memory took 1.4 ms in FP32.  NB shrinks as rows a thread grow, to stay in
+// 64 registers.
 // Magnitudes as integer keys (the bits of |a|^2; NaN counts as 0), so that the pivot search stays off the FP64 pipe.
 __device__ __forceinline__ unsigned pivot_key(float v) {
   const unsigned b = __float_as_uint(v);
@@ -675,7 +678,9 @@ __device__ __forceinline__ void split3x8(const float (&v)[8], __nv_bfloat16* p0,
 // Im U12[:, c]]: FP32 split into three BF16 parts p0, p1, p2 of [batch][m][TC_LDK], FP64 as digits dig
 // [batch][OZ_S][m][TC_LDK] with the row scales usc [batch][m].  b0: the batch's first matrix within the operand's
 // sub-batch.  olim: elements of the operand (an index beyond is recorded in *err, code 65, and skipped).
-// FMA-bound in FP32 (16 FMAs a shared-memory read); the triangular solve it replaces ran column by column.
+// Bound by the latency of its loads: two CTAs an SM fit, the loads of one have only the other's FMAs (a tenth of the
+// time) to hide behind, and DRAM runs at 11 % (0.47 ms for 160 matrices of n 1800).  The triangular solve it replaces ran
+// column by column.
 template <typename T>
 __global__ void __launch_bounds__(256) lu_cols_kernel(T* Ar_base, T* Ai_base, long stride, int n, int k0, int kend,
                                                       const int* __restrict__ sw_base, const T* __restrict__ linv_base,

@@ -516,7 +516,7 @@ __global__ void tri_back_kernel(const double* __restrict__ H, const double* __re
   for (int i = lane; i < N; i += 32) Zs[i] = z[i];
 }
 
-// Refinement of rows V (V M V^T = S, V V^T = G): E_st = (S_st + lam_t R_st) / (lam_t - lam_s) off the diagonal (R_st / 2
+// Refinement (Ogita and Aishima) of rows V (V M V^T = S, V V^T = G): E_st = (S_st + lam_t R_st) / (lam_t - lam_s) off the diagonal (R_st / 2
 // where the two are closer than `close`), E_ss = R_ss / 2, R = I - G, lam_s = S_ss / (1 - R_ss); rows V_t <- V_t + sum_s
 // E_st V_s, so G is overwritten by I + E^T.  norms: [0] off-diagonal and [1] diagonal squares of S, [2] squares of R.
 __global__ void __launch_bounds__(256) eig_norms_kernel(const double* __restrict__ S, const double* __restrict__ G, int N,

@@ -1,9 +1,8 @@
-// tcgen05 (5th-generation tensor core) batched GEMM with BF16 hi+lo split operands, used for every
-// dense contraction of the mixed-precision path:
-//   out_b[m][n] = f( sum_k A_b[m][k] * Bm[n][k] ),   A_b = Ahi_b + Alo_b,  Bm = Bhi + Blo  (BF16)
-// computed as Ahi*Bhi + Ahi*Blo + Alo*Bhi with FP32 accumulation in tensor memory (TMEM).
-//  * Pi(i xi_b) (Sec. 3.3): A_b = B_ia o w_b with w_b,ia = -4 D_ia/(D_ia^2 + xi_b^2), Bm = B_ia, lower tiles.
-//  * dense real-axis Pi(x_j) for the residue fallback: A = B_ia o Re c(x_j) and B_ia o Im c(x_j).
+// tcgen05 (5th-generation tensor core) batched GEMM with BF16 split operands, used for the dense contractions of the
+// mixed-precision path other than Pi (pi_fused.cu): Newton-Schulz products and the W reduction, the MINRES and
+// refinement operators, the LU's trailing updates:
+//   out_b[m][n] = f( sum_k A_b[m][k] * B_b[n][k] ),   A = Ahi + Alo (+ Alo2),  B = Bhi + Blo (+ Blo2)  (BF16)
+// as Ahi*Bhi + Ahi*Blo + Alo*Bhi, or the six products of three parts, with FP32 accumulation in tensor memory (TMEM).
 // Operands are staged by TMA (cp.async.bulk.tensor, 128-byte swizzle) into a 3-stage shared-memory
 // ring; one elected thread issues tcgen05.mma; the accumulator is read back with tcgen05.ld.
 // Every mbarrier wait is bounded: on timeout the kernel records an error code and unwinds.
