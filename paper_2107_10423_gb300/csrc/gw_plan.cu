@@ -598,7 +598,8 @@ gw_status oz_weighted_syrk(gw_plan* P, const int* kinds, const double* params, i
     for (int k0 = 0; k0 < K; k0 += slab) {
       const int kc = std::min(slab, K - k0);
       CK(gw::oz_split_weighted(P->d_B_ia, n, k0, kc, K, f, h, K, ne, dA, scA, dB, scB, P->stream));
-      if (checked) CK(gw::oz_cover(dA, dB, n, kc, ne, as<int>(P->oz_part), P->stream));
+      const gw::OzOperand A{dA, scA, 1}, B{dB, scB, 1};
+      if (checked) CK(gw::oz_cover(A, B, n, kc, ne, as<int>(P->oz_part), P->stream));
       gw::OzEpi ep{};
       ep.kind = gw::OZ_EPI_STORE;
       ep.lower = 1;
@@ -608,8 +609,7 @@ gw_status oz_weighted_syrk(gw_plan* P, const int* kinds, const double* params, i
       ep.out = out + (size_t)b0 * n * n;
       ep.out_bstride = (long)n * n;
       ep.ldo = n;
-      CK(gw::oz_gemm(gw::OzOperand{dA, scA, 1}, gw::OzOperand{dB, scB, 1}, ne, n, n, kc, ep, as<int>(P->tc_err),
-                     P->stream));
+      CK(gw::oz_gemm(A, B, ne, n, n, kc, ep, as<int>(P->tc_err), P->stream));
       P->stats.n_kernel_launches += checked ? 3 : 2;
     }
     P->stats.n_kernel_launches += 1;

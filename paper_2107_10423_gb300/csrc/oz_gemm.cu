@@ -13,7 +13,8 @@
 // 2^-62; typical is sqrt(K) 2^-62).  That is relative to the rows' largest elements, not to the sum of |terms| as an FP64
 // chain's K 2^-53: it is the smaller of the two unless the sum of |terms| is below 2^-6 sa sb, which takes rows whose
 // largest elements meet small ones.  Where that matters:
-//   * weighted products sum_k x_mk w_k x_nk share the weight between the rows (x w 2^-h and x 2^h, 4^h ~ |w|): whatever
+//   * weighted products sum_k x_mk w_k x_nk share the weight between the rows (x w 2^-h, rounded to FP64 once as a chain
+//     rounds x w, and x 2^h, 4^h ~ |w|): whatever
 //     the spread of the weights (a pair in resonance has 2/eta), sa sb is at most 8 times the geometric mean of the two
 //     diagonal sums of |terms|, t_m and t_n.  The error is then below K 2^-56 sqrt(t_m t_n), an eighth of an FP64 chain's
 //     bound in the same terms, which are those of the Cholesky factorisation that follows;
@@ -402,13 +403,14 @@ __global__ void __launch_bounds__(128) oz_split_weighted_kernel(const double* __
 }
 
 // Sums of |terms| of the lower 64 x 64 tiles of a digit product, from the two leading digits of each element in FP32: a
-// tile where one is below sa sb / 8 (and neither row is zero) gets its flag.  flags [batch][tiles], tiles in the order of
-// pi_syrk_kernel.  1/36 of the product's multiply-adds on the FP32 pipes: 2.3 ms for 129 entries of n 504, K 3040 at
+// tile where one is below sa sb / 8 (and neither row is zero), or where a row holds a NaN or an infinity (its scale is
+// NaN), gets its flag.  flags [batch][tiles], tiles in the order of pi_syrk_kernel.  1/36 of the product's multiply-adds on the FP32 pipes: 2.3 ms for 129 entries of n 504, K 3040 at
 // their peak, for products handed to the caller only.
 constexpr int CT = 64, CKK = 16;
 __global__ void __launch_bounds__(256) oz_cover_kernel(const __nv_bfloat16* __restrict__ digA,
-                                                       const __nv_bfloat16* __restrict__ digB, int n, int ldd,
-                                                       int* __restrict__ flags) {
+                                                       const __nv_bfloat16* __restrict__ digB,
+                                                       const double* __restrict__ scA, const double* __restrict__ scB,
+                                                       int n, int ldd, int* __restrict__ flags) {
   __shared__ float As[CKK][CT + 4], Bs[CKK][CT + 4];
   const int t = blockIdx.x, b = blockIdx.y;
   int bi = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
@@ -470,7 +472,9 @@ __global__ void __launch_bounds__(256) oz_cover_kernel(const __nv_bfloat16* __re
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int p = p0 + ty + 16 * i, q = q0 + tx + 16 * j;
-      if (p < n && q <= p && sa[i] > 0.f && sb[j] > 0.f && !(acc[i][j] >= 0.125f)) low = true;
+      if (p >= n || q > p) continue;
+      if (sa[i] > 0.f && sb[j] > 0.f && !(acc[i][j] >= 0.125f)) low = true;
+      if (isnan(scA[(long)b * n + p]) || isnan(scB[(long)b * n + q])) low = true;
     }
   if (__syncthreads_or(low) && tid == 0) flags[(long)b * gridDim.x + t] = 1;
 }
@@ -700,11 +704,10 @@ cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long 
 
 int oz_cover_tiles(int n) { return (n + CT - 1) / CT * ((n + CT - 1) / CT + 1) / 2; }
 
-cudaError_t oz_cover(const __nv_bfloat16* digA, const __nv_bfloat16* digB, int n, int cols, int nb, int* flags,
-                     cudaStream_t s) {
-  if (nb > 65535) return cudaErrorInvalidValue;
+cudaError_t oz_cover(const OzOperand& A, const OzOperand& B, int n, int cols, int nb, int* flags, cudaStream_t s) {
+  if (nb > 65535 || !A.batched || !B.batched) return cudaErrorInvalidValue;
   if (n > 0 && cols > 0 && nb > 0)
-    oz_cover_kernel<<<dim3(oz_cover_tiles(n), nb), 256, 0, s>>>(digA, digB, n, oz_ld(cols), flags);
+    oz_cover_kernel<<<dim3(oz_cover_tiles(n), nb), 256, 0, s>>>(A.dig, B.dig, A.sc, B.sc, n, oz_ld(cols), flags);
   return cudaGetLastError();
 }
 

@@ -60,10 +60,10 @@ cudaError_t oz_split_weighted(const double* x, int rows, int k0, int cols, long 
 cudaError_t oz_pair_weights(const double* Dk, int K, const int* kinds, const double* params, double eta, int nb,
                             double* f, int* h, cudaStream_t s);
 // flags[b][t] = 1 for the lower 64 x 64 tiles t of entry b that hold an element whose sum of |terms| is below an eighth of
-// its two scales' product (others are left as they are); operands of `cols` columns, oz_cover_tiles(n) tiles an entry.
+// its two scales' product, or of a row with a NaN or an infinity (others are left as they are); batched operands of n rows
+// and `cols` columns, oz_cover_tiles(n) tiles an entry.
 int oz_cover_tiles(int n);
-cudaError_t oz_cover(const __nv_bfloat16* digA, const __nv_bfloat16* digB, int n, int cols, int nb, int* flags,
-                     cudaStream_t s);
+cudaError_t oz_cover(const OzOperand& A, const OzOperand& B, int n, int cols, int nb, int* flags, cudaStream_t s);
 
 // Row scales and digits of x [rows][cols] (row length ld) in one launch.
 cudaError_t oz_row_digits(const double* x, int rows, int cols, long ld, double* sc, __nv_bfloat16* dig,

@@ -65,3 +65,24 @@ def test_dense_residue_at_a_resonance(gwlib, eta):
         w = b @ np.linalg.solve(np.eye(n_aux) - pi, b.astype(complex)) - b @ b
         tol = 4 * n_aux * 2.0 ** -53 * cond * (b @ b)
         assert abs(out["w_re"][j] - w.real) < tol and abs(out["w_im"][j] - w.imag) < tol, (j, out["w_re"][j], w, tol)
+
+
+@pytest.mark.parametrize("ws", [0, 1])
+def test_polarizability_of_non_finite_rows(gwlib, ws):
+    from paper_2107_10423_gb300 import gw
+    s = _system(200, 13, 79)
+    B, Bn = s.b_ia(), s.b_nm()
+    B[3, 17], B[70, 1000], B[71, 1000], B[150, 5] = np.inf, -np.inf, np.inf, np.nan
+    with gw.Plan(s.eps, s.n_occ, B, Bn, s.targets, workspace_mb=ws) as p:
+        Pi = p.polarizability(np.array([0.0, 1.3]))
+    D = O.pair_energies(s.eps, s.n_occ)
+    for g, x in enumerate((0.0, 1.3)):
+        w = -4.0 * D / (D * D + x * x)
+        # every product of an infinite element is infinite (no zeros here), its sign that of the other factors
+        with np.errstate(invalid="ignore"):
+            want = np.array([[np.sum(B[p] * w * B[q]) for q in range(200)] for p in range(200)])
+        assert np.array_equal(np.isnan(Pi[g]), np.isnan(want))
+        inf = np.isinf(want)
+        assert np.array_equal(Pi[g][inf], want[inf])
+        ok = np.isfinite(want)
+        assert ok.sum() == 196 ** 2 and np.allclose(Pi[g][ok], want[ok], rtol=0, atol=1e-12)
